@@ -66,6 +66,7 @@ Params params_of(const hh_ctx *ctx)
     p.eta_s = ctx->cfg.eta_s;
     p.dt_min = ctx->cfg.dt_min;
     p.dt_max = ctx->cfg.dt_max;
+    p.unit = 1.0;
     return p;
 }
 

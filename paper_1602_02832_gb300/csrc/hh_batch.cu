@@ -755,8 +755,8 @@ __global__ void __launch_bounds__(kBlock, 1) k_batch(BatchDev B)
                 }
                 unsigned long long n_int = 0;
                 const bool done = force_item<Rec, TJ, false>(sd.st, (const Rec *)sd.rec, sd.L,
-                                                             (typename Traits<Rec>::Eps)sd.prm.eps2, it, sm, n_int,
-                                                             gt, bar);
+                                                             (typename Traits<Rec>::Eps)sd.prm.eps2, sd.prm.unit, it,
+                                                             sm, n_int, gt, bar);
                 if (gt == 0 && n_int) atomicAdd(&sd.ds->interactions, n_int);
                 if (done) {
                     group_sync(bar);  // the tile's new forces are visible to the group
@@ -1076,6 +1076,7 @@ extern "C" int hh_batch_run(hh_batch *b, int32_t n, hh_ctx *const *ctxs, const d
         d.prm.eta_s = c->cfg.eta_s;
         d.prm.dt_min = c->cfg.dt_min;
         d.prm.dt_max = c->cfg.dt_max;
+        d.prm.unit = 1.0;
         d.t_end = t_end[s];
         jb[s + 1] = jb[s] + c->nj;
         pb[s + 1] = pb[s] + c->n;

@@ -17,6 +17,8 @@
 #include <type_traits>
 #include <cuda_runtime.h>
 
+#include "hh_pair64.cuh"
+
 namespace hh {
 
 constexpr int kThreads = 128;  // threads per force CTA (4 warps)
@@ -59,7 +61,8 @@ struct StepCtl {
 };
 
 // ---------------------------------------------------------------- records
-// Predicted j record, plain form: (x, y, z, m), (vx, vy, vz, 0) in FP64.
+// Predicted j record, plain form: (x, y, z, m), (vx, vy, vz, -) in FP64; the
+// last word holds the mass's bits for the integer pair term (mass_bits).
 struct __align__(32) RecF64 {
     double4 xm;
     double4 v;
@@ -135,6 +138,7 @@ struct Lists {
 
 struct Params {
     double eps2, eta, eta_s, dt_min, dt_max;
+    double unit;  // 1.0, as a value the compiler cannot see (pair_diff)
 };
 
 __device__ __forceinline__ double bits_to_time(unsigned long long b) { return __longlong_as_double((long long)b); }
@@ -266,7 +270,7 @@ __device__ __forceinline__ void store_rec<RecF64>(RecF64 *out, int64_t e, const 
 {
     RecF64 r;
     r.xm = make_double4(xp[0], xp[1], xp[2], m);
-    r.v = make_double4(vp[0], vp[1], vp[2], 0.0);
+    r.v = make_double4(vp[0], vp[1], vp[2], __longlong_as_double((long long)mass_bits(m)));
     out[e] = r;
 }
 
@@ -475,6 +479,21 @@ __device__ __forceinline__ void interact(const IF64 &I, const RecF64 &J, bool se
     A.jz = fma(mr3, fma(-al, dz, wz), A.jz);
 }
 
+// Differences as fused multiply-adds with 1: an FP64 add issues in 76 cycles
+// here, a fused multiply-add in 64.
+__device__ __forceinline__ void interact_int(const IF64 &I, const RecF64 &J, bool self, const Soft64 &eps, double unit,
+                                             int smin, AccI64 &A)
+{
+    double d[3], w[3];
+    d[0] = fma(J.xm.x, unit, -I.x);
+    d[1] = fma(J.xm.y, unit, -I.y);
+    d[2] = fma(J.xm.z, unit, -I.z);
+    w[0] = fma(J.v.x, unit, -I.vx);
+    w[1] = fma(J.v.y, unit, -I.vy);
+    w[2] = fma(J.v.z, unit, -I.vz);
+    pair_add(d, w, J.xm.w, (uint64_t)__double_as_longlong(J.v.w), self, eps, smin, A);
+}
+
 // Mixed: chunk partials in FP32, folded into (hi, lo) pairs after each
 // staged chunk with Knuth's TwoSum, so that the running sum is carried to
 // about 2^-48 relative while the inner loop stays plain FP32.
@@ -644,6 +663,15 @@ __device__ __forceinline__ void to_red(const AccF64 &A, RedF64 &r)
 {
     r.v[0] = A.ax; r.v[1] = A.ay; r.v[2] = A.az; r.v[3] = A.jx; r.v[4] = A.jy; r.v[5] = A.jz; r.v[6] = A.p;
 }
+__device__ __forceinline__ void to_red(const AccI64 &A, RedF64 &r)
+{
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        r.v[k] = sum_get(A.a.u[k], A.a.o[k], A.a.e);
+        r.v[3 + k] = sum_get(A.j.u[k], A.j.o[k], A.j.e);
+    }
+    r.v[6] = sum_get(A.p.u[0], A.p.o[0], A.p.e);
+}
 __device__ __forceinline__ void to_red(const AccMix &A, RedMix &r)
 {
     r.v[0] = A.Ax; r.v[1] = A.Ay; r.v[2] = A.Az; r.v[3] = A.Jx; r.v[4] = A.Jy; r.v[5] = A.Jz; r.v[6] = A.P;
@@ -678,7 +706,7 @@ struct Traits;
 template <>
 struct Traits<RecF64> {
     using I = IF64;
-    using Acc = AccF64;
+    using Acc = AccI64;
     using Red = RedF64;
     using Eps = double;
 };
@@ -690,7 +718,6 @@ struct Traits<RecMix> {
     using Eps = float;
 };
 
-__device__ __forceinline__ void fold_chunk(AccF64 &) {}
 __device__ __forceinline__ void fold_chunk(AccMix &A) { A.fold(); }
 
 // ------------------------------------------------------------ list force
@@ -777,12 +804,42 @@ __device__ __forceinline__ void group_sync(int bar_id)
     else asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "r"(kThreads) : "memory");
 }
 
+// The same, returning whether `pred` holds in any thread of the group.
+__device__ __forceinline__ bool group_any(int bar_id, bool pred)
+{
+    if (bar_id == 0) return __syncthreads_or(pred) != 0;
+    int r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.s32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, %2, %3, p;\n\t"
+        "selp.s32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"((int)pred), "r"(bar_id), "r"(kThreads)
+        : "memory");
+    return r != 0;
+}
+
+// A thread's sums over its entries of a list part in FP64 arithmetic (jslice,
+// jslice + S, ... of each chunk of tj entries), straight from the records: the
+// parts that the integer pair term does not take.
+static __device__ __noinline__ void part_sums_f64(const RecF64 *__restrict__ rec, const int32_t *idx, int64_t len, int tj,
+                                                  int jslice, int S, int64_t pi, const IF64 &I, double eps2, RedF64 &out)
+{
+    AccF64 A;
+    A.zero();
+    for (int64_t c = 0; c < len; c += tj)
+        for (int64_t e = c + jslice; e < min(len, c + (int64_t)tj); e += S) {
+            const int32_t j = idx[e];
+            interact(I, rec[j], (int64_t)j == pi, eps2, A);
+        }
+    to_red(A, out);
+}
+
 // item = (tile, part | sim << 16, active mask, parts of the tile); tid is
 // the thread's index in its 128-thread group.  Returns true (in every thread
 // of the group) for the item that wrote the tile's final forces.
 template <typename Rec, int TJ, bool kMapI>
 __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict__ rec, const Lists &L,
-                                           typename Traits<Rec>::Eps eps2, const WorkItem &it,
+                                           typename Traits<Rec>::Eps eps2, double unit, const WorkItem &it,
                                            ForceSmem<Rec, TJ> &sm, unsigned long long &n_int, const int tid,
                                            const int bar_id)
 {
@@ -865,6 +922,15 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
         }
         load_idx(kStages - 1);
     }
+    constexpr bool kPlain = std::is_same<Rec, RecF64>::value;
+    // plain form: softening in integers, room in the sums for a thread's terms
+    Soft64 soft{};
+    int smin = 0;
+    if constexpr (kPlain) {
+        soft = soft_of(eps2);
+        smin = max(2, 32 - __clz((int)(len / S + 1 + (int64_t)n_chunks)));
+        A.bad = !soft.ok;
+    }
     for (int c = 0; c < n_chunks; c++) {
         const int b = c % kStages;
         const int nc = (len - (int64_t)c * TJ < (int64_t)TJ) ? (int)(len - (int64_t)c * TJ) : TJ;
@@ -872,16 +938,21 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
         load_idx(c + kStages);
         cp_async_wait<kStages - 1>();
         group_sync(bar_id);
-        // FP32 partials are folded into the compensated sums every
-        // kFold terms per thread (short plain-FP32 runs keep the
-        // partial-sum rounding below the per-term rounding).
-        for (int e = idle ? nc : jslice; e < nc;) {
-            const int e_end = min(nc, e + kFold * S);
-            for (; e < e_end; e += S) {
-                const int32_t j = sm.idx[b][e];
-                interact(Iv, sm.rec[b][e], (int64_t)j == pi, eps2, A);
+        if constexpr (kPlain) {
+            for (int e = idle ? nc : jslice; e < nc; e += S)
+                interact_int(Iv, sm.rec[b][e], (int64_t)sm.idx[b][e] == pi, soft, unit, smin, A);
+        } else {
+            // FP32 partials are folded into the compensated sums every
+            // kFold terms per thread (short plain-FP32 runs keep the
+            // partial-sum rounding below the per-term rounding).
+            for (int e = idle ? nc : jslice; e < nc;) {
+                const int e_end = min(nc, e + kFold * S);
+                for (; e < e_end; e += S) {
+                    const int32_t j = sm.idx[b][e];
+                    interact(Iv, sm.rec[b][e], (int64_t)j == pi, eps2, A);
+                }
+                fold_chunk(A);
             }
-            fold_chunk(A);
         }
         group_sync(bar_id);  // buffer b is refilled by the next step's issue
     }
@@ -895,8 +966,8 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
     // two outputs (7 n_a <= 224).  Mixed form (FP32 pair adds are cheap, the
     // extra barriers are not): a butterfly over the lanes when n_a is a power
     // of two, else a tree towards slice 0, then a sum over the four warps.
-    constexpr bool kTreeTail = std::is_same<Rec, RecF64>::value;
-    if (!kTreeTail) {
+    constexpr bool kTreeTail = kPlain;
+    if constexpr (!kTreeTail) {
         if ((I & (I - 1)) == 0) {
             for (int off = I; off < 32; off <<= 1) acc_shfl_add(A, off);
         } else {
@@ -909,7 +980,16 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
         to_red(A, rr);
         sm.red[warp][lane] = rr;
     }
-    group_sync(bar_id);
+    if constexpr (kPlain) {
+        // a term that the integers do not take (a number beyond their range,
+        // a mass that is not positive): the whole part again in FP64
+        if (group_any(bar_id, A.bad)) {
+            if (!idle) part_sums_f64(rec, L.idx + lb, len, TJ, jslice, S, pi, Iv, eps2, sm.red[warp][lane]);
+            group_sync(bar_id);
+        }
+    } else {
+        group_sync(bar_id);
+    }
     using E = typename std::remove_reference<decltype(sm.red[0][0].v[0])>::type;
     const int n_out = 7 * n_a;
     const int n_sl = kTreeTail ? (kThreads / 32) * K : kThreads / 32;  // terms per output
@@ -1045,7 +1125,7 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
 }
 
 template <typename Rec, int TJ, bool kMapI = false>
-__global__ void __launch_bounds__(kThreads, 6) k_force(State s, const Rec *__restrict__ rec, Lists L, DevScalars *ds,
+__global__ void __launch_bounds__(kThreads, std::is_same<Rec, RecF64>::value ? 4 : 6) k_force(State s, const Rec *__restrict__ rec, Lists L, DevScalars *ds,
                                                     StepCtl c, Params prm)
 {
     double tnow;
@@ -1059,7 +1139,7 @@ __global__ void __launch_bounds__(kThreads, 6) k_force(State s, const Rec *__res
         __syncthreads();
         const int item = sm.item;
         if (item >= n_items) break;
-        force_item<Rec, TJ, kMapI>(s, rec, L, eps2, L.items[item], sm, n_int, threadIdx.x, 0);
+        force_item<Rec, TJ, kMapI>(s, rec, L, eps2, prm.unit, L.items[item], sm, n_int, threadIdx.x, 0);
         // the next iteration's first barrier protects sm reuse
     }
     if (threadIdx.x == 0 && n_int) atomicAdd(&ds->interactions, n_int);

@@ -220,6 +220,7 @@ extern "C" int hh_force_static(int device, int precision, double eps2, int64_t n
     Params prm;
     std::memset(&prm, 0, sizeof(prm));
     prm.eps2 = eps2;
+    prm.unit = 1.0;
     StepCtl c{1, 0, 1, 0, 0.0};
     if (precision == HH_MIXED)
         k_static_pack<RecMix><<<st.elem_grid, 256, 0, s>>>(reinterpret_cast<RecMix *>(base + kOffRec), xj, vj, mj, n_j);
