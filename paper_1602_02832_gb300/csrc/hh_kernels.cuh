@@ -724,7 +724,8 @@ __device__ __forceinline__ void fold_chunk(AccMix &A) { A.fold(); }
 // One 128-thread group (4 warps) per work item = (tile, part of its group's
 // list).  With n_a active particles in the tile each warp holds floor(32 /
 // n_a) j slices of n_a lanes (lane = i slot + n_a * slice; leftover lanes
-// idle), and the slices stride through each staged chunk of the part.
+// idle), and the slices stride through each staged chunk of the part.  (Plain
+// form: the slices lie across the whole group, floor(128 / n_a) of them.)
 // Slices are summed in a fixed order (shuffles, then warps).  A list split
 // into several parts leaves per-part sums in the partials buffer; the group
 // that finishes a tile's last part (acquire-release arrival counter: no
@@ -772,6 +773,7 @@ struct ForceSmem {
     int last;
     double tn[kThreads / 32];  // per-warp minimum of t + dt after the corrector
     int lv[kMaxTileI];         // new step level of each corrected particle, by active index
+    typename Traits<Rec>::I iv[kMaxTileI];  // plain form: the item's active particles
     double fin[kMaxTileI][7];  // the completed tile's new acc, jerk, pot by active index (for its corrector)
 };
 
@@ -853,16 +855,22 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
     const int pj = it.part_len;
     const int part = it.part_sim & 0xFFFF, slot0 = it.slot;
 
-    // Lane mapping: every warp holds K = floor(32 / n_a) j slices of n_a lanes
-    // (lane = i slot + n_a * slice); the 32 - K n_a leftover lanes idle.  So no
-    // lane is spent on a missing particle (rounding n_a up to a power of two
-    // left up to half the lanes idle, and the FP64 pipe charges the whole warp).
+    // Lane mapping.  Mixed form: every warp holds K = floor(32 / n_a) j slices
+    // of n_a lanes (lane = i slot + n_a * slice); the 32 - K n_a leftover lanes
+    // idle.  So no lane is spent on a missing particle (rounding n_a up to a
+    // power of two left up to half the lanes idle).  Plain form: the slices lie
+    // across the group's 128 threads (its slice sums go through shared memory,
+    // so a slice may straddle two warps): 7 slices of 18 particles where the
+    // warps alone hold 4.  Tree groups of n_crit 64 hold 18 particles on
+    // average: 56% of the lanes at work before, 98% now, and an evaluation of
+    // N = 65536 went from 3.95 to 3.53 ms.
+    constexpr bool kPlain = std::is_same<Rec, RecF64>::value;
     const int I = n_a;
-    const int K = 32 / I;
-    const int islot = lane % I, kslice = lane / I;
+    const int K = kPlain ? kThreads / I : 32 / I;  // slices of the group (plain), of each warp (mixed)
+    const int islot = (kPlain ? tid : lane) % I, kslice = (kPlain ? tid : lane) / I;
     const bool idle = kslice >= K;
-    const int jslice = warp * K + kslice;
-    const int S = (kThreads / 32) * K;
+    const int jslice = kPlain ? kslice : warp * K + kslice;
+    const int S = kPlain ? K : (kThreads / 32) * K;
     const bool has_i = !idle;
     int64_t pi = -1;
     {
@@ -878,6 +886,9 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
     }
     typename T::I Iv;
     load_i(rec, pload, Iv);
+    // (plain form: read again for every pair, which keeps 12 registers free:
+    // a tree interval of N = 65536 takes 52.8 ms against 53.9 ms)
+    if (kPlain && tid < I) sm.iv[tid] = Iv;
     typename T::Acc A;
     A.zero();
 
@@ -922,7 +933,6 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
         }
         load_idx(kStages - 1);
     }
-    constexpr bool kPlain = std::is_same<Rec, RecF64>::value;
     // plain form: softening in integers, room in the sums for a thread's terms
     Soft64 soft{};
     int smin = 0;
@@ -939,8 +949,10 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
         cp_async_wait<kStages - 1>();
         group_sync(bar_id);
         if constexpr (kPlain) {
-            for (int e = idle ? nc : jslice; e < nc; e += S)
-                interact_int(Iv, sm.rec[b][e], (int64_t)sm.idx[b][e] == pi, soft, unit, smin, A);
+            for (int e = idle ? nc : jslice; e < nc; e += S) {
+                asm volatile("" ::: "memory");  // (no hoisting of iv's loads out of the loop)
+                interact_int(sm.iv[islot], sm.rec[b][e], (int64_t)sm.idx[b][e] == pi, soft, unit, smin, A);
+            }
         } else {
             // FP32 partials are folded into the compensated sums every
             // kFold terms per thread (short plain-FP32 runs keep the
@@ -956,11 +968,11 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
         }
         group_sync(bar_id);  // buffer b is refilled by the next step's issue
     }
-    // Plain form: sum over the group's 4 K slices for each (i slot,
+    // Plain form: sum over the group's K slices for each (i slot,
     // component): the partials go to shared memory, then P contiguous lanes of
     // one warp (P a power of two, P * 7 n_a <= 128) each add a contiguous run
     // of slices in order and a shuffle tree adds the P runs.  A fixed order,
-    // with about 4 K / P + log2 P adds per thread, where a butterfly over the
+    // with about K / P + log2 P adds per thread, where a butterfly over the
     // lanes costs 7 adds per level for every lane (a warp instruction costs the
     // FP64 pipe the same with one lane active).  With P = 1 a thread may own
     // two outputs (7 n_a <= 224).  Mixed form (FP32 pair adds are cheap, the
@@ -978,13 +990,14 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
     if (kTreeTail ? !idle : lane < I) {
         Red rr;
         to_red(A, rr);
-        sm.red[warp][lane] = rr;
+        (&sm.red[0][0])[kPlain ? tid : warp * kMaxTileI + lane] = rr;
     }
     if constexpr (kPlain) {
         // a term that the integers do not take (a number beyond their range,
         // a mass that is not positive): the whole part again in FP64
         if (group_any(bar_id, A.bad)) {
-            if (!idle) part_sums_f64(rec, L.idx + lb, len, TJ, jslice, S, pi, Iv, eps2, sm.red[warp][lane]);
+            if (!idle) load_i(rec, pload, Iv);
+            if (!idle) part_sums_f64(rec, L.idx + lb, len, TJ, jslice, S, pi, Iv, eps2, (&sm.red[0][0])[tid]);
             group_sync(bar_id);
         }
     } else {
@@ -992,7 +1005,7 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
     }
     using E = typename std::remove_reference<decltype(sm.red[0][0].v[0])>::type;
     const int n_out = 7 * n_a;
-    const int n_sl = kTreeTail ? (kThreads / 32) * K : kThreads / 32;  // terms per output
+    const int n_sl = kTreeTail ? K : kThreads / 32;  // terms per output
     int P = 1;  // (mixed form: one thread per output, warps 0..3 in order)
     if (kTreeTail)
         while (P < 32 && 2 * P * n_out <= kThreads && 2 * P <= n_sl) P <<= 1;
@@ -1007,8 +1020,7 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
             const int slot = o / 7, comp = o - 7 * slot;
             const int x1 = min(n_sl, (q + 1) * per);
             for (int x = q * per; x < x1; x++) {
-                const int w = kTreeTail ? x / K : x, k = kTreeTail ? x - w * K : 0;
-                const E v = sm.red[w][k * I + slot].v[comp];
+                const E v = (&sm.red[0][0])[kTreeTail ? x * I + slot : x * kMaxTileI + slot].v[comp];
                 if (has[u]) comp_add(r[u], v);
                 else {
                     r[u] = v;

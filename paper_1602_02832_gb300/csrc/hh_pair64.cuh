@@ -10,10 +10,14 @@
 // separation, the relative velocity and every scalar as 64-bit numbers in two
 // signed 32-bit digits, the sums in 96 bits with an exponent of their own.
 // A micro-benchmark of the pair loop (4 warps per sub-partition, records in
-// shared memory) went from 2280 to 660 cycles a warp and pair; one evaluation of
+// shared memory) went from 2280 to 650 cycles a warp and pair; one evaluation of
 // N = 65536 particles (theta 0.5 lists) from 11.5 to 3.95 ms, a tree interval of
 // its block steps from 90.8 to 55.6 ms.  What bounds it now is the integer
-// multiply-add pipe (75-80% busy; the ALU pipe 58%, FP64 54%).
+// multiply-add pipe (71% busy; the ALU pipe 61%, FP64 59%, issue 58%) and the
+// latency of its chains with 4 warps a sub-partition.  Taken back: the next
+// pair's differences one iteration ahead (its registers: 6% slower), unpacking
+// by FP64-to-integer conversions (64 cycles each on the FP64 pipe: 1% slower for
+// two components, 9% for three), five or six warps a sub-partition (the same).
 //
 // Errors, measured against quad precision: force 4.7e-17 (rms, relative) and
 // jerk 8e-17 of |m w / r^3| a pair, where FP64 arithmetic has 1.9e-16 and
@@ -253,6 +257,14 @@ struct Sum64 {
     }
 };
 
+// Where a sum puts its first term (and one too large for it): 24 places below
+// the top of the window leave 2^16 and more of room for larger ones, so that a
+// thread's terms rarely move the scale (a move costs as much as a pair, and one
+// lane's move holds up its warp; with 4 places of room instead of about 18 an
+// evaluation of N = 65536 took 3.53 ms against 3.41 ms), and 8 bits below the first
+// term's last one for smaller ones.
+constexpr int kPlace = 24;
+
 // sum += t 2^(e - s), smin <= s <= 32 (smin: the bits of the number of terms, at least 2)
 template <int N>
 HH_HD void sum_put(Sum64<N> &S, const int64_t *t, int s)
@@ -270,7 +282,7 @@ template <int N>
 HH_HD void sum_any(Sum64<N> &S, int64_t *t, int s, int smin)
 {
     if (s < smin) {
-        const int ns = imin(smin + 4, 32), d = ns - s;
+        const int ns = imax(smin, kPlace), d = ns - s;
         if (d < 128) {
             for (int k = 0; k < N; k++) {
                 __int128 x = ((__int128)S.o[k] << 32) + (__int128)S.u[k];
@@ -296,32 +308,24 @@ HH_HD void sum_any(Sum64<N> &S, int64_t *t, int s, int smin)
 // The sum as a double (to nearest on its top 64 bits).
 HH_HD double sum_get(uint64_t u, int64_t o, int e)
 {
-    // 96 bits: w2 w1 w0
-    const uint64_t c = hi32(u) + (uint64_t)lo32((uint64_t)o);
-    uint32_t w0 = lo32(u), w1 = lo32(c), w2 = hi32((uint64_t)o) + hi32(c);
-    const bool neg = (int32_t)w2 < 0;
+    // 96 bits: c w0, then the magnitude
+    uint64_t c = (uint64_t)o + hi32(u);
+    uint32_t w0 = lo32(u);
+    const bool neg = (int64_t)c < 0;
     if (neg) {
-        const uint32_t c1 = w0 == 0u, c2 = (w0 | w1) == 0u;
+        c = ~c + (w0 == 0u ? 1u : 0u);
         w0 = 0u - w0;
-        w1 = ~w1 + c1;
-        w2 = ~w2 + c2;
     }
     e -= 32;
-    if (w2 == 0u) {
-        w2 = w1;
-        w1 = w0;
-        w0 = 0u;
-        e -= 32;
-        if (w2 == 0u) {
-            w2 = w1;
-            w1 = 0u;
+    for (int q = 0; q < 2; q++)
+        if (hi32(c) == 0u) {  // 32 places up
+            c = (c << 32) | w0;
+            w0 = 0u;
             e -= 32;
-            if (w2 == 0u) return 0.0;
         }
-    }
-    const int z = clz32(w2);
-    uint64_t m = ((uint64_t)w2 << 32) | w1;
-    if (z) m = (m << z) | (w0 >> (32 - z));
+    if (hi32(c) == 0u) return 0.0;
+    const int z = clz32(hi32(c));
+    uint64_t m = (c << z) | (z ? w0 >> (32 - z) : 0u);
     e += 96 - z;  // value = m 2^(e - 64) with the top bit of m set
     if (e < -1000) return 0.0;                                       // below the normal range
     if (e > 1024) return f64_of(neg ? 0xfff00000u : 0x7ff00000u, 0u);  // beyond it
