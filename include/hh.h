@@ -216,11 +216,18 @@ int hh_init_forces(hh_ctx *ctx, double t);
 int hh_step(hh_ctx *ctx, double *t_next_out, int32_t *n_act_out);
 
 /* Block steps on the device until the next block time would exceed t_end,
- * without host round trips per step (CUDA graph of unrolled block steps,
- * replayed; each kernel becomes a no-op once done).  *n_steps_out (may be
- * NULL) receives the number of block steps taken.  Errors: HH_ESTATE
- * without lists and steps; HH_EINVAL for a NaN t_end or an error found on
- * the device; HH_ETIMEOUT if the replays stop making progress; HH_ECUDA. */
+ * without host round trips per step: one persistent cooperative launch per
+ * 256 steps (the kernel of hh_batch_run, with the same results as the graph
+ * loop: list parts of tile_j, or of work_item when work_split is 0, every
+ * entry predicted at every step).  Contexts that advance at the same time
+ * from several threads share the SMs.  With hh_force_timing on, and for a
+ * state that breaks the block rule (see hh_batch_run), a CUDA graph of
+ * unrolled block steps is replayed instead (each kernel becomes a no-op once
+ * done).  The first call allocates the launch's buffers (some 40 KB, counted
+ * in hh_ctx_device_bytes).  *n_steps_out (may be NULL) receives the number of
+ * block steps taken.  Errors: HH_ESTATE without lists and steps; HH_EINVAL
+ * for a NaN t_end or an error found on the device; HH_ETIMEOUT for a grid
+ * barrier that gave up, or if the replays stop making progress; HH_ECUDA. */
 int hh_advance(hh_ctx *ctx, double t_end, int64_t *n_steps_out);
 
 /* Step 1 done by the library: copies the (synchronised) particle state to

@@ -38,6 +38,14 @@ int hh_finish_device_rebuild(hh_ctx *ctx, int64_t total_parts, int64_t lmax, boo
 // (when there are two or more), the others one by one.
 constexpr int64_t kBatchRebuildMaxN = 32768;
 int hh_rebuild_many(hh_ctx *const *ctxs, const double *ts, int k, int *rcs, RbScratch *r);
+// hh_advance's block steps in the persistent loop of the batched kernel, one
+// context alone (hh_batch.cu).  Returns HH_OK, an error, or kLoopNotTaken when
+// the loop cannot run here (no memory or no cooperative launch) or the state
+// breaks the block rule (nothing but the work counters may have changed then).
+constexpr int kLoopNotTaken = 1;
+struct LoopBuf;
+int hh_loop_run(hh_ctx *ctx, double t_end);
+void hh_loop_free(LoopBuf *b);
 // Block steps of the batched loop with at most this many due particles use
 // list parts of tile_j_small (when set).
 constexpr int kSmallDue = 16;
@@ -87,7 +95,8 @@ struct hh_ctx {
     std::vector<int32_t> h_group_of;
     // grid shapes
     int n_sm = 0, force_grid = 0, elem_grid = 0;
-    // loop graph
+    LoopBuf *loop = nullptr;   // buffers of the persistent loop (first hh_advance)
+    // loop graph (with per-launch timing, or for states that break the block rule)
     cudaGraphExec_t graph = nullptr;
     int graph_timed = -1;
     std::vector<cudaEvent_t> ev;  // 2 per unrolled step when timed
