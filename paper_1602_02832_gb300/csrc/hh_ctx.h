@@ -86,6 +86,10 @@ struct hh_ctx {
     hh::DevScalars *h_ds = nullptr;
     double *h_buf = nullptr;   // [14 * cap_j]
     int32_t *h_ibuf = nullptr; // [cap_n]
+    int32_t *h_flag = nullptr; // verdict of an explicit evaluation's checks
+    double *h_out = nullptr;   // results of small evaluations (first use)
+    std::vector<uint32_t> seen;  // last evaluation that listed each particle (repeats)
+    uint32_t seen_stamp = 0;
     double *h_jbuf = nullptr;  // [14 * cap_j] staging of the rebuilt j entries
     hh_tree *tree = nullptr;   // host tree reused by hh_rebuild
     GTreeBuf *gtree = nullptr; // device tree builder (rebuild_device)
@@ -105,6 +109,7 @@ struct hh_ctx {
     double force_ms = 0.0;
     int64_t force_launches = 0;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
+    cudaEvent_t begun = nullptr;  // behind the checks of an explicit evaluation
     // state flags
     bool have_j = false, have_lists = false, have_dt = false, predicted = false, have_forces = false;
     int64_t rebuilds = 0;

@@ -33,10 +33,10 @@ struct DevScalars {
     int32_t err;                 // device-detected error (HH_* code), 0 = none
     uint32_t work;               // force work-queue head
     uint32_t n_items;            // work items of this step
+    uint32_t slot_ctr;           // partial-sum slots handed out this step
     int32_t part_len;            // shortest list part (a multiple of the staging chunk)
     int32_t work_item;           // target interactions per work item (0: every part is part_len long)
     int32_t work_split;          // > 0: work_item applies only to batched steps with this many active particles
-    uint32_t slot_ctr;           // partial-sum slots handed out this step
     uint32_t slot_par[2];        // the same for the batched loop, by step parity
     int32_t n_act_last;          // active particles of the last corrected step
     int64_t n;                   // particles
@@ -238,6 +238,7 @@ __device__ __forceinline__ void select_tiles(const State &s, const Lists &L, Dev
 static __global__ void k_select(State s, Lists L, DevScalars *ds, StepCtl c)
 {
     double tnow;
+    if (c.mode == 1 && *(volatile const int32_t *)&ds->err) return;  // (k_mark_begin found a bad index)
     if (!step_time(ds, c, &tnow)) return;
     select_tiles(s, L, ds, c, tnow);
 }
@@ -1496,22 +1497,50 @@ static __global__ void k_refresh_base(State s, int64_t first, int64_t n)
         refresh_base(s, first + q);
 }
 
-static __global__ void k_set_marks(int32_t *mark, const int32_t *idx, int32_t n, int32_t value)
+// Start of an explicit evaluation: marks the listed particles and empties the
+// work queue.  An index outside [0, n_part) sets ds->err; *verdict (host
+// memory) is then set, as it is for an error that was pending.
+static __global__ void k_mark_begin(int32_t *mark, const int32_t *idx, int32_t n, int64_t n_part, DevScalars *ds,
+                                    volatile int32_t *verdict)
 {
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) mark[idx[q]] = value;
+    const int q0 = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q0 == 0) {
+        if (*(volatile int32_t *)&ds->err) *verdict = 1;
+        ds->work = 0u;
+        ds->n_items = 0u;
+        ds->slot_ctr = 0u;
+    }
+    for (int q = q0; q < n; q += gridDim.x * blockDim.x) {
+        const int32_t p = idx[q];
+        if (p < 0 || p >= n_part) {
+            atomicExch(&ds->err, -1);
+            *verdict = 1;
+        } else {
+            mark[p] = 1;
+        }
+    }
 }
 
-// out[3][n_act] (SoA) <- acc1 etc. at i_idx
-static __global__ void k_gather_out(State s, const int32_t *idx, int32_t n_act, double *acc, double *jerk, double *pot)
+// End of it: out[3][n_act] (SoA) <- acc1 etc. at idx (with out set), marks
+// cleared; *verdict (host memory, may be NULL) <- ds->err.
+static __global__ void k_mark_end(State s, const int32_t *idx, int32_t n_act, int64_t n_part, bool out, double *acc,
+                                  double *jerk, double *pot, const DevScalars *ds, volatile int32_t *verdict)
 {
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n_act; q += gridDim.x * blockDim.x) {
+    const int32_t err = *(volatile const int32_t *)&ds->err;
+    const int q0 = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q0 == 0 && verdict) *verdict = err;
+    for (int q = q0; q < n_act; q += gridDim.x * blockDim.x) {
         const int64_t p = idx[q];
+        if (p < 0 || p >= n_part) continue;
+        if (out && !err) {
 #pragma unroll
-        for (int d = 0; d < 3; d++) {
-            if (acc) acc[(int64_t)d * n_act + q] = s.acc1[d * s.cap_n + p];
-            if (jerk) jerk[(int64_t)d * n_act + q] = s.jerk1[d * s.cap_n + p];
+            for (int d = 0; d < 3; d++) {
+                if (acc) acc[(int64_t)d * n_act + q] = s.acc1[d * s.cap_n + p];
+                if (jerk) jerk[(int64_t)d * n_act + q] = s.jerk1[d * s.cap_n + p];
+            }
+            if (pot) pot[q] = s.pot1[p];
         }
-        if (pot) pot[q] = s.pot1[p];
+        s.mark[p] = 0;
     }
 }
 
@@ -1526,12 +1555,6 @@ static __global__ void k_check_j(const State s, int64_t first, int64_t n, DevSca
                  isfinite(s.a[d * s.cap_j + e]) && isfinite(s.jk[d * s.cap_j + e]);
         if (!ok) atomicExch(&ds->err, -1);
     }
-}
-
-static __global__ void k_check_idx(const int32_t *idx, int32_t n, int64_t n_part, DevScalars *ds)
-{
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x)
-        if (idx[q] < 0 || idx[q] >= n_part) atomicExch(&ds->err, -1);
 }
 
 }  // namespace hh
