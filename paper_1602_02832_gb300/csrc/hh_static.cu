@@ -19,14 +19,24 @@ namespace {
 constexpr int64_t kStaticMaxJ = 131072;    // j entries
 constexpr int64_t kStaticMaxAct = 65536;   // active particles (and tiles)
 constexpr int64_t kStaticMaxParts = 8192;  // (tile, list part) work items
-constexpr int32_t kStaticPartLen = 2048;   // list entries per part
+constexpr int32_t kStaticPartLen = 2048;   // list entries per part (the longest)
+// The plain form takes shorter parts while the work items stay within their
+// number: at level v > 0 a tile with n_a particles takes parts of about
+// 2048 << (4 - v) interactions, at least one chunk (256 entries); the highest
+// level that fits is used.  3001 of 12007 particles in tiles of one 2048-entry
+// part each left most of the chip waiting for the few tiles with 16 and more
+// particles: 375 us a call, 224 us with these parts (247 us with 256-entry parts for
+// every tile: eight iterations a part for four particles do not cover its start
+// and end).  The mixed form keeps 2048: its FP32 partial sums follow the parts.
+constexpr int kStaticLevels = 5;
 constexpr int kStaticTj = 256;             // staged chunk (both precisions)
 constexpr int kMaxDevices = 64;
 
 // byte layout of the scratch array (each region 256-byte aligned)
 constexpr size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 constexpr size_t kOffDs = 0;
-constexpr size_t kOffCnt = kOffDs + align256(sizeof(DevScalars));
+constexpr size_t kOffHdr = kOffDs + align256(sizeof(DevScalars));
+constexpr size_t kOffCnt = kOffHdr + align256(sizeof(uint32_t) * kStaticLevels);
 constexpr size_t kOffTiles = kOffCnt + align256(sizeof(int32_t) * kStaticMaxAct);
 constexpr size_t kOffItems = kOffTiles + align256(sizeof(int4) * kStaticMaxAct);
 constexpr size_t kOffParts = kOffItems + align256(sizeof(WorkItem) * kStaticMaxParts);
@@ -72,10 +82,34 @@ void setup_device(int device, DeviceSetup &st)
     st.rc = HH_OK;
 }
 
-template <typename Rec>
-__global__ void k_static_pack(Rec *rec, const double *x, const double *v, const double *m, int64_t n_j)
+__device__ __forceinline__ int32_t static_part_len(int v, int n_a)
 {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n_j; e += (int64_t)gridDim.x * blockDim.x) {
+    if (v == 0) return kStaticPartLen;
+    const int32_t want = (2048 << (kStaticLevels - 1 - v)) / n_a;
+    return min(kStaticPartLen, max(1, (want + kStaticTj - 1) / kStaticTj) * kStaticTj);
+}
+
+__device__ __forceinline__ int64_t parts_of64(int64_t len, int32_t pj) { return len > 0 ? (len + pj - 1) / pj : 1; }
+
+// Caller-supplied device inputs are checked before the force kernel reads
+// them: off[0] = 0 and non-decreasing, list and i indices inside [0, n_j), list
+// ids inside [0, n_groups).  One launch also packs the j records (as before:
+// from arrays whose size the caller states) and clears nothing: the header and
+// tile counters were cleared by the caller.
+template <typename Rec>
+__global__ void k_static_prepare(Rec *rec, const double *x, const double *v, const double *m, int64_t n_j,
+                                 const int64_t *off, int32_t n_groups, const int32_t *i_idx, const int32_t *gid,
+                                 int32_t n_act, DevScalars *ds)
+{
+    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t nth = (int64_t)gridDim.x * blockDim.x;
+    bool bad = tid == 0 && off[0] != 0;
+    for (int64_t g = tid; g < n_groups; g += nth)
+        if (off[g + 1] < off[g]) bad = true;
+    for (int64_t k = tid; k < n_act; k += nth)
+        if (i_idx[k] < 0 || i_idx[k] >= n_j || gid[k] < 0 || gid[k] >= n_groups) bad = true;
+    if (bad) atomicExch(&ds->err, HH_EINVAL);
+    for (int64_t e = tid; e < n_j; e += nth) {
         const double xp[3] = {x[e], x[n_j + e], x[2 * n_j + e]};
         const double vp[3] = {v[e], v[n_j + e], v[2 * n_j + e]};
         store_rec<Rec>(rec, e, xp, vp, m[e]);
@@ -83,82 +117,82 @@ __global__ void k_static_pack(Rec *rec, const double *x, const double *v, const 
 }
 
 // Tiles = runs of consecutive active positions with the same list, cut at
-// every 32nd position; one warp per 32 positions.  Every part of every tile
-// becomes a work item.  Overflowing the fixed item capacity sets ds->err and
-// writes nothing out of bounds.
-__global__ void k_static_tiles(const int32_t *gid, int32_t n_act, int32_t n_groups, const int64_t *off,
-                               int4 *tiles, WorkItem *items, DevScalars *ds)
+// every 32nd position; one warp per 32 positions: this lane's tile, if one
+// starts here (list id g, n_a particles).
+__device__ __forceinline__ bool static_tile(const int32_t *gid, int32_t n_act, int64_t c, int lane, int32_t &g, int &n_a)
 {
-    if (*(volatile int32_t *)&ds->err) return;  // inputs failed the checks
+    const int64_t k = c * 32 + lane;
+    const bool in = k < n_act;
+    g = in ? gid[k] : -1;
+    const int32_t gprev = __shfl_up_sync(0xffffffffu, g, 1);
+    const bool start = in && (lane == 0 || g != gprev);
+    const uint32_t starts = __ballot_sync(0xffffffffu, start);
+    const uint32_t valid = __ballot_sync(0xffffffffu, in);
+    // this tile spans [k, next start or end of valid lanes)
+    const uint32_t later = starts & ~((2u << lane) - 1u);
+    n_a = (later ? (__ffs(later) - 1) : (32 - __clz(valid))) - lane;
+    return start;
+}
+
+// Checks the list indices and counts the work items of each level.
+__global__ void k_static_count(const int64_t *off, int32_t n_groups, const int32_t *idx, int64_t n_j, const int32_t *gid,
+                               int32_t n_act, DevScalars *ds, uint32_t *level_items)
+{
+    if (*(volatile int32_t *)&ds->err) return;  // off itself is not trusted after a failed check
+    const int64_t L = off[n_groups];
+    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    bool bad = false;
+    for (int64_t e = tid; e < L; e += (int64_t)gridDim.x * blockDim.x)
+        if (idx[e] < 0 || idx[e] >= n_j) bad = true;
+    if (bad) atomicExch(&ds->err, HH_EINVAL);
     const int lane = threadIdx.x & 31;
-    const int64_t warp0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t c = warp0; c * 32 < n_act; c += nwarps) {
-        const int64_t k = c * 32 + lane;
-        const bool in = k < n_act;
-        const int32_t g = in ? gid[k] : -1;
-        const bool bad = in && (g < 0 || g >= n_groups);
-        if (__any_sync(0xffffffffu, bad)) {
-            if (lane == 0) atomicExch(&ds->err, HH_EINVAL);
-            continue;
-        }
-        const int32_t gprev = __shfl_up_sync(0xffffffffu, g, 1);
-        const bool start = in && (lane == 0 || g != gprev);
-        const uint32_t starts = __ballot_sync(0xffffffffu, start);
-        const uint32_t valid = __ballot_sync(0xffffffffu, in);
-        if (start) {
-            // this tile spans [k, next start or end of valid lanes)
-            const uint32_t later = starts & ~((2u << lane) - 1u);
-            const int end_lane = later ? (__ffs(later) - 1) : (32 - __clz(valid));
-            const int n_a = end_lane - lane;
-            const int64_t len = off[g + 1] - off[g];
-            const int n_parts = len > 0 ? (int)((len + kStaticPartLen - 1) / kStaticPartLen) : 1;
-            const int t = atomicAdd(&ds->n_tiles, 1);
-            const uint32_t base = atomicAdd(&ds->n_items, (uint32_t)n_parts);
-            if ((int64_t)base + n_parts > kStaticMaxParts) {
-                atomicExch(&ds->err, HH_ENOMEM);
-            } else {
-                const int4 td = make_int4((int)k, (int)k + n_a, g, (int)base);
-                tiles[t] = td;
-                const uint32_t mask = n_a == 32 ? 0xffffffffu : ((1u << n_a) - 1u);
-                for (int q = 0; q < n_parts; q++) items[base + q] = make_item(t, q, mask, (int)base, td, off[g], off[g + 1], kStaticPartLen);
-            }
+    for (int64_t c = tid >> 5; c * 32 < n_act; c += nwarps) {
+        int32_t g;
+        int n_a;
+        const bool start = static_tile(gid, n_act, c, lane, g, n_a);
+        const int64_t len = start ? off[g + 1] - off[g] : 0;
+#pragma unroll
+        for (int v = 0; v < kStaticLevels; v++) {
+            // (more than kStaticMaxParts parts of one tile count as that many and one: no overflow of the sums)
+            const int64_t p = !start ? 0 : parts_of64(len, static_part_len(v, n_a));
+            const uint32_t s = __reduce_add_sync(0xffffffffu, (uint32_t)min(p, kStaticMaxParts + 1));
+            if (lane == 0 && s) atomicAdd(&level_items[v], min(s, (uint32_t)kStaticMaxParts + 1u));
         }
     }
 }
 
-// Caller-supplied device inputs are checked before the force kernel reads
-// them: off[0] = 0 and non-decreasing, list and i indices inside [0, n_j).
-__global__ void k_static_check(const int64_t *off, int32_t n_groups, const int32_t *idx, const int32_t *i_idx,
-                               int32_t n_act, int64_t n_j, DevScalars *ds)
+// Every part of every tile becomes a work item.  More items than there is room
+// for set ds->err, and nothing is written.
+__global__ void k_static_tiles(const int32_t *gid, int32_t n_act, const int64_t *off, int4 *tiles, WorkItem *items,
+                               DevScalars *ds, const uint32_t *level_items, int levels)
 {
-    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t nth = (int64_t)gridDim.x * blockDim.x;
-    bool bad = false;
-    if (tid == 0 && off[0] != 0) bad = true;
-    for (int64_t g = tid; g < n_groups; g += nth)
-        if (off[g + 1] < off[g]) bad = true;
-    for (int64_t k = tid; k < n_act; k += nth)
-        if (i_idx[k] < 0 || i_idx[k] >= n_j) bad = true;
-    if (bad) atomicExch(&ds->err, HH_EINVAL);
-}
-
-__global__ void k_static_check_idx(const int64_t *off, int32_t n_groups, const int32_t *idx, int64_t n_j,
-                                   DevScalars *ds)
-{
-    if (ds->err) return;  // off itself is not trusted after a failed check
-    const int64_t L = off[n_groups];
-    bool bad = false;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < L; e += (int64_t)gridDim.x * blockDim.x)
-        if (idx[e] < 0 || idx[e] >= n_j) bad = true;
-    if (bad) atomicExch(&ds->err, HH_EINVAL);
-}
-
-__global__ void k_static_finish(DevScalars *ds)
-{
-    // the force kernel must see no items when tiling failed
-    if (ds->err) ds->n_items = 0u;
-    ds->part_len = kStaticPartLen;
+    if (*(volatile int32_t *)&ds->err) return;  // inputs failed the checks
+    if (level_items[0] > (uint32_t)kStaticMaxParts) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) atomicExch(&ds->err, HH_ENOMEM);
+        return;
+    }
+    int v = 0;
+    while (v + 1 < levels && level_items[v + 1] <= (uint32_t)kStaticMaxParts) v++;
+    const int lane = threadIdx.x & 31;
+    const int64_t warp0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t c = warp0; c * 32 < n_act; c += nwarps) {
+        int32_t g;
+        int n_a;
+        if (static_tile(gid, n_act, c, lane, g, n_a)) {
+            const int k = (int)(c * 32 + lane);
+            const int64_t gb = off[g], ge = off[g + 1];
+            const int32_t pj = static_part_len(v, n_a);
+            const int n_parts = parts_of(ge - gb, pj);
+            const int t = atomicAdd(&ds->n_tiles, 1);
+            const uint32_t base = atomicAdd(&ds->n_items, (uint32_t)n_parts);
+            const int4 td = make_int4(k, k + n_a, g, (int)base);
+            tiles[t] = td;
+            const uint32_t mask = n_a == 32 ? 0xffffffffu : ((1u << n_a) - 1u);
+            for (int q = 0; q < n_parts; q++) items[base + q] = make_item(t, q, mask, (int)base, td, gb, ge, pj);
+        }
+    }
 }
 
 // Restores the current device of the calling thread when it goes out of scope.
@@ -222,14 +256,16 @@ extern "C" int hh_force_static(int device, int precision, double eps2, int64_t n
     prm.eps2 = eps2;
     prm.unit = 1.0;
     StepCtl c{1, 0, 1, 0, 0.0};
+    uint32_t *level_items = reinterpret_cast<uint32_t *>(base + kOffHdr);
     if (precision == HH_MIXED)
-        k_static_pack<RecMix><<<st.elem_grid, 256, 0, s>>>(reinterpret_cast<RecMix *>(base + kOffRec), xj, vj, mj, n_j);
+        k_static_prepare<RecMix><<<st.elem_grid, 256, 0, s>>>(reinterpret_cast<RecMix *>(base + kOffRec), xj, vj, mj, n_j,
+                                                              off, n_groups, i_idx, gid, n_act, ds);
     else
-        k_static_pack<RecF64><<<st.elem_grid, 256, 0, s>>>(reinterpret_cast<RecF64 *>(base + kOffRec), xj, vj, mj, n_j);
-    k_static_check<<<st.elem_grid, 256, 0, s>>>(off, n_groups, idx, i_idx, n_act, n_j, ds);
-    k_static_check_idx<<<st.elem_grid, 256, 0, s>>>(off, n_groups, idx, n_j, ds);
-    k_static_tiles<<<st.elem_grid, 256, 0, s>>>(gid, n_act, n_groups, off, const_cast<int4 *>(L.tiles), L.items, ds);
-    k_static_finish<<<1, 1, 0, s>>>(ds);
+        k_static_prepare<RecF64><<<st.elem_grid, 256, 0, s>>>(reinterpret_cast<RecF64 *>(base + kOffRec), xj, vj, mj, n_j,
+                                                              off, n_groups, i_idx, gid, n_act, ds);
+    k_static_count<<<st.elem_grid, 256, 0, s>>>(off, n_groups, idx, n_j, gid, n_act, ds, level_items);
+    k_static_tiles<<<(n_act + 255) / 256, 256, 0, s>>>(gid, n_act, off, const_cast<int4 *>(L.tiles), L.items, ds,
+                                                       level_items, precision == HH_FP64 ? kStaticLevels : 1);
     if (precision == HH_MIXED)
         k_force<RecMix, kStaticTj, true><<<st.force_grid, kThreads, 0, s>>>(
             S, reinterpret_cast<const RecMix *>(base + kOffRec), L, ds, c, prm);

@@ -90,3 +90,25 @@ def test_parts_left_to_fp64(env, what):
     # FP64 sums in another order: at most 2048 terms a thread and part, 2^-41 of the sizes
     assert (np.abs(got - ref)[fine] <= 2.0 ** -41 * size[fine]).all()
     assert np.array_equal(np.isnan(ref), np.isnan(got)) and np.array_equal(np.isinf(ref), np.isinf(got))
+
+
+@pytest.mark.parametrize("n_act,n_list", [(4000, 250), (4000, 700), (4000, 1500), (8000, 2000), (8192, 2048)])
+def test_static_part_lengths(env, n_act, n_list):
+    # every active particle is a tile of its own (two lists in turn): at most 8192 parts of at most 2048 entries
+    hh, torch = env
+    rng = np.random.default_rng(n_act + n_list)
+    n, eps2 = 2 * n_list + 11, 1e-4
+    x, v, m = rng.normal(size=(3, n)), rng.normal(size=(3, n)), np.full(n, 1.0 / n)
+    lists = [np.sort(rng.choice(n, n_list, replace=False)) for _ in range(2)]
+    act, gid = rng.integers(0, n, n_act), np.arange(n_act) % 2
+    dev = torch.device("cuda", 0)
+    t = lambda u, dt: torch.tensor(np.ascontiguousarray(u), dtype=dt, device=dev)  # noqa: E731
+    out = [torch.zeros(s, dtype=torch.float64, device=dev) for s in ((3, n_act), (3, n_act), (n_act,))]
+    hh.hh_force_static(t(x, torch.float64), t(v, torch.float64), t(m, torch.float64),
+                       t([0, n_list, 2 * n_list], torch.int64), t(np.concatenate(lists), torch.int32),
+                       t(act, torch.int32), t(gid, torch.int32), *out, eps2=eps2, precision=hh.HH_FP64)
+    got = np.concatenate([out[0].cpu().numpy(), out[1].cpu().numpy(), out[2].cpu().numpy()[None]])
+    for g in range(2):
+        sel = np.flatnonzero(gid == g)[:: max(1, n_act // 400)]
+        ref, size = _reference(x, v, m, lists[g], act[sel], eps2, np.float64)
+        assert (np.abs(got[:, sel] - ref) <= 2.0 ** -41 * size).all()
