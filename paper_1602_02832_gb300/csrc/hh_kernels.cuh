@@ -72,7 +72,7 @@ struct __align__(32) RecF64 {
 struct __align__(16) RecMix {
     float4 hm;  // (x_hi, y_hi, z_hi, m)
     float4 lo;  // (x_lo, y_lo, z_lo, 0)
-    float4 v;   // (vx, vy, vz, 0)
+    float4 v;   // (vx, vy, vz, -): the last word holds the entry's index
 };
 
 // Mixed form: per j entry, the FP32 quantities the predictor needs,
@@ -288,7 +288,8 @@ __device__ __forceinline__ void store_rec<RecMix>(RecMix *out, int64_t e, const 
     RecMix r;
     r.hm = make_float4(hi[0], hi[1], hi[2], __double2float_rn(m));
     r.lo = make_float4(lo[0], lo[1], lo[2], 0.f);
-    r.v = make_float4(__double2float_rn(vp[0]), __double2float_rn(vp[1]), __double2float_rn(vp[2]), 0.f);
+    r.v = make_float4(__double2float_rn(vp[0]), __double2float_rn(vp[1]), __double2float_rn(vp[2]),
+                      __int_as_float((int)e));
     out[e] = r;
 }
 
@@ -331,7 +332,7 @@ __device__ __forceinline__ void refresh_base(const State &s, int64_t e)
 // Mixed predictor: the FP64 base position (as a float pair) plus an FP32
 // increment D (v + D (a/2 + D jerk/6)), added with TwoSum; v + D (a + D jerk/2)
 // in FP32.  D = t - t_e is exact in FP32 (a multiple of dt_min below dt_tree).
-__device__ __forceinline__ RecMix mix_from_base(const BaseMix &b, float D)
+__device__ __forceinline__ RecMix mix_from_base(const BaseMix &b, float D, int64_t e)
 {
     const float hx[3] = {b.hm.x, b.hm.y, b.hm.z}, lx[3] = {b.lo.x, b.lo.y, b.lo.z};
     const float vv[3] = {b.v.x, b.v.y, b.v.z}, aa[3] = {b.a2.x, b.a2.y, b.a2.z}, jj[3] = {b.j6.x, b.j6.y, b.j6.z};
@@ -349,7 +350,7 @@ __device__ __forceinline__ RecMix mix_from_base(const BaseMix &b, float D)
     RecMix r;
     r.hm = make_float4(ho[0], ho[1], ho[2], b.hm.w);
     r.lo = make_float4(lo[0], lo[1], lo[2], 0.f);
-    r.v = make_float4(vo[0], vo[1], vo[2], 0.f);
+    r.v = make_float4(vo[0], vo[1], vo[2], __int_as_float((int)e));
     return r;
 }
 
@@ -404,7 +405,7 @@ __device__ __forceinline__ void pred_store<RecF64>(const PredIn<RecF64> &in, Rec
 template <>
 __device__ __forceinline__ void pred_store<RecMix>(const PredIn<RecMix> &in, RecMix *rec, int64_t e, double tnow)
 {
-    rec[e] = mix_from_base(in.b, __double2float_rn(tnow - in.t));
+    rec[e] = mix_from_base(in.b, __double2float_rn(tnow - in.t), e);
 }
 
 // Predicted record of entry e at tnow, in the form's own arithmetic.
@@ -526,49 +527,79 @@ __device__ __forceinline__ F2 f2_add(F2 a, F2 b)
 }
 
 struct AccMix {
-    float ax, ay, az, jx, jy, jz, p;  // current chunk
+    float2 axy, jxy, azjz;  // current chunk: (ax, ay), (jx, jy), (az, jz)
+    float p;
     F2 Ax, Ay, Az, Jx, Jy, Jz, P;     // running compensated sums
     __device__ void zero()
     {
-        ax = ay = az = jx = jy = jz = p = 0.f;
+        axy = jxy = azjz = make_float2(0.f, 0.f);
+        p = 0.f;
         Ax = Ay = Az = Jx = Jy = Jz = P = F2{0.f, 0.f};
     }
     __device__ void fold()
     {
-        two_sum_into(Ax, ax); two_sum_into(Ay, ay); two_sum_into(Az, az);
-        two_sum_into(Jx, jx); two_sum_into(Jy, jy); two_sum_into(Jz, jz);
+        two_sum_into(Ax, axy.x); two_sum_into(Ay, axy.y); two_sum_into(Az, azjz.x);
+        two_sum_into(Jx, jxy.x); two_sum_into(Jy, jxy.y); two_sum_into(Jz, azjz.y);
         two_sum_into(P, p);
-        ax = ay = az = jx = jy = jz = p = 0.f;
+        axy = jxy = azjz = make_float2(0.f, 0.f);
+        p = 0.f;
     }
 };
 
+// The i particle, negated (differences are sums then), x and y together.
 struct IMix {
-    float xh, yh, zh, xl, yl, zl, vx, vy, vz;
+    float2 h, l, v;
+    float hz, lz, vz;
 };
 
 __device__ __forceinline__ void load_i(const RecMix *rec, int64_t i, IMix &o)
 {
     const RecMix r = rec[i];
-    o.xh = r.hm.x; o.yh = r.hm.y; o.zh = r.hm.z;
-    o.xl = r.lo.x; o.yl = r.lo.y; o.zl = r.lo.z;
-    o.vx = r.v.x; o.vy = r.v.y; o.vz = r.v.z;
+    o.h = make_float2(-r.hm.x, -r.hm.y);
+    o.l = make_float2(-r.lo.x, -r.lo.y);
+    o.v = make_float2(-r.v.x, -r.v.y);
+    o.hz = -r.hm.z;
+    o.lz = -r.lo.z;
+    o.vz = -r.v.z;
 }
 
+// 1/sqrt estimate.  With kNormal (the softening, and so every r2, is a normal
+// number) without the scaling of subnormal arguments: the same bits, three
+// instructions less.
+template <bool kNormal>
+__device__ __forceinline__ float rsqrt_est(float x)
+{
+    if (!kNormal) return rsqrtf(x);
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// Bound by instruction issue (60 a pair, 78% of the issue slots at 6 warps a
+// sub-partition), so the x and y components, and the z components of the two
+// sums, go two to an instruction (packed FP32: each half rounds as the single
+// instruction does, so the sums keep their bits), the self test reads the index
+// that comes with the record, and the estimate skips the subnormal scaling: 46
+// instructions, 82 -> 64 cycles a warp and pair (the FP32 pipe's own time is
+// about 45).  Two pairs at a time in packed scalars (39 instructions) measured 3%
+// more with 6 warps a sub-partition and is left out.
+template <bool kNormal>
 __device__ __forceinline__ void interact(const IMix &I, const RecMix &J, bool self, float eps2, AccMix &A)
 {
     // i-j difference of the float pairs: (hi_j - hi_i) + (lo_j - lo_i)
-    const float dx = __fadd_rn(__fsub_rn(J.hm.x, I.xh), __fsub_rn(J.lo.x, I.xl));
-    const float dy = __fadd_rn(__fsub_rn(J.hm.y, I.yh), __fsub_rn(J.lo.y, I.yl));
-    const float dz = __fadd_rn(__fsub_rn(J.hm.z, I.zh), __fsub_rn(J.lo.z, I.zl));
-    const float wx = J.v.x - I.vx, wy = J.v.y - I.vy, wz = J.v.z - I.vz;
-    float r2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, eps2)));
+    const float2 dxy = __fadd2_rn(__fadd2_rn(make_float2(J.hm.x, J.hm.y), I.h),
+                                  __fadd2_rn(make_float2(J.lo.x, J.lo.y), I.l));
+    const float dz = __fadd_rn(__fadd_rn(J.hm.z, I.hz), __fadd_rn(J.lo.z, I.lz));
+    const float2 wxy = __fadd2_rn(make_float2(J.v.x, J.v.y), I.v);
+    const float wz = __fadd_rn(J.v.z, I.vz);
+    float r2 = fmaf(dxy.x, dxy.x, fmaf(dxy.y, dxy.y, fmaf(dz, dz, eps2)));
     r2 = self ? 1.f : r2;
     const float mj = self ? 0.f : J.hm.w;
-    const float rw = fmaf(dx, wx, fmaf(dy, wy, dz * wz));
+    const float rw = fmaf(dxy.x, wxy.x, fmaf(dxy.y, wxy.y, dz * wz));
     // 1/sqrt: hardware estimate, then one Newton-Raphson step
     // y <- y + (y/2) h, h = 1 - r2 y^2, with the residual formed exactly
     // (r2 y = p + e by an FMA) so the step lands within ~1/2 ulp.
-    const float y0 = rsqrtf(r2);
+    const float y0 = rsqrt_est<kNormal>(r2);
     const float pr = r2 * y0;
     const float er = fmaf(r2, y0, -pr);
     const float hres = fmaf(-er, y0, fmaf(-pr, y0, 1.f));
@@ -577,13 +608,13 @@ __device__ __forceinline__ void interact(const IMix &I, const RecMix &J, bool se
     const float mr = mj * rinv;
     const float mr3 = mr * rinv2;
     const float al = 3.f * rw * rinv2;
+    const float2 m2 = make_float2(mr3, mr3);
+    const float2 ixy = __ffma2_rn(make_float2(-al, -al), dxy, wxy);
+    const float iz = fmaf(-al, dz, wz);
     A.p += mr;
-    A.ax = fmaf(mr3, dx, A.ax);
-    A.ay = fmaf(mr3, dy, A.ay);
-    A.az = fmaf(mr3, dz, A.az);
-    A.jx = fmaf(mr3, fmaf(-al, dx, wx), A.jx);
-    A.jy = fmaf(mr3, fmaf(-al, dy, wy), A.jy);
-    A.jz = fmaf(mr3, fmaf(-al, dz, wz), A.jz);
+    A.axy = __ffma2_rn(m2, dxy, A.axy);
+    A.jxy = __ffma2_rn(m2, ixy, A.jxy);
+    A.azjz = __ffma2_rn(m2, make_float2(dz, iz), A.azjz);
 }
 
 // ---------------------------------------------- cross-slice reductions
@@ -768,13 +799,13 @@ constexpr int kStages = 2;
 template <typename Rec, int TJ>
 struct ForceSmem {
     Rec rec[kStages][TJ];  // ring of staged list chunks
-    int32_t idx[kStages][TJ];
+    int32_t idx[kStages][std::is_same<Rec, RecF64>::value ? TJ : 1];  // plain form (mixed: in the records)
     typename Traits<Rec>::Red red[kThreads / 32][kMaxTileI];
     int item;
     int last;
     double tn[kThreads / 32];  // per-warp minimum of t + dt after the corrector
     int lv[kMaxTileI];         // new step level of each corrected particle, by active index
-    typename Traits<Rec>::I iv[kMaxTileI];  // plain form: the item's active particles
+    typename Traits<Rec>::I iv[std::is_same<Rec, RecF64>::value ? kMaxTileI : 1];  // plain form: the item's active particles
     double fin[kMaxTileI][7];  // the completed tile's new acc, jerk, pot by active index (for its corrector)
 };
 
@@ -920,7 +951,7 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
 #pragma unroll
             for (int q = 0; q < EPT; q++) {
                 const int e = q * kThreads + tid;
-                sm.idx[b][e] = nxt[q];
+                if constexpr (kPlain) sm.idx[b][e] = nxt[q];
                 if (nxt[q] >= 0) cp_async_rec(&sm.rec[b][e], &rec[nxt[q]]);
             }
         }
@@ -958,14 +989,18 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
             // FP32 partials are folded into the compensated sums every
             // kFold terms per thread (short plain-FP32 runs keep the
             // partial-sum rounding below the per-term rounding).
-            for (int e = idle ? nc : jslice; e < nc;) {
-                const int e_end = min(nc, e + kFold * S);
-                for (; e < e_end; e += S) {
-                    const int32_t j = sm.idx[b][e];
-                    interact(Iv, sm.rec[b][e], (int64_t)j == pi, eps2, A);
+            auto chunk = [&](auto normal) {
+                for (int e = idle ? nc : jslice; e < nc;) {
+                    const int e_end = min(nc, e + kFold * S);
+                    for (; e < e_end; e += S) {
+                        const RecMix &J = sm.rec[b][e];
+                        interact<decltype(normal)::value>(Iv, J, __float_as_int(J.v.w) == (int)pi, eps2, A);
+                    }
+                    fold_chunk(A);
                 }
-                fold_chunk(A);
-            }
+            };
+            if (eps2 >= 1.17549435e-38f) chunk(std::true_type{});
+            else chunk(std::false_type{});
         }
         group_sync(bar_id);  // buffer b is refilled by the next step's issue
     }
