@@ -290,10 +290,10 @@ __device__ __forceinline__ double correct_tile_3lane(const SimDesc &sd, const in
 struct StepCache {
     double t[kSimCache];
     double t_end[kSimCache];
-    int due[kSimCache];                  // particles due at t (levels >= kmin(t)); -1: not counted
     unsigned char list_mode[kSimCache];  // predict only the entries of this step's list parts
     int any_list;                        // some simulation of the batch is in list mode this step
     int any_full;                        // some live simulation predicts every entry this step
+    int any_live;                        // some simulation has a step to take
 };
 
 // Due particles of a simulation at block time tnow: its level histogram's
@@ -329,28 +329,34 @@ __device__ __forceinline__ bool list_mode_of(const SimDesc &sd, double tnow, int
     return (int64_t)due * sd.lbar * kDiv < sd.nj;
 }
 
-__device__ __forceinline__ void cache_times(StepCache &c, const SimDesc *sims, int n_sims, int par)
+template <typename SDF>
+__device__ __forceinline__ void cache_times(StepCache &c, SDF SD, int n_sims, int par)
 {
     if (threadIdx.x == 0) {
         c.any_list = 0;
         c.any_full = n_sims > kSimCache;  // (simulations beyond the cache predict every entry)
+        c.any_live = 0;
     }
     __syncthreads();
-    int any = 0, full = 0;
+    int any = 0, full = 0, live = 0;
     for (int s = threadIdx.x; s < n_sims && s < kSimCache; s += blockDim.x) {
-        c.t[s] = __longlong_as_double((long long)__ldcg(&sims[s].ds->tmin[par]));
-        c.t_end[s] = sims[s].t_end;
+        const SimDesc &sd = SD(s);
+        c.t[s] = __longlong_as_double((long long)__ldcg(&sd.ds->tmin[par]));
+        c.t_end[s] = sd.t_end;
         // (counted here only where list mode may apply: the count is one
         // more round trip to L2 on the path of every step)
-        const int due = sims[s].nj >= kListModeMinJ ? due_count(sims[s], c.t[s]) : -1;
-        c.due[s] = due;
-        const bool lm = due >= 0 && list_mode_of(sims[s], c.t[s], due);
+        const int due = sd.nj >= kListModeMinJ ? due_count(sd, c.t[s]) : -1;
+        const bool lm = due >= 0 && list_mode_of(sd, c.t[s], due);
         c.list_mode[s] = lm;
         any |= lm;
         full |= !lm && c.t[s] <= c.t_end[s];
+        live |= c.t[s] <= c.t_end[s];
     }
+    for (int s = kSimCache + threadIdx.x; s < n_sims; s += blockDim.x)
+        live |= __longlong_as_double((long long)__ldcg(&SD(s).ds->tmin[par])) <= SD(s).t_end;
     if (any) c.any_list = 1;
     if (full) c.any_full = 1;
+    if (live) c.any_live = 1;
     __syncthreads();
 }
 
@@ -549,23 +555,39 @@ __global__ void __launch_bounds__(kBlock, 1) k_batch(BatchDev B)
 
     int step = 0;
     bool prev_full = true;  // the last step predicted every entry of some simulation
+    // this lane's first tile of the selection (the same at every step)
+    const int lane = tid & 31;
+    const int64_t w0 = gtid >> 5, nw = nth >> 5;
+    const int64_t wt0 = w0 + (int64_t)lane * nw;
+    const int s_t0 = wt0 < NT ? find_sim(TB, n_sims, wt0) : 0;
     for (; step < max_steps; step++) {
         const int par = step & 1;
         // ---- phase 1: select + predict
-        // The inputs of this thread's first predicted entry (mixed form; the
-        // plain form's FP64 inputs would not fit in registers, and its
-        // predictor is bound by the FP64 pipe) do not depend on the block
-        // time: their loads go out before the block times are read, unless
-        // the last step predicted only list entries (then this one likely
-        // does too, and the loads would be wasted).
+        // What does not depend on the block time goes out before the block
+        // times are read: the first tile's levels and record, and the inputs
+        // of this thread's first predicted entry (mixed form; the plain form's
+        // FP64 inputs would not fit in registers, and its predictor is bound
+        // by the FP64 pipe), these unless the last step predicted only list
+        // entries (then this one likely does too, and the loads would be
+        // wasted).
         constexpr bool kEarly = std::is_same<Rec, RecMix>::value;
         constexpr bool kPlain = std::is_same<Rec, RecF64>::value;
         constexpr bool kExactChunks = std::is_same<Rec, RecMix>::value;
+        uint32_t lv0 = 0u;
+        int4 td0 = make_int4(0, 0, 0, 0);
+        if (wt0 < NT) {
+            const SimDesc &sd = SD(s_t0);
+            lv0 = sd.tile_lv[wt0 - TB[s_t0]];
+            td0 = sd.L.tiles[wt0 - TB[s_t0]];
+        }
         PredIn<Rec> in0;
         const int s_p0 = gtid < NJ ? find_sim(JB, n_sims, gtid) : 0;
         const bool early = kEarly && prev_full && gtid < NJ;
         if (early) pred_load<Rec>(SD(s_p0).st, gtid - JB[s_p0], in0);
-        cache_times(sc, B.sims, n_sims, par);
+        // (the block times are read once a step: whether any simulation goes
+        // on is known here, not after a read of its own at the step's end)
+        cache_times(sc, SD, n_sims, par);
+        if (step > 0 && !sc.any_live) break;
         prev_full = sc.any_full;
         // counters of the previous step (other parity) are free again
         if (blockIdx.x == 0 && tid == 0) {
@@ -574,45 +596,28 @@ __global__ void __launch_bounds__(kBlock, 1) k_batch(BatchDev B)
             B.bs->max_chunks[par ^ 1] = 0u;
         }
         {
-            // one warp per simulation, spread over the CTAs (a loop in one
-            // CTA put a latency chain per 16 simulations on every step)
-            const int wpb = (int)(blockDim.x >> 5);
-            for (int s = (int)blockIdx.x * wpb + (tid >> 5); s < n_sims; s += (int)gridDim.x * wpb) {
-                // the next block time starts from the due times of the levels
-                // not corrected now; the corrector lowers it with the
-                // corrected ones.  A finished simulation keeps its time.
-                DevScalars *ds = B.sims[s].ds;
-                const double tnow = cached_time(sc, B.sims, s, par);
-                const bool live = tnow <= B.sims[s].t_end;
-                const double below = due_below_warp(ds->lvl_cnt, tnow, kmin_of(tnow));
-                if ((tid & 31) == 0) {
-                    ds->tmin[par ^ 1] = live ? (unsigned long long)__double_as_longlong(below) : ds->tmin[par];
-                    ds->n_act_last = 0;
-                    ds->slot_par[par ^ 1] = 0u;
-                    if (live) ds->block_steps += 1ull;
-                    if (live && cached_list_mode(sc, s)) ds->list_steps += 1ull;
-                }
-            }
-        }
-        {
             // Tile selection: warp w takes tiles w + k W (W warps, k = 0,
-            // 1, ...); its lanes read the level masks of 32 of them per round
-            // trip, and the warp then builds the items of the due ones among
-            // them, one tile at a time.  It runs before the prediction: the
-            // few warps of a small step that find due tiles wait on chains of
-            // loads and atomics while the others' predictions use the pipes.
-            const int lane = tid & 31;
-            const int64_t w0 = gtid >> 5, nw = nth >> 5;
+            // 1, ...); its lanes read the level masks and records of 32 of
+            // them per round trip, and the warp then builds the items of the
+            // due ones among them, one tile at a time: one round trip for all
+            // that a tile's items need (its particles' times, its list's
+            // range, the level histogram), one for the queue's atomics.  It
+            // runs before the prediction: the few warps of a small step that
+            // find due tiles wait on these loads and atomics while the others'
+            // predictions use the pipes.
             for (int64_t k0 = 0; w0 + k0 * nw < NT; k0 += 32) {
                 const int64_t wt = w0 + (k0 + lane) * nw;
-                int s_l = 0;
+                int s_l = s_t0;
                 bool due_l = false;
                 if (wt < NT) {
-                    s_l = find_sim(TB, n_sims, wt);
-                    const SimDesc &sd = SD(s_l);
+                    if (k0 > 0) {
+                        s_l = find_sim(TB, n_sims, wt);
+                        const SimDesc &sd = SD(s_l);
+                        lv0 = sd.tile_lv[wt - TB[s_l]];
+                        td0 = sd.L.tiles[wt - TB[s_l]];
+                    }
                     const double tnow = cached_time(sc, B.sims, s_l, par);
-                    const uint32_t lv = sd.tile_lv[wt - TB[s_l]];
-                    due_l = tnow <= sd.t_end && (lv >> kmin_of(tnow)) != 0u;  // a due level in this tile
+                    due_l = tnow <= SD(s_l).t_end && (lv0 >> kmin_of(tnow)) != 0u;  // a due level in this tile
                 }
                 for (uint32_t dmask = __ballot_sync(0xffffffffu, due_l); dmask; dmask &= dmask - 1) {
                     const int l = __ffs(dmask) - 1;
@@ -620,9 +625,13 @@ __global__ void __launch_bounds__(kBlock, 1) k_batch(BatchDev B)
                     const SimDesc &sd = SD(s);
                     const double tnow = cached_time(sc, B.sims, s, par);
                     const int tile = (int)(w0 + (k0 + l) * nw - TB[s]);
-                    const int4 td = sd.L.tiles[tile];
-                    const int64_t p = td.x + lane;
-                    const bool act = (p < td.y) && (sd.st.t[p] + sd.st.dt[p] == tnow);
+                    const int4 td = make_int4(__shfl_sync(0xffffffffu, td0.x, l), __shfl_sync(0xffffffffu, td0.y, l),
+                                              __shfl_sync(0xffffffffu, td0.z, l), 0);
+                    const int64_t p = min((int64_t)td.x + lane, (int64_t)td.y - 1);
+                    const double t_p = sd.st.t[p], dt_p = sd.st.dt[p];
+                    const int64_t gb = sd.L.off[td.z], ge = sd.L.off[td.z + 1];
+                    const int cnt = __ldcg(&sd.ds->lvl_cnt[lane]);
+                    const bool act = (td.x + lane < td.y) && (t_p + dt_p == tnow);
                     // equal-cost items in this step?  With work_split the
                     // simulation's due particles (levels >= kmin, from its
                     // level histogram, fixed during this phase) must reach
@@ -634,13 +643,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_batch(BatchDev B)
                     // kSmallDue due particles take parts of that length
                     int work = sd.work, pj = sd.pj;
                     if (sd.work_split > 0 || sd.pj_small > 0) {
-                        int due;
-                        if (s < kSimCache && sc.due[s] >= 0) {
-                            due = sc.due[s];
-                        } else {
-                            const int cnt = __ldcg(&sd.ds->lvl_cnt[lane]);
-                            due = __reduce_add_sync(0xffffffffu, lane >= kmin_of(tnow) ? cnt : 0);
-                        }
+                        const int due = __reduce_add_sync(0xffffffffu, lane >= kmin_of(tnow) ? cnt : 0);
                         if (sd.work_split > 0 && due < sd.work_split) {
                             work = kPlain ? kMedWork * sd.pj : 0;
                             if (kPlain) pj = 32;
@@ -652,9 +655,30 @@ __global__ void __launch_bounds__(kBlock, 1) k_batch(BatchDev B)
                     }
                     const uint32_t mask = __ballot_sync(0xffffffffu, act);
                     if (mask)
-                        append_tile_items(sd.L, tile, td, mask, pj, work, &B.bs->n_items[par], &sd.ds->slot_par[par],
+                        append_tile_items(tile, td, gb, ge, mask, pj, work, &B.bs->n_items[par], &sd.ds->slot_par[par],
                                           items, s, sd.ds->na_hist,
                                           kExactChunks && cached_list_mode(sc, s) ? &B.bs->max_chunks[par] : nullptr);
+                }
+            }
+        }
+        {
+            // one warp per simulation, spread over the CTAs (a loop in one
+            // CTA put a latency chain per 16 simulations on every step)
+            const int wpb = (int)(blockDim.x >> 5);
+            for (int s = (int)blockIdx.x * wpb + (tid >> 5); s < n_sims; s += (int)gridDim.x * wpb) {
+                // the next block time starts from the due times of the levels
+                // not corrected now; the corrector lowers it with the
+                // corrected ones.  A finished simulation keeps its time.
+                DevScalars *ds = SD(s).ds;
+                const double tnow = cached_time(sc, B.sims, s, par);
+                const bool live = tnow <= SD(s).t_end;
+                const double below = due_below_warp(ds->lvl_cnt, tnow, kmin_of(tnow));
+                if (lane == 0) {
+                    ds->tmin[par ^ 1] = live ? (unsigned long long)__double_as_longlong(below) : ds->tmin[par];
+                    ds->n_act_last = 0;
+                    ds->slot_par[par ^ 1] = 0u;
+                    if (live) ds->block_steps += 1ull;
+                    if (live && cached_list_mode(sc, s)) ds->list_steps += 1ull;
                 }
             }
         }
@@ -694,8 +718,6 @@ __global__ void __launch_bounds__(kBlock, 1) k_batch(BatchDev B)
                         maxc = max(maxc, (min(plen, sd.lmax) + 31) / 32);
                     }
             }
-            const int lane = tid & 31;
-            const int64_t w0 = gtid >> 5, nw = nth >> 5;
             const int64_t n_tasks = (int64_t)n_items * maxc;
             for (int64_t task = w0; task < n_tasks; task += nw) {
                 const int64_t i = task / maxc;
@@ -815,14 +837,6 @@ __global__ void __launch_bounds__(kBlock, 1) k_batch(BatchDev B)
             const unsigned long long now = globaltimer_ns();
             B.step_ns[3 * step + 2] = now;
             B.step_ns[3 * step + 3] = now;  // the corrector ran inside the force phase
-        }
-
-        // any simulation still live for the next step?
-        int live = 0;
-        for (int s = tid; s < n_sims; s += blockDim.x) live |= sim_time(B.sims[s], par ^ 1) <= B.sims[s].t_end;
-        if (!__syncthreads_or(live)) {
-            step++;
-            break;
         }
     }
     if (blockIdx.x == 0) {

@@ -193,12 +193,11 @@ __device__ __forceinline__ int parts_of(int64_t len, int pj) { return len > 0 ? 
 // Warp-collective: appends one work item per part of tile `tile`'s list;
 // item = (tile, part | sim << 16, active mask, first partial-sum slot, part
 // length).  `work` is the equal-cost target of this step (0: parts of pj_min).
-__device__ __forceinline__ void append_tile_items(const Lists &L, int tile, const int4 td, uint32_t mask, int pj_min,
-                                                  int work, uint32_t *n_items, uint32_t *slot_ctr, WorkItem *items,
+__device__ __forceinline__ void append_tile_items(int tile, const int4 td, int64_t gb, int64_t ge, uint32_t mask,
+                                                  int pj_min, int work, uint32_t *n_items, uint32_t *slot_ctr, WorkItem *items,
                                                   int sim, unsigned long long *na_hist, uint32_t *max_chunks = nullptr)
 {
     const int lane = threadIdx.x & 31;
-    const int64_t gb = L.off[td.z], ge = L.off[td.z + 1];
     const int64_t len = ge - gb;
     const int pj = part_len_for(__popc(mask), pj_min, work);
     const int n_parts = parts_of(len, pj);
@@ -231,7 +230,8 @@ __device__ __forceinline__ void select_tiles(const State &s, const Lists &L, Dev
         const bool act = (p < td.y) && is_active(s, c, p, tnow);
         const uint32_t mask = __ballot_sync(0xffffffffu, act);
         if (mask == 0u) continue;
-        append_tile_items(L, (int)tile, td, mask, pj, work, &ds->n_items, &ds->slot_ctr, L.items, 0, ds->na_hist);
+        append_tile_items((int)tile, td, L.off[td.z], L.off[td.z + 1], mask, pj, work, &ds->n_items, &ds->slot_ctr, L.items,
+                          0, ds->na_hist);
     }
 }
 
