@@ -225,9 +225,10 @@ __device__ __forceinline__ double due_below_warp(const int32_t *lvl_cnt, double 
 // each corrected particle's new level in lv_out[its index among the active].
 // The new forces come from fin[active index] (the force tail's copy in
 // shared memory; the same values as acc1 / jerk1).
+template <bool kPlain>
 __device__ __forceinline__ double correct_tile_3lane(const SimDesc &sd, const int4 td, uint32_t mask, double tnow,
                                                      int lane, int k_first, int k_step, int *lv_out,
-                                                     const double (*fin)[7])
+                                                     const double (*fin)[7], const int *pidx)
 {
     const unsigned full = 0xffffffffu;
     const State &s = sd.st;
@@ -239,30 +240,38 @@ __device__ __forceinline__ double correct_tile_3lane(const SimDesc &sd, const in
     for (int base = k_first; base < na; base += k_step) {
         const int k = base + q;
         const bool on = lane < 30 && k < na;
-        const int64_t p = on ? td.x + (__fns(mask, 0, k + 1)) : td.x;
-        double sa = 0.0, sj = 0.0, ss = 0.0, st = 0.0, a1 = 0.0, j1 = 0.0, dt_old = 1.0;
+        const int64_t p = on ? pidx[k] : td.x;
+        double D = 1.0, a1 = 0.0, j1 = 0.0, dt_old = 1.0;
         CorrComp c{};
         if (on) {
             dt_old = s.dt[p];
-            const StepPowers P = step_powers(tnow - s.t[p]);
+            D = tnow - s.t[p];
             const double a0 = s.a[d * s.cap_j + p], j0 = s.jk[d * s.cap_j + p];
             a1 = fin[k][d];
             j1 = fin[k][3 + d];
-            c = correct_component(s.x[d * s.cap_j + p], s.v[d * s.cap_j + p], a0, j0, a1, j1, P);
-            sa = sq(a1);
-            sj = sq(j1);
-            ss = sq(c.a2e);
-            st = sq(c.a3);
+            c = correct_component<kPlain>(s.x[d * s.cap_j + p], s.v[d * s.cap_j + p], a0, j0, a1, j1, D);
         }
         // the particle's three lanes: g, g + 1, g + 2 (lanes 30, 31 are idle)
-        const double A = norm2_of(__shfl_sync(full, sa, g), __shfl_sync(full, sa, g + 1), __shfl_sync(full, sa, g + 2));
-        const double J = norm2_of(__shfl_sync(full, sj, g), __shfl_sync(full, sj, g + 1), __shfl_sync(full, sj, g + 2));
-        const double S = norm2_of(__shfl_sync(full, ss, g), __shfl_sync(full, ss, g + 1), __shfl_sync(full, ss, g + 2));
-        const double T = norm2_of(__shfl_sync(full, st, g), __shfl_sync(full, st, g + 1), __shfl_sync(full, st, g + 2));
+        auto sum3 = [&](float u) {
+            return __fadd_rn(__fadd_rn(__shfl_sync(full, u, g), __shfl_sync(full, u, g + 1)), __shfl_sync(full, u, g + 2));
+        };
+        int ea = biased_exp(a1);
+        ea = max(max(__shfl_sync(full, ea, g), __shfl_sync(full, ea, g + 1)), __shfl_sync(full, ea, g + 2));
+        const CritSquares u = crit_squares<kPlain>(a1, c, ea, D);
+        const float A = sum3(u.a), J = sum3(u.j), S = sum3(u.s), T = sum3(u.t);
+        double want = 0.0;
+        const bool certain = corrector_screen<kPlain>(A, J, S, T, D, sd.prm.eta, ea, want);
+        if (__any_sync(full, on && !certain)) {
+            auto norm3d = [&](double u) {
+                const double q2 = sq(u);
+                return norm2_of(__shfl_sync(full, q2, g), __shfl_sync(full, q2, g + 1), __shfl_sync(full, q2, g + 2));
+            };
+            const double A2 = norm3d(a1), J2 = norm3d(c.q), S2 = norm3d(c.s), T2 = norm3d(c.g);
+            if (!certain) want = corrector_want<kPlain>(A2, J2, S2, T2, D, sd.prm.eta);
+        }
         __syncwarp();  // every lane has read t and dt before any is rewritten
         if (on) {
-            const double dtn = block_dt(aarseth_want(A, J, S, T, sd.prm.eta), dt_old, tnow, sd.prm.dt_min,
-                                        sd.prm.dt_max);
+            const double dtn = block_dt(want, dt_old, tnow, sd.prm.dt_min, sd.prm.dt_max);
             s.x[d * s.cap_j + p] = c.x;
             s.v[d * s.cap_j + p] = c.v;
             s.a[d * s.cap_j + p] = a1;
@@ -792,7 +801,8 @@ __global__ void __launch_bounds__(kBlock, 1) k_batch(BatchDev B)
                     const int64_t pw = td.x + glane;
                     const double dt_keep = (gw == 0 && pw < td.y && !((mask >> glane) & 1u)) ? sdc.st.dt[pw] : 0.0;
                     const double tn =
-                        correct_tile_3lane(sdc, td, mask, tnow, glane, 10 * gw, 10 * (kThreads / 32), sm.lv, sm.fin);
+                        correct_tile_3lane<kPlain>(sdc, td, mask, tnow, glane, 10 * gw, 10 * (kThreads / 32), sm.lv, sm.fin,
+                                           sm.pidx);
                     if (glane == 0) sm.tn[gw] = tn;
                     group_sync(bar);  // new levels and times are visible to the group
                     if (gw == 0) {

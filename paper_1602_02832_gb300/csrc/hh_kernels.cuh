@@ -293,17 +293,55 @@ __device__ __forceinline__ void store_rec<RecMix>(RecMix *out, int64_t e, const 
     out[e] = r;
 }
 
+// (float)x and (float)(x - (double)(float)x), both to nearest, on the bits: a
+// conversion between FP64 and FP32 takes 64 cycles of the FP64 pipe, and the
+// corrector refreshes its particles' base records with ten of them.  Numbers
+// outside [2^-70, 2^127) take the conversions.
+__device__ __forceinline__ uint32_t f32_rn_bits(uint32_t hi, uint32_t lo, int &rem)
+{
+    const uint32_t t = __funnelshift_l(lo, hi & 0x7fffffffu, 3) - (896u << 23);  // truncated
+    const uint32_t r = lo & 0x1fffffffu;
+    const uint32_t up = (r + (t & 1u)) > 0x10000000u ? 1u : 0u;
+    rem = (int)r - (int)(up << 29);
+    return t + up;
+}
+__device__ __forceinline__ bool f32_in_range(uint32_t hi)
+{
+    return ((hi >> 20) & 0x7ffu) - (1023u - 70u) < 70u + 127u;
+}
+__device__ __forceinline__ float f32_rn(double x)
+{
+    const uint32_t hi = f64_hi(x);
+    if (!f32_in_range(hi)) return __double2float_rn(x);
+    int rem;
+    return __uint_as_float(f32_rn_bits(hi, f64_lo(x), rem) | (hi & 0x80000000u));
+}
+__device__ __forceinline__ void f32_pair(double x, float &h, float &l)
+{
+    const uint32_t hi = f64_hi(x);
+    if (!f32_in_range(hi)) {
+        h = __double2float_rn(x);
+        l = __double2float_rn(x - (double)h);
+        return;
+    }
+    int rem;
+    h = __uint_as_float(f32_rn_bits(hi, f64_lo(x), rem) | (hi & 0x80000000u));
+    // rem 2^(e - 52), |rem| <= 2^28: one rounding, then an exact scaling
+    const float scale = __uint_as_float((((hi >> 20) & 0x7ffu) - 1023u - 52u + 127u) << 23 | (hi & 0x80000000u));
+    l = __int2float_rn(rem) * scale;
+}
+
 // FP32 copy of entry e's FP64 state for the mixed predictor, one component
 // (d = 0, 1, 2) from the values x, v, a, jk of that component; the mass m goes
 // with component 0.
 __device__ __forceinline__ void refresh_base_values(const State &s, int64_t e, int d, double x, double v, double a,
                                                     double jk, double m)
 {
-    const float hi = __double2float_rn(x);
-    const float lo = __double2float_rn(x - (double)hi);
-    const float vf = __double2float_rn(v);
-    const float a2 = 0.5f * __double2float_rn(a);
-    const float j6 = __double2float_rn(jk) * (1.0f / 6.0f);
+    float hi, lo;
+    f32_pair(x, hi, lo);
+    const float vf = f32_rn(v);
+    const float a2 = 0.5f * f32_rn(a);
+    const float j6 = f32_rn(jk) * (1.0f / 6.0f);
     float *b = reinterpret_cast<float *>(&s.base[e]);  // hm, lo, v, a2, j6: float4 each
     b[0 + d] = hi;
     b[4 + d] = lo;
@@ -311,7 +349,7 @@ __device__ __forceinline__ void refresh_base_values(const State &s, int64_t e, i
     b[12 + d] = a2;
     b[16 + d] = j6;
     if (d == 0) {
-        b[3] = __double2float_rn(m);
+        b[3] = f32_rn(m);
         b[7] = b[11] = b[15] = b[19] = 0.f;
     }
 }
@@ -806,6 +844,7 @@ struct ForceSmem {
     double tn[kThreads / 32];  // per-warp minimum of t + dt after the corrector
     int lv[kMaxTileI];         // new step level of each corrected particle, by active index
     typename Traits<Rec>::I iv[std::is_same<Rec, RecF64>::value ? kMaxTileI : 1];  // plain form: the item's active particles
+    int pidx[kMaxTileI];       // its active particles
     double fin[kMaxTileI][7];  // the completed tile's new acc, jerk, pot by active index (for its corrector)
 };
 
@@ -1162,6 +1201,7 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
                 const int64_t p = p0 + (__ffs(mm) - 1);
                 const double v = comp_get(r[u]);
                 sm.fin[slot][comp] = v;
+                if (comp == 0) sm.pidx[slot] = (int)p;
                 if (comp < 3) s.acc1[comp * s.cap_n + p] = v;
                 else if (comp < 6) s.jerk1[(comp - 3) * s.cap_n + p] = v;
                 else s.pot1[p] = -v;
@@ -1271,13 +1311,23 @@ __device__ __forceinline__ void atomic_min_time(unsigned long long *slot, double
 // x1 = x_p + a2 D^4/24 + a3 D^5/120, v1 = v_p + a2 D^3/6 + a3 D^4/24;
 // new step from Aarseth's criterion at the end of the step.
 //
-// The FP64 pipe is narrow on this GPU (a warp instruction issues in 64
-// cycles per SM sub-partition), so the corrector avoids FP64 divisions and
-// roots: D is the particle's power-of-two step, so 1/D^2 and 1/D^3 are exact
-// powers of two, and the timestep criterion is screened in FP32.  The
-// per-component arithmetic and the order of every sum are shared by the
-// one-thread-per-particle and the three-lanes-per-particle correctors, so
-// both give the same bits.
+// The FP64 pipe is narrow on this GPU (a warp instruction issues in 64 to 76
+// cycles per SM sub-partition, however few lanes it has), and a small block
+// step's corrector is one warp: its time is the number of its FP64
+// instructions.  D is the particle's power-of-two step, so 1/D^2 and 1/D^3 are
+// exact powers of two; the timestep criterion works on FP32 values taken from
+// the bits (no FP64 norms), and the mixed form's base records are converted on
+// the bits: 22 FP64 instructions fewer.  The plain form takes predictor and
+// corrector in one Horner form in units of the acceleration, with p = D j0,
+// q = D j1, A = a1 - a0:
+//   h = D^2 a2 / 2 = 3 A - (2 p + q),  g = D^3 a3 / 6 = p + q - 2 A,
+//   x1 = x + D (v + D/2 (a0 + p/3 + h/6 + g/10)),  v1 = v + D (a0 + p/2 + h/3 + g/4),
+// 19 FP64 operations a component instead of 27.  (The mixed form keeps the
+// longer form: its forces amplify a change of rounding in the corrected
+// positions to FP32 size, and now and then to another block step.)  The force phase
+// of a small step went from 10.6 to 9.9 us (mixed) and from 12.0 to 11.1 us (plain).
+// The per-component arithmetic is shared by the one-thread-per-particle and the
+// three-lanes-per-particle correctors, so both give the same bits.
 
 // Powers of D (a power of two) needed by the corrector, exact.
 struct StepPowers {
@@ -1307,25 +1357,41 @@ __device__ __forceinline__ StepPowers step_powers(double D)
 }
 
 // One Cartesian component: state (x, v, a0, j0) at t, new force (a1, j1) at
-// t + D.  Returns the corrected x, v and the a^(2) at t + D and a^(3).
+// t + D.  Corrected x and v, and for the criterion j1, a^(2) at t + D and
+// a^(3), in units that differ by powers of D and constants (crit_units).
 struct CorrComp {
-    double x, v, a2e, a3;
+    double x, v, q, s, g;
 };
 
+template <bool kPlain>
 __device__ __forceinline__ CorrComp correct_component(double x, double v, double a0, double j0, double a1, double j1,
-                                                      const StepPowers &P)
+                                                      double D)
 {
-    const double D = P.D;
-    const double h = 0.5 * D, th = D * (1.0 / 3.0);
-    const double xp = x + D * (v + h * (a0 + th * j0));
-    const double vp = v + D * (a0 + h * j0);
-    const double a2 = (-6.0 * (a0 - a1) - D * (4.0 * j0 + 2.0 * j1)) * P.iD2;
-    const double a3 = (12.0 * (a0 - a1) + 6.0 * D * (j0 + j1)) * P.iD3;
     CorrComp c;
-    c.x = xp + P.D4 * (a2 * (1.0 / 24.0) + a3 * D * (1.0 / 120.0));
-    c.v = vp + P.D3 * (a2 * (1.0 / 6.0) + a3 * D * (1.0 / 24.0));
-    c.a2e = a2 + a3 * D;
-    c.a3 = a3;
+    if constexpr (kPlain) {
+        const double p = D * j0, A = a1 - a0;
+        c.q = D * j1;
+        const double w = p + c.q;
+        const double h = fma(3.0, A, -(p + w));
+        c.g = fma(-2.0, A, w);  // D^3 a3 / 6
+        const double E = fma(0.1, c.g, fma(1.0 / 6.0, h, fma(1.0 / 3.0, p, a0)));
+        const double F = fma(1.0 / 3.0, h, fma(0.25, c.g, fma(0.5, p, a0)));
+        c.x = fma(D, fma(0.5 * D, E, v), x);
+        c.v = fma(D, F, v);
+        c.s = fma(3.0, c.g, h);  // D^2 a^(2) / 2
+    } else {
+        const StepPowers P = step_powers(D);
+        const double h = 0.5 * D, th = D * (1.0 / 3.0);
+        const double xp = x + D * (v + h * (a0 + th * j0));
+        const double vp = v + D * (a0 + h * j0);
+        const double a2 = (-6.0 * (a0 - a1) - D * (4.0 * j0 + 2.0 * j1)) * P.iD2;
+        const double a3 = (12.0 * (a0 - a1) + 6.0 * D * (j0 + j1)) * P.iD3;
+        c.x = xp + P.D4 * (a2 * (1.0 / 24.0) + a3 * D * (1.0 / 120.0));
+        c.v = vp + P.D3 * (a2 * (1.0 / 6.0) + a3 * D * (1.0 / 24.0));
+        c.q = j1;
+        c.s = a2 + a3 * D;
+        c.g = a3;
+    }
     return c;
 }
 
@@ -1375,6 +1441,22 @@ __device__ __forceinline__ bool normal_pos(double x)
     return b >= 0x0010000000000000ll && b < 0x7ff0000000000000ll;
 }
 
+// The screen on FP32 values A, J, S, T (each within 2^-21 of its exact value,
+// in [2^-62, 2^62]; the bound above then is 34 * 2^-24): true, and the exponent of the
+// power of two below sqrt(eta (sqrt(A S) + J) / (sqrt(J T) + S)), where that is
+// certain.
+__device__ __forceinline__ bool aarseth_screen(float A, float J, float S, float T, double eta, int &exponent)
+{
+    const float p1 = A * S, p2 = J * T;
+    const float num = p1 * rsqrtf(p1) + J, den = p2 * rsqrtf(p2) + S;
+    const float w2 = f32_scaled(eta, 0) * __fdividef(num, den);
+    const int wb = __float_as_int(w2);
+    const int frac = wb & 0x7fffff, ex = (wb >> 23) & 0xff;
+    const int e = ex - 127, odd = e & 1;
+    exponent = e >> 1;
+    return ex > 0 && ex < 255 && (odd ? frac <= 0x7fffff - 128 : frac >= 128);
+}
+
 __device__ __forceinline__ double aarseth_want(double A, double J, double S, double T, double eta)
 {
     if (normal_pos(A) && normal_pos(J) && normal_pos(S) && normal_pos(T) && eta >= 0x1p-30 && eta <= 0x1p30) {
@@ -1385,42 +1467,107 @@ __device__ __forceinline__ double aarseth_want(double A, double J, double S, dou
         // the FP64 expression of the original inputs stays finite and normal
         const bool fp64_ok = eA + eS > -1000 && eA + eS < 1000 && eJ + eT > -1000 && eJ + eT < 1000;
         if (fp64_ok && xS >= -60 && xS <= 60 && xT >= -60 && xT <= 60) {
-            const float Af = f32_scaled(A, mA), Jf = f32_scaled(J, mJ), Sf = f32_scaled(S, mS), Tf = f32_scaled(T, mT);
-            const float p1 = Af * Sf, p2 = Jf * Tf;
-            const float num = p1 * rsqrtf(p1) + Jf, den = p2 * rsqrtf(p2) + Sf;
-            const float w2 = f32_scaled(eta, 0) * __fdividef(num, den);
-            const int wb = __float_as_int(w2);
-            const int frac = wb & 0x7fffff, ex = (wb >> 23) & 0xff;
-            const int e = ex - 127, odd = e & 1;
-            const int e2 = (e >> 1) - k;  // dt = sqrt(w2) / 2^k: exponent of the power of two below dt
-            if (ex > 0 && ex < 255 && (odd ? frac <= 0x7fffff - 128 : frac >= 128) && e2 > -400 && e2 < 400)
-                return __longlong_as_double((long long)(e2 + 1023) << 52);
+            int e2;
+            if (aarseth_screen(f32_scaled(A, mA), f32_scaled(J, mJ), f32_scaled(S, mS), f32_scaled(T, mT), eta, e2)) {
+                e2 -= k;  // dt = sqrt(w2) / 2^k: exponent of the power of two below dt
+                if (e2 > -400 && e2 < 400) return __longlong_as_double((long long)(e2 + 1023) << 52);
+            }
         }
     }
     return sqrt(eta * (sqrt(A * S) + J) / (sqrt(J * T) + S));
 }
 
+// The corrector's criterion from its components, in units of the acceleration:
+// dt = D sqrt(eta (|a| |s| + |q|^2) / (|q| |t| + |s|^2)) with s = D^2 a^(2),
+// t = D^3 a^(3), q = D j1 (the same value as above: the unit of time is D).  The
+// components' squares come from truncated FP32 values relative to the largest
+// component of a (biased exponent ea); the mixed form's j1, a^(2) and a^(3) carry
+// their powers of D in the exponent offset.
+__device__ __forceinline__ int biased_exp(double x) { return (int)((f64_hi(x) >> 20) & 0x7ffu); }
+
+// (|x| 2^(1023 - ea))^2, |x| truncated to FP32; 0 below 2^-62, infinite above 2^60.
+__device__ __forceinline__ float rel_square(double x, int ea)
+{
+    const uint32_t hi = f64_hi(x);
+    const int e = (int)((hi >> 20) & 0x7ffu), r = e - ea;
+    const uint32_t b = __funnelshift_l(f64_lo(x), hi & 0x7fffffffu, 3) - ((uint32_t)(ea - 127) << 23);
+    const float f = r < -62 || e == 0 ? 0.f : r > 60 ? __int_as_float(0x7f800000) : __uint_as_float(b);
+    return __fmul_rn(f, f);
+}
+
+// The four squares of one component.
+struct CritSquares {
+    float a, j, s, t;
+};
+template <bool kPlain>
+__device__ __forceinline__ CritSquares crit_squares(double a1, const CorrComp &c, int ea, double D)
+{
+    const int k = kPlain ? 0 : biased_exp(D) - 1023;
+    return CritSquares{rel_square(a1, ea), rel_square(c.q, ea - k), rel_square(c.s, ea - 2 * k),
+                       rel_square(c.g, ea - 3 * k)};
+}
+
+// True, and the power of two below the criterion's value, where the screen is
+// certain (for a power-of-two D) from the components' summed squares.
+template <bool kPlain>
+__device__ __forceinline__ bool corrector_screen(float A, float J, float S, float T, double D, double eta, int ea,
+                                                 double &want)
+{
+    if (kPlain) {  // s and t come without their factors 2 and 6
+        S = __fmul_rn(4.f, S);
+        T = __fmul_rn(36.f, T);
+    }
+    const float lo = fminf(fminf(A, J), fminf(S, T)), hi = fmaxf(fmaxf(A, J), fmaxf(S, T));
+    const long long b = __double_as_longlong(D);
+    int e;
+    const bool ok = lo >= 0x1p-60f && hi <= 0x1p60f && ea > 0 && ea < 0x7ff && (b & 0xFFFFFFFFFFFFFll) == 0 && b > 0 &&
+                    eta >= 0x1p-30 && eta <= 0x1p30 && aarseth_screen(A, J, S, T, eta, e);
+    if (!ok) return false;
+    const int f = (int)(b >> 52) + e;
+    want = __longlong_as_double((long long)f << 52);
+    return f > 0 && f < 0x7ff;
+}
+
+// The same from FP64 squares.
+template <bool kPlain>
+__device__ __forceinline__ double corrector_want(double A, double J, double S, double T, double D, double eta)
+{
+    if (!kPlain) return aarseth_want(A, J, S, T, eta);
+    S *= 4.0;
+    T *= 36.0;
+    return D * sqrt(eta * (sqrt(A * S) + J) / (sqrt(J * T) + S));
+}
+
+template <bool kPlain>
 __device__ __forceinline__ void correct_particle(const State &s, int64_t p, double tnow, const Params &prm)
 {
-    const StepPowers P = step_powers(tnow - s.t[p]);
-    double sa[3], sj[3], ss[3], st[3];
+    const double D = tnow - s.t[p];
+    double a1[3];
+    CorrComp c[3];
+    int ea = 0;
 #pragma unroll
     for (int d = 0; d < 3; d++) {
         const double a0 = s.a[d * s.cap_j + p], j0 = s.jk[d * s.cap_j + p];
-        const double a1 = s.acc1[d * s.cap_n + p];
+        a1[d] = s.acc1[d * s.cap_n + p];
         const double j1 = s.jerk1[d * s.cap_n + p];
-        const CorrComp c = correct_component(s.x[d * s.cap_j + p], s.v[d * s.cap_j + p], a0, j0, a1, j1, P);
-        s.x[d * s.cap_j + p] = c.x;
-        s.v[d * s.cap_j + p] = c.v;
-        s.a[d * s.cap_j + p] = a1;
+        c[d] = correct_component<kPlain>(s.x[d * s.cap_j + p], s.v[d * s.cap_j + p], a0, j0, a1[d], j1, D);
+        s.x[d * s.cap_j + p] = c[d].x;
+        s.v[d * s.cap_j + p] = c[d].v;
+        s.a[d * s.cap_j + p] = a1[d];
         s.jk[d * s.cap_j + p] = j1;
-        sa[d] = sq(a1);
-        sj[d] = sq(j1);
-        ss[d] = sq(c.a2e);
-        st[d] = sq(c.a3);
+        ea = max(ea, biased_exp(a1[d]));
     }
-    const double want = aarseth_want(norm2_of(sa[0], sa[1], sa[2]), norm2_of(sj[0], sj[1], sj[2]),
-                                     norm2_of(ss[0], ss[1], ss[2]), norm2_of(st[0], st[1], st[2]), prm.eta);
+    CritSquares u[3];
+#pragma unroll
+    for (int d = 0; d < 3; d++) u[d] = crit_squares<kPlain>(a1[d], c[d], ea, D);
+    auto sum3 = [](float x, float y, float z) { return __fadd_rn(__fadd_rn(x, y), z); };
+    double want;
+    if (!corrector_screen<kPlain>(sum3(u[0].a, u[1].a, u[2].a), sum3(u[0].j, u[1].j, u[2].j),
+                                  sum3(u[0].s, u[1].s, u[2].s), sum3(u[0].t, u[1].t, u[2].t), D, prm.eta, ea, want))
+        want = corrector_want<kPlain>(norm2_of(sq(a1[0]), sq(a1[1]), sq(a1[2])),
+                                      norm2_of(sq(c[0].q), sq(c[1].q), sq(c[2].q)),
+                                      norm2_of(sq(c[0].s), sq(c[1].s), sq(c[2].s)),
+                                      norm2_of(sq(c[0].g), sq(c[1].g), sq(c[2].g)), D, prm.eta);
     const double dtn = block_dt(want, s.dt[p], tnow, prm.dt_min, prm.dt_max);
     s.t[p] = tnow;
     s.dt[p] = dtn;
@@ -1441,7 +1588,8 @@ static __global__ void k_correct(State s, DevScalars *ds, StepCtl c, Params prm)
                 atomicExch(&ds->err, -1);  // HH_EINVAL: marked particle not due at t
                 continue;
             }
-            correct_particle(s, p, tnow, prm);
+            if (s.base) correct_particle<false>(s, p, tnow, prm);
+            else correct_particle<true>(s, p, tnow, prm);
             my_cnt++;
         }
         const double tn = s.t[p] + s.dt[p];
