@@ -794,7 +794,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_batch(BatchDev B)
                     group_sync(bar);  // the tile's new forces are visible to the group
                     const SimDesc &sdc = s < kSdCache ? sd_all[s] : sd_sm[group];  // copied at the item's start
                     const double tnow = cached_time(sc, B.sims, s, par);
-                    const int4 td = make_int4(it.p_begin, it.p_end, it.group, it.slot);
+                    const int4 td = make_int4(it.p_begin, it.p_end, 0, it.slot);
                     const uint32_t mask = it.mask;
                     // steps of the tile's particles that are not corrected now,
                     // loaded while the corrector runs

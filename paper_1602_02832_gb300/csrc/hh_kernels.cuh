@@ -104,13 +104,14 @@ struct __align__(16) WorkItem {
     int32_t part_sim;  // list part | simulation << 16
     uint32_t mask;     // active lanes of the tile
     int32_t slot;      // first partial-sum slot of the tile's parts (0 with one part)
-    int32_t p_begin, p_end, group;  // the tile's particles and list group
+    int32_t p_begin, p_end;  // the tile's particles
+    int32_t n_parts;         // parts of its list
     int32_t part_len;               // list entries per part of this tile (the last part may be shorter)
     int64_t gb, ge;    // the group's list [gb, ge) in idx
 };
 
 __device__ __forceinline__ WorkItem make_item(int tile, int part_sim, uint32_t mask, int slot, const int4 td, int64_t gb,
-                                              int64_t ge, int part_len)
+                                              int64_t ge, int part_len, int n_parts)
 {
     WorkItem w;
     w.tile = tile;
@@ -119,7 +120,7 @@ __device__ __forceinline__ WorkItem make_item(int tile, int part_sim, uint32_t m
     w.slot = slot;
     w.p_begin = td.x;
     w.p_end = td.y;
-    w.group = td.z;
+    w.n_parts = n_parts;
     w.part_len = part_len;
     w.gb = gb;
     w.ge = ge;
@@ -188,7 +189,12 @@ __device__ __forceinline__ int part_len_for(int n_a, int pj_min, int work)
     return (k < 1 ? 1 : k) * pj_min;
 }
 
-__device__ __forceinline__ int parts_of(int64_t len, int pj) { return len > 0 ? (int)((len + pj - 1) / pj) : 1; }
+// (A list's length fits 32 bits: a 64-bit division would take a microsecond of
+// a step's chain.)
+__device__ __forceinline__ int parts_of(int64_t len, int pj)
+{
+    return len > 0 ? (int)(((uint32_t)len + (uint32_t)pj - 1u) / (uint32_t)pj) : 1;
+}
 
 // Warp-collective: appends one work item per part of tile `tile`'s list;
 // item = (tile, part | sim << 16, active mask, first partial-sum slot, part
@@ -211,7 +217,7 @@ __device__ __forceinline__ void append_tile_items(int tile, const int4 td, int64
     }
     base = __shfl_sync(0xffffffffu, base, 0);
     slot = __shfl_sync(0xffffffffu, slot, 0);
-    for (int q = lane; q < n_parts; q += 32) items[base + q] = make_item(tile, q | (sim << 16), mask, slot, td, gb, ge, pj);
+    for (int q = lane; q < n_parts; q += 32) items[base + q] = make_item(tile, q | (sim << 16), mask, slot, td, gb, ge, pj, n_parts);
 }
 
 __device__ __forceinline__ void select_tiles(const State &s, const Lists &L, DevScalars *ds, const StepCtl &c,
@@ -537,7 +543,7 @@ __device__ __forceinline__ void interact_int(const IF64 &I, const RecF64 &J, boo
 // Mixed: chunk partials in FP32, folded into (hi, lo) pairs after each
 // staged chunk with Knuth's TwoSum, so that the running sum is carried to
 // about 2^-48 relative while the inner loop stays plain FP32.
-struct F2 {
+struct __align__(8) F2 {
     float h, l;
 };
 
@@ -765,10 +771,8 @@ __device__ __forceinline__ double comp_get(const F2 &a) { return (double)a.h + (
 __device__ __forceinline__ double ld_comp_cg(const double *p) { return __ldcg(p); }
 __device__ __forceinline__ F2 ld_comp_cg(const F2 *p)
 {
-    F2 r;
-    r.h = __ldcg(&p->h);
-    r.l = __ldcg(&p->l);
-    return r;
+    const float2 u = __ldcg(reinterpret_cast<const float2 *>(p));
+    return F2{u.x, u.y};
 }
 
 template <typename Rec>
@@ -907,6 +911,11 @@ static __device__ __noinline__ void part_sums_f64(const RecF64 *__restrict__ rec
     to_red(A, out);
 }
 
+// a / b for 0 <= a < 2^14, 0 < b <= 2^8: one reciprocal and a product instead of
+// an integer division's chain, of which a part's path has five ((a + 1/2) / b
+// keeps 2^-9 from every integer, the error is below 2^-16).
+__device__ __forceinline__ int small_div(int a, int b) { return (int)__fdividef((float)a + 0.5f, (float)b); }
+
 // item = (tile, part | sim << 16, active mask, parts of the tile); tid is
 // the thread's index in its 128-thread group.  Returns true (in every thread
 // of the group) for the item that wrote the tile's final forces.
@@ -937,8 +946,8 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
     // N = 65536 went from 3.95 to 3.53 ms.
     constexpr bool kPlain = std::is_same<Rec, RecF64>::value;
     const int I = n_a;
-    const int K = kPlain ? kThreads / I : 32 / I;  // slices of the group (plain), of each warp (mixed)
-    const int islot = (kPlain ? tid : lane) % I, kslice = (kPlain ? tid : lane) / I;
+    const int K = small_div(kPlain ? kThreads : 32, I);  // slices of the group (plain), of each warp (mixed)
+    const int kslice = small_div(kPlain ? tid : lane, I), islot = (kPlain ? tid : lane) - kslice * I;
     const bool idle = kslice >= K;
     const int jslice = kPlain ? kslice : warp * K + kslice;
     const int S = kPlain ? K : (kThreads / 32) * K;
@@ -964,7 +973,7 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
     A.zero();
 
     const int64_t gb = it.gb, ge = it.ge;
-    const int n_parts = parts_of(ge - gb, pj);
+    const int n_parts = it.n_parts;
     const int64_t lb = gb + (int64_t)part * pj;
     const int64_t le = min(ge, lb + (int64_t)pj);
     const int64_t len = le - lb;
@@ -1009,7 +1018,7 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
     int smin = 0;
     if constexpr (kPlain) {
         soft = soft_of(eps2);
-        smin = max(2, 32 - __clz((int)(len / S + 1 + (int64_t)n_chunks)));
+        smin = max(2, 32 - __clz((int)((uint32_t)len / (uint32_t)S + 1u + (uint32_t)n_chunks)));
         A.bad = !soft.ok;
     }
     for (int c = 0; c < n_chunks; c++) {
@@ -1081,16 +1090,16 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
     using E = typename std::remove_reference<decltype(sm.red[0][0].v[0])>::type;
     const int n_out = 7 * n_a;
     const int n_sl = kTreeTail ? K : kThreads / 32;  // terms per output
-    int P = 1;  // (mixed form: one thread per output, warps 0..3 in order)
+    int lgP = 0;  // (mixed form: one thread per output, warps 0..3 in order)
     if (kTreeTail)
-        while (P < 32 && 2 * P * n_out <= kThreads && 2 * P <= n_sl) P <<= 1;
-    const int per = (n_sl + P - 1) / P;
+        while (lgP < 5 && (2 << lgP) * n_out <= kThreads && (2 << lgP) <= n_sl) lgP++;
+    const int P = 1 << lgP, per = (n_sl + P - 1) >> lgP;
     E r[2] = {E{}, E{}};
     bool has[2] = {false, false};
 #pragma unroll
     for (int u = 0; u < 2; u++) {
         const int t = tid + u * kThreads;
-        const int o = t / P, q = t - o * P;
+        const int o = t >> lgP, q = t & (P - 1);
         if ((u == 0 || P == 1) && o < n_out) {
             const int slot = o / 7, comp = o - 7 * slot;
             const int x1 = min(n_sl, (q + 1) * per);
@@ -1121,8 +1130,8 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
     if (P > 1) {
         group_sync(bar_id);
         E *outv = &sm.red[0][0].v[0];
-        const int o = tid / P;
-        if (o < n_out && tid - o * P == 0) outv[o] = r[0];
+        const int o = tid >> lgP;
+        if (o < n_out && (tid & (P - 1)) == 0) outv[o] = r[0];
         group_sync(bar_id);
         if (tid < n_out) r[0] = outv[tid];
     }
@@ -1159,11 +1168,13 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
             E *buf = reinterpret_cast<E *>(&sm.rec[0][0]);
             constexpr int kBuf = (int)(sizeof(sm.rec) / sizeof(E));
             constexpr int kMergeBlock = 8;
-            int blk = kMergeBlock;
-            while ((int64_t)n_out * ((n_parts + blk - 1) / blk) > kBuf) blk *= 2;
-            const int n_blk = (n_parts + blk - 1) / blk;
+            static_assert(kBuf <= (1 << 14), "small_div");
+            static_assert(kMergeBlock == 8, "lgb starts at 3");
+            int lgb = 3;
+            while (n_out * ((n_parts + (1 << lgb) - 1) >> lgb) > kBuf) lgb++;
+            const int blk = 1 << lgb, n_blk = (n_parts + blk - 1) >> lgb;
             for (int x = tid; x < n_out * n_blk; x += kThreads) {
-                const int b = x / n_out, o = x - b * n_out;
+                const int b = small_div(x, n_out), o = x - b * n_out;  // x < kBuf
                 const int q0 = b * blk, q1 = min(n_parts, q0 + blk);
                 const Red *src = base + o / 7;
                 const int comp = o - 7 * (o / 7);
