@@ -28,6 +28,7 @@ namespace {
 
 constexpr int kBits = 21;
 constexpr int kMaxDepth = 21;
+constexpr int kPath = 24;  // entries of a chunk's path (at most kMaxDepth ancestors)
 
 // ------------------------------------------------------------ small helpers
 __device__ __forceinline__ unsigned long long order_bits(double v)  // monotone map double -> u64
@@ -103,7 +104,7 @@ struct Cells {
 struct GCounts {
     int32_t lvl_c0[kMaxDepth + 2];
     int32_t lvl_n[kMaxDepth + 2];
-    int32_t ncells, overflow, bad, G, R, A, pad[2];
+    int32_t ncells, overflow, bad, G;
     int64_t L, n_tiles, total_parts;
     unsigned long long lmax;  // longest list
 };
@@ -119,61 +120,6 @@ struct PCells {
 };
 
 enum : int { kOpen = 0, kEmitParticles = 1, kEmitNode = 2 };
-
-// The opening decision of cell c for group g (rules of hh_tree_build): the
-// group's own cell and single particles go in as particles; a cell that does
-// not contain the group goes in as a node when side < theta * (distance of its
-// centre of mass to the group's box), else as particles when it is a leaf;
-// everything else is opened.
-//
-// The distance test is screened in FP32 (FP64 throughput is low on this part).
-// With X a bound on |coordinates|, rounding centre, box and side to FP32 and
-// evaluating gaps, squares, sum, sqrtf and the product with theta in FP32
-// moves side - theta * distance by less than
-// 2^-21 (side + theta * distance) + 2^-21 theta X; the screen's margin is
-// 2^-18 (side + theta * distance) + 2^-19 theta X.  Inside the margin the test
-// is redone in FP64 with the roundings of the sequential builder (no
-// contraction), so the decision is always the FP64 one.
-struct GroupView {
-    int32_t gc, gb, ge;
-    double lo[3], hi[3];
-    float3 lof, hif;
-};
-
-__device__ __forceinline__ int decide(const State &s, const PCells &P, int64_t n, double theta, float theta_f,
-                                      float tol_abs, const GroupView &G, int32_t c, int4 &pk)
-{
-    // both records are loaded before any test, so that a walk step waits for
-    // one memory round trip, not two (the tables are read-only here)
-    pk = __ldg(&P.pack[c]);
-    const float4 cf = __ldg(&P.cf[c]);
-    if (c == G.gc) return kEmitParticles;
-    if (pk.x <= G.gb && G.ge <= pk.y) return kOpen;
-    if (pk.y - pk.x == 1) return kEmitParticles;
-    const float gx = fmaxf(fmaxf(G.lof.x - cf.x, cf.x - G.hif.x), 0.f);
-    const float gy = fmaxf(fmaxf(G.lof.y - cf.y, cf.y - G.hif.y), 0.f);
-    const float gz = fmaxf(fmaxf(G.lof.z - cf.z, cf.z - G.hif.z), 0.f);
-    const float rhs = theta_f * sqrtf(gx * gx + gy * gy + gz * gz);
-    const float tol = 0x1p-18f * (cf.w + rhs) + tol_abs;
-    bool accept;
-    if (cf.w < rhs - tol) {
-        accept = true;
-    } else if (cf.w > rhs + tol) {
-        accept = false;
-    } else {
-        double d2 = 0.0;
-        for (int d = 0; d < 3; d++) {
-            const double cm = s.x[d * s.cap_j + n + c];
-            double gap = 0.0;
-            if (cm < G.lo[d]) gap = __dsub_rn(G.lo[d], cm);
-            else if (cm > G.hi[d]) gap = __dsub_rn(cm, G.hi[d]);
-            d2 = __dadd_rn(d2, __dmul_rn(gap, gap));
-        }
-        accept = P.side[c] < __dmul_rn(theta, __dsqrt_rn(d2));
-    }
-    if (accept) return kEmitNode;
-    return pk.z == 0 ? kEmitParticles : kOpen;
-}
 
 // Everything a rebuild kernel reads or writes for one simulation.  A kernel
 // runs for one simulation (the record passed by value) or for many (an array
@@ -193,8 +139,8 @@ struct RbSim {
     uint64_t *ckey, *ckey2;   // cell keys (first particle, depth), and sorted
     int32_t *cval, *cval2;    // cell indices, and in key order
     double *mom;              // [13][cap_c] cell sums (BFS order)
-    int32_t *flag3, *pos3;    // [3][ncells] selection flags and their exclusive scan
-    int32_t *g_cell, *cut, *above;
+    int32_t *flag, *pos;      // [ncells + 1] group cells' flags and their exclusive scan
+    int32_t *g_cell;
     double *box_lo, *box_hi;  // [3][G] group boxes
     float4 *box_f;
     int64_t *ids, *ids2;
@@ -203,14 +149,15 @@ struct RbSim {
     int32_t *lidx;            // list entries
     int4 *tiles;
     int64_t *nt2, *tscan2;    // [tile counts | part counts], G + 1 each, and their scan
-    int64_t *pair2, *pscan2;  // [particle | node entries per (group, cut cell)], pairs + 1 each, and their scan
-    int32_t *top;             // [G][A] topmost unopened cell above the cut
+    int64_t *pair2, *pscan2;  // [particle | node entries per (group, chunk)], pairs + 1 each, and their scan
+    int32_t *path;            // [R][kPath] ancestors of each chunk's first cell, from the root (right-aligned)
     DevScalars *ds;           // the context's device sizes (set by k_finish)
     double t, theta;
     float theta_f;
     int64_t n, cap_c, pairs;
     int32_t cap_g, cap_cells, leaf, n_crit, order, tile_i, part_len, work_item, work_split;
-    int32_t ncells, S, G, R, A;  // set by the host as they become known
+    int32_t ncells, G;           // set by the host as they become known
+    int32_t chunk, R;            // cells of a walk chunk, and chunks
 };
 
 #define RB_ARGS const RbSim one, const RbSim *many
@@ -339,7 +286,7 @@ __global__ void k_root_init(RB_ARGS)
     a.C.pre[0] = 0;
     for (int d = 0; d < kMaxDepth + 2; d++) gc->lvl_c0[d] = gc->lvl_n[d] = 0;
     gc->lvl_n[0] = 1;
-    gc->ncells = gc->overflow = gc->bad = gc->G = gc->R = gc->A = 0;
+    gc->ncells = gc->overflow = gc->bad = gc->G = 0;
     gc->lmax = 0ull;
 }
 
@@ -615,75 +562,104 @@ __global__ void k_group_box(RB_ARGS)
     }
 }
 
-// Groups (Barnes 1990): maximal cells with <= n_crit particles (or leaves).
-// Cut through the tree: the maximal cells whose subtree holds <= S cells.
-// They partition the cells at or below the cut; every cell above it is an
-// ancestor of some cut cell.  The three selections at once: flags [groups |
-// cut cells | cells above the cut], each ncells long, in pre-order,
-// compacted by one exclusive scan (positions of the second and third
-// selections are offset by the counts before them).
+// Groups (Barnes 1990): maximal cells with <= n_crit particles (or leaves),
+// flagged in pre-order and compacted by one exclusive scan.
 template <bool kMany>
-__global__ void k_flags3(RB_ARGS)
+__global__ void k_flags(RB_ARGS)
 {
     RB_SIM;
     const PCells &P = a.P;
-    const int32_t ncells = a.ncells, S = a.S;
-    int32_t *flag = a.flag3;
+    const int32_t ncells = a.ncells;
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.flag[ncells] = 0;  // terminal entry of the scan
     for (int32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < ncells; c += gridDim.x * blockDim.x) {
         const int32_t cnt = P.end[c] - P.begin[c];
         const bool small = cnt <= a.n_crit || P.nchild[c] == 0;
         const int32_t par = P.parent[c];
         const bool parent_big = par < 0 || !((P.end[par] - P.begin[par]) <= a.n_crit || P.nchild[par] == 0);
-        flag[c] = (small && parent_big) ? 1 : 0;                                         // group
-        flag[ncells + c] = (P.size[c] <= S && (par < 0 || P.size[par] > S)) ? 1 : 0;     // cut cell
-        flag[2 * ncells + c] = P.size[c] > S ? 1 : 0;                                    // above the cut
+        a.flag[c] = (small && parent_big) ? 1 : 0;
     }
 }
 
-// one thread per simulation
+// The group cells in pre-order (g_cell, group_of) and their number (cells
+// beyond cap_g are not stored: the host reports the overflow).
 template <bool kMany>
-__global__ void k_counts3(RB_ARGS)
+__global__ void k_groups(RB_ARGS)
 {
     RB_SIM;
-    const int32_t *pos = a.pos3, *flag = a.flag3;
-    const int32_t ncells = a.ncells;
-    a.gc->G = pos[ncells] - pos[0];
-    a.gc->R = pos[2 * ncells] - pos[ncells];
-    a.gc->A = pos[3 * ncells - 1] + flag[3 * ncells - 1] - pos[2 * ncells];
-}
-
-// groups (g_cell, group_of), cut cells and cells above the cut, in pre-order
-// (group cells beyond cap_g are not stored: the host reports the overflow)
-template <bool kMany>
-__global__ void k_write3(RB_ARGS)
-{
-    RB_SIM;
-    const int32_t *pos = a.pos3, *flag = a.flag3;
-    const int32_t ncells = a.ncells;
-    const int32_t g0 = pos[0], r0 = pos[ncells], a0 = pos[2 * ncells];
-    for (int32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < ncells; c += gridDim.x * blockDim.x) {
-        if (flag[c]) {
-            const int32_t g = pos[c] - g0;
+    const int32_t ncells = a.ncells, g0 = a.pos[0];
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.gc->G = a.pos[ncells] - g0;
+    for (int32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < ncells; c += gridDim.x * blockDim.x)
+        if (a.flag[c]) {
+            const int32_t g = a.pos[c] - g0;
             if (g < a.cap_g) a.g_cell[g] = c;
             for (int32_t p = a.P.begin[c]; p < a.P.end[c]; p++) a.group_of[p] = g;
         }
-        if (flag[ncells + c]) a.cut[pos[ncells + c] - r0] = c;
-        if (flag[2 * ncells + c]) a.above[pos[2 * ncells + c] - a0] = c;
-    }
 }
 
-// The group's cell, its particle range and its box (FP64 and FP32), as the
-// list walk reads them.
+// The opening decision of cell c for group g (rules of hh_tree_build): the
+// group's own cell and single particles go in as particles; a cell that does
+// not contain the group goes in as a node when side < theta * (distance of its
+// centre of mass to the group's box), else as particles when it is a leaf;
+// everything else is opened.
+//
+// The distance test is screened in FP32 (FP64 throughput is low on this part).
+// With X a bound on |coordinates|, rounding centre, box and side to FP32 and
+// evaluating gaps, squares, sum, sqrtf and the product with theta in FP32
+// moves side - theta * distance by less than
+// 2^-21 (side + theta * distance) + 2^-21 theta X; the screen's margin is
+// 2^-18 (side + theta * distance) + 2^-19 theta X.  Inside the margin the test
+// is redone in FP64 with the roundings of the sequential builder (no
+// contraction), so the decision is always the FP64 one.
+struct GroupView {
+    int32_t g, gc, gb, ge;
+    float3 lof, hif;
+};
+
+__device__ __forceinline__ int decide(const RbSim &a, float tol_abs, const GroupView &G, int32_t c, int4 &pk)
+{
+    // both records are loaded before any test, so that a walk step waits for
+    // one memory round trip, not two (the tables are read-only here)
+    pk = __ldg(&a.P.pack[c]);
+    const float4 cf = __ldg(&a.P.cf[c]);
+    if (c == G.gc) return kEmitParticles;
+    if (pk.x <= G.gb && G.ge <= pk.y) return kOpen;
+    if (pk.y - pk.x == 1) return kEmitParticles;
+    const float gx = fmaxf(fmaxf(G.lof.x - cf.x, cf.x - G.hif.x), 0.f);
+    const float gy = fmaxf(fmaxf(G.lof.y - cf.y, cf.y - G.hif.y), 0.f);
+    const float gz = fmaxf(fmaxf(G.lof.z - cf.z, cf.z - G.hif.z), 0.f);
+    const float rhs = a.theta_f * sqrtf(gx * gx + gy * gy + gz * gz);
+    const float tol = 0x1p-18f * (cf.w + rhs) + tol_abs;
+    bool accept;
+    if (cf.w < rhs - tol) {
+        accept = true;
+    } else if (cf.w > rhs + tol) {
+        accept = false;
+    } else {
+        double d2 = 0.0;
+        for (int d = 0; d < 3; d++) {
+            const double cm = a.st.x[d * a.st.cap_j + a.n + c];
+            const double lo = a.box_lo[d * a.G + G.g], hi = a.box_hi[d * a.G + G.g];
+            double gap = 0.0;
+            if (cm < lo) gap = __dsub_rn(lo, cm);
+            else if (cm > hi) gap = __dsub_rn(cm, hi);
+            d2 = __dadd_rn(d2, __dmul_rn(gap, gap));
+        }
+        accept = a.P.side[c] < __dmul_rn(a.theta, __dsqrt_rn(d2));
+    }
+    if (accept) return kEmitNode;
+    return pk.z == 0 ? kEmitParticles : kOpen;
+}
+
+// The group's cell, its particle range and its FP32 box, as the list walk
+// reads them (the FP64 box only where the screen cannot decide).
 __device__ __forceinline__ GroupView group_view(const RbSim &a, int32_t g)
 {
     GroupView V;
+    V.g = g;
     V.gc = a.g_cell[g];
-    V.gb = a.P.begin[V.gc];
-    V.ge = a.P.end[V.gc];
-    for (int d = 0; d < 3; d++) {
-        V.lo[d] = a.box_lo[d * a.G + g];
-        V.hi[d] = a.box_hi[d * a.G + g];
-    }
+    const int4 pk = __ldg(&a.P.pack[V.gc]);
+    V.gb = pk.x;
+    V.ge = pk.y;
     const float4 l = a.box_f[2 * g], h = a.box_f[2 * g + 1];
     V.lof = make_float3(l.x, l.y, l.z);
     V.hif = make_float3(h.x, h.y, h.z);
@@ -693,111 +669,90 @@ __device__ __forceinline__ GroupView group_view(const RbSim &a, int32_t g)
 // the FP32 screen's absolute margin, 2^-19 theta X
 __device__ __forceinline__ float walk_tol(const RbSim &a) { return 0x1p-19f * a.theta_f * *a.xmax; }
 
-
-// For every (group g, cell above the cut a = above[i]): the topmost cell on
-// the path root -> a that the walk of g does not open (-1: all opened).
-// Cells above the cut are few; this replaces a walk up the tree per
-// (group, cut cell) pair by one table lookup.
+// The ancestors of each chunk's first cell, one thread per chunk: from the
+// root to the parent in path[chunk][..kPath - 1], the entries before the root
+// -1.  (A cell has at most kMaxDepth ancestors.)
 template <bool kMany>
-__global__ void k_top_above(RB_ARGS)
+__global__ void k_paths(RB_ARGS)
 {
     RB_SIM;
-    const float tol = walk_tol(a);
-    const int32_t A = a.A;
-    const int64_t total = int64_t(a.G) * A;
-    // neighbouring threads take neighbouring groups under the same cell: the
-    // same path, similar decisions, coalesced group records
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t i = int32_t(t / a.G), g = int32_t(t - int64_t(i) * a.G);
-        const int64_t q = int64_t(g) * A + i;
-        const GroupView V = group_view(a, g);
-        int32_t top = -1;
-        int4 pk;
-        for (int32_t c = a.above[i]; c >= 0; c = a.P.parent[c])
-            if (decide(a.st, a.P, a.n, a.theta, a.theta_f, tol, V, c, pk) != kOpen) top = c;
-        a.top[q] = top;
+    for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < a.R; k += gridDim.x * blockDim.x) {
+        int32_t *row = a.path + int64_t(k) * kPath;
+        int32_t q = kPath;
+        for (int32_t c = a.P.parent[k * a.chunk]; c >= 0 && q > 0; c = a.P.parent[c]) row[--q] = c;
+        while (q > 0) row[--q] = -1;
     }
 }
 
-// One thread per (group g, cut cell k).  The topmost cell on the path
-// root -> cut[k] that the walk does not open comes from the table of the
-// parent (above the cut) and the decision on cut[k] itself; if there is one,
-// the leftmost cut cell below it emits it (once); otherwise the thread walks
-// the subtree of cut[k] in pre-order, skipping every emitted cell's subtree.
-// The list of a group is then the concatenation over k in pre-order:
+// The list walk, cut into chunks of `chunk` cells in pre-order: one thread per
+// (group, chunk), a warp taking 32 neighbouring groups (close in space) at one
+// chunk, so that its lanes walk nearly the same cells.  A thread first takes
+// the decisions on the ancestors of the chunk's first cell, from the root
+// down, until one is not opened: that cell is emitted by the chunk that holds
+// it, and the walk here goes on behind its subtree (most chunks end there).
+// Then it walks the chunk's cells in pre-order, skipping every emitted cell's
+// subtree.  The list of a group is the concatenation over the chunks:
 // particles ascending, then nodes ascending, as in the sequential walk.
 // Pass 0 counts into cnt_p/cnt_n[g * R + k] (and zeroes both arrays'
 // terminal entries); pass 1 writes at the scanned offsets.  cnt_n follows
 // cnt_p's terminal entry, so one exclusive scan covers both (each read
 // relative to its first entry).
+// Bound by the decisions' latency and by the scattered stores of pass 1.  A
+// thread per (group, subtree of ncells / 256 cells), with a table of the
+// topmost unopened cells above those subtrees, spent most of its time on its
+// start: rebuild of 32 clusters with 1k to 32k particles 775 us (table and
+// counts) and 787 us (entries), here 198 and 404 us; of 262144 particles 583
+// and 730 us, here 427 and 620 us.
 template <bool kMany, bool kWrite>
-__global__ void k_lists_cut(RB_ARGS)
+__global__ void __launch_bounds__(128) k_lists(RB_ARGS)
 {
     RB_SIM;
     const float tol = walk_tol(a);
-    const int32_t R = a.R, A = a.A;
-    const int64_t total = int64_t(a.G) * R;
+    const int32_t R = a.R, n_gb = (a.G + 31) >> 5;
     const int64_t n = a.n;
-    const int32_t *cut = a.cut, *above_pos = a.pos3 + 2 * int64_t(a.ncells);
     int64_t *cnt_p = a.pair2, *cnt_n = a.pair2 + a.pairs + 1;
     const int64_t *scan_p = a.pscan2, *scan_n = a.pscan2 + a.pairs + 1;
-    if (!kWrite && blockIdx.x == 0 && threadIdx.x == 0) cnt_p[total] = cnt_n[total] = 0;
+    if (!kWrite && blockIdx.x == 0 && threadIdx.x == 0) cnt_p[a.pairs] = cnt_n[a.pairs] = 0;
     const int64_t pb = kWrite ? scan_p[0] : 0, nb = kWrite ? scan_n[0] : 0;
-    // neighbouring threads take neighbouring groups (in space too) under the
-    // same cut cell: they walk the same subtree, mostly alike, and read the
-    // same cells; the counts stay indexed by g * R + k
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t k = int32_t(t / a.G), g = int32_t(t - int64_t(k) * a.G);
-        const int64_t q = int64_t(g) * R + k;
-        const int32_t r = cut[k], par = a.P.parent[r];
-        int32_t top = par >= 0 ? a.top[int64_t(g) * A + (above_pos[par] - above_pos[0])] : -1;
-        if (top >= 0 && k > 0 && cut[k - 1] >= top) {  // emitted by an earlier cut cell
-            if (!kWrite) cnt_p[q] = cnt_n[q] = 0;
-            continue;
-        }
+    const int32_t total = R * n_gb, lane = threadIdx.x & 31;
+    const int32_t stride = int32_t(gridDim.x * (blockDim.x >> 5));
+    for (int32_t w = int32_t(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); w < total; w += stride) {
+        const int32_t k = w / n_gb, g = (w - k * n_gb) * 32 + lane;
+        if (g >= a.G) continue;
+        const int32_t *row = a.path + int64_t(k) * kPath;
         const GroupView V = group_view(a, g);
+        const int32_t end = min((k + 1) * a.chunk, a.ncells);
+        int32_t c = k * a.chunk;
+        int4 pk;
+        for (int q = 0; q < kPath; q++) {
+            const int32_t up = __ldg(&row[q]);
+            if (up >= 0 && decide(a, tol, V, up, pk) != kOpen) {
+                c = up + pk.w;
+                break;
+            }
+        }
+        const int64_t q = int64_t(g) * R + k;
         int64_t wp = 0, wn = 0;
-        if (kWrite) {
+        if (kWrite && c < end) {
             wp = (scan_p[q] - pb) + (scan_n[int64_t(g) * R] - nb);
             wn = (scan_p[int64_t(g + 1) * R] - pb) + (scan_n[q] - nb);
         }
-        int64_t np = 0, nn = 0;
-        int4 pk;
-        int top_dec;
-        if (top >= 0) {
-            top_dec = decide(a.st, a.P, n, a.theta, a.theta_f, tol, V, top, pk);
-        } else {
-            top_dec = decide(a.st, a.P, n, a.theta, a.theta_f, tol, V, r, pk);
-            if (top_dec != kOpen) top = r;
-        }
-        if (top >= 0) {
-            if (top_dec == kEmitNode) {
-                if (kWrite) a.lidx[wn] = int32_t(n + top);
-                nn = 1;
+        int32_t np = 0, nn = 0;
+        while (c < end) {
+            const int dec = decide(a, tol, V, c, pk);
+            if (dec == kOpen) {
+                c++;
+                continue;
+            }
+            if (dec == kEmitNode) {
+                if (kWrite) a.lidx[wn++] = int32_t(n + c);
+                nn++;
             } else {
                 if (kWrite)
                     for (int32_t p = pk.x; p < pk.y; p++) a.lidx[wp++] = p;
-                np = pk.y - pk.x;
+                np += pk.y - pk.x;
             }
-        } else {
-            const int32_t end = r + pk.w;
-            int32_t c = r + 1;
-            while (c < end) {
-                const int dec = decide(a.st, a.P, n, a.theta, a.theta_f, tol, V, c, pk);
-                if (dec == kOpen) {
-                    c++;
-                    continue;
-                }
-                if (dec == kEmitNode) {
-                    if (kWrite) a.lidx[wn++] = int32_t(n + c);
-                    nn++;
-                } else {
-                    if (kWrite)
-                        for (int32_t p = pk.x; p < pk.y; p++) a.lidx[wp++] = p;
-                    np += pk.y - pk.x;
-                }
-                c += pk.w;
-            }
+            c += pk.w;
         }
         if (!kWrite) {
             cnt_p[q] = np;
@@ -937,19 +892,19 @@ struct GTreeBuf {
     float4 *box_f = nullptr;
     Cells C{};
     PCells P{};
-    int32_t *flag3 = nullptr, *pos3 = nullptr;  // [3][cap_c] selection flags and their scan
-    int32_t *g_cell = nullptr, *cut = nullptr, *above = nullptr;
+    int32_t *flag = nullptr, *pos = nullptr;  // [cap_c + 1] group cells' flags and their scan
+    int32_t *g_cell = nullptr;
     // [tile counts | part counts] and their one scan, each 2 (G + 1) long
     int64_t *ntile = nullptr, *tile_off = nullptr;
     double *mom = nullptr;                    // [13][cap_c] cell sums (BFS order)
     double *box_lo = nullptr, *box_hi = nullptr;  // [3][cap_g] group boxes
     State alt{};                 // second particle-state buffer for the reordering
     int64_t *ids = nullptr, *ids2 = nullptr;
-    // (group, cut cell) counts and their scans, grown on demand
+    // (group, chunk) counts and their scans, grown on demand
     int64_t *pair_buf = nullptr;
     int64_t pair_cap = 0;
-    int32_t *top_buf = nullptr;  // [G][A] topmost unopened cell above the cut
-    int64_t top_cap = 0;
+    int32_t *path_buf = nullptr;  // [R][kPath] ancestors of the chunks' first cells
+    int64_t path_cap = 0;
     int depth = -1;              // depth of the last tree (-1: none yet)
     void *tmp = nullptr;
     size_t tmp_bytes = 0;
@@ -980,7 +935,7 @@ void hh_gtree_free(GTreeBuf *g)
         if (p) cudaFree(p);
     if (g->tmp) cudaFree(g->tmp);
     if (g->pair_buf) cudaFree(g->pair_buf);
-    if (g->top_buf) cudaFree(g->top_buf);
+    if (g->path_buf) cudaFree(g->path_buf);
     if (g->gc_host) cudaFreeHost(g->gc_host);
     delete g;
 }
@@ -1019,8 +974,8 @@ GTreeBuf *gtree_alloc(hh_ctx *ctx)
               galloc(g, &g->P.nchild, cc) && galloc(g, &g->P.parent, cc) && galloc(g, &g->P.child, 8 * cc) &&
               galloc(g, &g->P.side, cc) && galloc(g, &g->P.size, cc) && galloc(g, &g->P.pack, cc) &&
               galloc(g, &g->P.cf, cc) && galloc(g, &g->xmax, 1) && galloc(g, &g->gc, 1) &&
-              galloc(g, &g->box_f, 2 * ctx->cap_g) && galloc(g, &g->flag3, 3 * cc) && galloc(g, &g->pos3, 3 * cc) &&
-              galloc(g, &g->g_cell, ctx->cap_g) && galloc(g, &g->cut, cc) && galloc(g, &g->above, cc) &&
+              galloc(g, &g->box_f, 2 * ctx->cap_g) && galloc(g, &g->flag, cc + 1) && galloc(g, &g->pos, cc + 1) &&
+              galloc(g, &g->g_cell, ctx->cap_g) &&
               galloc(g, &g->mom, 13 * cc) && galloc(g, &g->box_lo, 3 * ctx->cap_g) &&
               galloc(g, &g->box_hi, 3 * ctx->cap_g) &&
               galloc(g, &g->ntile, 2 * (ctx->cap_g + 1)) && galloc(g, &g->tile_off, 2 * (ctx->cap_g + 1)) &&
@@ -1047,7 +1002,7 @@ GTreeBuf *gtree_alloc(hh_ctx *ctx)
 int64_t gtree_bytes(const hh_ctx *ctx)
 {
     const int64_t n = ctx->cap_n, cc = ctx->cap_j, G = ctx->cap_g + 1;
-    return n * (8 * 2 + 4 * 2 + 8 * 2) + cc * (4 * 8 + 4 * 5 + 32 + 8 + 4 * 8 + 13 * 8 + 32) +
+    return n * (8 * 2 + 4 * 2 + 8 * 2) + cc * (4 * 8 + 4 * 5 + 32 + 8 + 4 * 8 + 13 * 8 + 4 * 2) +
            G * (4 + 8 * 4 + 6 * 8 + 32) + ctx->cap_j * 8 * (12 + 2) + n * 8;
 }
 
@@ -1077,14 +1032,12 @@ RbSim rb_sim(hh_ctx *ctx, GTreeBuf *g, double t)
     // selection arrays, not yet in use when the cells are sorted
     a.ckey = reinterpret_cast<uint64_t *>(g->mom);
     a.ckey2 = a.ckey + g->cap_c;
-    a.cval = g->flag3;
-    a.cval2 = g->pos3;
+    a.cval = g->flag;
+    a.cval2 = g->pos;
     a.mom = g->mom;
-    a.flag3 = g->flag3;
-    a.pos3 = g->pos3;
+    a.flag = g->flag;
+    a.pos = g->pos;
     a.g_cell = g->g_cell;
-    a.cut = g->cut;
-    a.above = g->above;
     a.box_lo = g->box_lo;
     a.box_hi = g->box_hi;
     a.box_f = g->box_f;
@@ -1098,7 +1051,7 @@ RbSim rb_sim(hh_ctx *ctx, GTreeBuf *g, double t)
     a.tscan2 = g->tile_off;
     a.pair2 = g->pair_buf;
     a.pscan2 = nullptr;
-    a.top = g->top_buf;
+    a.path = g->path_buf;
     a.t = t;
     a.theta = ctx->cfg.theta;
     a.theta_f = float(ctx->cfg.theta);
@@ -1179,6 +1132,26 @@ int grow_list(hh_ctx *ctx, int64_t L)
     return HH_OK;
 }
 
+// Cells of a walk chunk: small enough that all (group, chunk) threads fill the
+// chip, large enough that a thread's start (its group's record, the path, one
+// pair of counts) is spread over many cells, and at most about 512 chunks per
+// tree, so that the pair counts stay linear in the groups.  Rebuild of 32
+// clusters with 1k to 32k particles at 32, 128, 256, 512 cells: 2.45, 2.35,
+// 2.40, 2.41 ms; of 262144 particles at 128, 256, 512: 1.92, 1.92, 1.85 ms.
+int32_t walk_chunk(double group_cells, int32_t max_cells)
+{
+    int32_t c = 32;
+    while (c < 512 && group_cells / (2.0 * c) >= 600e3) c *= 2;
+    while (c < max_cells / 512) c *= 2;
+    return c;
+}
+
+// blocks of 4 warps for the walk: a warp per (32 groups, chunk)
+int64_t walk_blocks(int32_t G, int32_t R)
+{
+    return std::max<int64_t>(1, std::min<int64_t>((int64_t((G + 31) / 32) * R + 3) / 4, int64_t(1) << 28));
+}
+
 // bits of a cell key: begin (< 2^b with 2^b > n) above 5 bits of depth
 int cell_key_bits(int64_t n)
 {
@@ -1248,7 +1221,6 @@ int hh_rebuild_device(hh_ctx *ctx, double t)
         return gfail(ctx, HH_ENOMEM, "hh_rebuild: tree exceeds nj_max (more cells than room for nodes)");
     const int32_t ncells = g->gc_host->ncells;
     a.ncells = ncells;
-    a.S = std::max<int32_t>(32, ncells / 256);
     // the deepest level that holds cells: the moment loop runs from there
     int depth = 0;
     for (int d = 0; d <= kMaxDepth; d++)
@@ -1268,42 +1240,37 @@ int hh_rebuild_device(hh_ctx *ctx, double t)
     a.alt = g->alt;
     a.ids = g->ids;
     a.ids2 = g->ids2;
-    // 4. node records (bottom-up moments); groups, and (5.) the cut of
-    //    subtrees of <= S cells and the cells above it: flags, one scan,
-    //    counts and the three compacted tables; group boxes
+    // 4. node records (bottom-up moments); groups (flags, one scan, the
+    //    compacted table) and their boxes
     for (int d = depth; d >= 0; d--) k_moments_level<false><<<grid, 256, 0, st>>>(a, nullptr, d);
     k_node_records<false><<<grid, 256, 0, st>>>(a, nullptr);
-    k_flags3<false><<<grid, 256, 0, st>>>(a, nullptr);
-    if ((rc = cub_exclusive_sum(g->tmp, g->tmp_bytes, g->flag3, g->pos3, 3 * int64_t(ncells), st)))
+    k_flags<false><<<grid, 256, 0, st>>>(a, nullptr);
+    if ((rc = cub_exclusive_sum(g->tmp, g->tmp_bytes, a.flag, a.pos, int64_t(ncells) + 1, st)))
         return gfail(ctx, rc, "hh_rebuild: scan failed");
-    k_counts3<false><<<1, 1, 0, st>>>(a, nullptr);
-    k_write3<false><<<grid, 256, 0, st>>>(a, nullptr);
+    k_groups<false><<<grid, 256, 0, st>>>(a, nullptr);
     k_group_box<false><<<grid, 256, 0, st>>>(a, nullptr);
-    launches += 6 + (depth + 1) + 6;
+    launches += 4 + (depth + 1) + 4;
     if (!read_counts()) return gfail(ctx, HH_ECUDA, "hh_rebuild: group build failed");
-    const int32_t G = g->gc_host->G, R = g->gc_host->R, A = g->gc_host->A;
+    const int32_t G = g->gc_host->G;
     if (G > ctx->cap_g) return gfail(ctx, HH_ENOMEM, "hh_rebuild: more groups than groups_max");
     a.G = G;
-    a.R = R;
-    a.A = A;
-    // then per-(group, cut cell) list counts, one scan, offsets, tiles, write
-    if (!grow(g->top_buf, g->top_cap, std::max<int64_t>(1, int64_t(G) * A)))
+    // 5. per-(group, chunk) list counts, one scan, offsets, tiles, write
+    a.chunk = walk_chunk(double(G) * ncells, ncells);
+    a.R = (ncells + a.chunk - 1) / a.chunk;
+    if (!grow(g->path_buf, g->path_cap, int64_t(a.R) * kPath))
         return gfail(ctx, HH_ENOMEM, "hh_rebuild: list walk table does not fit");
-    a.top = g->top_buf;
-    if (A > 0) {
-        k_top_above<false><<<unsigned((int64_t(G) * A + 127) / 128), 128, 0, st>>>(a, nullptr);
-        launches++;
-    }
-    const int64_t pairs = int64_t(G) * R;
+    a.path = g->path_buf;
+    k_paths<false><<<(a.R + 127) / 128, 128, 0, st>>>(a, nullptr);
+    const int64_t pairs = int64_t(G) * a.R;
     if (2 * (pairs + 1) >= int64_t(INT32_MAX))  // (one scan covers both count arrays)
-        return gfail(ctx, HH_ENOMEM, "hh_rebuild: too many (group, subtree) pairs");
+        return gfail(ctx, HH_ENOMEM, "hh_rebuild: too many (group, chunk) pairs");
     if (!grow(g->pair_buf, g->pair_cap, 4 * (pairs + 1)))
         return gfail(ctx, HH_ENOMEM, "hh_rebuild: list count buffers do not fit");
     a.pairs = pairs;
     a.pair2 = g->pair_buf;
     a.pscan2 = g->pair_buf + 2 * (pairs + 1);
-    const int64_t lgrid = std::min<int64_t>((pairs + 127) / 128, int64_t(1) << 30);
-    k_lists_cut<false, false><<<unsigned(lgrid), 128, 0, st>>>(a, nullptr);
+    const int64_t lgrid = walk_blocks(G, a.R);
+    k_lists<false, false><<<unsigned(lgrid), 128, 0, st>>>(a, nullptr);
     if ((rc = cub_exclusive_sum(g->tmp, g->tmp_bytes, a.pair2, a.pscan2, 2 * (pairs + 1), st)))  // cnt_p, cnt_n at once
         return gfail(ctx, rc, "hh_rebuild: scan failed");
     k_list_off<false><<<grid, 256, 0, st>>>(a, nullptr);
@@ -1312,13 +1279,13 @@ int hh_rebuild_device(hh_ctx *ctx, double t)
     if ((rc = cub_exclusive_sum(g->tmp, g->tmp_bytes, g->ntile, g->tile_off, 2 * (int64_t(G) + 1), st)))
         return gfail(ctx, rc, "hh_rebuild: scan failed");
     k_store_totals<false><<<1, 1, 0, st>>>(a, nullptr);
-    launches += 4;
+    launches += 5;
     if (!read_counts()) return gfail(ctx, HH_ECUDA, "hh_rebuild: list count failed");
     const int64_t L = g->gc_host->L, n_tiles = g->gc_host->n_tiles, total_parts = g->gc_host->total_parts;
     if (n_tiles > ctx->cap_tiles) return gfail(ctx, HH_ENOMEM, "hh_rebuild: too many tiles");
     if ((rc = grow_list(ctx, L))) return rc;
     a.lidx = ctx->idx;
-    k_lists_cut<false, true><<<unsigned(lgrid), 128, 0, st>>>(a, nullptr);
+    k_lists<false, true><<<unsigned(lgrid), 128, 0, st>>>(a, nullptr);
     k_tiles<false><<<grid, 256, 0, st>>>(a, nullptr);
     launches += 2;
     const cudaError_t ce = cudaGetLastError();
@@ -1349,12 +1316,12 @@ struct RbScratch {
     uint64_t *ckey = nullptr, *ckey2 = nullptr;
     int32_t *cval = nullptr, *cval2 = nullptr;
     int64_t cap_ckey = 0, cap_ckey2 = 0, cap_cval = 0, cap_cval2 = 0;
-    int32_t *flag3 = nullptr, *pos3 = nullptr;
-    int64_t cap_flag3 = 0, cap_pos3 = 0;
+    int32_t *flag = nullptr, *pos = nullptr;
+    int64_t cap_flag = 0, cap_pos = 0;
     int64_t *pair2 = nullptr, *pscan2 = nullptr;
     int64_t cap_pair2 = 0, cap_pscan2 = 0;
-    int32_t *top = nullptr;
-    int64_t cap_top = 0;
+    int32_t *path = nullptr;
+    int64_t cap_path = 0;
     int64_t *nt2 = nullptr, *tscan2 = nullptr;
     int64_t cap_nt2 = 0, cap_tscan2 = 0;
     void *tmp = nullptr;
@@ -1446,8 +1413,8 @@ void hh_rb_scratch_free(RbScratch *r)
     cudaStreamSynchronize(r->stream);
     rb_free_sims(r);
     for (void *p : {(void *)r->key, (void *)r->key2, (void *)r->idx, (void *)r->perm, (void *)r->ckey,
-                    (void *)r->ckey2, (void *)r->cval, (void *)r->cval2, (void *)r->flag3, (void *)r->pos3,
-                    (void *)r->pair2, (void *)r->pscan2, (void *)r->top, (void *)r->nt2, (void *)r->tscan2, r->tmp})
+                    (void *)r->ckey2, (void *)r->cval, (void *)r->cval2, (void *)r->flag, (void *)r->pos,
+                    (void *)r->pair2, (void *)r->pscan2, (void *)r->path, (void *)r->nt2, (void *)r->tscan2, r->tmp})
         if (p) cudaFree(p);
     cudaStreamDestroy(r->stream);
     delete r;
@@ -1585,13 +1552,14 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
     });
     if (act.empty()) return HH_OK;
     // 2. one segmented cell sort, pre-order, reordering, moments, node
-    //    records, the three selections (one scan), group boxes
+    //    records, groups (one scan), group boxes
     int64_t tcells = 0;
     if (!segments(1, [&](size_t q) { return int64_t(cnt(q).ncells); }, &tcells))
         return fail_all(HH_ENOMEM, "hh_rebuild: batch too large");
     if (!rb_grow(r->ckey, r->cap_ckey, tcells) || !rb_grow(r->ckey2, r->cap_ckey2, tcells) ||
         !rb_grow(r->cval, r->cap_cval, tcells) || !rb_grow(r->cval2, r->cap_cval2, tcells) ||
-        !rb_grow(r->flag3, r->cap_flag3, 3 * tcells) || !rb_grow(r->pos3, r->cap_pos3, 3 * tcells))
+        !rb_grow(r->flag, r->cap_flag, tcells + int64_t(act.size())) ||
+        !rb_grow(r->pos, r->cap_pos, tcells + int64_t(act.size())))
         return fail_all(HH_ENOMEM, "hh_rebuild: batch cell buffers do not fit");
     const int32_t *hs1 = r->h_seg + (r->cap_sims + 1);
     int depth = 0;
@@ -1599,7 +1567,6 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
         RbSim &a = H(int(q));
         GTreeBuf *g = ctxs[act[q]]->gtree;
         a.ncells = cnt(q).ncells;
-        a.S = std::max<int32_t>(32, a.ncells / 256);
         int dq = 0;
         for (int d = 0; d <= kMaxDepth; d++)
             if (cnt(q).lvl_n[d] > 0) dq = d;
@@ -1610,8 +1577,8 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
         a.ckey2 = r->ckey2 + o;
         a.cval = r->cval + o;
         a.cval2 = r->cval2 + o;
-        a.flag3 = r->flag3 + 3 * o;
-        a.pos3 = r->pos3 + 3 * o;
+        a.flag = r->flag + o + int64_t(q);  // (a terminal entry each)
+        a.pos = r->pos + o + int64_t(q);
     }
     const int K2 = int(act.size());
     const dim3 g2 = dim3(unsigned(gx), unsigned(K2)), one2(1, unsigned(K2));
@@ -1637,13 +1604,12 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
     if (!upload()) return fail_all(HH_ECUDA, "hh_rebuild: batch upload failed");
     for (int d = depth; d >= 0; d--) k_moments_level<true><<<g2, 256, 0, st>>>(RbSim{}, D(), d);
     k_node_records<true><<<g2, 256, 0, st>>>(RbSim{}, D());
-    k_flags3<true><<<g2, 256, 0, st>>>(RbSim{}, D());
-    if ((rc = cub_exclusive_sum(r->tmp, r->tmp_bytes, r->flag3, r->pos3, 3 * tcells, st)))
+    k_flags<true><<<g2, 256, 0, st>>>(RbSim{}, D());
+    if ((rc = cub_exclusive_sum(r->tmp, r->tmp_bytes, r->flag, r->pos, tcells + int64_t(K2), st)))
         return fail_all(rc, "hh_rebuild: batch scan failed");
-    k_counts3<true><<<one2, 1, 0, st>>>(RbSim{}, D());
-    k_write3<true><<<g2, 256, 0, st>>>(RbSim{}, D());
+    k_groups<true><<<g2, 256, 0, st>>>(RbSim{}, D());
     k_group_box<true><<<dim3(unsigned(gx_full), unsigned(K2)), 256, 0, st>>>(RbSim{}, D());
-    launches += 6 + (depth + 1) + 6;
+    launches += 4 + (depth + 1) + 4;
     if (!read_counts()) return fail_all(HH_ECUDA, "hh_rebuild: group build failed");
     next_stage([&](size_t q) {
         if (cnt(q).G > ctxs[act[q]]->cap_g) {
@@ -1653,34 +1619,40 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
         return true;
     });
     if (act.empty()) return HH_OK;
-    // 3. per-(group, cut cell) list counts (one scan), offsets, tiles (one scan)
-    int64_t t_top = 0, t_pair = 0, t_nt = 0, tgrid = 1, lgrid = 1;
+    // 3. per-(group, chunk) list counts (one scan), offsets, tiles (one scan)
+    int64_t t_path = 0, t_pair = 0, t_nt = 0, lgrid = 1;
+    int32_t max_cells = 0, max_R = 1;
+    double group_cells = 0.0;
+    for (size_t q = 0; q < act.size(); q++) {
+        group_cells += double(cnt(q).G) * cnt(q).ncells;
+        max_cells = std::max(max_cells, cnt(q).ncells);
+    }
     for (size_t q = 0; q < act.size(); q++) {
         RbSim &a = H(int(q));
         a.G = cnt(q).G;
-        a.R = cnt(q).R;
-        a.A = cnt(q).A;
+        a.chunk = walk_chunk(group_cells, max_cells);
+        a.R = (a.ncells + a.chunk - 1) / a.chunk;
         a.pairs = int64_t(a.G) * a.R;
-        a.top = reinterpret_cast<int32_t *>(t_top);  // offsets for now
+        a.path = reinterpret_cast<int32_t *>(t_path);  // offsets for now
         a.pair2 = reinterpret_cast<int64_t *>(t_pair);
         a.nt2 = reinterpret_cast<int64_t *>(t_nt);
-        t_top += std::max<int64_t>(1, int64_t(a.G) * a.A);
+        t_path += int64_t(a.R) * kPath;
         t_pair += 2 * (a.pairs + 1);
         t_nt += 2 * (int64_t(a.G) + 1);
-        tgrid = std::max<int64_t>(tgrid, (int64_t(a.G) * a.A + 127) / 128);
-        lgrid = std::max<int64_t>(lgrid, (a.pairs + 127) / 128);
+        max_R = std::max(max_R, a.R);
+        lgrid = std::max<int64_t>(lgrid, walk_blocks(a.G, a.R));
     }
     if (t_pair >= int64_t(INT32_MAX) || t_nt >= int64_t(INT32_MAX))  // (one CUB scan each)
-        return fail_all(HH_ENOMEM, "hh_rebuild: too many (group, subtree) pairs in one batch");
-    if (!rb_grow(r->top, r->cap_top, t_top) || !rb_grow(r->pair2, r->cap_pair2, t_pair) ||
+        return fail_all(HH_ENOMEM, "hh_rebuild: too many (group, chunk) pairs in one batch");
+    if (!rb_grow(r->path, r->cap_path, t_path) || !rb_grow(r->pair2, r->cap_pair2, t_pair) ||
         !rb_grow(r->pscan2, r->cap_pscan2, t_pair) || !rb_grow(r->nt2, r->cap_nt2, t_nt) ||
         !rb_grow(r->tscan2, r->cap_tscan2, t_nt))
         return fail_all(HH_ENOMEM, "hh_rebuild: batch list buffers do not fit");
     for (size_t q = 0; q < act.size(); q++) {
         RbSim &a = H(int(q));
-        const int64_t o_top = reinterpret_cast<int64_t>(a.top), o_pair = reinterpret_cast<int64_t>(a.pair2),
+        const int64_t o_path = reinterpret_cast<int64_t>(a.path), o_pair = reinterpret_cast<int64_t>(a.pair2),
                       o_nt = reinterpret_cast<int64_t>(a.nt2);
-        a.top = r->top + o_top;
+        a.path = r->path + o_path;
         a.pair2 = r->pair2 + o_pair;
         a.pscan2 = r->pscan2 + o_pair;
         a.nt2 = r->nt2 + o_nt;
@@ -1688,11 +1660,10 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
     }
     const int K3 = int(act.size());
     const dim3 g3 = dim3(unsigned(gx), unsigned(K3)), one3(1, unsigned(K3));
-    const dim3 lg3(unsigned(std::min<int64_t>(lgrid, int64_t(1) << 30)), unsigned(K3));
+    const dim3 lg3 = dim3(unsigned(lgrid), unsigned(K3));
     if (!upload()) return fail_all(HH_ECUDA, "hh_rebuild: batch upload failed");
-    k_top_above<true><<<dim3(unsigned(std::min<int64_t>(tgrid, int64_t(1) << 30)), unsigned(K3)), 128, 0, st>>>(
-        RbSim{}, D());
-    k_lists_cut<true, false><<<lg3, 128, 0, st>>>(RbSim{}, D());
+    k_paths<true><<<dim3(unsigned((max_R + 127) / 128), unsigned(K3)), 128, 0, st>>>(RbSim{}, D());
+    k_lists<true, false><<<lg3, 128, 0, st>>>(RbSim{}, D());
     if ((rc = cub_exclusive_sum(r->tmp, r->tmp_bytes, r->pair2, r->pscan2, t_pair, st)))
         return fail_all(rc, "hh_rebuild: batch scan failed");
     k_list_off<true><<<g3, 256, 0, st>>>(RbSim{}, D());
@@ -1716,9 +1687,9 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
     for (size_t q = 0; q < act.size(); q++) H(int(q)).lidx = ctxs[act[q]]->idx;
     const int K4 = int(act.size());
     const dim3 g4 = dim3(unsigned(gx), unsigned(K4));
-    const dim3 lg4(unsigned(std::min<int64_t>(lgrid, int64_t(1) << 30)), unsigned(K4));
+    const dim3 lg4 = dim3(unsigned(lgrid), unsigned(K4));
     if (!upload()) return fail_all(HH_ECUDA, "hh_rebuild: batch upload failed");
-    k_lists_cut<true, true><<<lg4, 128, 0, st>>>(RbSim{}, D());
+    k_lists<true, true><<<lg4, 128, 0, st>>>(RbSim{}, D());
     k_tiles<true><<<g4, 256, 0, st>>>(RbSim{}, D());
     launches += 2;
     const cudaError_t ce = cudaGetLastError();
