@@ -113,8 +113,8 @@ struct GCounts {
 struct PCells {
     int32_t *begin, *end, *nchild, *parent;
     int32_t *size;   // cells in the subtree: the subtree of p is [p, p + size)
-    int4 *pack;      // {begin, end, nchild, size}: what the list walk reads per cell
-    float4 *cf;      // {centre of mass x, y, z, side} rounded to FP32 (screening)
+    int4 *pack;      // {begin, end, FP32 bits of the reject bound, size}: what the list walk reads per cell
+    float4 *cf;      // {centre of mass x, y, z in the tree's unit, accept bound}
     int32_t *child;  // [8 * n]
     double *side;
 };
@@ -133,7 +133,7 @@ struct RbSim {
     GCounts *gc;
     Box *box;
     double *root_side;
-    float *xmax;
+    double *unit;             // power of two that brings every |coordinate| below 1
     uint64_t *key, *key2;     // particle keys, and sorted
     int32_t *idx, *perm;      // particle indices, and in key order
     uint64_t *ckey, *ckey2;   // cell keys (first particle, depth), and sorted
@@ -153,7 +153,6 @@ struct RbSim {
     int32_t *path;            // [R][kPath] ancestors of each chunk's first cell, from the root (right-aligned)
     DevScalars *ds;           // the context's device sizes (set by k_finish)
     double t, theta;
-    float theta_f;
     int64_t n, cap_c, pairs;
     int32_t cap_g, cap_cells, leaf, n_crit, order, tile_i, part_len, work_item, work_split;
     int32_t ncells, G;           // set by the host as they become known
@@ -251,7 +250,9 @@ __global__ void k_keys(RB_ARGS)
         *a.root_side = side;
         double xm = 0.0;  // bound on |coordinate| of every particle, node and group box
         for (int d = 0; d < 3; d++) xm = fmax(xm, fmax(fabs(lo[d]), fabs(from_order_bits(b->hi[d]))));
-        *a.xmax = float(xm) * 1.0001f;
+        int e = 0;
+        if (xm > 0.0) frexp(xm, &e);
+        *a.unit = ldexp(1.0, min(max(-e, -1000), 1000));
     }
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * blockDim.x) {
         uint32_t u[3];
@@ -427,7 +428,6 @@ __global__ void k_to_preorder(RB_ARGS)
         P.end[p] = C.end[c];
         P.nchild[p] = C.nchild[c];
         P.size[p] = C.size[c];
-        P.pack[p] = make_int4(C.begin[c], C.end[c], C.nchild[c], C.size[c]);
         P.parent[p] = C.parent[c] >= 0 ? C.pre[C.parent[c]] : -1;
         double side = s0;
         for (int d = 0; d < C.depth[c]; d++) side *= 0.5;
@@ -520,7 +520,16 @@ __global__ void k_node_records(RB_ARGS)
             s.a[d * s.cap_j + j] = mom[(7 + d) * cap + c] / M;
             s.jk[d * s.cap_j + j] = mom[(10 + d) * cap + c] / M;
         }
-        a.P.cf[p] = make_float4(float(x[0]), float(x[1]), float(x[2]), float(a.P.side[p]));
+        // what the list walk reads of the cell: its FP32 centre and bounds on
+        // the squared distance (see decide)
+        const double u = *a.unit, side = a.P.side[p] * u, tol = 0x1p-19 * a.theta;
+        const double far = (side * (1.0 + 0x1p-17) + tol) / a.theta, near = (side * (1.0 - 0x1p-17) - tol) / a.theta;
+        const int32_t b = a.C.begin[c], e = a.C.end[c];
+        float hi = __double2float_ru(far * far * (1.0 + 0x1p-20));
+        float lo = near > 0.0 ? __double2float_rd(near * near * (1.0 - 0x1p-20)) : -1.0f;
+        if (e - b == 1) hi = lo = __int_as_float(0x7f800000);  // a single particle always goes in as such
+        a.P.cf[p] = make_float4(float(x[0] * u), float(x[1] * u), float(x[2] * u), hi);
+        a.P.pack[p] = make_int4(b, e, __float_as_int(lo), a.C.size[c]);
     }
 }
 
@@ -555,9 +564,11 @@ __global__ void k_group_box(RB_ARGS)
             }
         }
         if (lane == 0) {
-            a.box_f[2 * g] = make_float4(float(a.box_lo[g]), float(a.box_lo[G + g]), float(a.box_lo[2 * G + g]), 0.f);
-            a.box_f[2 * g + 1] =
-                make_float4(float(a.box_hi[g]), float(a.box_hi[G + g]), float(a.box_hi[2 * G + g]), 0.f);
+            const double u = *a.unit;
+            a.box_f[2 * g] = make_float4(float(a.box_lo[g] * u), float(a.box_lo[G + g] * u),
+                                         float(a.box_lo[2 * G + g] * u), 0.f);
+            a.box_f[2 * g + 1] = make_float4(float(a.box_hi[g] * u), float(a.box_hi[G + g] * u),
+                                             float(a.box_hi[2 * G + g] * u), 0.f);
         }
     }
 }
@@ -602,39 +613,45 @@ __global__ void k_groups(RB_ARGS)
 // centre of mass to the group's box), else as particles when it is a leaf;
 // everything else is opened.
 //
-// The distance test is screened in FP32 (FP64 throughput is low on this part).
-// With X a bound on |coordinates|, rounding centre, box and side to FP32 and
-// evaluating gaps, squares, sum, sqrtf and the product with theta in FP32
-// moves side - theta * distance by less than
-// 2^-21 (side + theta * distance) + 2^-21 theta X; the screen's margin is
-// 2^-18 (side + theta * distance) + 2^-19 theta X.  Inside the margin the test
-// is redone in FP64 with the roundings of the sequential builder (no
-// contraction), so the decision is always the FP64 one.
+// The distance test is screened in FP32 (FP64 throughput is low on this part),
+// with two bounds on the squared distance that each cell carries (node
+// records), in the tree's unit: the power of two that brings every
+// |coordinate| below 1, so that no square leaves FP32's range.  Rounding centre
+// and box to FP32 and taking gaps, squares and sum in FP32 moves the distance
+// by less than 2^-21 + 2^-22 distance.  A cell is accepted above
+// ((1 + 2^-17) side + 2^-19 theta)^2 / theta^2 (and 2^-20 more, rounded up) and
+// not accepted below ((1 - 2^-17) side - 2^-19 theta)^2 / theta^2 (and 2^-20
+// less, rounded down; never when that difference is negative), which covers
+// those errors and the roundings of the FP64 test.  Between the bounds (and for
+// any NaN) the test is redone in FP64 with the roundings of the sequential
+// builder (no contraction), so the decision is always the FP64 one.  A single
+// particle carries infinite bounds: it is a leaf and goes in as a particle.
+// (With the two bounds instead of a square root and a tolerance per decision,
+// the walk's counts of 262144 particles take 339 us, 427 before.)
 struct GroupView {
     int32_t g, gc, gb, ge;
     float3 lof, hif;
 };
 
-__device__ __forceinline__ int decide(const RbSim &a, float tol_abs, const GroupView &G, int32_t c, int4 &pk)
+struct CellRec {
+    int4 pk;
+    float4 cf;
+};
+
+__device__ __forceinline__ CellRec load_cell(const RbSim &a, int32_t c)
 {
-    // both records are loaded before any test, so that a walk step waits for
-    // one memory round trip, not two (the tables are read-only here)
-    pk = __ldg(&a.P.pack[c]);
-    const float4 cf = __ldg(&a.P.cf[c]);
-    if (c == G.gc) return kEmitParticles;
-    if (pk.x <= G.gb && G.ge <= pk.y) return kOpen;
-    if (pk.y - pk.x == 1) return kEmitParticles;
-    const float gx = fmaxf(fmaxf(G.lof.x - cf.x, cf.x - G.hif.x), 0.f);
-    const float gy = fmaxf(fmaxf(G.lof.y - cf.y, cf.y - G.hif.y), 0.f);
-    const float gz = fmaxf(fmaxf(G.lof.z - cf.z, cf.z - G.hif.z), 0.f);
-    const float rhs = a.theta_f * sqrtf(gx * gx + gy * gy + gz * gz);
-    const float tol = 0x1p-18f * (cf.w + rhs) + tol_abs;
-    bool accept;
-    if (cf.w < rhs - tol) {
-        accept = true;
-    } else if (cf.w > rhs + tol) {
-        accept = false;
-    } else {
+    return {__ldg(&a.P.pack[c]), __ldg(&a.P.cf[c])};
+}
+
+__device__ __forceinline__ int decide(const RbSim &a, const GroupView &G, int32_t c, const CellRec &r)
+{
+    if (r.pk.x <= G.gb && G.ge <= r.pk.y) return c == G.gc ? kEmitParticles : kOpen;
+    const float gx = fmaxf(fmaxf(G.lof.x - r.cf.x, r.cf.x - G.hif.x), 0.f);
+    const float gy = fmaxf(fmaxf(G.lof.y - r.cf.y, r.cf.y - G.hif.y), 0.f);
+    const float gz = fmaxf(fmaxf(G.lof.z - r.cf.z, r.cf.z - G.hif.z), 0.f);
+    const float d2f = gx * gx + gy * gy + gz * gz;
+    bool accept = d2f > r.cf.w;
+    if (!accept && !(d2f < __int_as_float(r.pk.z))) {
         double d2 = 0.0;
         for (int d = 0; d < 3; d++) {
             const double cm = a.st.x[d * a.st.cap_j + a.n + c];
@@ -647,7 +664,7 @@ __device__ __forceinline__ int decide(const RbSim &a, float tol_abs, const Group
         accept = a.P.side[c] < __dmul_rn(a.theta, __dsqrt_rn(d2));
     }
     if (accept) return kEmitNode;
-    return pk.z == 0 ? kEmitParticles : kOpen;
+    return r.pk.w == 1 ? kEmitParticles : kOpen;  // (only a leaf is its whole subtree)
 }
 
 // The group's cell, its particle range and its FP32 box, as the list walk
@@ -665,9 +682,6 @@ __device__ __forceinline__ GroupView group_view(const RbSim &a, int32_t g)
     V.hif = make_float3(h.x, h.y, h.z);
     return V;
 }
-
-// the FP32 screen's absolute margin, 2^-19 theta X
-__device__ __forceinline__ float walk_tol(const RbSim &a) { return 0x1p-19f * a.theta_f * *a.xmax; }
 
 // The ancestors of each chunk's first cell, one thread per chunk: from the
 // root to the parent in path[chunk][..kPath - 1], the entries before the root
@@ -701,13 +715,14 @@ __global__ void k_paths(RB_ARGS)
 // thread per (group, subtree of ncells / 256 cells), with a table of the
 // topmost unopened cells above those subtrees, spent most of its time on its
 // start: rebuild of 32 clusters with 1k to 32k particles 775 us (table and
-// counts) and 787 us (entries), here 198 and 404 us; of 262144 particles 583
-// and 730 us, here 427 and 620 us.
+// counts) and 787 us (entries), here 180 and 328 us; of 262144 particles 583
+// and 730 us, here 339 and 570 us.  (Gathering each lane's entries into 16-byte
+// stores made it slower, 796 us: it is bound by instructions issued, not by
+// the stores.)
 template <bool kMany, bool kWrite>
 __global__ void __launch_bounds__(128) k_lists(RB_ARGS)
 {
     RB_SIM;
-    const float tol = walk_tol(a);
     const int32_t R = a.R, n_gb = (a.G + 31) >> 5;
     const int64_t n = a.n;
     int64_t *cnt_p = a.pair2, *cnt_n = a.pair2 + a.pairs + 1;
@@ -723,11 +738,12 @@ __global__ void __launch_bounds__(128) k_lists(RB_ARGS)
         const GroupView V = group_view(a, g);
         const int32_t end = min((k + 1) * a.chunk, a.ncells);
         int32_t c = k * a.chunk;
-        int4 pk;
         for (int q = 0; q < kPath; q++) {
             const int32_t up = __ldg(&row[q]);
-            if (up >= 0 && decide(a, tol, V, up, pk) != kOpen) {
-                c = up + pk.w;
+            if (up < 0) continue;
+            const CellRec r = load_cell(a, up);
+            if (decide(a, V, up, r) != kOpen) {
+                c = up + r.pk.w;
                 break;
             }
         }
@@ -739,20 +755,17 @@ __global__ void __launch_bounds__(128) k_lists(RB_ARGS)
         }
         int32_t np = 0, nn = 0;
         while (c < end) {
-            const int dec = decide(a, tol, V, c, pk);
-            if (dec == kOpen) {
-                c++;
-                continue;
-            }
+            const CellRec r = load_cell(a, c);
+            const int dec = decide(a, V, c, r);
             if (dec == kEmitNode) {
                 if (kWrite) a.lidx[wn++] = int32_t(n + c);
                 nn++;
-            } else {
+            } else if (dec == kEmitParticles) {
                 if (kWrite)
-                    for (int32_t p = pk.x; p < pk.y; p++) a.lidx[wp++] = p;
-                np += pk.y - pk.x;
+                    for (int32_t p = r.pk.x; p < r.pk.y; p++) a.lidx[wp++] = p;
+                np += r.pk.y - r.pk.x;
             }
-            c += pk.w;
+            c += dec == kOpen ? 1 : r.pk.w;
         }
         if (!kWrite) {
             cnt_p[q] = np;
@@ -886,7 +899,7 @@ struct GTreeBuf {
     int32_t *idx = nullptr, *perm = nullptr;
     Box *box = nullptr;
     double *root_side = nullptr;
-    float *xmax = nullptr;
+    double *unit = nullptr;
     GCounts *gc = nullptr;      // device
     GCounts *gc_host = nullptr;  // pinned mirror
     float4 *box_f = nullptr;
@@ -973,7 +986,7 @@ GTreeBuf *gtree_alloc(hh_ctx *ctx)
               galloc(g, &g->C.pre, cc) && galloc(g, &g->P.begin, cc) && galloc(g, &g->P.end, cc) &&
               galloc(g, &g->P.nchild, cc) && galloc(g, &g->P.parent, cc) && galloc(g, &g->P.child, 8 * cc) &&
               galloc(g, &g->P.side, cc) && galloc(g, &g->P.size, cc) && galloc(g, &g->P.pack, cc) &&
-              galloc(g, &g->P.cf, cc) && galloc(g, &g->xmax, 1) && galloc(g, &g->gc, 1) &&
+              galloc(g, &g->P.cf, cc) && galloc(g, &g->unit, 1) && galloc(g, &g->gc, 1) &&
               galloc(g, &g->box_f, 2 * ctx->cap_g) && galloc(g, &g->flag, cc + 1) && galloc(g, &g->pos, cc + 1) &&
               galloc(g, &g->g_cell, ctx->cap_g) &&
               galloc(g, &g->mom, 13 * cc) && galloc(g, &g->box_lo, 3 * ctx->cap_g) &&
@@ -1023,7 +1036,7 @@ RbSim rb_sim(hh_ctx *ctx, GTreeBuf *g, double t)
     a.gc = g->gc;
     a.box = g->box;
     a.root_side = g->root_side;
-    a.xmax = g->xmax;
+    a.unit = g->unit;
     a.key = g->key;
     a.key2 = g->key2;
     a.idx = g->idx;
@@ -1054,7 +1067,6 @@ RbSim rb_sim(hh_ctx *ctx, GTreeBuf *g, double t)
     a.path = g->path_buf;
     a.t = t;
     a.theta = ctx->cfg.theta;
-    a.theta_f = float(ctx->cfg.theta);
     a.n = ctx->n;
     a.cap_c = g->cap_c;
     a.cap_g = ctx->cap_g;

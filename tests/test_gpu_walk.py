@@ -20,7 +20,9 @@ def hh():
 
 def _positions(form, n):
     x, v, m = synth.plummer(n, 61)
-    if form == "huge":
+    if form == "tiny":
+        x = x * 2.0 ** -90
+    elif form == "huge":
         x = x * 2.0 ** 90
     elif form == "far":
         x = x + np.array([4096.0, -512.0, 7.0])
@@ -38,7 +40,7 @@ def _positions(form, n):
     ("plummer", 9, 8, 4, 0.5, "hilbert"), ("plummer", 33, 1, 8, 0.7, "morton"), ("plummer", 150, 8, 32, 0.5, "morton"),
     ("plummer", 2049, 32, 8, 0.6, "morton"), ("plummer", 5000, 1, 300, 0.8, "hilbert"),
     ("plummer", 4000, 8, 64, 0.0, "hilbert"), ("plummer", 4000, 8, 64, 30.0, "morton"),
-    ("huge", 3000, 8, 64, 0.5, "hilbert"), ("far", 3000, 8, 64, 0.5, "morton"),
+    ("tiny", 3000, 8, 64, 0.5, "morton"), ("huge", 3000, 8, 64, 0.5, "hilbert"), ("far", 3000, 8, 64, 0.5, "morton"),
     ("pairs", 3001, 1, 16, 0.5, "morton"), ("clump", 900, 8, 64, 0.5, "hilbert"), ("line", 3000, 4, 40, 0.6, "morton"),
     ("plummer", 120000, 8, 256, 0.75, "morton")])
 def test_device_tree_forms(hh, orc, form, n, leaf, n_crit, theta, order):
