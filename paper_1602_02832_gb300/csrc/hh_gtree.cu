@@ -5,7 +5,7 @@
 // (include/hh.h, hh_tree_build): root cube from the bounding box, 21-bit
 // Morton keys, cells split while they hold more than `leaf` particles,
 // pre-order cell numbering, groups = maximal cells with <= n_crit particles,
-// the same opening walk.  Node moments are warp sums (the host sums in
+// the same opening walk.  Node moments are summed from the leaves up (the host sums in
 // index order), so a node's centre of mass may differ in the last bits.
 //
 // CUB (shipped with the CUDA toolkit) provides the radix sort of the keys and
@@ -88,38 +88,27 @@ struct Box {
     int32_t bad;                      // a particle not at the tree time
 };
 
-// BFS level arrays: cells of one level are contiguous; the children of a cell
-// are one contiguous block of the next level, in octant order (the blocks of
-// different cells are placed in whatever order the reservations happen, which
-// changes no pre-order number: those follow from the tree alone).
-struct Cells {
-    int32_t *begin, *end, *depth, *nchild, *first;  // first: BFS index of the first child
-    int32_t *parent;                                 // BFS index of the parent (-1 root)
-    int32_t *size;                                   // cells in the subtree
-    int32_t *pre;                                    // pre-order number
-};
-
-// Sizes the build keeps on the device, so that no step waits for the host:
-// level d holds cells [lvl_c0[d], lvl_c0[d] + lvl_n[d]).
+// Sizes the build keeps on the device, so that no step waits for the host.
 struct GCounts {
-    int32_t lvl_c0[kMaxDepth + 2];
-    int32_t lvl_n[kMaxDepth + 2];
     int32_t ncells, overflow, bad, G;
     int64_t L, n_tiles, total_parts;
     unsigned long long lmax;  // longest list
 };
 
-// Pre-order cell table used by the group and list kernels.
+// Cell table in pre-order (a cell's subtree is the `size` cells from it on).
 struct PCells {
-    int32_t *begin, *end, *nchild, *parent;
-    int32_t *size;   // cells in the subtree: the subtree of p is [p, p + size)
-    int4 *pack;      // {begin, end, FP32 bits of the reject bound, size}: what the list walk reads per cell
-    float4 *cf;      // {centre of mass x, y, z in the tree's unit, accept bound}
-    int32_t *child;  // [8 * n]
-    double *side;
+    int32_t *begin, *end, *depth, *parent, *size;
+    int32_t *arrived;  // particles below whose moments are summed
+    int4 *child;       // [2 * n] children in order, -1 behind the last
+    int4 *pack;        // {begin, end, FP32 bits of the reject bound, size}: what the list walk reads per cell
+    float4 *cf;        // {centre of mass x, y, z in the tree's unit, accept bound}
 };
 
 enum : int { kOpen = 0, kEmitParticles = 1, kEmitNode = 2 };
+
+// cells | groups in one word: cells below bit 34 (at most 22 per particle),
+// groups above
+constexpr int kCellBits = 34;
 
 // Everything a rebuild kernel reads or writes for one simulation.  A kernel
 // runs for one simulation (the record passed by value) or for many (an array
@@ -128,7 +117,6 @@ enum : int { kOpen = 0, kEmitParticles = 1, kEmitNode = 2 };
 // one scan over many simulations' arrays reads like its own scan.
 struct RbSim {
     State st, alt;            // particle state and the buffer it is reordered into
-    Cells C;
     PCells P;
     GCounts *gc;
     Box *box;
@@ -136,10 +124,9 @@ struct RbSim {
     double *unit;             // power of two that brings every |coordinate| below 1
     uint64_t *key, *key2;     // particle keys, and sorted
     int32_t *idx, *perm;      // particle indices, and in key order
-    uint64_t *ckey, *ckey2;   // cell keys (first particle, depth), and sorted
-    int32_t *cval, *cval2;    // cell indices, and in key order
-    double *mom;              // [13][cap_c] cell sums (BFS order)
-    int32_t *flag, *pos;      // [ncells + 1] group cells' flags and their exclusive scan
+    int64_t *cnt, *pos;       // [n + 1] cells and groups that begin at a particle, and their exclusive scan
+    int32_t *chain;           // [n] depths of the cells that begin at a particle (see k_chains)
+    double *mom;              // [ncells][16] cell sums
     int32_t *g_cell;
     double *box_lo, *box_hi;  // [3][G] group boxes
     float4 *box_f;
@@ -153,7 +140,7 @@ struct RbSim {
     int32_t *path;            // [R][kPath] ancestors of each chunk's first cell, from the root (right-aligned)
     DevScalars *ds;           // the context's device sizes (set by k_finish)
     double t, theta;
-    int64_t n, cap_c, pairs;
+    int64_t n, pairs;
     int32_t cap_g, cap_cells, leaf, n_crit, order, tile_i, part_len, work_item, work_split;
     int32_t ncells, G;           // set by the host as they become known
     int32_t chunk, R;            // cells of a walk chunk, and chunks
@@ -177,6 +164,12 @@ __device__ __forceinline__ const RbSim &rb_sim_of(const RbSim &one, const RbSim 
 #define RB_SIM                                                      \
     __shared__ __align__(16) unsigned char rb_rec_[sizeof(RbSim)]; \
     const RbSim &a = rb_sim_of<kMany>(one, many, rb_rec_)
+
+// side of cell c: the root's, halved at each level
+__device__ __forceinline__ double cell_side(const RbSim &a, int32_t c)
+{
+    return *a.root_side * __longlong_as_double((long long)(1023 - a.P.depth[c]) << 52);
+}
 
 template <bool kMany>
 __global__ void k_box(RB_ARGS)
@@ -280,159 +273,171 @@ __global__ void k_root_init(RB_ARGS)
         b->hi[d] = 0ull;
     }
     b->bad = 0;
-    a.C.begin[0] = 0;
-    a.C.end[0] = int32_t(a.n);
-    a.C.depth[0] = 0;
-    a.C.parent[0] = -1;
-    a.C.pre[0] = 0;
-    for (int d = 0; d < kMaxDepth + 2; d++) gc->lvl_c0[d] = gc->lvl_n[d] = 0;
-    gc->lvl_n[0] = 1;
     gc->ncells = gc->overflow = gc->bad = gc->G = 0;
     gc->lmax = 0ull;
 }
 
-// Splits the cells of level d that hold more than `leaf` particles (and are
-// above the depth limit): the octant boundaries come from binary searches of
-// the sorted keys, and each cell reserves its block of children in level d+1.
+// Leading octal digits that two keys share (0..21).
+__device__ __forceinline__ int shared_digits(uint64_t a, uint64_t b)
+{
+    const uint64_t x = a ^ b;
+    return x ? (__clzll((long long)x) - 1) / 3 : kMaxDepth;
+}
+
+// Whether the cell of depth d that holds sorted particles i - 1 and i has more
+// than `most` particles: its first particle (or i - most, if it begins before
+// that) by a binary search, then the particle `most` behind it.
+__device__ __forceinline__ bool more_than(const uint64_t *key, int64_t n, int64_t i, uint64_t ki, int d, int64_t most)
+{
+    int64_t l = max(int64_t(0), i - most), h = i - 1;
+    while (l < h) {
+        const int64_t mid = (l + h) >> 1;
+        if (shared_digits(key[mid], ki) >= d) h = mid;
+        else l = mid + 1;
+    }
+    return l + most < n && shared_digits(key[l + most], ki) >= d;
+}
+
+// The cells, from the sorted keys alone.  A cell is a range of particles that
+// share `depth` leading digits, and it exists when its parent holds more than
+// `leaf` particles.  The cells that begin at sorted particle i are nested, so
+// they are one run of depths: from one more than the digits that i shares with
+// i - 1 (if the cell of that many digits, i's and i - 1's common one, is
+// split) down to a leaf; the cell of depth d is split when particle i + leaf
+// shares d digits too.  In pre-order the cells follow their first particle,
+// then their depth: the scan of the runs' lengths gives every cell's number.
+// A group (Barnes 1990: maximal cells with <= n_crit particles, or leaves)
+// begins at i when the common cell of i - 1 and i has more than n_crit: it is
+// the run's first cell without them.
+// Splitting level by level (up to 22 launches, each with octant searches),
+// sorting the cells into pre-order and selecting the groups from them took 215
+// us for 262144 particles and 430 us for 32 clusters with 1k to 32k; this
+// kernel, its scan and the two after it take 45 and 70 us.
+// chain[i] = top | group depth << 8 | leaf depth << 16.
 template <bool kMany>
-__global__ void k_level(RB_ARGS, int d)
+__global__ void k_chains(RB_ARGS)
 {
     RB_SIM;
-    const Cells &C = a.C;
     const uint64_t *key = a.key2;
-    GCounts *gc = a.gc;
-    // after an overflow the level counts include blocks that were not written:
-    // nothing below reads them, and the host reports HH_ENOMEM
-    if (gc->overflow) return;
-    const int32_t c0 = gc->lvl_c0[d], nc = gc->lvl_n[d], next0 = c0 + nc;
-    if (blockIdx.x == 0 && threadIdx.x == 0) gc->lvl_c0[d + 1] = next0;
-    // Eight lanes per cell: lane o finds where octant o ends (the first
-    // index of the cell's sorted range whose digit at this depth exceeds o)
-    // by its own binary search, so a large cell costs one search, not
-    // eight in a row.  The digit is monotone over the range, so these ends
-    // are the octant boundaries.
-    const int lane = threadIdx.x & 31;
-    const int64_t n_q = (int64_t)nc * 8;
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.cnt[a.n] = 0;  // terminal entry of the scan
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * blockDim.x) {
+        const uint64_t k = key[i];
+        const int top = i > 0 ? shared_digits(key[i - 1], k) + 1 : 0;
+        int64_t word = 0;
+        if (top <= kMaxDepth) {
+            const int low = i + a.leaf < a.n ? min(kMaxDepth, shared_digits(k, key[i + a.leaf]) + 1) : 0;
+            if (i == 0 || low >= top || more_than(key, a.n, i, k, top - 1, a.leaf)) {
+                const int leaf_d = max(low, top);
+                const int big = i + a.n_crit < a.n ? shared_digits(k, key[i + a.n_crit]) + 1 : 0;
+                const bool group = i == 0 || big >= top || more_than(key, a.n, i, k, top - 1, a.n_crit);
+                const int group_d = min(leaf_d, max(big, top));
+                word = (leaf_d - top + 1) | (int64_t(group) << kCellBits);
+                a.chain[i] = top | (group_d << 8) | (leaf_d << 16);
+            }
+        }
+        a.cnt[i] = word;
+    }
+}
+
+// cells (low part) and groups (high part) before sorted particle i
+__device__ __forceinline__ uint64_t before(const RbSim &a, int64_t i) { return uint64_t(a.pos[i]) - uint64_t(a.pos[0]); }
+__device__ __forceinline__ int64_t cells_of(uint64_t w) { return int64_t(w & ((uint64_t(1) << kCellBits) - 1)); }
+
+// First particle and depth of every cell, the group cells, and the sizes (no
+// cell is written when they do not fit: the host reports HH_ENOMEM; group
+// cells beyond cap_g are not stored, likewise).
+template <bool kMany>
+__global__ void k_begin_cells(RB_ARGS)
+{
+    RB_SIM;
+    const uint64_t all = before(a, a.n);
+    const int64_t ncells = cells_of(all);
+    const bool overflow = ncells > a.cap_cells;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.gc->ncells = overflow ? 0 : int32_t(ncells);
+        a.gc->overflow = overflow;
+        a.gc->bad = a.box->bad;
+        a.gc->G = int32_t(all >> kCellBits);
+    }
+    if (overflow) return;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t word = a.cnt[i];
+        if (word == 0) continue;
+        const int32_t ch = a.chain[i], top = ch & 255;
+        const uint64_t w = before(a, i);
+        const int32_t p = int32_t(cells_of(w));
+        for (int d = top; d <= (ch >> 16); d++) {
+            a.P.begin[p + d - top] = int32_t(i);
+            a.P.depth[p + d - top] = d;
+        }
+        if (word >> kCellBits) {
+            const int32_t g = int32_t(w >> kCellBits);
+            if (g < a.cap_g) a.g_cell[g] = p + ((ch >> 8) & 255) - top;
+        }
+    }
+}
+
+// Ends, subtree sizes, children and parents: eight lanes per cell, lane o
+// finding where octant o of a split cell ends (the cell's own end is octant
+// 7's) by a search that doubles its step from the cell's first particle.  A
+// child that begins behind its parent's first particle is the first of the
+// cells beginning there.
+template <bool kMany>
+__global__ void k_cells(RB_ARGS)
+{
+    RB_SIM;
+    const uint64_t *key = a.key2;
+    const int32_t n = int32_t(a.n), ncells = a.gc->ncells;
+    const int lane = threadIdx.x & 31, o = lane & 7;
+    const int64_t n_q = (int64_t)ncells * 8;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;  // a multiple of 32: warps stay whole
     for (int64_t q0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; q0 < n_q; q0 += stride) {
-        const int64_t q = q0 + lane;
-        const bool valid = q < n_q;
-        const int32_t c = c0 + (int32_t)(q >> 3);
-        const int o = (int)(q & 7);
-        int32_t b = 0, e = 0, hi = 0;
+        const bool valid = q0 + lane < n_q;
+        const int32_t p = int32_t((q0 + lane) >> 3);
+        int32_t b = 0, d = 0, hi = 0;
         bool split = false;
         if (valid) {
-            b = C.begin[c];
-            e = C.end[c];
-            split = e - b > a.leaf && d < kMaxDepth;
-            if (split) {
-                int32_t l = b, h = e;
+            b = a.P.begin[p];
+            d = a.P.depth[p];
+            split = d < (a.chain[b] >> 16);
+            // the first key behind octant o (a leaf: behind the cell)
+            const int sh = 3 * (kBits - (split ? d + 1 : d));
+            const uint64_t k = key[b];
+            const uint64_t lim = (split ? ((((k >> sh) & ~uint64_t(7)) | uint64_t(o)) + 1) : ((k >> sh) + 1)) << sh;
+            if (split || o == 7) {
+                int32_t l = b, step = 8;
+                while (n - l > step && key[l + step] < lim) {
+                    l += step;
+                    step *= 2;
+                }
+                int32_t h = n - l > step ? l + step : n;
                 while (l < h) {
-                    const int32_t mid = (l + h) >> 1;
-                    if (digit_at(key[mid], d) <= o) l = mid + 1;
+                    const int32_t mid = l + ((h - l) >> 1);
+                    if (key[mid] < lim) l = mid + 1;
                     else h = mid;
                 }
                 hi = l;
             }
         }
-        int32_t ends[8];
-#pragma unroll
-        for (int k = 0; k < 8; k++) ends[k] = __shfl_sync(0xffffffffu, hi, (lane & ~7) | k);
-        if (!valid || o != 0) continue;
-        int32_t bound[9];
-        int nch = 0;
-        if (split) {
-            int32_t lo = b;
-            for (int k = 0; k < 8 && lo < e; k++) {
-                if (ends[k] > lo) bound[nch++] = lo;
-                lo = ends[k];
-            }
-            bound[nch] = e;
+        // children: the octants that are not empty; a lane's begins where the one before it ends
+        const int prev = __shfl_up_sync(0xffffffffu, hi, 1);
+        const int32_t from = o == 0 ? b : prev, end = __shfl_sync(0xffffffffu, hi, lane | 7);
+        const bool has = valid && split && hi > from;
+        const uint32_t oct = (__ballot_sync(0xffffffffu, has) >> (lane & 24)) & 0xffu;
+        if (!valid) continue;
+        int32_t *child = reinterpret_cast<int32_t *>(a.P.child) + 8 * int64_t(p);
+        if (has) {
+            const int32_t c = from == b ? p + 1 : int32_t(cells_of(before(a, from)));
+            child[__popc(oct & ((1u << o) - 1u))] = c;
+            a.P.parent[c] = p;
         }
-        C.first[c] = next0;
-        C.nchild[c] = 0;
-        if (nch == 0) continue;
-        const int32_t w = next0 + atomicAdd(&gc->lvl_n[d + 1], nch);
-        if ((int64_t)w + nch > a.cap_cells) {
-            atomicExch(&gc->overflow, 1);
-            continue;
+        if (o >= __popc(oct)) child[o] = -1;
+        if (o == 0) {
+            a.P.end[p] = end;
+            a.P.size[p] = int32_t(cells_of(before(a, end))) - p;
+            a.P.arrived[p] = 0;
+            if (p == 0) a.P.parent[0] = -1;
         }
-        C.first[c] = w;
-        C.nchild[c] = nch;
-        for (int k = 0; k < nch; k++) {
-            C.begin[w + k] = bound[k];
-            C.end[w + k] = bound[k + 1];
-            C.depth[w + k] = d + 1;
-            C.parent[w + k] = c;
-        }
-    }
-}
-
-// After the levels 0..d: the cells made so far (complete when level d made
-// no children, i.e. lvl_n[d + 1] == 0), and the synchronisation flag of the
-// bounding-box pass.  One thread per simulation.
-template <bool kMany>
-__global__ void k_cells_done(RB_ARGS, int d)
-{
-    RB_SIM;
-    a.gc->ncells = a.gc->lvl_c0[d + 1] + a.gc->lvl_n[d + 1];
-    a.gc->bad = a.box->bad;
-}
-
-// Pre-order numbers and subtree sizes without a pass per level: the cells
-// sorted by (first particle, depth) are in pre-order (children follow their
-// parent in octant order, which is particle order, and a cell's descendants
-// are the cells after it that start before it ends).  Key of a cell:
-// begin << 5 | depth (depth <= kMaxDepth < 32).
-template <bool kMany>
-__global__ void k_cell_keys(RB_ARGS)
-{
-    RB_SIM;
-    for (int32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < a.ncells; c += gridDim.x * blockDim.x) {
-        a.ckey[c] = (uint64_t(a.C.begin[c]) << 5) | uint64_t(a.C.depth[c]);
-        a.cval[c] = c;
-    }
-}
-
-// From the sorted keys and cells: pre[c] = its rank; size[c] = the cells from
-// it to the first one that starts at or after its end.
-template <bool kMany>
-__global__ void k_pre_size(RB_ARGS)
-{
-    RB_SIM;
-    const int32_t ncells = a.ncells;
-    for (int32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < ncells; p += gridDim.x * blockDim.x) {
-        const int32_t c = a.cval2[p];
-        a.C.pre[c] = p;
-        const uint64_t lim = uint64_t(a.C.end[c]) << 5;
-        int32_t lo = p + 1, hi = ncells;
-        while (lo < hi) {
-            const int32_t mid = (lo + hi) >> 1;
-            if (a.ckey2[mid] < lim) lo = mid + 1;
-            else hi = mid;
-        }
-        a.C.size[c] = lo - p;
-    }
-}
-
-template <bool kMany>
-__global__ void k_to_preorder(RB_ARGS)
-{
-    RB_SIM;
-    const Cells &C = a.C;
-    const PCells &P = a.P;
-    const double s0 = *a.root_side;
-    for (int32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < a.ncells; c += gridDim.x * blockDim.x) {
-        const int32_t p = C.pre[c];
-        P.begin[p] = C.begin[c];
-        P.end[p] = C.end[c];
-        P.nchild[p] = C.nchild[c];
-        P.size[p] = C.size[c];
-        P.parent[p] = C.parent[c] >= 0 ? C.pre[C.parent[c]] : -1;
-        double side = s0;
-        for (int d = 0; d < C.depth[c]; d++) side *= 0.5;
-        P.side[p] = side;
-        for (int k = 0; k < C.nchild[c]; k++) P.child[8 * p + k] = C.pre[C.first[c] + k];
     }
 }
 
@@ -458,94 +463,126 @@ __global__ void k_permute(RB_ARGS)
     }
 }
 
-// Node records (pseudo-particles): mass and mass-weighted sums of x, v, a, jk
-// of the members, bottom-up one tree level per launch: a leaf sums its
-// particles, an inner cell the sums of its children.  mom is [13][cap] in BFS
-// cell order.  (st is the reordered state.)
+// Mass and mass-weighted sums of x, v, a, jk of every cell's particles, in one
+// pass from the leaves up.  Sixteen lanes take a leaf, lane w one of its 13
+// sums (0: mass; 1 + 3k + dim: mass times x, v, a, jerk), which a single
+// thread's order keeps: a leaf over its particles, a split cell over its
+// children.  The lanes then add the cell's particles to its parent's arrivals;
+// the last child to arrive has its lanes sum the parent and goes on, the others
+// stop.  Nothing waits.  (A launch per level took 122 us for 262144 particles
+// and 170 us for 32 clusters with 1k to 32k, here 94 and 106 us: FP64 sums and,
+// at the top, a round trip to L2 per level.)
 template <bool kMany>
-__global__ void k_moments_level(RB_ARGS, int d)
+__global__ void __launch_bounds__(256) k_moments(RB_ARGS)
 {
     RB_SIM;
-    const State &s = a.st;
-    const Cells &C = a.C;
-    const int64_t cap = a.cap_c;
-    double *mom = a.mom;
-    if (a.gc->overflow) return;
-    const int32_t c0 = a.gc->lvl_c0[d], nc = a.gc->lvl_n[d];
-    // one thread per (cell, moment): the 13 sums of a cell run side by side
-    // (each in the same order as a single thread would take them), since a
-    // warp's FP64 instruction costs the pipe the same however few lanes use it
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < (int64_t)nc * 13;
-         q += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t c = c0 + (int32_t)(q / 13);
-        const int w = (int)(q - (q / 13) * 13);
+    const State &s = a.alt;  // (the reordered particles)
+    const int32_t ncells = a.gc->ncells;
+    const int w = threadIdx.x & 15, half = (threadIdx.x >> 4) & 1;
+    const uint32_t mask = 0xffffu << (16 * half);
+    const int32_t stride = int32_t(gridDim.x * blockDim.x) >> 4;
+    const int field = w == 0 ? 0 : (w - 1) / 3, dim = w == 0 ? 0 : (w - 1) % 3;
+    double *const f = (field == 0 ? s.x : field == 1 ? s.v : field == 2 ? s.a : s.jk) + int64_t(dim) * s.cap_j;
+    for (int32_t leaf = int32_t(blockIdx.x * blockDim.x + threadIdx.x) >> 4; leaf < ncells; leaf += stride) {
+        if (a.P.size[leaf] != 1) continue;
         double acc = 0.0;
-        const int nch = C.nchild[c];
-        if (nch == 0) {
-            // w = 0: mass; 1 + 3k + dim: mass times x, v, a, jerk (k = 0..3)
-            const double *f = w == 0 ? nullptr : (w < 4 ? s.x : w < 7 ? s.v : w < 10 ? s.a : s.jk) +
-                                                     (int64_t)((w - 1) % 3) * s.cap_j;
-            for (int32_t p = C.begin[c]; p < C.end[c]; p++) {
+        int32_t c = leaf, b = a.P.begin[leaf], e = a.P.end[leaf];
+        if (w < 13)
+            for (int32_t p = b; p < e; p++) {
                 const double mi = s.m[p];
                 acc = w == 0 ? acc + mi : fma(mi, f[p], acc);
             }
-        } else {
-            const int32_t f = C.first[c];
-            for (int k = 0; k < nch; k++) acc += mom[w * cap + f + k];
+        while (true) {
+            a.mom[int64_t(c) * 16 + w] = acc;
+            const int32_t par = a.P.parent[c];
+            bool last = false;
+            __syncwarp(mask);
+            if (w == 0 && par >= 0)
+                last = int32_t(atom_add_acq_rel_gpu(reinterpret_cast<unsigned int *>(&a.P.arrived[par]),
+                                                    (unsigned int)(e - b))) + (e - b) == a.P.end[par] - a.P.begin[par];
+            if (!__shfl_sync(mask, int(last), 0, 16)) break;
+            __syncwarp(mask);
+            // the parent's sums
+            c = par;
+            b = a.P.begin[c];
+            e = a.P.end[c];
+            const int4 k0 = a.P.child[2 * int64_t(c)], k1 = a.P.child[2 * int64_t(c) + 1];
+            const int32_t kid[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
+            double part[8];
+#pragma unroll
+            for (int k = 0; k < 8; k++) part[k] = kid[k] >= 0 ? __ldcg(&a.mom[int64_t(kid[k]) * 16 + w]) : 0.0;
+            acc = 0.0;
+#pragma unroll
+            for (int k = 0; k < 8; k++)
+                if (kid[k] >= 0) acc += part[k];
         }
-        mom[w * cap + c] = acc;
     }
 }
 
-// j entry n + (pre-order number) of every cell: centre of mass and
-// mass-weighted mean velocity, acceleration and jerk at the tree time.
+// Node records (pseudo-particles), j entry n + (pre-order number) of every
+// cell: centre of mass and mass-weighted mean velocity, acceleration and jerk
+// at the tree time.  And what the list walk reads of the cell: its centre in
+// FP32 and the bounds on the squared distance (see decide).  A thread per cell
+// (the divisions bound this kernel; sixteen lanes per cell, as the sums have
+// them, leave a quarter of the lanes idle: 79 against 47 us for 112233 cells).
 template <bool kMany>
-__global__ void k_node_records(RB_ARGS)
+__global__ void __launch_bounds__(128) k_node_records(RB_ARGS)
 {
     RB_SIM;
-    const State &s = a.st;
-    const int64_t cap = a.cap_c;
-    const double *mom = a.mom;
-    for (int32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < a.ncells; c += gridDim.x * blockDim.x) {
-        const int32_t p = a.C.pre[c];
-        const int64_t j = a.n + p;
-        const double M = mom[c];
+    const State &s = a.alt;
+    const int32_t ncells = a.gc->ncells;
+    const double u = *a.unit;
+    const float theta = float(a.theta), inv_theta = 1.0f / theta, root = float(*a.root_side * u);
+    for (int32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < ncells; c += gridDim.x * blockDim.x) {
+        const double2 *mom = reinterpret_cast<const double2 *>(a.mom + int64_t(c) * 16);
+        double sum[14];
+#pragma unroll
+        for (int k = 0; k < 7; k++) {
+            const double2 v = mom[k];
+            sum[2 * k] = v.x;
+            sum[2 * k + 1] = v.y;
+        }
+        const double M = sum[0];
+        const int64_t j = a.n + c;
+        float xf[3];
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+            const int64_t q = d * s.cap_j + j;
+            const double x = sum[1 + d] / M;
+            xf[d] = float(x * u);
+            s.x[q] = x;
+            s.v[q] = sum[4 + d] / M;
+            s.a[q] = sum[7 + d] / M;
+            s.jk[q] = sum[10 + d] / M;
+        }
         s.m[j] = M;
         s.t[j] = a.t;
-        double x[3];
-        for (int d = 0; d < 3; d++) {
-            x[d] = mom[(1 + d) * cap + c] / M;
-            s.x[d * s.cap_j + j] = x[d];
-            s.v[d * s.cap_j + j] = mom[(4 + d) * cap + c] / M;
-            s.a[d * s.cap_j + j] = mom[(7 + d) * cap + c] / M;
-            s.jk[d * s.cap_j + j] = mom[(10 + d) * cap + c] / M;
-        }
-        // what the list walk reads of the cell: its FP32 centre and bounds on
-        // the squared distance (see decide)
-        const double u = *a.unit, side = a.P.side[p] * u, tol = 0x1p-19 * a.theta;
-        const double far = (side * (1.0 + 0x1p-17) + tol) / a.theta, near = (side * (1.0 - 0x1p-17) - tol) / a.theta;
-        const int32_t b = a.C.begin[c], e = a.C.end[c];
-        float hi = __double2float_ru(far * far * (1.0 + 0x1p-20));
-        float lo = near > 0.0 ? __double2float_rd(near * near * (1.0 - 0x1p-20)) : -1.0f;
+        const int32_t b = a.P.begin[c], e = a.P.end[c];
+        const float side = root * __int_as_float((127 - a.P.depth[c]) << 23);
+        const float far = (side * (1.0f + 0x1p-16f) + 0x1p-18f * theta) * inv_theta;
+        const float near = (side * (1.0f - 0x1p-16f) - 0x1p-18f * theta) * inv_theta;
+        float hi = far * far * (1.0f + 0x1p-17f), lo = near > 0.0f ? near * near * (1.0f - 0x1p-17f) : -1.0f;
         if (e - b == 1) hi = lo = __int_as_float(0x7f800000);  // a single particle always goes in as such
-        a.P.cf[p] = make_float4(float(x[0] * u), float(x[1] * u), float(x[2] * u), hi);
-        a.P.pack[p] = make_int4(b, e, __float_as_int(lo), a.C.size[c]);
+        a.P.cf[c] = make_float4(xf[0], xf[1], xf[2], hi);
+        a.P.pack[c] = make_int4(b, e, __float_as_int(lo), a.P.size[c]);
     }
 }
 
-// Bounding box of each group's particles ([3][G] lo and hi), one warp per group
+// Bounding box of each group's particles ([3][G] lo and hi) and the particles'
+// group numbers, one warp per group
 // (none beyond cap_g groups: the host then reports the overflow).
 template <bool kMany>
 __global__ void k_group_box(RB_ARGS)
 {
     RB_SIM;
-    const State &s = a.st;
+    const State &s = a.alt;
     const int32_t G = a.gc->G;
     if (G > a.cap_g) return;
     const int lane = threadIdx.x & 31;
     const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t g = w0; g < G; g += nw) {
         const int32_t c = a.g_cell[g], b = a.P.begin[c], e = a.P.end[c];
+        for (int32_t p = b + lane; p < e; p += 32) a.group_of[p] = int32_t(g);
         for (int d = 0; d < 3; d++) {
             double lo = s.x[d * s.cap_j + b], hi = lo;
             for (int32_t p = b + lane; p < e; p += 32) {
@@ -573,40 +610,6 @@ __global__ void k_group_box(RB_ARGS)
     }
 }
 
-// Groups (Barnes 1990): maximal cells with <= n_crit particles (or leaves),
-// flagged in pre-order and compacted by one exclusive scan.
-template <bool kMany>
-__global__ void k_flags(RB_ARGS)
-{
-    RB_SIM;
-    const PCells &P = a.P;
-    const int32_t ncells = a.ncells;
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.flag[ncells] = 0;  // terminal entry of the scan
-    for (int32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < ncells; c += gridDim.x * blockDim.x) {
-        const int32_t cnt = P.end[c] - P.begin[c];
-        const bool small = cnt <= a.n_crit || P.nchild[c] == 0;
-        const int32_t par = P.parent[c];
-        const bool parent_big = par < 0 || !((P.end[par] - P.begin[par]) <= a.n_crit || P.nchild[par] == 0);
-        a.flag[c] = (small && parent_big) ? 1 : 0;
-    }
-}
-
-// The group cells in pre-order (g_cell, group_of) and their number (cells
-// beyond cap_g are not stored: the host reports the overflow).
-template <bool kMany>
-__global__ void k_groups(RB_ARGS)
-{
-    RB_SIM;
-    const int32_t ncells = a.ncells, g0 = a.pos[0];
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.gc->G = a.pos[ncells] - g0;
-    for (int32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < ncells; c += gridDim.x * blockDim.x)
-        if (a.flag[c]) {
-            const int32_t g = a.pos[c] - g0;
-            if (g < a.cap_g) a.g_cell[g] = c;
-            for (int32_t p = a.P.begin[c]; p < a.P.end[c]; p++) a.group_of[p] = g;
-        }
-}
-
 // The opening decision of cell c for group g (rules of hh_tree_build): the
 // group's own cell and single particles go in as particles; a cell that does
 // not contain the group goes in as a node when side < theta * (distance of its
@@ -619,9 +622,9 @@ __global__ void k_groups(RB_ARGS)
 // |coordinate| below 1, so that no square leaves FP32's range.  Rounding centre
 // and box to FP32 and taking gaps, squares and sum in FP32 moves the distance
 // by less than 2^-21 + 2^-22 distance.  A cell is accepted above
-// ((1 + 2^-17) side + 2^-19 theta)^2 / theta^2 (and 2^-20 more, rounded up) and
-// not accepted below ((1 - 2^-17) side - 2^-19 theta)^2 / theta^2 (and 2^-20
-// less, rounded down; never when that difference is negative), which covers
+// ((1 + 2^-16) side + 2^-18 theta)^2 / theta^2 (and 2^-17 more) and not accepted
+// below ((1 - 2^-16) side - 2^-18 theta)^2 / theta^2 (and 2^-17 less; never when
+// that difference is negative), both evaluated in FP32 to 2^-20, which covers
 // those errors and the roundings of the FP64 test.  Between the bounds (and for
 // any NaN) the test is redone in FP64 with the roundings of the sequential
 // builder (no contraction), so the decision is always the FP64 one.  A single
@@ -661,7 +664,7 @@ __device__ __forceinline__ int decide(const RbSim &a, const GroupView &G, int32_
             else if (cm > hi) gap = __dsub_rn(cm, hi);
             d2 = __dadd_rn(d2, __dmul_rn(gap, gap));
         }
-        accept = a.P.side[c] < __dmul_rn(a.theta, __dsqrt_rn(d2));
+        accept = cell_side(a, c) < __dmul_rn(a.theta, __dsqrt_rn(d2));
     }
     if (accept) return kEmitNode;
     return r.pk.w == 1 ? kEmitParticles : kOpen;  // (only a leaf is its whole subtree)
@@ -903,13 +906,12 @@ struct GTreeBuf {
     GCounts *gc = nullptr;      // device
     GCounts *gc_host = nullptr;  // pinned mirror
     float4 *box_f = nullptr;
-    Cells C{};
     PCells P{};
-    int32_t *flag = nullptr, *pos = nullptr;  // [cap_c + 1] group cells' flags and their scan
+    int64_t *cnt = nullptr, *pos = nullptr;  // [n + 1] cells and groups by first particle, and their scan
     int32_t *g_cell = nullptr;
     // [tile counts | part counts] and their one scan, each 2 (G + 1) long
     int64_t *ntile = nullptr, *tile_off = nullptr;
-    double *mom = nullptr;                    // [13][cap_c] cell sums (BFS order)
+    double *mom = nullptr;                    // [cap_c][16] cell sums
     double *box_lo = nullptr, *box_hi = nullptr;  // [3][cap_g] group boxes
     State alt{};                 // second particle-state buffer for the reordering
     int64_t *ids = nullptr, *ids2 = nullptr;
@@ -918,7 +920,6 @@ struct GTreeBuf {
     int64_t pair_cap = 0;
     int32_t *path_buf = nullptr;  // [R][kPath] ancestors of the chunks' first cells
     int64_t path_cap = 0;
-    int depth = -1;              // depth of the last tree (-1: none yet)
     void *tmp = nullptr;
     size_t tmp_bytes = 0;
     std::vector<void *> all;
@@ -980,16 +981,13 @@ GTreeBuf *gtree_alloc(hh_ctx *ctx)
     g->cap_n = n;
     g->cap_c = cc;
     bool ok = galloc(g, &g->key, n) && galloc(g, &g->key2, n) && galloc(g, &g->idx, n) && galloc(g, &g->perm, n) &&
-              galloc(g, &g->box, 1) && galloc(g, &g->root_side, 1) && galloc(g, &g->C.begin, cc) &&
-              galloc(g, &g->C.end, cc) && galloc(g, &g->C.depth, cc) && galloc(g, &g->C.nchild, cc) &&
-              galloc(g, &g->C.first, cc) && galloc(g, &g->C.parent, cc) && galloc(g, &g->C.size, cc) &&
-              galloc(g, &g->C.pre, cc) && galloc(g, &g->P.begin, cc) && galloc(g, &g->P.end, cc) &&
-              galloc(g, &g->P.nchild, cc) && galloc(g, &g->P.parent, cc) && galloc(g, &g->P.child, 8 * cc) &&
-              galloc(g, &g->P.side, cc) && galloc(g, &g->P.size, cc) && galloc(g, &g->P.pack, cc) &&
-              galloc(g, &g->P.cf, cc) && galloc(g, &g->unit, 1) && galloc(g, &g->gc, 1) &&
-              galloc(g, &g->box_f, 2 * ctx->cap_g) && galloc(g, &g->flag, cc + 1) && galloc(g, &g->pos, cc + 1) &&
+              galloc(g, &g->box, 1) && galloc(g, &g->root_side, 1) && galloc(g, &g->P.begin, cc) &&
+              galloc(g, &g->P.end, cc) && galloc(g, &g->P.depth, cc) && galloc(g, &g->P.parent, cc) &&
+              galloc(g, &g->P.size, cc) && galloc(g, &g->P.arrived, cc) && galloc(g, &g->P.child, 2 * cc) &&
+              galloc(g, &g->P.pack, cc) && galloc(g, &g->P.cf, cc) && galloc(g, &g->unit, 1) && galloc(g, &g->gc, 1) &&
+              galloc(g, &g->box_f, 2 * ctx->cap_g) && galloc(g, &g->cnt, n + 1) && galloc(g, &g->pos, n + 1) &&
               galloc(g, &g->g_cell, ctx->cap_g) &&
-              galloc(g, &g->mom, 13 * cc) && galloc(g, &g->box_lo, 3 * ctx->cap_g) &&
+              galloc(g, &g->mom, 16 * cc) && galloc(g, &g->box_lo, 3 * ctx->cap_g) &&
               galloc(g, &g->box_hi, 3 * ctx->cap_g) &&
               galloc(g, &g->ntile, 2 * (ctx->cap_g + 1)) && galloc(g, &g->tile_off, 2 * (ctx->cap_g + 1)) &&
               galloc(g, &g->ids, n) && galloc(g, &g->ids2, n);
@@ -1015,7 +1013,7 @@ GTreeBuf *gtree_alloc(hh_ctx *ctx)
 int64_t gtree_bytes(const hh_ctx *ctx)
 {
     const int64_t n = ctx->cap_n, cc = ctx->cap_j, G = ctx->cap_g + 1;
-    return n * (8 * 2 + 4 * 2 + 8 * 2) + cc * (4 * 8 + 4 * 5 + 32 + 8 + 4 * 8 + 13 * 8 + 4 * 2) +
+    return n * (8 * 2 + 4 * 2 + 8 * 2) + (n + 1) * 8 * 2 + cc * (4 * 6 + 32 + 32 + 16 * 8) +
            G * (4 + 8 * 4 + 6 * 8 + 32) + ctx->cap_j * 8 * (12 + 2) + n * 8;
 }
 
@@ -1031,7 +1029,6 @@ RbSim rb_sim(hh_ctx *ctx, GTreeBuf *g, double t)
     RbSim a{};
     a.st = ctx->st;
     a.alt = g->alt;
-    a.C = g->C;
     a.P = g->P;
     a.gc = g->gc;
     a.box = g->box;
@@ -1041,15 +1038,10 @@ RbSim rb_sim(hh_ctx *ctx, GTreeBuf *g, double t)
     a.key2 = g->key2;
     a.idx = g->idx;
     a.perm = g->perm;
-    // the cell sort's keys and values live in the moment sums and the
-    // selection arrays, not yet in use when the cells are sorted
-    a.ckey = reinterpret_cast<uint64_t *>(g->mom);
-    a.ckey2 = a.ckey + g->cap_c;
-    a.cval = g->flag;
-    a.cval2 = g->pos;
-    a.mom = g->mom;
-    a.flag = g->flag;
+    a.cnt = g->cnt;
     a.pos = g->pos;
+    a.chain = g->idx;  // (the sort's input, not used after it)
+    a.mom = g->mom;
     a.g_cell = g->g_cell;
     a.box_lo = g->box_lo;
     a.box_hi = g->box_hi;
@@ -1068,7 +1060,6 @@ RbSim rb_sim(hh_ctx *ctx, GTreeBuf *g, double t)
     a.t = t;
     a.theta = ctx->cfg.theta;
     a.n = ctx->n;
-    a.cap_c = g->cap_c;
     a.cap_g = ctx->cap_g;
     a.cap_cells = int32_t(std::min<int64_t>(ctx->cap_j - ctx->n, INT32_MAX));
     a.leaf = ctx->cfg.leaf;
@@ -1164,14 +1155,6 @@ int64_t walk_blocks(int32_t G, int32_t R)
     return std::max<int64_t>(1, std::min<int64_t>((int64_t((G + 31) / 32) * R + 3) / 4, int64_t(1) << 28));
 }
 
-// bits of a cell key: begin (< 2^b with 2^b > n) above 5 bits of depth
-int cell_key_bits(int64_t n)
-{
-    int bits = 5;
-    while (bits < 64 && (int64_t(1) << (bits - 5)) <= n) bits++;
-    return bits;
-}
-
 }  // namespace
 
 // Called by hh_rebuild when the context builds on the device.
@@ -1185,10 +1168,13 @@ int hh_rebuild_device(hh_ctx *ctx, double t)
     // element-wise kernels: a thread per particle at most (they stride over
     // cells, groups and particles alike), so a small tree launches few blocks
     const int grid = int(std::max<int64_t>(1, std::min<int64_t>(ctx->elem_grid, (n + 255) / 256)));
+    // (those with 8 or 16 lanes per cell, or a warp per group: about four
+    // lanes per particle)
+    const int grid8 = int(std::max<int64_t>(1, std::min<int64_t>(2 * ctx->elem_grid, (4 * n + 255) / 256)));
     int64_t launches = 0;
     RbSim a = rb_sim(ctx, g, t);
-    // Sizes stay on the device (GCounts) and the host reads them three times:
-    // after the cells, after groups and cut, and after the list counts.
+    // Sizes stay on the device (GCounts) and the host reads them twice: after
+    // the tree and the groups, and after the list counts.
     auto read_counts = [&]() {
         cudaMemcpyAsync(g->gc_host, g->gc, sizeof(GCounts), cudaMemcpyDeviceToHost, st);
         return cudaStreamSynchronize(st) == cudaSuccess;
@@ -1214,59 +1200,34 @@ int hh_rebuild_device(hh_ctx *ctx, double t)
             cudaSuccess)
             return gfail(ctx, HH_ECUDA, "hh_rebuild: key sort failed");
     }
-    // 2. cells level by level (BFS).  The levels run up to two below the last
-    //    tree's depth (the tree changes little in one dt_tree); if the last of
-    //    them still made children, the rest follow after the read of the counts.
-    const int d_guess = g->depth < 0 ? kMaxDepth : std::min(kMaxDepth, g->depth + 2);
-    for (int d = 0; d <= d_guess; d++) k_level<false><<<grid, 256, 0, st>>>(a, nullptr, d);
-    k_cells_done<false><<<1, 1, 0, st>>>(a, nullptr, d_guess);
-    launches += (d_guess + 1) + 1;
+    // 2. cells and groups, particles into Morton order and node records, group
+    //    boxes: all into the builder's buffers, which become the context's when
+    //    the tree is known to fit
+    k_chains<false><<<grid, 256, 0, st>>>(a, nullptr);
+    if ((rc = cub_exclusive_sum(g->tmp, g->tmp_bytes, a.cnt, a.pos, n + 1, st)))
+        return gfail(ctx, rc, "hh_rebuild: scan failed");
+    k_begin_cells<false><<<grid, 256, 0, st>>>(a, nullptr);
+    k_cells<false><<<grid8, 256, 0, st>>>(a, nullptr);
+    k_permute<false><<<grid, 256, 0, st>>>(a, nullptr);
+    k_moments<false><<<grid8, 256, 0, st>>>(a, nullptr);
+    k_node_records<false><<<grid, 128, 0, st>>>(a, nullptr);
+    k_group_box<false><<<grid8, 256, 0, st>>>(a, nullptr);
+    launches += 7;
     if (!read_counts()) return gfail(ctx, HH_ECUDA, "hh_rebuild: tree build failed");
-    if (!g->gc_host->overflow && g->gc_host->lvl_n[d_guess + 1] > 0) {
-        for (int d = d_guess + 1; d <= kMaxDepth; d++) k_level<false><<<grid, 256, 0, st>>>(a, nullptr, d);
-        k_cells_done<false><<<1, 1, 0, st>>>(a, nullptr, kMaxDepth);
-        launches += (kMaxDepth - d_guess) + 1;
-        if (!read_counts()) return gfail(ctx, HH_ECUDA, "hh_rebuild: tree build failed");
-    }
     if (g->gc_host->bad) return gfail(ctx, HH_ESTATE, "hh_rebuild: particles are not synchronised at t");
     if (g->gc_host->overflow)
         return gfail(ctx, HH_ENOMEM, "hh_rebuild: tree exceeds nj_max (more cells than room for nodes)");
     const int32_t ncells = g->gc_host->ncells;
     a.ncells = ncells;
-    // the deepest level that holds cells: the moment loop runs from there
-    int depth = 0;
-    for (int d = 0; d <= kMaxDepth; d++)
-        if (g->gc_host->lvl_n[d] > 0) depth = d;
-    g->depth = depth;
-    // pre-order numbers and subtree sizes from one sort of the cells by
-    // (first particle, depth)
-    k_cell_keys<false><<<grid, 256, 0, st>>>(a, nullptr);
-    if ((rc = cub_sort_pairs(g->tmp, g->tmp_bytes, a.ckey, a.ckey2, a.cval, a.cval2, ncells, cell_key_bits(n), st)))
-        return gfail(ctx, rc, "hh_rebuild: cell sort failed");
-    k_pre_size<false><<<grid, 256, 0, st>>>(a, nullptr);
-    k_to_preorder<false><<<grid, 256, 0, st>>>(a, nullptr);
-    // 3. particles into Morton order (into the second buffer), then swap
-    k_permute<false><<<grid, 256, 0, st>>>(a, nullptr);
     swap_state(ctx, g);
     a.st = ctx->st;
     a.alt = g->alt;
     a.ids = g->ids;
     a.ids2 = g->ids2;
-    // 4. node records (bottom-up moments); groups (flags, one scan, the
-    //    compacted table) and their boxes
-    for (int d = depth; d >= 0; d--) k_moments_level<false><<<grid, 256, 0, st>>>(a, nullptr, d);
-    k_node_records<false><<<grid, 256, 0, st>>>(a, nullptr);
-    k_flags<false><<<grid, 256, 0, st>>>(a, nullptr);
-    if ((rc = cub_exclusive_sum(g->tmp, g->tmp_bytes, a.flag, a.pos, int64_t(ncells) + 1, st)))
-        return gfail(ctx, rc, "hh_rebuild: scan failed");
-    k_groups<false><<<grid, 256, 0, st>>>(a, nullptr);
-    k_group_box<false><<<grid, 256, 0, st>>>(a, nullptr);
-    launches += 4 + (depth + 1) + 4;
-    if (!read_counts()) return gfail(ctx, HH_ECUDA, "hh_rebuild: group build failed");
     const int32_t G = g->gc_host->G;
     if (G > ctx->cap_g) return gfail(ctx, HH_ENOMEM, "hh_rebuild: more groups than groups_max");
     a.G = G;
-    // 5. per-(group, chunk) list counts, one scan, offsets, tiles, write
+    // 3. per-(group, chunk) list counts, one scan, offsets, tiles, write
     a.chunk = walk_chunk(double(G) * ncells, ncells);
     a.R = (ncells + a.chunk - 1) / a.chunk;
     if (!grow(g->path_buf, g->path_cap, int64_t(a.R) * kPath))
@@ -1286,7 +1247,7 @@ int hh_rebuild_device(hh_ctx *ctx, double t)
     if ((rc = cub_exclusive_sum(g->tmp, g->tmp_bytes, a.pair2, a.pscan2, 2 * (pairs + 1), st)))  // cnt_p, cnt_n at once
         return gfail(ctx, rc, "hh_rebuild: scan failed");
     k_list_off<false><<<grid, 256, 0, st>>>(a, nullptr);
-    // 6. tiles and their work-item capacity (from the list lengths)
+    // 4. tiles and their work-item capacity (from the list lengths)
     k_tile_counts<false><<<grid, 256, 0, st>>>(a, nullptr);
     if ((rc = cub_exclusive_sum(g->tmp, g->tmp_bytes, g->ntile, g->tile_off, 2 * (int64_t(G) + 1), st)))
         return gfail(ctx, rc, "hh_rebuild: scan failed");
@@ -1320,16 +1281,13 @@ struct RbScratch {
     cudaStream_t stream = nullptr;
     RbSim *h_sims = nullptr, *d_sims = nullptr;  // [kStages][cap_sims]
     GCounts *h_gc = nullptr, *d_gc = nullptr;     // [cap_sims], by the simulation's slot
-    int32_t *h_seg = nullptr, *d_seg = nullptr;   // [2][cap_sims + 1]: particles, cells
+    int32_t *h_seg = nullptr, *d_seg = nullptr;   // [cap_sims + 1] particle segments
     int64_t cap_sims = 0;
     uint64_t *key = nullptr, *key2 = nullptr;
     int32_t *idx = nullptr, *perm = nullptr;
     int64_t cap_key = 0, cap_key2 = 0, cap_idx = 0, cap_perm = 0;
-    uint64_t *ckey = nullptr, *ckey2 = nullptr;
-    int32_t *cval = nullptr, *cval2 = nullptr;
-    int64_t cap_ckey = 0, cap_ckey2 = 0, cap_cval = 0, cap_cval2 = 0;
-    int32_t *flag = nullptr, *pos = nullptr;
-    int64_t cap_flag = 0, cap_pos = 0;
+    int64_t *cnt = nullptr, *pos = nullptr;
+    int64_t cap_cnt = 0, cap_pos = 0;
     int64_t *pair2 = nullptr, *pscan2 = nullptr;
     int64_t cap_pair2 = 0, cap_pscan2 = 0;
     int32_t *path = nullptr;
@@ -1363,10 +1321,10 @@ bool rb_reserve_sims(RbScratch *r, int64_t k)
     const int64_t cap = k + k / 2 + 8;
     if (cudaMalloc(&r->d_sims, sizeof(RbSim) * kStages * cap) != cudaSuccess ||
         cudaMalloc(&r->d_gc, sizeof(GCounts) * cap) != cudaSuccess ||
-        cudaMalloc(&r->d_seg, sizeof(int32_t) * 2 * (cap + 1)) != cudaSuccess ||
+        cudaMalloc(&r->d_seg, sizeof(int32_t) * (cap + 1)) != cudaSuccess ||
         cudaHostAlloc((void **)&r->h_sims, sizeof(RbSim) * kStages * cap, cudaHostAllocDefault) != cudaSuccess ||
         cudaHostAlloc((void **)&r->h_gc, sizeof(GCounts) * cap, cudaHostAllocDefault) != cudaSuccess ||
-        cudaHostAlloc((void **)&r->h_seg, sizeof(int32_t) * 2 * (cap + 1), cudaHostAllocDefault) != cudaSuccess) {
+        cudaHostAlloc((void **)&r->h_seg, sizeof(int32_t) * (cap + 1), cudaHostAllocDefault) != cudaSuccess) {
         cudaGetLastError();
         rb_free_sims(r);
         return false;
@@ -1424,9 +1382,7 @@ void hh_rb_scratch_free(RbScratch *r)
     if (!r) return;
     cudaStreamSynchronize(r->stream);
     rb_free_sims(r);
-    for (void *p : {(void *)r->key, (void *)r->key2, (void *)r->idx, (void *)r->perm, (void *)r->ckey,
-                    (void *)r->ckey2, (void *)r->cval, (void *)r->cval2, (void *)r->flag, (void *)r->pos,
-                    (void *)r->pair2, (void *)r->pscan2, (void *)r->path, (void *)r->nt2, (void *)r->tscan2, r->tmp})
+    for (void *p : {(void *)r->key, (void *)r->key2, (void *)r->idx, (void *)r->perm, (void *)r->cnt, (void *)r->pos, (void *)r->pair2, (void *)r->pscan2, (void *)r->path, (void *)r->nt2, (void *)r->tscan2, r->tmp})
         if (p) cudaFree(p);
     cudaStreamDestroy(r->stream);
     delete r;
@@ -1483,39 +1439,36 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
         act.clear();
         return HH_OK;
     };
-    // exclusive prefix of per-context sizes into segment offsets `which`
-    auto segments = [&](int which, const std::function<int64_t(size_t)> &size, int64_t *total) {
-        int32_t *h = r->h_seg + which * (r->cap_sims + 1);
+    // exclusive prefix of the particle counts as segment offsets
+    auto segments = [&](int64_t *total) {
         int64_t acc = 0;
         for (size_t q = 0; q < act.size(); q++) {
-            h[q] = int32_t(acc);
-            acc += size(q);
+            r->h_seg[q] = int32_t(acc);
+            acc += ctxs[act[q]]->n;
             if (acc >= int64_t(INT32_MAX)) return false;
         }
-        h[act.size()] = int32_t(acc);
+        r->h_seg[act.size()] = int32_t(acc);
         *total = acc;
-        return cudaMemcpyAsync(r->d_seg + which * (r->cap_sims + 1), h, sizeof(int32_t) * (act.size() + 1),
-                               cudaMemcpyHostToDevice, st) == cudaSuccess;
+        return cudaMemcpyAsync(r->d_seg, r->h_seg, sizeof(int32_t) * (act.size() + 1), cudaMemcpyHostToDevice, st) ==
+               cudaSuccess;
     };
     // blocks per simulation of the element-wise kernels (they stride over
     // cells, groups and particles alike): a thread per particle of the
     // largest one, but no more than about twice the threads the SMs hold in
-    // all, since a level or a moment pass has little work for most blocks
-    int64_t launches = 0, gx = 1, max_n = 1;
-    for (int s : act) {
-        gx = std::max<int64_t>(gx, std::min<int64_t>(ctxs[s]->elem_grid, (ctxs[s]->n + 255) / 256));
-        max_n = std::max<int64_t>(max_n, ctxs[s]->n);
-    }
-    const int64_t gx_full = gx;  // (the group boxes, a warp per group, take every block)
+    // all
+    int64_t launches = 0, gx = 1;
+    for (int s : act) gx = std::max<int64_t>(gx, std::min<int64_t>(ctxs[s]->elem_grid, (ctxs[s]->n + 255) / 256));
+    // (those with 8 or 16 lanes per cell, or a warp per group)
+    const int64_t gx8 = std::max<int64_t>(
+        1, std::min<int64_t>(4 * gx, 8 * int64_t(ctxs[act[0]]->elem_grid) / int64_t(act.size())));
     gx = std::max<int64_t>(1, std::min<int64_t>(gx, 2 * int64_t(ctxs[act[0]]->elem_grid) / int64_t(act.size())));
-    // 1. bounding boxes, keys, one segmented key sort, levels, counts
+    // 1. bounding boxes, keys, one segmented key sort
     int64_t tot = 0;
-    if (!segments(0, [&](size_t q) { return ctxs[act[q]]->n; }, &tot))
-        return fail_all(HH_ENOMEM, "hh_rebuild: batch too large");
+    if (!segments(&tot)) return fail_all(HH_ENOMEM, "hh_rebuild: batch too large");
     if (!rb_grow(r->key, r->cap_key, tot) || !rb_grow(r->key2, r->cap_key2, tot) || !rb_grow(r->idx, r->cap_idx, tot) ||
-        !rb_grow(r->perm, r->cap_perm, tot))
+        !rb_grow(r->perm, r->cap_perm, tot) || !rb_grow(r->cnt, r->cap_cnt, tot + K0) ||
+        !rb_grow(r->pos, r->cap_pos, tot + K0))
         return fail_all(HH_ENOMEM, "hh_rebuild: batch key buffers do not fit");
-    int d_guess = 0;
     for (size_t q = 0; q < act.size(); q++) {
         hh_ctx *ctx = ctxs[act[q]];
         GTreeBuf *g = ctx->gtree;
@@ -1527,29 +1480,32 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
         a.key2 = r->key2 + o;
         a.idx = r->idx + o;
         a.perm = r->perm + o;
+        a.chain = a.idx;  // (the sort's input, not used after it)
+        a.cnt = r->cnt + o + int64_t(q);  // (a terminal entry each)
+        a.pos = r->pos + o + int64_t(q);
         slot.push_back(int(q));
-        d_guess = std::max(d_guess, g->depth < 0 ? kMaxDepth : std::min(kMaxDepth, g->depth + 2));
     }
     if (!upload()) return fail_all(HH_ECUDA, "hh_rebuild: batch upload failed");
-    const dim3 g1 = dim3(unsigned(gx), unsigned(K0)), one1(1, unsigned(K0));
+    const dim3 g1 = dim3(unsigned(gx), unsigned(K0)), one1(1, unsigned(K0)), g8 = dim3(unsigned(gx8), unsigned(K0));
     k_root_init<true><<<one1, 1, 0, st>>>(RbSim{}, D());
     k_box<true><<<g1, 256, 0, st>>>(RbSim{}, D());
     k_keys<true><<<g1, 256, 0, st>>>(RbSim{}, D());
     launches += 3;
     int rc = rb_seg_sort(r, r->key, r->key2, r->idx, r->perm, tot, K0, r->d_seg, 63);
     if (rc) return fail_all(rc, "hh_rebuild: batch key sort failed");
-    for (int d = 0; d <= d_guess; d++) k_level<true><<<g1, 256, 0, st>>>(RbSim{}, D(), d);
-    k_cells_done<true><<<one1, 1, 0, st>>>(RbSim{}, D(), d_guess);
-    launches += (d_guess + 1) + 1;
+    // 2. cells and groups, reordering, node records, group boxes, all into the
+    //    builders' buffers
+    k_chains<true><<<g1, 256, 0, st>>>(RbSim{}, D());
+    if ((rc = cub_exclusive_sum(r->tmp, r->tmp_bytes, r->cnt, r->pos, tot + K0, st)))
+        return fail_all(rc, "hh_rebuild: batch scan failed");
+    k_begin_cells<true><<<g1, 256, 0, st>>>(RbSim{}, D());
+    k_cells<true><<<g8, 256, 0, st>>>(RbSim{}, D());
+    k_permute<true><<<g1, 256, 0, st>>>(RbSim{}, D());
+    k_moments<true><<<g8, 256, 0, st>>>(RbSim{}, D());
+    k_node_records<true><<<g1, 128, 0, st>>>(RbSim{}, D());
+    k_group_box<true><<<g8, 256, 0, st>>>(RbSim{}, D());
+    launches += 7;
     if (!read_counts()) return fail_all(HH_ECUDA, "hh_rebuild: tree build failed");
-    bool deeper = false;
-    for (size_t q = 0; q < act.size(); q++) deeper |= !cnt(q).overflow && cnt(q).lvl_n[d_guess + 1] > 0;
-    if (deeper) {  // (a context that is complete gains empty levels)
-        for (int d = d_guess + 1; d <= kMaxDepth; d++) k_level<true><<<g1, 256, 0, st>>>(RbSim{}, D(), d);
-        k_cells_done<true><<<one1, 1, 0, st>>>(RbSim{}, D(), kMaxDepth);
-        launches += (kMaxDepth - d_guess) + 1;
-        if (!read_counts()) return fail_all(HH_ECUDA, "hh_rebuild: tree build failed");
-    }
     next_stage([&](size_t q) {
         if (cnt(q).bad) {
             rcs[act[q]] = gfail(ctxs[act[q]], HH_ESTATE, "hh_rebuild: particles are not synchronised at t");
@@ -1563,46 +1519,6 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
         return true;
     });
     if (act.empty()) return HH_OK;
-    // 2. one segmented cell sort, pre-order, reordering, moments, node
-    //    records, groups (one scan), group boxes
-    int64_t tcells = 0;
-    if (!segments(1, [&](size_t q) { return int64_t(cnt(q).ncells); }, &tcells))
-        return fail_all(HH_ENOMEM, "hh_rebuild: batch too large");
-    if (!rb_grow(r->ckey, r->cap_ckey, tcells) || !rb_grow(r->ckey2, r->cap_ckey2, tcells) ||
-        !rb_grow(r->cval, r->cap_cval, tcells) || !rb_grow(r->cval2, r->cap_cval2, tcells) ||
-        !rb_grow(r->flag, r->cap_flag, tcells + int64_t(act.size())) ||
-        !rb_grow(r->pos, r->cap_pos, tcells + int64_t(act.size())))
-        return fail_all(HH_ENOMEM, "hh_rebuild: batch cell buffers do not fit");
-    const int32_t *hs1 = r->h_seg + (r->cap_sims + 1);
-    int depth = 0;
-    for (size_t q = 0; q < act.size(); q++) {
-        RbSim &a = H(int(q));
-        GTreeBuf *g = ctxs[act[q]]->gtree;
-        a.ncells = cnt(q).ncells;
-        int dq = 0;
-        for (int d = 0; d <= kMaxDepth; d++)
-            if (cnt(q).lvl_n[d] > 0) dq = d;
-        g->depth = dq;
-        depth = std::max(depth, dq);
-        const int64_t o = hs1[q];
-        a.ckey = r->ckey + o;
-        a.ckey2 = r->ckey2 + o;
-        a.cval = r->cval + o;
-        a.cval2 = r->cval2 + o;
-        a.flag = r->flag + o + int64_t(q);  // (a terminal entry each)
-        a.pos = r->pos + o + int64_t(q);
-    }
-    const int K2 = int(act.size());
-    const dim3 g2 = dim3(unsigned(gx), unsigned(K2)), one2(1, unsigned(K2));
-    if (!upload()) return fail_all(HH_ECUDA, "hh_rebuild: batch upload failed");
-    k_cell_keys<true><<<g2, 256, 0, st>>>(RbSim{}, D());
-    if ((rc = rb_seg_sort(r, r->ckey, r->ckey2, r->cval, r->cval2, tcells, K2, r->d_seg + (r->cap_sims + 1),
-                          cell_key_bits(max_n))))
-        return fail_all(rc, "hh_rebuild: batch cell sort failed");
-    k_pre_size<true><<<g2, 256, 0, st>>>(RbSim{}, D());
-    k_to_preorder<true><<<g2, 256, 0, st>>>(RbSim{}, D());
-    k_permute<true><<<g2, 256, 0, st>>>(RbSim{}, D());
-    next_stage([](size_t) { return true; });
     for (size_t q = 0; q < act.size(); q++) {  // the reordered state becomes the context's
         hh_ctx *ctx = ctxs[act[q]];
         GTreeBuf *g = ctx->gtree;
@@ -1612,17 +1528,8 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
         a.alt = g->alt;
         a.ids = g->ids;
         a.ids2 = g->ids2;
+        a.ncells = cnt(q).ncells;
     }
-    if (!upload()) return fail_all(HH_ECUDA, "hh_rebuild: batch upload failed");
-    for (int d = depth; d >= 0; d--) k_moments_level<true><<<g2, 256, 0, st>>>(RbSim{}, D(), d);
-    k_node_records<true><<<g2, 256, 0, st>>>(RbSim{}, D());
-    k_flags<true><<<g2, 256, 0, st>>>(RbSim{}, D());
-    if ((rc = cub_exclusive_sum(r->tmp, r->tmp_bytes, r->flag, r->pos, tcells + int64_t(K2), st)))
-        return fail_all(rc, "hh_rebuild: batch scan failed");
-    k_groups<true><<<g2, 256, 0, st>>>(RbSim{}, D());
-    k_group_box<true><<<dim3(unsigned(gx_full), unsigned(K2)), 256, 0, st>>>(RbSim{}, D());
-    launches += 4 + (depth + 1) + 4;
-    if (!read_counts()) return fail_all(HH_ECUDA, "hh_rebuild: group build failed");
     next_stage([&](size_t q) {
         if (cnt(q).G > ctxs[act[q]]->cap_g) {
             rcs[act[q]] = gfail(ctxs[act[q]], HH_ENOMEM, "hh_rebuild: more groups than groups_max");
