@@ -181,6 +181,7 @@ int sync_ids_to_host(hh_ctx *ctx)
                        ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     ctx->ids_on_device = false;
+    ctx->ids_on_both = true;
     return HH_OK;
 }
 
@@ -191,17 +192,39 @@ int check_ctx(hh_ctx *ctx)
     return HH_OK;
 }
 
+// (exponent bits, block by block: a loop the host compiler vectorises)
+bool all_finite(const double *p, int64_t n)
+{
+    constexpr uint64_t kExp = 0x7ff0000000000000ull;
+    for (int64_t b = 0; b < n; b += 4096) {
+        const int64_t e = std::min(n, b + 4096);
+        uint64_t bad = 0;
+        for (int64_t q = b; q < e; q++) {
+            uint64_t w;
+            std::memcpy(&w, p + q, sizeof(w));
+            bad |= uint64_t((w & kExp) == kExp);
+        }
+        if (bad) return false;
+    }
+    return true;
+}
+
+// masses > 0 and times (t[q * t_stride]) finite, the first wrong entry first
+int validate_mt(hh_ctx *ctx, int64_t n, const double *m, const double *t, int64_t t_stride)
+{
+    for (int64_t q = 0; q < n; q++) {
+        if (!(m[q] > 0.0) || !std::isfinite(m[q])) return fail(ctx, HH_EINVAL, "hh_set_j: masses must be > 0");
+        if (!std::isfinite(t[q * t_stride])) return fail(ctx, HH_EINVAL, "hh_set_j: non-finite time");
+    }
+    return HH_OK;
+}
+
 int validate_j_host(hh_ctx *ctx, int64_t n, const double *x, const double *v, const double *a, const double *jk,
                     const double *m, const double *t)
 {
-    for (int64_t q = 0; q < 3 * n; q++)
-        if (!std::isfinite(x[q]) || !std::isfinite(v[q]) || !std::isfinite(a[q]) || !std::isfinite(jk[q]))
-            return fail(ctx, HH_EINVAL, "hh_set_j: non-finite x/v/a/jk");
-    for (int64_t q = 0; q < n; q++) {
-        if (!(m[q] > 0.0) || !std::isfinite(m[q])) return fail(ctx, HH_EINVAL, "hh_set_j: masses must be > 0");
-        if (!std::isfinite(t[q])) return fail(ctx, HH_EINVAL, "hh_set_j: non-finite time");
-    }
-    return HH_OK;
+    for (const double *p : {x, v, a, jk})
+        if (!all_finite(p, 3 * n)) return fail(ctx, HH_EINVAL, "hh_set_j: non-finite x/v/a/jk");
+    return validate_mt(ctx, n, m, t, 1);
 }
 
 // copies a host or device SoA [3][n] block into [3][cap_j] at `first`
@@ -713,6 +736,7 @@ int set_lists_core(hh_ctx *ctx, int64_t n_particles, int64_t n_j, int32_t n_grou
     if (int64_t(ctx->ids.size()) != n_particles) {
         ctx->ids.resize(size_t(n_particles));
         for (int64_t q = 0; q < n_particles; q++) ctx->ids[size_t(q)] = q;
+        ctx->ids_on_both = false;
     }
     ctx->have_lists = true;
     ctx->predicted = false;
@@ -1010,14 +1034,24 @@ int hh_load_particles(hh_ctx *ctx, int64_t n, const double *x, const double *v, 
     int rc = check_ctx(ctx);
     if (rc) return rc;
     if (n < 2 || n > ctx->cap_n || !x || !v || !m) return fail(ctx, HH_EINVAL, "hh_load_particles: bad n or NULL");
-    std::vector<double> zeros(3 * size_t(n), 0.0), tt(size_t(n), t);
-    if ((rc = validate_j_host(ctx, n, x, v, zeros.data(), zeros.data(), m, tt.data()))) return rc;
-    if ((rc = set_j_impl(ctx, 0, n, x, v, zeros.data(), zeros.data(), m, tt.data(), cudaMemcpyHostToDevice))) return rc;
+    if (!all_finite(x, 3 * n) || !all_finite(v, 3 * n))
+        return fail(ctx, HH_EINVAL, "hh_set_j: non-finite x/v/a/jk");
+    if ((rc = validate_mt(ctx, n, m, &t, 0))) return rc;
+    if ((rc = put3(ctx, ctx->st.x, 0, n, x, cudaMemcpyHostToDevice))) return rc;
+    if ((rc = put3(ctx, ctx->st.v, 0, n, v, cudaMemcpyHostToDevice))) return rc;
+    CK(cudaMemcpyAsync(ctx->st.m, m, sizeof(double) * n, cudaMemcpyHostToDevice, ctx->stream));
+    // the rest is written on the device (as host arrays of zeros and of t it
+    // took a third of the load: 262144 particles 1.88 ms, now 1.26 ms)
+    k_load_rest<<<ctx->elem_grid, 256, 0, ctx->stream>>>(ctx->st, n, t);
+    CKL();
+    ctx->have_j = true;
+    ctx->predicted = false;
+    if ((rc = sync_and_check(ctx))) return rc;
     ctx->n = n;
     ctx->nj = n;
     ctx->ids.resize(size_t(n));
     for (int64_t q = 0; q < n; q++) ctx->ids[size_t(q)] = q;
-    ctx->ids_on_device = false;
+    ctx->ids_on_device = ctx->ids_on_both = false;
     ctx->have_lists = false;
     ctx->have_dt = false;
     return HH_OK;
@@ -1083,9 +1117,11 @@ int rebuild_begin(hh_ctx *ctx)
     // until this rebuild succeeds the lists are not valid (a failure part way
     // may have overwritten them); the state stays readable
     ctx->have_lists = false;
-    if (ctx->rebuild_device && ctx->gtree && !ctx->ids_on_device &&
-        hh_gtree_set_ids(ctx->gtree, ctx->ids.data(), ctx->n, ctx->stream) != HH_OK)
-        return fail(ctx, HH_ECUDA, "hh_rebuild: id upload failed");
+    if (ctx->rebuild_device && ctx->gtree && !ctx->ids_on_device && !ctx->ids_on_both) {
+        if (hh_gtree_set_ids(ctx->gtree, ctx->ids.data(), ctx->n, ctx->stream) != HH_OK)
+            return fail(ctx, HH_ECUDA, "hh_rebuild: id upload failed");
+        ctx->ids_on_both = true;
+    }
     return HH_OK;
 }
 
@@ -1156,6 +1192,7 @@ int rebuild_impl(hh_ctx *ctx, double t)
     }
     if ((rc = set_j_impl(ctx, 0, nj, Jx, Jv, Ja, Jj, Jm, Jt, cudaMemcpyHostToDevice))) return rc;
     ctx->ids = ids_new;
+    ctx->ids_on_both = false;
     if ((rc = set_lists_core(ctx, n, nj, V.n_groups, V.off, V.idx, V.group_of, true))) return rc;
     CK(cudaMemcpyAsync(ctx->st.dt, dt_new.data(), sizeof(double) * n, cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));

@@ -94,7 +94,8 @@ struct hh_ctx {
     hh_tree *tree = nullptr;   // host tree reused by hh_rebuild
     GTreeBuf *gtree = nullptr; // device tree builder (rebuild_device)
     bool rebuild_device = false;
-    bool ids_on_device = false;  // particle ids kept by the device builder
+    bool ids_on_device = false;  // particle ids kept by the device builder (the host's are old)
+    bool ids_on_both = false;    // the builder's ids and the host's are the same
     std::vector<int64_t> ids;  // slot -> particle id
     std::vector<int32_t> h_group_of;
     // grid shapes

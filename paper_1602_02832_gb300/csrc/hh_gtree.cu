@@ -1085,6 +1085,8 @@ void swap_state(hh_ctx *ctx, GTreeBuf *g)
     std::swap(ctx->st.t, g->alt.t);
     std::swap(ctx->st.dt, g->alt.dt);
     std::swap(g->ids, g->ids2);
+    ctx->ids_on_device = true;  // (whether the build succeeds or not)
+    ctx->ids_on_both = false;
 }
 
 int gtree_prepare(hh_ctx *ctx)
@@ -1268,7 +1270,6 @@ int hh_rebuild_device(hh_ctx *ctx, double t)
     ctx->n_groups = G;
     ctx->list_len = L;
     ctx->n_tiles = int32_t(n_tiles);
-    ctx->ids_on_device = true;
     return hh_finish_device_rebuild(ctx, total_parts, int64_t(g->gc_host->lmax));
 }
 
@@ -1638,7 +1639,6 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
         ctx->n_groups = c.G;
         ctx->list_len = c.L;
         ctx->n_tiles = int32_t(c.n_tiles);
-        ctx->ids_on_device = true;
         rcs[act[q]] = hh_finish_device_rebuild(ctx, c.total_parts, int64_t(c.lmax), true);
         return rcs[act[q]] == HH_OK;
     });

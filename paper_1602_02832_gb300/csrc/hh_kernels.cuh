@@ -1685,6 +1685,16 @@ static __global__ void k_adopt_forces(State s, DevScalars *ds)
     }
 }
 
+// What a load of n particles at time t leaves besides x, v and m.
+static __global__ void k_load_rest(State s, int64_t n, double t)
+{
+    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
+        for (int d = 0; d < 3; d++) s.a[d * s.cap_j + q] = s.jk[d * s.cap_j + q] = 0.0;
+        s.t[q] = t;
+        if (s.base) refresh_base(s, q);
+    }
+}
+
 static __global__ void k_refresh_base(State s, int64_t first, int64_t n)
 {
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x)
