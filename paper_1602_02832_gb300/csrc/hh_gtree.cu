@@ -569,7 +569,8 @@ __global__ void __launch_bounds__(128) k_node_records(RB_ARGS)
 }
 
 // Bounding box of each group's particles ([3][G] lo and hi) and the particles'
-// group numbers, one warp per group
+// group numbers, one warp per group (17k groups of 262144 particles: 16 us; with
+// FP64 comparisons and one lane's conversions 52 us)
 // (none beyond cap_g groups: the host then reports the overflow).
 template <bool kMany>
 __global__ void k_group_box(RB_ARGS)
@@ -580,32 +581,37 @@ __global__ void k_group_box(RB_ARGS)
     if (G > a.cap_g) return;
     const int lane = threadIdx.x & 31;
     const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const double u = *a.unit;
     for (int64_t g = w0; g < G; g += nw) {
         const int32_t c = a.g_cell[g], b = a.P.begin[c], e = a.P.end[c];
+        // (as ordered integers: an FP64 comparison takes the pipe 64 cycles)
+        unsigned long long lo[3], hi[3];
         for (int32_t p = b + lane; p < e; p += 32) a.group_of[p] = int32_t(g);
+#pragma unroll
         for (int d = 0; d < 3; d++) {
-            double lo = s.x[d * s.cap_j + b], hi = lo;
-            for (int32_t p = b + lane; p < e; p += 32) {
-                const double u = s.x[d * s.cap_j + p];
-                lo = u < lo ? u : lo;
-                hi = u > hi ? u : hi;
-            }
-            for (int off = 16; off > 0; off >>= 1) {
-                const double l2 = __shfl_xor_sync(0xffffffffu, lo, off), h2 = __shfl_xor_sync(0xffffffffu, hi, off);
-                lo = l2 < lo ? l2 : lo;
-                hi = h2 > hi ? h2 : hi;
-            }
-            if (lane == 0) {
-                a.box_lo[d * G + g] = lo;
-                a.box_hi[d * G + g] = hi;
+            lo[d] = hi[d] = order_bits(s.x[d * s.cap_j + min(b + lane, e - 1)]);
+            for (int32_t p = b + lane + 32; p < e; p += 32) {
+                const unsigned long long o = order_bits(s.x[d * s.cap_j + p]);
+                lo[d] = o < lo[d] ? o : lo[d];
+                hi[d] = o > hi[d] ? o : hi[d];
             }
         }
-        if (lane == 0) {
-            const double u = *a.unit;
-            a.box_f[2 * g] = make_float4(float(a.box_lo[g] * u), float(a.box_lo[G + g] * u),
-                                         float(a.box_lo[2 * G + g] * u), 0.f);
-            a.box_f[2 * g + 1] = make_float4(float(a.box_hi[g] * u), float(a.box_hi[G + g] * u),
-                                             float(a.box_hi[2 * G + g] * u), 0.f);
+        for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+            for (int d = 0; d < 3; d++) {
+                const unsigned long long l2 = __shfl_xor_sync(0xffffffffu, lo[d], off);
+                const unsigned long long h2 = __shfl_xor_sync(0xffffffffu, hi[d], off);
+                lo[d] = l2 < lo[d] ? l2 : lo[d];
+                hi[d] = h2 > hi[d] ? h2 : hi[d];
+            }
+        if (lane < 8) {  // lanes 0..2: the lower bounds, 4..6: the upper ones
+            const int d = lane & 3;
+            const bool upper = lane >= 4;
+            const unsigned long long o = d == 0 ? (upper ? hi[0] : lo[0]) : d == 1 ? (upper ? hi[1] : lo[1])
+                                                                                  : (upper ? hi[2] : lo[2]);
+            const double v = from_order_bits(o);
+            if (d < 3) (upper ? a.box_hi : a.box_lo)[d * int64_t(G) + g] = v;
+            reinterpret_cast<float *>(a.box_f)[8 * g + lane] = d < 3 ? float(v * u) : 0.f;
         }
     }
 }
@@ -718,8 +724,8 @@ __global__ void k_paths(RB_ARGS)
 // thread per (group, subtree of ncells / 256 cells), with a table of the
 // topmost unopened cells above those subtrees, spent most of its time on its
 // start: rebuild of 32 clusters with 1k to 32k particles 775 us (table and
-// counts) and 787 us (entries), here 180 and 328 us; of 262144 particles 583
-// and 730 us, here 339 and 570 us.  (Gathering each lane's entries into 16-byte
+// counts) and 787 us (entries), here 180 and 308 us; of 262144 particles 583
+// and 730 us, here 339 and 538 us.  (Gathering each lane's entries into 16-byte
 // stores made it slower, 796 us: it is bound by instructions issued, not by
 // the stores.)
 template <bool kMany, bool kWrite>
@@ -764,9 +770,16 @@ __global__ void __launch_bounds__(128) k_lists(RB_ARGS)
                 if (kWrite) a.lidx[wn++] = int32_t(n + c);
                 nn++;
             } else if (dec == kEmitParticles) {
-                if (kWrite)
-                    for (int32_t p = r.pk.x; p < r.pk.y; p++) a.lidx[wp++] = p;
-                np += r.pk.y - r.pk.x;
+                const int32_t cnt = r.pk.y - r.pk.x;
+                if (kWrite) {  // (four predicated stores a turn: half the instructions of a store a turn)
+                    int32_t *const o = a.lidx + wp;
+                    for (int32_t k = 0; k < cnt; k += 4)
+#pragma unroll
+                        for (int u = 0; u < 4; u++)
+                            if (k + u < cnt) o[k + u] = r.pk.x + k + u;
+                    wp += cnt;
+                }
+                np += cnt;
             }
             c += dec == kOpen ? 1 : r.pk.w;
         }
