@@ -935,8 +935,11 @@ int hh_get_state(hh_ctx *ctx, double *x, double *v, double *a, double *jk, doubl
 int hh_get_ids(hh_ctx *ctx, int64_t *ids)
 {
     if (!ctx || !ids) return hh_set_global_error(HH_EINVAL, "hh_get_ids: NULL");
-    int rc = sync_ids_to_host(ctx);
-    if (rc) return rc;
+    if (ctx->ids_on_device && ctx->gtree) {  // straight to the caller; the device keeps them
+        CK(cudaMemcpyAsync(ids, hh_gtree_ids(ctx->gtree), sizeof(int64_t) * ctx->n, cudaMemcpyDeviceToHost, ctx->stream));
+        CK(cudaStreamSynchronize(ctx->stream));
+        return HH_OK;
+    }
     std::copy(ctx->ids.begin(), ctx->ids.end(), ids);
     return HH_OK;
 }
