@@ -27,6 +27,8 @@ namespace {
 
 constexpr int kBits = 21;
 constexpr int kMaxDepth = 21;
+constexpr int kWalkThreads = 128;  // threads of a walk block
+constexpr int kWalkStage = 512;    // cells that it stages
 constexpr int kPath = 24;  // entries of a chunk's path (at most kMaxDepth ancestors)
 
 // ------------------------------------------------------------ small helpers
@@ -708,85 +710,97 @@ __global__ void k_paths(RB_ARGS)
 }
 
 // The list walk, cut into chunks of `chunk` cells in pre-order: one thread per
-// (group, chunk), a warp taking 32 neighbouring groups (close in space) at one
-// chunk, so that its lanes walk nearly the same cells.  A thread first takes
-// the decisions on the ancestors of the chunk's first cell, from the root
-// down, until one is not opened: that cell is emitted by the chunk that holds
-// it, and the walk here goes on behind its subtree (most chunks end there).
-// Then it walks the chunk's cells in pre-order, skipping every emitted cell's
-// subtree.  The list of a group is the concatenation over the chunks:
-// particles ascending, then nodes ascending, as in the sequential walk.
+// (group, chunk), a block taking kWalkThreads neighbouring groups (close in
+// space) at one chunk, so that its lanes walk nearly the same cells, which the
+// block stages first (a chunk of more than kWalkStage cells, in trees of more
+// than 262144 cells, is read in place).  A thread first takes the decisions on the
+// ancestors of the chunk's first cell, from the root down, until one is not
+// opened: that cell is emitted by the chunk that holds it, and the walk here
+// goes on behind its subtree (most chunks end there).  Then it walks the
+// chunk's cells in pre-order, skipping every emitted cell's subtree.  The list
+// of a group is the concatenation over the chunks: particles ascending, then
+// nodes ascending, as in the sequential walk.
+// The chunks around the groups' own cells take longest, so all rows of groups
+// take those first (turn 0, then outwards on either side): otherwise a few of
+// them run alone at the end.
 // Pass 0 counts into cnt_p/cnt_n[g * R + k] (and zeroes both arrays'
 // terminal entries); pass 1 writes at the scanned offsets.  cnt_n follows
 // cnt_p's terminal entry, so one exclusive scan covers both (each read
 // relative to its first entry).
-// Bound by the decisions' latency and by the scattered stores of pass 1.  A
-// thread per (group, subtree of ncells / 256 cells), with a table of the
-// topmost unopened cells above those subtrees, spent most of its time on its
-// start: rebuild of 32 clusters with 1k to 32k particles 775 us (table and
-// counts) and 787 us (entries), here 180 and 308 us; of 262144 particles 583
-// and 730 us, here 339 and 538 us.  (Gathering each lane's entries into 16-byte
-// stores made it slower, 796 us: it is bound by instructions issued, not by
-// the stores.)
+// Bound by the decisions' latency.  Counts and entries of a rebuild of 32
+// clusters with 1k to 32k particles, and of 262144 particles: a thread per
+// (group, subtree of ncells / 256 cells) with a table of the topmost unopened
+// cells above those subtrees, which spent most of its time on its start, 775 and
+// 787 us, 583 and 730 us; a thread per chunk in launch order 180 and 308 us, 339
+// and 538 us; with the staging and this order 164 and 275 us, 290 and 399 us.
+// (Gathering each lane's entries into 16-byte stores, prefetching the next cell
+// and more warps by fewer registers each made it slower.)
 template <bool kMany, bool kWrite>
-__global__ void __launch_bounds__(128) k_lists(RB_ARGS)
+__global__ void __launch_bounds__(kWalkThreads) k_lists(RB_ARGS)
 {
     RB_SIM;
-    const int32_t R = a.R, n_gb = (a.G + 31) >> 5;
+    __shared__ CellRec s_cell[kWalkStage];
+    const int32_t R = a.R, n_row = (a.G + kWalkThreads - 1) / kWalkThreads;
     const int64_t n = a.n;
     int64_t *cnt_p = a.pair2, *cnt_n = a.pair2 + a.pairs + 1;
     const int64_t *scan_p = a.pscan2, *scan_n = a.pscan2 + a.pairs + 1;
     if (!kWrite && blockIdx.x == 0 && threadIdx.x == 0) cnt_p[a.pairs] = cnt_n[a.pairs] = 0;
     const int64_t pb = kWrite ? scan_p[0] : 0, nb = kWrite ? scan_n[0] : 0;
-    const int32_t total = R * n_gb, lane = threadIdx.x & 31;
-    const int32_t stride = int32_t(gridDim.x * (blockDim.x >> 5));
-    for (int32_t w = int32_t(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); w < total; w += stride) {
-        const int32_t k = w / n_gb, g = (w - k * n_gb) * 32 + lane;
-        if (g >= a.G) continue;
-        const int32_t *row = a.path + int64_t(k) * kPath;
-        const GroupView V = group_view(a, g);
-        const int32_t end = min((k + 1) * a.chunk, a.ncells);
-        int32_t c = k * a.chunk;
-        for (int q = 0; q < kPath; q++) {
-            const int32_t up = __ldg(&row[q]);
-            if (up < 0) continue;
-            const CellRec r = load_cell(a, up);
-            if (decide(a, V, up, r) != kOpen) {
-                c = up + r.pk.w;
-                break;
-            }
+    const int32_t turn = int32_t(blockIdx.x) / n_row, row = int32_t(blockIdx.x) - turn * n_row;
+    if (turn >= R) return;  // (another simulation's grid)
+    const int32_t g = row * kWalkThreads + int32_t(threadIdx.x);
+    int32_t k = a.g_cell[min(row * kWalkThreads + kWalkThreads / 2, a.G - 1)] / a.chunk +
+                ((turn & 1) ? (turn + 1) / 2 : -(turn / 2));
+    if (k < 0) k += R;
+    if (k >= R) k -= R;
+    const int32_t first = k * a.chunk, end = min(first + a.chunk, a.ncells);
+    const bool staged = a.chunk <= kWalkStage;
+    if (staged)
+        for (int32_t c = first + int32_t(threadIdx.x); c < end; c += kWalkThreads) s_cell[c - first] = load_cell(a, c);
+    __syncthreads();
+    if (g >= a.G) return;
+    const int32_t *path = a.path + int64_t(k) * kPath;
+    const GroupView V = group_view(a, g);
+    int32_t c = first;
+    for (int q = 0; q < kPath; q++) {
+        const int32_t up = __ldg(&path[q]);
+        if (up < 0) continue;
+        const CellRec r = load_cell(a, up);
+        if (decide(a, V, up, r) != kOpen) {
+            c = up + r.pk.w;
+            break;
         }
-        const int64_t q = int64_t(g) * R + k;
-        int64_t wp = 0, wn = 0;
-        if (kWrite && c < end) {
-            wp = (scan_p[q] - pb) + (scan_n[int64_t(g) * R] - nb);
-            wn = (scan_p[int64_t(g + 1) * R] - pb) + (scan_n[q] - nb);
-        }
-        int32_t np = 0, nn = 0;
-        while (c < end) {
-            const CellRec r = load_cell(a, c);
-            const int dec = decide(a, V, c, r);
-            if (dec == kEmitNode) {
-                if (kWrite) a.lidx[wn++] = int32_t(n + c);
-                nn++;
-            } else if (dec == kEmitParticles) {
-                const int32_t cnt = r.pk.y - r.pk.x;
-                if (kWrite) {  // (four predicated stores a turn: half the instructions of a store a turn)
-                    int32_t *const o = a.lidx + wp;
-                    for (int32_t k = 0; k < cnt; k += 4)
+    }
+    const int64_t q = int64_t(g) * R + k;
+    int64_t wp = 0, wn = 0;
+    if (kWrite && c < end) {
+        wp = (scan_p[q] - pb) + (scan_n[int64_t(g) * R] - nb);
+        wn = (scan_p[int64_t(g + 1) * R] - pb) + (scan_n[q] - nb);
+    }
+    int32_t np = 0, nn = 0;
+    while (c < end) {
+        const CellRec r = staged ? s_cell[c - first] : load_cell(a, c);
+        const int dec = decide(a, V, c, r);
+        if (dec == kEmitNode) {
+            if (kWrite) a.lidx[wn++] = int32_t(n + c);
+            nn++;
+        } else if (dec == kEmitParticles) {
+            const int32_t cnt = r.pk.y - r.pk.x;
+            if (kWrite) {  // (four predicated stores a turn: half the instructions of a store a turn)
+                int32_t *const o = a.lidx + wp;
+                for (int32_t k = 0; k < cnt; k += 4)
 #pragma unroll
-                        for (int u = 0; u < 4; u++)
-                            if (k + u < cnt) o[k + u] = r.pk.x + k + u;
-                    wp += cnt;
-                }
-                np += cnt;
+                    for (int u = 0; u < 4; u++)
+                        if (k + u < cnt) o[k + u] = r.pk.x + k + u;
+                wp += cnt;
             }
-            c += dec == kOpen ? 1 : r.pk.w;
+            np += cnt;
         }
-        if (!kWrite) {
-            cnt_p[q] = np;
-            cnt_n[q] = nn;
-        }
+        c += dec == kOpen ? 1 : r.pk.w;
+    }
+    if (!kWrite) {
+        cnt_p[q] = np;
+        cnt_n[q] = nn;
     }
 }
 
@@ -1164,11 +1178,8 @@ int32_t walk_chunk(double group_cells, int32_t max_cells)
     return c;
 }
 
-// blocks of 4 warps for the walk: a warp per (32 groups, chunk)
-int64_t walk_blocks(int32_t G, int32_t R)
-{
-    return std::max<int64_t>(1, std::min<int64_t>((int64_t((G + 31) / 32) * R + 3) / 4, int64_t(1) << 28));
-}
+// blocks of the walk: one per (kWalkThreads groups, chunk)
+int64_t walk_blocks(int32_t G, int32_t R) { return int64_t(R) * ((G + kWalkThreads - 1) / kWalkThreads); }
 
 }  // namespace
 
@@ -1258,7 +1269,7 @@ int hh_rebuild_device(hh_ctx *ctx, double t)
     a.pair2 = g->pair_buf;
     a.pscan2 = g->pair_buf + 2 * (pairs + 1);
     const int64_t lgrid = walk_blocks(G, a.R);
-    k_lists<false, false><<<unsigned(lgrid), 128, 0, st>>>(a, nullptr);
+    k_lists<false, false><<<unsigned(lgrid), kWalkThreads, 0, st>>>(a, nullptr);
     if ((rc = cub_exclusive_sum(g->tmp, g->tmp_bytes, a.pair2, a.pscan2, 2 * (pairs + 1), st)))  // cnt_p, cnt_n at once
         return gfail(ctx, rc, "hh_rebuild: scan failed");
     k_list_off<false><<<grid, 256, 0, st>>>(a, nullptr);
@@ -1273,7 +1284,7 @@ int hh_rebuild_device(hh_ctx *ctx, double t)
     if (n_tiles > ctx->cap_tiles) return gfail(ctx, HH_ENOMEM, "hh_rebuild: too many tiles");
     if ((rc = grow_list(ctx, L))) return rc;
     a.lidx = ctx->idx;
-    k_lists<false, true><<<unsigned(lgrid), 128, 0, st>>>(a, nullptr);
+    k_lists<false, true><<<unsigned(lgrid), kWalkThreads, 0, st>>>(a, nullptr);
     k_tiles<false><<<grid, 256, 0, st>>>(a, nullptr);
     launches += 2;
     const cudaError_t ce = cudaGetLastError();
@@ -1423,6 +1434,8 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
         if (rcs[s] == HH_OK) act.push_back(s);
     }
     if (act.empty()) return HH_OK;
+    // (the largest first: the blocks that take longest do not start last)
+    std::stable_sort(act.begin(), act.end(), [&](int p, int q) { return ctxs[p]->n > ctxs[q]->n; });
     const int K0 = int(act.size());
     int stage = 0;
     auto H = [&](int q) -> RbSim & { return r->h_sims[stage * r->cap_sims + q]; };
@@ -1576,10 +1589,11 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
         group_cells += double(cnt(q).G) * cnt(q).ncells;
         max_cells = std::max(max_cells, cnt(q).ncells);
     }
+    const int32_t chunk = walk_chunk(group_cells, max_cells);
     for (size_t q = 0; q < act.size(); q++) {
         RbSim &a = H(int(q));
         a.G = cnt(q).G;
-        a.chunk = walk_chunk(group_cells, max_cells);
+        a.chunk = chunk;
         a.R = (a.ncells + a.chunk - 1) / a.chunk;
         a.pairs = int64_t(a.G) * a.R;
         a.path = reinterpret_cast<int32_t *>(t_path);  // offsets for now
@@ -1612,7 +1626,7 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
     const dim3 lg3 = dim3(unsigned(lgrid), unsigned(K3));
     if (!upload()) return fail_all(HH_ECUDA, "hh_rebuild: batch upload failed");
     k_paths<true><<<dim3(unsigned((max_R + 127) / 128), unsigned(K3)), 128, 0, st>>>(RbSim{}, D());
-    k_lists<true, false><<<lg3, 128, 0, st>>>(RbSim{}, D());
+    k_lists<true, false><<<lg3, kWalkThreads, 0, st>>>(RbSim{}, D());
     if ((rc = cub_exclusive_sum(r->tmp, r->tmp_bytes, r->pair2, r->pscan2, t_pair, st)))
         return fail_all(rc, "hh_rebuild: batch scan failed");
     k_list_off<true><<<g3, 256, 0, st>>>(RbSim{}, D());
@@ -1638,7 +1652,7 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
     const dim3 g4 = dim3(unsigned(gx), unsigned(K4));
     const dim3 lg4 = dim3(unsigned(lgrid), unsigned(K4));
     if (!upload()) return fail_all(HH_ECUDA, "hh_rebuild: batch upload failed");
-    k_lists<true, true><<<lg4, 128, 0, st>>>(RbSim{}, D());
+    k_lists<true, true><<<lg4, kWalkThreads, 0, st>>>(RbSim{}, D());
     k_tiles<true><<<g4, 256, 0, st>>>(RbSim{}, D());
     launches += 2;
     const cudaError_t ce = cudaGetLastError();

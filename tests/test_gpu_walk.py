@@ -42,7 +42,7 @@ def _positions(form, n):
     ("plummer", 4000, 8, 64, 0.0, "hilbert"), ("plummer", 4000, 8, 64, 30.0, "morton"),
     ("tiny", 3000, 8, 64, 0.5, "morton"), ("huge", 3000, 8, 64, 0.5, "hilbert"), ("far", 3000, 8, 64, 0.5, "morton"),
     ("pairs", 3001, 1, 16, 0.5, "morton"), ("clump", 900, 8, 64, 0.5, "hilbert"), ("line", 3000, 4, 40, 0.6, "morton"),
-    ("plummer", 120000, 8, 256, 0.75, "morton")])
+    ("plummer", 120000, 8, 256, 0.75, "morton"), ("plummer", 190000, 1, 512, 1.2, "morton")])
 def test_device_tree_forms(hh, orc, form, n, leaf, n_crit, theta, order):
     x, v, m = _positions(form, n)
     z = np.zeros_like(x)
