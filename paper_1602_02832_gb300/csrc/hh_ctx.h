@@ -28,11 +28,10 @@ struct RbScratch;
 RbScratch *hh_rb_scratch_create();
 void hh_rb_scratch_free(RbScratch *r);
 int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rcs, RbScratch *r);
-// Ends a device rebuild (hh_api.cu): work-item capacity, then the sizes on the
-// device and the mixed form's base records on the context's stream,
-// synchronised.  batched: the batched build's closing kernel (k_finish) sets
-// the sizes and base records, and it synchronises.
-int hh_finish_device_rebuild(hh_ctx *ctx, int64_t total_parts, int64_t lmax, bool batched = false);
+// Ends a device rebuild (hh_api.cu) on the host: work-item capacity and sizes
+// (the builder's closing kernel has set those on the device, and the mixed
+// form's base records).
+int hh_finish_device_rebuild(hh_ctx *ctx, int64_t total_parts, int64_t lmax);
 // hh_rebuild for k contexts (hh_api.cu): device builders of at most
 // kBatchRebuildMaxN particles are rebuilt together by hh_rebuild_device_many
 // (when there are two or more), the others one by one.

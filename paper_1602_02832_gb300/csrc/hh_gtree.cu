@@ -142,6 +142,7 @@ struct RbSim {
     DevScalars *ds;           // the context's device sizes (set by k_finish)
     double t, theta;
     int64_t n, pairs;
+    int64_t cap_list, cap_tiles;  // entries and tiles that fit
     int32_t cap_g, cap_cells, leaf, n_crit, order, tile_i, part_len, work_item, work_split;
     int32_t seg;                 // where its particles begin among a batch's
     int32_t ncells, G;           // set by the host as they become known
@@ -746,6 +747,7 @@ __global__ void __launch_bounds__(kWalkThreads) k_lists(RB_ARGS)
     const int64_t *scan_p = a.pscan2, *scan_n = a.pscan2 + a.pairs + 1;
     if (!kWrite && blockIdx.x == 0 && threadIdx.x == 0) cnt_p[a.pairs] = cnt_n[a.pairs] = 0;
     const int64_t pb = kWrite ? scan_p[0] : 0, nb = kWrite ? scan_n[0] : 0;
+    if (kWrite && (scan_p[a.pairs] - pb) + (scan_n[a.pairs] - nb) > a.cap_list) return;  // (the host grows the lists)
     const int32_t turn = int32_t(blockIdx.x) / n_row, row = int32_t(blockIdx.x) - turn * n_row;
     if (turn >= R) return;  // (another simulation's grid)
     const int32_t g = row * kWalkThreads + int32_t(threadIdx.x);
@@ -804,32 +806,29 @@ __global__ void __launch_bounds__(kWalkThreads) k_lists(RB_ARGS)
     }
 }
 
-// off[g] = entries of all lists before group g (g = 0..G)
-template <bool kMany>
-__global__ void k_list_off(RB_ARGS)
-{
-    RB_SIM;
-    const int32_t G = a.G, R = a.R;
-    const int64_t *scan_p = a.pscan2, *scan_n = a.pscan2 + a.pairs + 1;
-    const int64_t pb = scan_p[0], nb = scan_n[0];
-    for (int32_t g = blockIdx.x * blockDim.x + threadIdx.x; g <= G; g += gridDim.x * blockDim.x)
-        a.off[g] = (scan_p[int64_t(g) * R] - pb) + (scan_n[int64_t(g) * R] - nb);
-}
-
-// tiles of <= tile_i particles per group and their list parts; the longest list
+// off[g] = entries of all lists before group g (g = 0..G); tiles of <= tile_i
+// particles per group and their list parts; the longest list
 template <bool kMany>
 __global__ void k_tile_counts(RB_ARGS)
 {
     RB_SIM;
-    const int32_t G = a.G;
+    const int32_t G = a.G, R = a.R;
+    const int64_t *scan_p = a.pscan2, *scan_n = a.pscan2 + a.pairs + 1;
+    const int64_t base = scan_p[0] + scan_n[0];
     int64_t *ntile = a.nt2, *nparts = a.nt2 + G + 1;
-    if (blockIdx.x == 0 && threadIdx.x == 0) ntile[G] = nparts[G] = 0;  // terminal entries of the scan
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        ntile[G] = nparts[G] = 0;  // terminal entries of the scan
+        a.off[G] = scan_p[a.pairs] + scan_n[a.pairs] - base;
+    }
     unsigned long long lmax = 0ull;
     for (int32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x) {
+        const int64_t q = int64_t(g) * R;
+        const int64_t off = scan_p[q] + scan_n[q] - base;
+        const int64_t L = scan_p[q + R] + scan_n[q + R] - base - off;
+        a.off[g] = off;
         const int32_t c = a.g_cell[g];
         const int64_t cnt = a.P.end[c] - a.P.begin[c];
         const int64_t nt = (cnt + a.tile_i - 1) / a.tile_i;
-        const int64_t L = a.off[g + 1] - a.off[g];
         const int64_t parts = L > 0 ? (L + a.part_len - 1) / a.part_len : 1;
         ntile[g] = nt;
         nparts[g] = nt * parts;
@@ -838,23 +837,20 @@ __global__ void k_tile_counts(RB_ARGS)
     if (lmax) atomicMax(&a.gc->lmax, lmax);
 }
 
-// list length and tile / work-item totals (one thread per simulation)
-template <bool kMany>
-__global__ void k_store_totals(RB_ARGS)
-{
-    RB_SIM;
-    const int32_t G = a.G;
-    const int64_t *tile_off = a.tscan2, *parts_off = a.tscan2 + G + 1;
-    a.gc->L = a.off[G];
-    a.gc->n_tiles = tile_off[G] - tile_off[0];
-    a.gc->total_parts = parts_off[G] - parts_off[0];
-}
-
+// tiles (none when they do not fit: the host reports it), and the list length
+// and tile / work-item totals
 template <bool kMany>
 __global__ void k_tiles(RB_ARGS)
 {
     RB_SIM;
-    const int64_t t0 = a.tscan2[0];
+    const int64_t *parts_off = a.tscan2 + a.G + 1;
+    const int64_t t0 = a.tscan2[0], n_tiles = a.tscan2[a.G] - t0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.gc->L = a.off[a.G];
+        a.gc->n_tiles = n_tiles;
+        a.gc->total_parts = parts_off[a.G] - parts_off[0];
+    }
+    if (n_tiles > a.cap_tiles) return;
     for (int32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < a.G; g += gridDim.x * blockDim.x) {
         const int32_t c = a.g_cell[g];
         const int32_t b = a.P.begin[c], e = a.P.end[c];
@@ -863,14 +859,16 @@ __global__ void k_tiles(RB_ARGS)
     }
 }
 
-// Closing step of a batched build: the context's sizes on the device and,
-// for the mixed form, the base records of every j entry (particles in their
-// new order, then the new nodes).
+// Closing step: the context's sizes on the device and, for the mixed form, the
+// base records of every j entry (particles in their new order, then the new
+// nodes).  Nothing when the lists or the tiles do not fit: the host then grows
+// the lists and takes this step again, or fails.
 template <bool kMany>
 __global__ void k_finish(RB_ARGS)
 {
     RB_SIM;
     const GCounts *gc = a.gc;
+    if (gc->L > a.cap_list || gc->n_tiles > a.cap_tiles) return;
     const int64_t nj = a.n + gc->ncells;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         a.ds->n = a.n;
@@ -1078,7 +1076,9 @@ RbSim rb_sim(hh_ctx *ctx, GTreeBuf *g, double t)
     a.group_of = ctx->group_of;
     a.off = ctx->off;
     a.lidx = ctx->idx;
+    a.cap_list = ctx->cap_list;
     a.tiles = ctx->tiles;
+    a.cap_tiles = ctx->cap_tiles;
     a.nt2 = g->ntile;
     a.tscan2 = g->tile_off;
     a.pair2 = g->pair_buf;
@@ -1200,7 +1200,7 @@ int hh_rebuild_device(hh_ctx *ctx, double t)
     int64_t launches = 0;
     RbSim a = rb_sim(ctx, g, t);
     // Sizes stay on the device (GCounts) and the host reads them twice: after
-    // the tree and the groups, and after the list counts.
+    // the tree and the groups, and at the end.
     auto read_counts = [&]() {
         cudaMemcpyAsync(g->gc_host, g->gc, sizeof(GCounts), cudaMemcpyDeviceToHost, st);
         return cudaStreamSynchronize(st) == cudaSuccess;
@@ -1272,21 +1272,29 @@ int hh_rebuild_device(hh_ctx *ctx, double t)
     k_lists<false, false><<<unsigned(lgrid), kWalkThreads, 0, st>>>(a, nullptr);
     if ((rc = cub_exclusive_sum(g->tmp, g->tmp_bytes, a.pair2, a.pscan2, 2 * (pairs + 1), st)))  // cnt_p, cnt_n at once
         return gfail(ctx, rc, "hh_rebuild: scan failed");
-    k_list_off<false><<<grid, 256, 0, st>>>(a, nullptr);
-    // 4. tiles and their work-item capacity (from the list lengths)
+    // 4. tiles and their work-item capacity (from the list lengths), entries and
+    //    closing step: the host reads the sizes after all of it, and takes the
+    //    last two again if the lists had to grow
     k_tile_counts<false><<<grid, 256, 0, st>>>(a, nullptr);
     if ((rc = cub_exclusive_sum(g->tmp, g->tmp_bytes, g->ntile, g->tile_off, 2 * (int64_t(G) + 1), st)))
         return gfail(ctx, rc, "hh_rebuild: scan failed");
-    k_store_totals<false><<<1, 1, 0, st>>>(a, nullptr);
-    launches += 5;
-    if (!read_counts()) return gfail(ctx, HH_ECUDA, "hh_rebuild: list count failed");
-    const int64_t L = g->gc_host->L, n_tiles = g->gc_host->n_tiles, total_parts = g->gc_host->total_parts;
-    if (n_tiles > ctx->cap_tiles) return gfail(ctx, HH_ENOMEM, "hh_rebuild: too many tiles");
-    if ((rc = grow_list(ctx, L))) return rc;
-    a.lidx = ctx->idx;
-    k_lists<false, true><<<unsigned(lgrid), kWalkThreads, 0, st>>>(a, nullptr);
     k_tiles<false><<<grid, 256, 0, st>>>(a, nullptr);
-    launches += 2;
+    launches += 4;
+    int64_t L = 0, n_tiles = 0;
+    const int fgrid = int(std::min<int64_t>(ctx->elem_grid, (n + ncells + 255) / 256));
+    for (int pass = 0; pass < 2; pass++) {
+        k_lists<false, true><<<unsigned(lgrid), kWalkThreads, 0, st>>>(a, nullptr);
+        k_finish<false><<<fgrid, 256, 0, st>>>(a, nullptr);
+        launches += 2;
+        if (!read_counts()) return gfail(ctx, HH_ECUDA, "hh_rebuild: list count failed");
+        L = g->gc_host->L;
+        n_tiles = g->gc_host->n_tiles;
+        if (n_tiles > ctx->cap_tiles) return gfail(ctx, HH_ENOMEM, "hh_rebuild: too many tiles");
+        if (L <= ctx->cap_list) break;
+        if ((rc = grow_list(ctx, L))) return rc;
+        a.lidx = ctx->idx;
+        a.cap_list = ctx->cap_list;
+    }
     const cudaError_t ce = cudaGetLastError();
     if (ce != cudaSuccess) return gfail(ctx, HH_ECUDA, cudaGetErrorString(ce));
     hh_count_launches(launches);  // kernels of this file; the radix sort and the scans are CUB's
@@ -1294,7 +1302,7 @@ int hh_rebuild_device(hh_ctx *ctx, double t)
     ctx->n_groups = G;
     ctx->list_len = L;
     ctx->n_tiles = int32_t(n_tiles);
-    return hh_finish_device_rebuild(ctx, total_parts, int64_t(g->gc_host->lmax));
+    return hh_finish_device_rebuild(ctx, g->gc_host->total_parts, int64_t(g->gc_host->lmax));
 }
 
 // ---------------------------------------------------------------- many at once
@@ -1629,58 +1637,64 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
     k_lists<true, false><<<lg3, kWalkThreads, 0, st>>>(RbSim{}, D());
     if ((rc = cub_exclusive_sum(r->tmp, r->tmp_bytes, r->pair2, r->pscan2, t_pair, st)))
         return fail_all(rc, "hh_rebuild: batch scan failed");
-    k_list_off<true><<<g3, 256, 0, st>>>(RbSim{}, D());
     k_tile_counts<true><<<g3, 256, 0, st>>>(RbSim{}, D());
     if ((rc = cub_exclusive_sum(r->tmp, r->tmp_bytes, r->nt2, r->tscan2, t_nt, st)))
         return fail_all(rc, "hh_rebuild: batch scan failed");
-    k_store_totals<true><<<one3, 1, 0, st>>>(RbSim{}, D());
-    launches += 5;
+    k_tiles<true><<<g3, 256, 0, st>>>(RbSim{}, D());
+    // 4. entries and closing step, again for the contexts whose lists had to
+    //    grow; then per context on the host: work-item capacity and sizes
+    int64_t fx = 1;
+    for (size_t q = 0; q < act.size(); q++)
+        fx = std::max<int64_t>(fx, std::min<int64_t>(ctxs[act[q]]->elem_grid, (ctxs[act[q]]->n + cnt(q).ncells + 255) / 256));
+    auto entries = [&]() {
+        const unsigned k = unsigned(act.size());
+        k_lists<true, true><<<dim3(unsigned(lgrid), k), kWalkThreads, 0, st>>>(RbSim{}, D());
+        k_finish<true><<<dim3(unsigned(fx), k), 256, 0, st>>>(RbSim{}, D());
+        launches += 2;
+    };
+    entries();
+    launches += 4;
     if (!read_counts()) return fail_all(HH_ECUDA, "hh_rebuild: list count failed");
+    const std::vector<int> all_act = act, all_slot = slot;
+    std::vector<char> done(all_act.size(), 0);  // (by position in all_act)
     next_stage([&](size_t q) {
         hh_ctx *ctx = ctxs[act[q]];
         if (cnt(q).n_tiles > ctx->cap_tiles) {
             rcs[act[q]] = gfail(ctx, HH_ENOMEM, "hh_rebuild: too many tiles");
             return false;
         }
+        if (cnt(q).L <= ctx->cap_list) {
+            done[q] = 1;
+            return false;
+        }
         if ((rcs[act[q]] = grow_list(ctx, cnt(q).L)) != HH_OK) return false;
+        done[q] = 1;
         return true;
     });
-    if (act.empty()) return HH_OK;
-    // 4. lists and tiles
-    for (size_t q = 0; q < act.size(); q++) H(int(q)).lidx = ctxs[act[q]]->idx;
-    const int K4 = int(act.size());
-    const dim3 g4 = dim3(unsigned(gx), unsigned(K4));
-    const dim3 lg4 = dim3(unsigned(lgrid), unsigned(K4));
-    if (!upload()) return fail_all(HH_ECUDA, "hh_rebuild: batch upload failed");
-    k_lists<true, true><<<lg4, kWalkThreads, 0, st>>>(RbSim{}, D());
-    k_tiles<true><<<g4, 256, 0, st>>>(RbSim{}, D());
-    launches += 2;
+    if (!act.empty()) {
+        for (size_t q = 0; q < act.size(); q++) {
+            H(int(q)).lidx = ctxs[act[q]]->idx;
+            H(int(q)).cap_list = ctxs[act[q]]->cap_list;
+        }
+        if (!upload()) return fail_all(HH_ECUDA, "hh_rebuild: batch upload failed");
+        entries();
+    }
     const cudaError_t ce = cudaGetLastError();
-    if (ce != cudaSuccess) return fail_all(HH_ECUDA, cudaGetErrorString(ce));
-    // 5. per context on the host: work-item capacity and sizes; then one
-    //    closing kernel over those that got them
-    next_stage([&](size_t q) {
-        hh_ctx *ctx = ctxs[act[q]];
-        const GCounts &c = cnt(q);
+    const bool ok = ce == cudaSuccess && cudaStreamSynchronize(st) == cudaSuccess;
+    for (size_t q = 0; q < all_act.size(); q++) {
+        if (!done[q]) continue;
+        hh_ctx *ctx = ctxs[all_act[q]];
+        const GCounts &c = r->h_gc[all_slot[q]];
+        if (!ok) {
+            rcs[all_act[q]] = gfail(ctx, HH_ECUDA, "hh_rebuild: batch build failed");
+            continue;
+        }
         ctx->nj = ctx->n + c.ncells;
         ctx->n_groups = c.G;
         ctx->list_len = c.L;
         ctx->n_tiles = int32_t(c.n_tiles);
-        rcs[act[q]] = hh_finish_device_rebuild(ctx, c.total_parts, int64_t(c.lmax), true);
-        return rcs[act[q]] == HH_OK;
-    });
-    if (!act.empty()) {
-        int64_t fx = 1;
-        for (int s : act) fx = std::max<int64_t>(fx, std::min<int64_t>(ctxs[s]->elem_grid, (ctxs[s]->nj + 255) / 256));
-        if (!upload()) return fail_all(HH_ECUDA, "hh_rebuild: batch upload failed");
-        k_finish<true><<<dim3(unsigned(fx), unsigned(act.size())), 256, 0, st>>>(RbSim{}, D());
-        launches++;
+        rcs[all_act[q]] = hh_finish_device_rebuild(ctx, c.total_parts, int64_t(c.lmax));
     }
     hh_count_launches(launches);  // kernels of this file; the sorts and scans are CUB's
-    const cudaError_t ce2 = cudaGetLastError();
-    if (ce2 != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) {
-        for (int s : act) ctxs[s]->have_lists = false;
-        return fail_all(HH_ECUDA, "hh_rebuild: batch build failed");
-    }
     return HH_OK;
 }

@@ -68,3 +68,29 @@ def test_device_tree_forms(hh, orc, form, n, leaf, n_crit, theta, order):
     diff = sum(1 for g in range(T.n_groups)
                if not np.array_equal(idx[off[g]:off[g + 1]], T.list_idx[T.list_off[g]:T.list_off[g + 1]]))
     assert diff <= T.n_groups // 1000, diff   # (a tie of an opening test at its last bit)
+
+
+def test_batched_rebuild_grows_some_lists(hh):
+    # contexts of a batch whose lists do not fit take the entries again; the
+    # others keep theirs: all equal a build alone with room enough
+    sizes, ctxs, alone = (700, 3000, 1500, 3000), [], []
+    cfg = hh.hh_config_default()
+    cfg.precision = hh.HH_MIXED
+    for k, n in enumerate(sizes):
+        x, v, m = synth.plummer(n, 70 + k)
+        for lst, room in ((ctxs, 16 if k % 2 else 400 * n), (alone, 400 * n)):
+            c = hh.Context(cfg, n, 3 * n, room, n)
+            c.hh_load_particles(x.T, v.T, m)
+            c.hh_set_rebuild_device(True)
+            lst.append(c)
+    with hh.Batch(hh.HH_MIXED, max_sims=len(sizes), max_steps=8) as b:
+        assert b.hh_batch_rebuild(ctxs, 0.0) == [hh.HH_OK] * len(sizes)
+    for c, d in zip(ctxs, alone):
+        d.hh_rebuild(0.0)
+        assert c.nj == d.nj and all(np.array_equal(p, q) for p, q in zip(c.hh_get_lists(), d.hh_get_lists()))
+        act = np.arange(c.n, dtype=np.int32)
+        for e in (c, d):
+            e.hh_predict(0.0)
+        assert all(np.array_equal(p, q) for p, q in zip(c.hh_force(act), d.hh_force(act)))
+        c.close()
+        d.close()
