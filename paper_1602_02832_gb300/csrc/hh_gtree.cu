@@ -165,6 +165,7 @@ __device__ __forceinline__ const RbSim &rb_sim_of(const RbSim &one, const RbSim 
     return *reinterpret_cast<const RbSim *>(sh);
 }
 #define RB_SIM                                                      \
+    after_previous();                                               \
     __shared__ __align__(16) unsigned char rb_rec_[sizeof(RbSim)]; \
     const RbSim &a = rb_sim_of<kMany>(one, many, rb_rec_)
 
@@ -1206,9 +1207,9 @@ int hh_rebuild_device(hh_ctx *ctx, double t)
         return cudaStreamSynchronize(st) == cudaSuccess;
     };
     // 1. bounding box, synchronisation check, keys, sort
-    k_root_init<false><<<1, 1, 0, st>>>(a, nullptr);
-    k_box<false><<<grid, 256, 0, st>>>(a, nullptr);
-    k_keys<false><<<grid, 256, 0, st>>>(a, nullptr);
+    launch_after(k_root_init<false>, dim3(1), dim3(1), st, true, a, nullptr);
+    launch_after(k_box<false>, dim3(grid), dim3(256), st, true, a, nullptr);
+    launch_after(k_keys<false>, dim3(grid), dim3(256), st, true, a, nullptr);
     launches += 3;
     {
         size_t need = 0;
@@ -1229,15 +1230,15 @@ int hh_rebuild_device(hh_ctx *ctx, double t)
     // 2. cells and groups, particles into Morton order and node records, group
     //    boxes: all into the builder's buffers, which become the context's when
     //    the tree is known to fit
-    k_chains<false><<<grid, 256, 0, st>>>(a, nullptr);
+    launch_after(k_chains<false>, dim3(grid), dim3(256), st, true, a, nullptr);
     if ((rc = cub_exclusive_sum(g->tmp, g->tmp_bytes, a.cnt, a.pos, n + 1, st)))
         return gfail(ctx, rc, "hh_rebuild: scan failed");
-    k_begin_cells<false><<<grid, 256, 0, st>>>(a, nullptr);
-    k_cells<false><<<grid8, 256, 0, st>>>(a, nullptr);
-    k_permute<false><<<grid, 256, 0, st>>>(a, nullptr);
-    k_moments<false><<<grid8, 256, 0, st>>>(a, nullptr);
-    k_node_records<false><<<grid, 128, 0, st>>>(a, nullptr);
-    k_group_box<false><<<grid8, 256, 0, st>>>(a, nullptr);
+    launch_after(k_begin_cells<false>, dim3(grid), dim3(256), st, true, a, nullptr);
+    launch_after(k_cells<false>, dim3(grid8), dim3(256), st, true, a, nullptr);
+    launch_after(k_permute<false>, dim3(grid), dim3(256), st, true, a, nullptr);
+    launch_after(k_moments<false>, dim3(grid8), dim3(256), st, true, a, nullptr);
+    launch_after(k_node_records<false>, dim3(grid), dim3(128), st, true, a, nullptr);
+    launch_after(k_group_box<false>, dim3(grid8), dim3(256), st, true, a, nullptr);
     launches += 7;
     if (!read_counts()) return gfail(ctx, HH_ECUDA, "hh_rebuild: tree build failed");
     if (g->gc_host->bad) return gfail(ctx, HH_ESTATE, "hh_rebuild: particles are not synchronised at t");
@@ -1259,7 +1260,7 @@ int hh_rebuild_device(hh_ctx *ctx, double t)
     if (!grow(g->path_buf, g->path_cap, int64_t(a.R) * kPath))
         return gfail(ctx, HH_ENOMEM, "hh_rebuild: list walk table does not fit");
     a.path = g->path_buf;
-    k_paths<false><<<(a.R + 127) / 128, 128, 0, st>>>(a, nullptr);
+    launch_after(k_paths<false>, dim3((a.R + 127) / 128), dim3(128), st, true, a, nullptr);
     const int64_t pairs = int64_t(G) * a.R;
     if (2 * (pairs + 1) >= int64_t(INT32_MAX))  // (one scan covers both count arrays)
         return gfail(ctx, HH_ENOMEM, "hh_rebuild: too many (group, chunk) pairs");
@@ -1269,22 +1270,22 @@ int hh_rebuild_device(hh_ctx *ctx, double t)
     a.pair2 = g->pair_buf;
     a.pscan2 = g->pair_buf + 2 * (pairs + 1);
     const int64_t lgrid = walk_blocks(G, a.R);
-    k_lists<false, false><<<unsigned(lgrid), kWalkThreads, 0, st>>>(a, nullptr);
+    launch_after(k_lists<false, false>, dim3(unsigned(lgrid)), dim3(kWalkThreads), st, true, a, nullptr);
     if ((rc = cub_exclusive_sum(g->tmp, g->tmp_bytes, a.pair2, a.pscan2, 2 * (pairs + 1), st)))  // cnt_p, cnt_n at once
         return gfail(ctx, rc, "hh_rebuild: scan failed");
     // 4. tiles and their work-item capacity (from the list lengths), entries and
     //    closing step: the host reads the sizes after all of it, and takes the
     //    last two again if the lists had to grow
-    k_tile_counts<false><<<grid, 256, 0, st>>>(a, nullptr);
+    launch_after(k_tile_counts<false>, dim3(grid), dim3(256), st, true, a, nullptr);
     if ((rc = cub_exclusive_sum(g->tmp, g->tmp_bytes, g->ntile, g->tile_off, 2 * (int64_t(G) + 1), st)))
         return gfail(ctx, rc, "hh_rebuild: scan failed");
-    k_tiles<false><<<grid, 256, 0, st>>>(a, nullptr);
+    launch_after(k_tiles<false>, dim3(grid), dim3(256), st, true, a, nullptr);
     launches += 4;
     int64_t L = 0, n_tiles = 0;
     const int fgrid = int(std::min<int64_t>(ctx->elem_grid, (n + ncells + 255) / 256));
     for (int pass = 0; pass < 2; pass++) {
-        k_lists<false, true><<<unsigned(lgrid), kWalkThreads, 0, st>>>(a, nullptr);
-        k_finish<false><<<fgrid, 256, 0, st>>>(a, nullptr);
+        launch_after(k_lists<false, true>, dim3(unsigned(lgrid)), dim3(kWalkThreads), st, true, a, nullptr);
+        launch_after(k_finish<false>, dim3(fgrid), dim3(256), st, true, a, nullptr);
         launches += 2;
         if (!read_counts()) return gfail(ctx, HH_ECUDA, "hh_rebuild: list count failed");
         L = g->gc_host->L;
@@ -1524,9 +1525,9 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
     }
     if (!upload()) return fail_all(HH_ECUDA, "hh_rebuild: batch upload failed");
     const dim3 g1 = dim3(unsigned(gx), unsigned(K0)), one1(1, unsigned(K0)), g8 = dim3(unsigned(gx8), unsigned(K0));
-    k_root_init<true><<<one1, 1, 0, st>>>(RbSim{}, D());
-    k_box<true><<<g1, 256, 0, st>>>(RbSim{}, D());
-    k_keys<true><<<g1, 256, 0, st>>>(RbSim{}, D());
+    launch_after(k_root_init<true>, one1, dim3(1), st, true, RbSim{}, D());
+    launch_after(k_box<true>, g1, dim3(256), st, true, RbSim{}, D());
+    launch_after(k_keys<true>, g1, dim3(256), st, true, RbSim{}, D());
     launches += 3;
     // one stable sort of all keys, then one by simulation (a segmented sort
     // gives each simulation one block: a rebuild of 32 clusters with 1k to 32k
@@ -1546,15 +1547,15 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
     }
     // 2. cells and groups, reordering, node records, group boxes, all into the
     //    builders' buffers
-    k_chains<true><<<g1, 256, 0, st>>>(RbSim{}, D());
+    launch_after(k_chains<true>, g1, dim3(256), st, true, RbSim{}, D());
     if ((rc = cub_exclusive_sum(r->tmp, r->tmp_bytes, r->cnt, r->pos, tot + K0, st)))
         return fail_all(rc, "hh_rebuild: batch scan failed");
-    k_begin_cells<true><<<g1, 256, 0, st>>>(RbSim{}, D());
-    k_cells<true><<<g8, 256, 0, st>>>(RbSim{}, D());
-    k_permute<true><<<g1, 256, 0, st>>>(RbSim{}, D());
-    k_moments<true><<<g8, 256, 0, st>>>(RbSim{}, D());
-    k_node_records<true><<<g1, 128, 0, st>>>(RbSim{}, D());
-    k_group_box<true><<<g8, 256, 0, st>>>(RbSim{}, D());
+    launch_after(k_begin_cells<true>, g1, dim3(256), st, true, RbSim{}, D());
+    launch_after(k_cells<true>, g8, dim3(256), st, true, RbSim{}, D());
+    launch_after(k_permute<true>, g1, dim3(256), st, true, RbSim{}, D());
+    launch_after(k_moments<true>, g8, dim3(256), st, true, RbSim{}, D());
+    launch_after(k_node_records<true>, g1, dim3(128), st, true, RbSim{}, D());
+    launch_after(k_group_box<true>, g8, dim3(256), st, true, RbSim{}, D());
     launches += 7;
     if (!read_counts()) return fail_all(HH_ECUDA, "hh_rebuild: tree build failed");
     next_stage([&](size_t q) {
@@ -1633,14 +1634,14 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
     const dim3 g3 = dim3(unsigned(gx), unsigned(K3)), one3(1, unsigned(K3));
     const dim3 lg3 = dim3(unsigned(lgrid), unsigned(K3));
     if (!upload()) return fail_all(HH_ECUDA, "hh_rebuild: batch upload failed");
-    k_paths<true><<<dim3(unsigned((max_R + 127) / 128), unsigned(K3)), 128, 0, st>>>(RbSim{}, D());
-    k_lists<true, false><<<lg3, kWalkThreads, 0, st>>>(RbSim{}, D());
+    launch_after(k_paths<true>, dim3(unsigned((max_R + 127) / 128), unsigned(K3)), dim3(128), st, true, RbSim{}, D());
+    launch_after(k_lists<true, false>, lg3, dim3(kWalkThreads), st, true, RbSim{}, D());
     if ((rc = cub_exclusive_sum(r->tmp, r->tmp_bytes, r->pair2, r->pscan2, t_pair, st)))
         return fail_all(rc, "hh_rebuild: batch scan failed");
-    k_tile_counts<true><<<g3, 256, 0, st>>>(RbSim{}, D());
+    launch_after(k_tile_counts<true>, g3, dim3(256), st, true, RbSim{}, D());
     if ((rc = cub_exclusive_sum(r->tmp, r->tmp_bytes, r->nt2, r->tscan2, t_nt, st)))
         return fail_all(rc, "hh_rebuild: batch scan failed");
-    k_tiles<true><<<g3, 256, 0, st>>>(RbSim{}, D());
+    launch_after(k_tiles<true>, g3, dim3(256), st, true, RbSim{}, D());
     // 4. entries and closing step, again for the contexts whose lists had to
     //    grow; then per context on the host: work-item capacity and sizes
     int64_t fx = 1;
@@ -1648,8 +1649,8 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
         fx = std::max<int64_t>(fx, std::min<int64_t>(ctxs[act[q]]->elem_grid, (ctxs[act[q]]->n + cnt(q).ncells + 255) / 256));
     auto entries = [&]() {
         const unsigned k = unsigned(act.size());
-        k_lists<true, true><<<dim3(unsigned(lgrid), k), kWalkThreads, 0, st>>>(RbSim{}, D());
-        k_finish<true><<<dim3(unsigned(fx), k), 256, 0, st>>>(RbSim{}, D());
+        launch_after(k_lists<true, true>, dim3(unsigned(lgrid), k), dim3(kWalkThreads), st, true, RbSim{}, D());
+        launch_after(k_finish<true>, dim3(unsigned(fx), k), dim3(256), st, true, RbSim{}, D());
         launches += 2;
     };
     entries();
