@@ -84,7 +84,9 @@ typedef struct hh_config {
                           ones the mixed form takes parts of tile_j and the plain form
                           equal-cost parts of 2 x tile_j interactions (at least 32 entries):
                           short parts spread a small step over more SMs, equal-cost parts
-                          balance a large one.  The other loops then use parts of tile_j.
+                          balance a large one.  The plain form doubles both where the step has
+                          particles enough (512 and 4096 due), and takes four times work_item
+                          from 16384 on.  The other loops then use parts of tile_j.
                           The count is the simulation's own, so results still do not depend
                           on the rest of a batch */
     int32_t tile_j_small; /* 0 (default): off.  Otherwise a multiple of 32 in [32, tile_j]: the

@@ -649,13 +649,26 @@ __global__ void __launch_bounds__(kBlock, 1) k_batch(BatchDev B)
                     // kMedWork x tile_j interactions (an item's FP64 work
                     // bounds its time, so smaller items spread such a step
                     // over more SMs), and with tile_j_small, steps of at most
-                    // kSmallDue due particles take parts of that length
+                    // kSmallDue due particles take parts of that length.
+                    // An item's start and end cost the plain form about as
+                    // much as six of its thread's pairs, so as soon as a step
+                    // keeps every group busy with fewer of them, its items are
+                    // longer: twice from 512 due particles (83 steps of 256 to
+                    // 1024, N = 65536: 86.3 -> 79.2 us; below 512 the step
+                    // lacks items), and of work_item's, twice from 4096 (690 ->
+                    // 659 us; half there: 745 us) and four times from 16384
+                    // (2066 -> 1898 us; twice 1948, eight times 1906).  (Not in
+                    // list mode: its prediction covers parts of the plain rule.)
                     int work = sd.work, pj = sd.pj;
                     if (sd.work_split > 0 || sd.pj_small > 0) {
                         const int due = __reduce_add_sync(0xffffffffu, lane >= kmin_of(tnow) ? cnt : 0);
+                        const bool longer = kPlain && sd.work_split > 0 && work <= (1 << 28) && !cached_list_mode(sc, s);
                         if (sd.work_split > 0 && due < sd.work_split) {
                             work = kPlain ? kMedWork * sd.pj : 0;
                             if (kPlain) pj = 32;
+                            if (longer && due >= 512) work *= 2;
+                        } else if (longer) {
+                            work *= due >= 16384 ? 4 : due >= 4096 ? 2 : 1;
                         }
                         if (sd.pj_small > 0 && due <= kSmallDue) {
                             work = 0;
