@@ -56,7 +56,7 @@ struct StepCtl {
     int32_t mode;       // 0: active = {t_i + dt_i == t_next}; 1: marked; 2: all particles
     int32_t slot_cur;   // tmin slot holding this step's time (mode 0)
     int32_t slot_next;  // tmin slot that receives the next step's time (mode 0)
-    int32_t pad;
+    int32_t part_shift; // list parts of tile_j << part_shift entries (modes 1 and 2)
     double t_arg;       // step time for modes 1 and 2
 };
 
@@ -260,7 +260,8 @@ __device__ __forceinline__ void select_tiles(const State &s, const Lists &L, Dev
     const int n_tiles = ds->n_tiles;
     // (this loop does not count a step's active particles first, so a
     // work_item limited to large steps, work_split > 0, is not used here)
-    const int pj = ds->part_len, work = ds->work_split > 0 ? 0 : ds->work_item;
+    const int work = ds->work_split > 0 ? 0 : ds->work_item;
+    const int pj = work > 0 ? ds->part_len : ds->part_len << c.part_shift;
     for (int64_t tile = warp0; tile < n_tiles; tile += nwarps) {
         const int4 td = L.tiles[tile];
         const int64_t p = td.x + lane;
