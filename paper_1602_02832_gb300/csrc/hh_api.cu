@@ -754,7 +754,7 @@ int set_lists_core(hh_ctx *ctx, int64_t n_particles, int64_t n_j, int32_t n_grou
     if (int64_t(ctx->ids.size()) != n_particles) {
         ctx->ids.resize(size_t(n_particles));
         for (int64_t q = 0; q < n_particles; q++) ctx->ids[size_t(q)] = q;
-        ctx->ids_on_both = false;
+        ctx->ids_on_device = ctx->ids_on_both = false;
     }
     ctx->have_lists = true;
     ctx->predicted = false;

@@ -75,3 +75,18 @@ def test_refused_load_changes_nothing(hh, what, q, value, word):
     assert all(np.array_equal(a[f], b[f]) for f in a)
     c.close()
     d.close()
+
+
+def test_ids_after_lists_of_fewer_particles(hh):
+    # lists set by the caller for another number of particles start new ids,
+    # also when the last ones were kept by the device builder
+    c = _ctx(hh, hh.HH_FP64, 1000)
+    x, v, m = synth.plummer(1000, 9)
+    c.hh_load_particles(x.T, v.T, m)
+    c.hh_rebuild(0.0)
+    assert not np.array_equal(c.hh_get_ids(), np.arange(1000))
+    z = np.zeros((3, 10))
+    c.hh_set_j(0, x[:10].T, v[:10].T, z, z, m[:10], np.zeros(10))
+    c.hh_set_lists(10, 10, np.array([0, 10]), np.arange(10, dtype=np.int32), np.zeros(10, np.int32))
+    assert np.array_equal(c.hh_get_ids(), np.arange(10))
+    c.close()
