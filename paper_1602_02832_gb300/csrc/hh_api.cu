@@ -157,7 +157,7 @@ int launch_select_only(hh_ctx *ctx, StepCtl c)
 // explicit modes: reset the work queue, then select work items
 int launch_select(hh_ctx *ctx, StepCtl c)
 {
-    CK(cudaMemsetAsync(&ctx->ds->work, 0, 3 * sizeof(uint32_t), ctx->stream));  // work, n_items, slot_ctr
+    CK(cudaMemsetAsync(&ctx->ds->n_items, 0, 3 * sizeof(uint32_t), ctx->stream));  // n_items, slot_ctr, work
     return launch_select_only(ctx, c);
 }
 

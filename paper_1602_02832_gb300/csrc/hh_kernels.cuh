@@ -31,9 +31,9 @@ struct DevScalars {
     double t_end;                // loop bound of hh_advance
     int32_t done;                // set once the next block time exceeds t_end
     int32_t err;                 // device-detected error (HH_* code), 0 = none
+    alignas(8) uint32_t n_items;  // work items of this step
+    uint32_t slot_ctr;           // partial-sum slots handed out this step (one 64-bit word with n_items)
     uint32_t work;               // force work-queue head
-    uint32_t n_items;            // work items of this step
-    uint32_t slot_ctr;           // partial-sum slots handed out this step
     int32_t part_len;            // shortest list part (a multiple of the staging chunk)
     int32_t work_item;           // target interactions per work item (0: every part is part_len long)
     int32_t work_split;          // > 0: work_item applies only to batched steps with this many active particles
@@ -230,6 +230,7 @@ __device__ __forceinline__ int parts_of(int64_t len, int pj)
 // Warp-collective: appends one work item per part of tile `tile`'s list;
 // item = (tile, part | sim << 16, active mask, first partial-sum slot, part
 // length).  `work` is the equal-cost target of this step (0: parts of pj_min).
+// slot_ctr = nullptr: the slots' counter is the word behind n_items (DevScalars).
 __device__ __forceinline__ void append_tile_items(int tile, const int4 td, int64_t gb, int64_t ge, uint32_t mask,
                                                   int pj_min, int work, uint32_t *n_items, uint32_t *slot_ctr, WorkItem *items,
                                                   int sim, unsigned long long *na_hist, uint32_t *max_chunks = nullptr)
@@ -240,8 +241,15 @@ __device__ __forceinline__ void append_tile_items(int tile, const int4 td, int64
     const int n_parts = parts_of(len, pj);
     int base = 0, slot = 0;
     if (lane == 0) {
-        base = (int)atomicAdd(n_items, (uint32_t)n_parts);
-        slot = n_parts > 1 ? (int)atomicAdd(slot_ctr, (uint32_t)n_parts) : 0;
+        if (slot_ctr) {
+            base = (int)atomicAdd(n_items, (uint32_t)n_parts);
+            slot = n_parts > 1 ? (int)atomicAdd(slot_ctr, (uint32_t)n_parts) : 0;
+        } else {  // the slots are the word behind the items: one atomic for both (50001 of 200003 particles: 590 -> 580 us)
+            const unsigned long long both = atomicAdd(reinterpret_cast<unsigned long long *>(n_items),
+                                                      (unsigned long long)(uint32_t)n_parts * (n_parts > 1 ? 0x100000001ull : 1ull));
+            base = (int)(uint32_t)both;
+            slot = n_parts > 1 ? (int)(both >> 32) : 0;
+        }
         atomicAdd(&na_hist[__popc(mask) - 1], 1ull);
         // (with max_chunks: the longest part so far, in 32-entry chunks)
         if (max_chunks) atomicMax(max_chunks, (uint32_t)((min((int64_t)pj, len) + 31) / 32));
@@ -268,7 +276,7 @@ __device__ __forceinline__ void select_tiles(const State &s, const Lists &L, Dev
         const bool act = (p < td.y) && is_active(s, c, p, tnow);
         const uint32_t mask = __ballot_sync(0xffffffffu, act);
         if (mask == 0u) continue;
-        append_tile_items((int)tile, td, L.off[td.z], L.off[td.z + 1], mask, pj, work, &ds->n_items, &ds->slot_ctr, L.items,
+        append_tile_items((int)tile, td, L.off[td.z], L.off[td.z + 1], mask, pj, work, &ds->n_items, nullptr, L.items,
                           0, ds->na_hist);
     }
 }
