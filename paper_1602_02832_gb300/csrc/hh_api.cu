@@ -319,7 +319,8 @@ int ensure_graph(hh_ctx *ctx)
 // two or four times that where the evaluation has eight parts of that length
 // for every group that works on them all the same (a part's start and end cost
 // about six of its thread's pairs, tile_j = 256 entries of a tile of 14 are 28:
-// N = 65536 takes 3.23 ms against 3.37 ms).  The mixed form's sums follow its parts, which stay.
+// N = 65536 takes 3.23 ms against 3.37 ms; four or two parts per group, or up to
+// eight times tile_j: the same).  The mixed form's sums follow its parts, which stay.
 int part_shift(const hh_ctx *ctx, int32_t n_act)
 {
     if (ctx->cfg.precision != HH_FP64 || ctx->n_groups < 1) return 0;
