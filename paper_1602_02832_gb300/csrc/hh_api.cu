@@ -488,7 +488,6 @@ int hh_destroy(hh_ctx *ctx)
     if (ctx->h_buf) cudaFreeHost(ctx->h_buf);
     if (ctx->h_ibuf) cudaFreeHost(ctx->h_ibuf);
     if (ctx->h_out) cudaFreeHost(ctx->h_out);
-    if (ctx->h_flag) cudaFreeHost(ctx->h_flag);
     if (ctx->begun) cudaEventDestroy(ctx->begun);
     if (ctx->h_jbuf) cudaFreeHost(ctx->h_jbuf);
     if (ctx->tree) hh_tree_free(ctx->tree);
@@ -596,11 +595,11 @@ int hh_create(hh_ctx **out, int device, const hh_config *cfg, int64_t n_max, int
     // the pinned staging of the host tree build (h_buf, h_jbuf) is allocated by
     // the first host rebuild: contexts that rebuild on the device never need it
     if (cudaHostAlloc((void **)&ctx->h_ds, sizeof(DevScalars), cudaHostAllocDefault) != cudaSuccess ||
-        cudaHostAlloc((void **)&ctx->h_ibuf, sizeof(int32_t) * n_max, cudaHostAllocDefault) != cudaSuccess ||
-        cudaHostAlloc((void **)&ctx->h_flag, sizeof(int32_t), cudaHostAllocDefault) != cudaSuccess) {
+        cudaHostAlloc((void **)&ctx->h_ibuf, sizeof(int32_t) * (n_max + 64), cudaHostAllocDefault) != cudaSuccess) {
         cudaGetLastError();
         return bail(HH_ENOMEM, "pinned host allocation failed");
     }
+    ctx->h_flag = ctx->h_ibuf + (n_max + 31) / 32 * 32;  // (a cache line of its own)
     if (cudaMemsetAsync(ctx->ds, 0, sizeof(DevScalars), ctx->stream) != cudaSuccess ||
         cudaMemsetAsync(ctx->st.mark, 0, sizeof(int32_t) * n_max, ctx->stream) != cudaSuccess ||
         cudaMemsetAsync(ctx->tile_cnt, 0, sizeof(int32_t) * ctx->cap_tiles, ctx->stream) != cudaSuccess ||

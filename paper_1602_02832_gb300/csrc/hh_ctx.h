@@ -90,7 +90,7 @@ struct hh_ctx {
     hh::DevScalars *h_ds = nullptr;
     double *h_buf = nullptr;   // [14 * cap_j]
     int32_t *h_ibuf = nullptr; // [cap_n]
-    int32_t *h_flag = nullptr; // verdict of an explicit evaluation's checks
+    int32_t *h_flag = nullptr; // verdict of an evaluation's or a load's checks (behind h_ibuf, in its allocation)
     double *h_out = nullptr;   // results of small evaluations (first use)
     std::vector<uint32_t> seen;  // last evaluation that listed each particle (repeats)
     uint32_t seen_stamp = 0;
