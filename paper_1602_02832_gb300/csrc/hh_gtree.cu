@@ -1343,7 +1343,7 @@ struct RbScratch {
 
 namespace {
 
-constexpr int kStages = 6;  // the records of stages 0..5 (a stage per read of the counts, and the close)
+constexpr int kStages = 4;  // the records of stages 0..3 (after each read of the counts, and as groups are known)
 
 void rb_free_sims(RbScratch *r)
 {
@@ -1427,7 +1427,8 @@ void hh_rb_scratch_free(RbScratch *r)
     if (!r) return;
     cudaStreamSynchronize(r->stream);
     rb_free_sims(r);
-    for (void *p : {(void *)r->key, (void *)r->key2, (void *)r->idx, (void *)r->perm, (void *)r->cnt, (void *)r->pos, (void *)r->pair2, (void *)r->pscan2, (void *)r->path, (void *)r->nt2, (void *)r->tscan2, r->tmp})
+    for (void *p : {(void *)r->key, (void *)r->key2, (void *)r->idx, (void *)r->perm, (void *)r->cnt, (void *)r->pos,
+                    (void *)r->pair2, (void *)r->pscan2, (void *)r->path, (void *)r->nt2, (void *)r->tscan2, r->tmp})
         if (p) cudaFree(p);
     cudaStreamDestroy(r->stream);
     delete r;
@@ -1655,7 +1656,8 @@ int hh_rebuild_device_many(hh_ctx *const *ctxs, const double *ts, int k, int *rc
     //    grow; then per context on the host: work-item capacity and sizes
     int64_t fx = 1;
     for (size_t q = 0; q < act.size(); q++)
-        fx = std::max<int64_t>(fx, std::min<int64_t>(ctxs[act[q]]->elem_grid, (ctxs[act[q]]->n + cnt(q).ncells + 255) / 256));
+        fx = std::max<int64_t>(
+            fx, std::min<int64_t>(ctxs[act[q]]->elem_grid, (ctxs[act[q]]->n + cnt(q).ncells + 255) / 256));
     auto entries = [&]() {
         const unsigned k = unsigned(act.size());
         launch_after(k_lists<true, true>, dim3(unsigned(lgrid), k), dim3(kWalkThreads), st, true, RbSim{}, D());
