@@ -347,9 +347,11 @@ __global__ void k_chains(RB_ARGS)
 __device__ __forceinline__ uint64_t before(const RbSim &a, int64_t i) { return uint64_t(a.pos[i]) - uint64_t(a.pos[0]); }
 __device__ __forceinline__ int64_t cells_of(uint64_t w) { return int64_t(w & ((uint64_t(1) << kCellBits) - 1)); }
 
-// First particle and depth of every cell, the group cells, and the sizes (no
-// cell is written when they do not fit: the host reports HH_ENOMEM; group
-// cells beyond cap_g are not stored, likewise).
+// First particle and depth of every cell, the group cells, and the sizes.  When
+// the cells do not fit, none is written and both counts are zero, so that the
+// kernels already queued behind this one (they run before the host reads the
+// overflow and reports HH_ENOMEM) find nothing to read; group cells beyond cap_g
+// are not stored, likewise.
 template <bool kMany>
 __global__ void k_begin_cells(RB_ARGS)
 {
@@ -361,7 +363,7 @@ __global__ void k_begin_cells(RB_ARGS)
         a.gc->ncells = overflow ? 0 : int32_t(ncells);
         a.gc->overflow = overflow;
         a.gc->bad = a.box->bad;
-        a.gc->G = int32_t(all >> kCellBits);
+        a.gc->G = overflow ? 0 : int32_t(all >> kCellBits);
     }
     if (overflow) return;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * blockDim.x) {
