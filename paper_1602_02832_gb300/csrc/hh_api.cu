@@ -895,14 +895,14 @@ int hh_advance(hh_ctx *ctx, double t_end, int64_t *n_steps_out)
     // in the mixed form against 2.1 / 7.1 / 41 ms (plain: 1.4 / 5.7 / 51 against
     // 2.8 / 9.5 / 66 ms), with the same bits; and no graph is captured and
     // instantiated after each device rebuild (about 1 ms).  The graph loop stays
-    // for per-launch timing, and for states that break the block rule.
+    // for per-launch timing, and for steps and states outside the block rule.
     if (!ctx->timing) {
         if ((rc = sync_and_check(ctx))) return rc;
         const DevScalars before = *ctx->h_ds;
+        ctx->predicted = false;
         rc = hh_loop_run(ctx, t_end);
         if (rc < 0) return rc;
         if (rc == HH_OK) {
-            ctx->predicted = false;
             if ((rc = sync_and_check(ctx))) return rc;
             if (n_steps_out) *n_steps_out = int64_t(ctx->h_ds->block_steps - before.block_steps);
             return HH_OK;

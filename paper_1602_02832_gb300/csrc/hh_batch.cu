@@ -1256,6 +1256,10 @@ void hh_loop_free(LoopBuf *b)
 
 int hh_loop_run(hh_ctx *ctx, double t_end)
 {
+    // The kernel keeps steps as levels 0 to 31 (2^-31 to 1); it checks the state
+    // when a launch begins, so the corrector must not be able to leave that range
+    // within one (the particles due would be lost): block_dt clamps to the limits.
+    if (ctx->cfg.dt_min < std::ldexp(1.0, -31) || ctx->cfg.dt_max > 1.0) return kLoopNotTaken;
     if (!ctx->loop && !(ctx->loop = loop_buf(ctx))) return kLoopNotTaken;
     LoopBuf *b = ctx->loop;
     const BatchLayout &L = b->lay;
@@ -1287,12 +1291,12 @@ int hh_loop_run(hh_ctx *ctx, double t_end)
         explicit Running(std::atomic<int> &c) : n(c) { n.fetch_add(1); }
         ~Running() { n.fetch_sub(1); }
     } running(g_loops[unsigned(ctx->device) % 64u]);
-    for (;;) {
+    for (bool first = true;; first = false) {  // (only before any step was taken is the loop left to the caller)
         const int grid = loop_ctas(ctx, b->sms, running.n.load());
         std::memset(b->h_blk + L.bs, 0, sizeof(BatchScalars));
         cudaError_t e = cudaMemcpyAsync(b->d_blk, b->h_blk, L.up_bytes(), cudaMemcpyHostToDevice, ctx->stream);
         if (e == cudaSuccess) e = cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kBlock), args, smem, ctx->stream);
-        if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+        if (first && (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported)) {
             cudaGetLastError();
             return kLoopNotTaken;
         }
@@ -1303,8 +1307,10 @@ int hh_loop_run(hh_ctx *ctx, double t_end)
         if (e != cudaSuccess) return lfail(HH_ECUDA, cudaGetErrorString(e));
         hh_count_launches(1);
         const BatchScalars *bs = reinterpret_cast<const BatchScalars *>(b->h_blk + L.bs);
-        if (bs->err == HH_EINVAL) return kLoopNotTaken;
-        if (bs->err) return lfail(bs->err, "hh_advance: grid barrier timed out");
+        if (bs->err == HH_EINVAL && first) return kLoopNotTaken;
+        if (bs->err)
+            return lfail(bs->err, bs->err == HH_EINVAL ? "hh_advance: the steps taken broke the block rule"
+                                                       : "hh_advance: grid barrier timed out");
         if (*reinterpret_cast<const double *>(b->h_blk + L.tnext) > t_end) return HH_OK;
     }
 }

@@ -44,8 +44,9 @@ constexpr int64_t kBatchRebuildMaxN = 32768;
 int hh_rebuild_many(hh_ctx *const *ctxs, const double *ts, int k, int *rcs, RbScratch *r);
 // hh_advance's block steps in the persistent loop of the batched kernel, one
 // context alone (hh_batch.cu).  Returns HH_OK, an error, or kLoopNotTaken when
-// the loop cannot run here (no memory or no cooperative launch) or the state
-// breaks the block rule (nothing but the work counters may have changed then).
+// the loop cannot run here (no memory or no cooperative launch), the step limits
+// go beyond [2^-31, 1] or the state breaks the block rule (no step was taken
+// then, and nothing but the work counters may have changed).
 constexpr int kLoopNotTaken = 1;
 struct LoopBuf;
 int hh_loop_run(hh_ctx *ctx, double t_end);
@@ -105,7 +106,7 @@ struct hh_ctx {
     // grid shapes
     int n_sm = 0, force_grid = 0, elem_grid = 0;
     LoopBuf *loop = nullptr;   // buffers of the persistent loop (first hh_advance)
-    // loop graph (with per-launch timing, or for states that break the block rule)
+    // loop graph (with per-launch timing, or for limits and states outside the block rule)
     cudaGraphExec_t graph = nullptr;
     int graph_timed = -1;
     std::vector<cudaEvent_t> ev;  // 2 per unrolled step when timed
