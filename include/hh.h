@@ -357,8 +357,11 @@ const char *hh_last_error(const hh_ctx *ctx);
  *   Every particle must follow the block rule (dt a power of two in
  *   [2^-31, 1], t a multiple of dt, t + dt after the latest t), as states
  *   made by hh_init_dt, hh_step, hh_advance and hh_rebuild do; otherwise
- *   HH_EINVAL.  The loop keeps a per-simulation histogram of step levels
- *   and per-tile level masks, so a block step touches only the due tiles. */
+ *   HH_EINVAL, also when the corrector asks for a step outside that range
+ *   on the way (dt_min below 2^-31 or dt_max above 1; the contexts have then
+ *   advanced in part and have to be loaded again).  The loop keeps a
+ *   per-simulation histogram of step levels and per-tile level masks, so a
+ *   block step touches only the due tiles. */
 typedef struct hh_batch hh_batch;
 /* Errors of hh_batch_create (message in hh_last_error(NULL)): HH_EINVAL for a
  * NULL out, a bad precision, max_sims or max_steps; HH_ECUDA for a bad device,

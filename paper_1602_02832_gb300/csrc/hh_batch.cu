@@ -226,8 +226,8 @@ __device__ __forceinline__ double due_below_warp(const int32_t *lvl_cnt, double 
 // The new forces come from fin[active index] (the force tail's copy in
 // shared memory; the same values as acc1 / jerk1).
 template <bool kPlain>
-__device__ __forceinline__ double correct_tile_3lane(const SimDesc &sd, const int4 td, uint32_t mask, double tnow,
-                                                     int lane, int k_first, int k_step, int *lv_out,
+__device__ __forceinline__ double correct_tile_3lane(BatchScalars *bs, const SimDesc &sd, const int4 td, uint32_t mask,
+                                                     double tnow, int lane, int k_first, int k_step, int *lv_out,
                                                      const double (*fin)[7], const int *pidx)
 {
     const unsigned full = 0xffffffffu;
@@ -282,9 +282,12 @@ __device__ __forceinline__ double correct_tile_3lane(const SimDesc &sd, const in
                 s.dt[p] = dtn;
                 const int lv_old = level_of(dt_old), lv_new = level_of(dtn);
                 lv_out[k] = lv_new;
-                if (lv_new != lv_old) {
+                // (limits beyond the levels, dt_min < 2^-31 or dt_max > 1: the
+                // run ends instead of writing outside the histogram)
+                if ((unsigned)lv_new > 31u) raise_error(bs, HH_EINVAL);
+                else if (lv_new != lv_old) {
                     atomicSub(&sd.ds->lvl_cnt[lv_old], 1);
-                    atomicAdd(&sd.ds->lvl_cnt[lv_new & 31], 1);
+                    atomicAdd(&sd.ds->lvl_cnt[lv_new], 1);
                 }
                 tn_min = min(tn_min, (unsigned long long)__double_as_longlong(tnow + dtn));
             }
@@ -814,8 +817,8 @@ __global__ void __launch_bounds__(kBlock, 1) k_batch(BatchDev B)
                     const int64_t pw = td.x + glane;
                     const double dt_keep = (gw == 0 && pw < td.y && !((mask >> glane) & 1u)) ? sdc.st.dt[pw] : 0.0;
                     const double tn =
-                        correct_tile_3lane<kPlain>(sdc, td, mask, tnow, glane, 10 * gw, 10 * (kThreads / 32), sm.lv, sm.fin,
-                                           sm.pidx);
+                        correct_tile_3lane<kPlain>(B.bs, sdc, td, mask, tnow, glane, 10 * gw, 10 * (kThreads / 32), sm.lv,
+                                           sm.fin, sm.pidx);
                     if (glane == 0) sm.tn[gw] = tn;
                     group_sync(bar);  // new levels and times are visible to the group
                     if (gw == 0) {
@@ -1164,14 +1167,12 @@ extern "C" int hh_batch_run(hh_batch *b, int32_t n, hh_ctx *const *ctxs, const d
         return bfail(b, HH_ECUDA, "hh_batch_run: kernel execution failed");
     BatchScalars hbs;
     std::memcpy(&hbs, b->h_blk + Ly.bs, sizeof(hbs));
+    for (int32_t s = 0; s < n; s++) ctxs[s]->predicted = false;
     if (hbs.err == HH_ETIMEOUT) return bfail(b, hbs.err, "hh_batch_run: grid barrier timed out");
     if (hbs.err)
         return bfail(b, hbs.err, "hh_batch_run: block-step state breaks the block rule (a step that is not a power "
                                  "of two in [2^-31, 1], a time not a multiple of its step, or an overdue particle)");
-    for (int32_t s = 0; s < n; s++) {
-        ctxs[s]->predicted = false;
-        ctxs[s]->have_forces = true;
-    }
+    for (int32_t s = 0; s < n; s++) ctxs[s]->have_forces = true;
     if (steps_out) *steps_out = hbs.steps_done;
     if (t_next_out) std::memcpy(t_next_out, b->h_blk + Ly.tnext, sizeof(double) * size_t(n));
     const unsigned long long *T = reinterpret_cast<const unsigned long long *>(b->h_blk + Ly.step_ns);

@@ -67,3 +67,28 @@ def test_steps_above_the_levels(hh, prec):
     x, v, m = synth.plummer(300, 12)
     steps, got = _both(hh, 64.0, prec, 60.0 * x, v / 8.0, m, np.full(300, 0.25), dt_tree=64.0, dt_max=64.0, eps2=4.0)
     assert steps > 20 and got.max() > 1.0
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_batched_run_refuses_steps_outside_the_levels(hh, prec):
+    x, v, m = (u.copy() for u in synth.plummer(64, 11))
+    x[1] = x[0] + np.array([2e-7, 0.0, 0.0])
+    v[1] = v[0] + np.array([0.0, 0.9 * np.sqrt(2 * m[0] / 2e-7), 0.0])
+    dt = np.full(64, 2.0 ** -20)
+    dt[:2] = 2.0 ** -31
+    c = _ctx(hh, prec, x, v, m, dt, dt_min=2.0 ** -40, eps2=0.0)
+    new = _ctx(hh, prec, x, v, m, dt, dt_min=2.0 ** -40, eps2=0.0)
+    lists = c.hh_get_lists()
+    with hh.Batch(c.cfg.precision, max_sims=1, max_steps=64) as b:
+        with pytest.raises(hh.HHError) as e:
+            b.hh_batch_run([c], [2.0 ** -25])
+        assert e.value.code == hh.HH_EINVAL
+    assert all(np.array_equal(p, q) for p, q in zip(lists, c.hh_get_lists()))
+    y, u, k = synth.plummer(64, 13)
+    for q in (c, new):  # loaded again, the context is as good as another
+        q.hh_load_particles(y.T, u.T, k)
+        q.hh_run(0.0, 2.0 ** -6)
+    s0, s1 = c.hh_get_state(), new.hh_get_state()
+    assert all(np.array_equal(s0[f], s1[f]) for f in s0)
+    c.close()
+    new.close()
