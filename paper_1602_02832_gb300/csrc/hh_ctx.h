@@ -21,11 +21,10 @@ void hh_gtree_free(GTreeBuf *g);
 int64_t *hh_gtree_ids(GTreeBuf *g);
 int hh_gtree_set_ids(GTreeBuf *g, const int64_t *ids, int64_t n, cudaStream_t st);
 struct hh_ctx;
-// The builder's second set of state buffers (as large as the context's), a
-// device flag, and the exchange of the two sets (all but the steps).
+// The builder's second set of state buffers (as large as the context's; their
+// contents are scratch between two builds), and a device flag.
 hh::State hh_gtree_second(const hh_ctx *ctx);
 int32_t *hh_gtree_flag(GTreeBuf *g);
-void hh_gtree_swap(hh_ctx *ctx);
 int hh_rebuild_device(hh_ctx *ctx, double t);        // hh_gtree.cu
 // Batched device rebuild of k contexts (hh_gtree.cu): rcs[s] gets context
 // s's result; the scratch (and its stream) belongs to the caller.

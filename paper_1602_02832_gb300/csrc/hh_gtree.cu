@@ -958,17 +958,6 @@ int64_t *hh_gtree_ids(GTreeBuf *g) { return g->ids; }
 State hh_gtree_second(const hh_ctx *ctx) { return ctx->gtree->alt; }
 int32_t *hh_gtree_flag(GTreeBuf *g) { return &g->gc->bad; }
 
-void hh_gtree_swap(hh_ctx *ctx)
-{
-    GTreeBuf *g = ctx->gtree;
-    std::swap(ctx->st.x, g->alt.x);
-    std::swap(ctx->st.v, g->alt.v);
-    std::swap(ctx->st.a, g->alt.a);
-    std::swap(ctx->st.jk, g->alt.jk);
-    std::swap(ctx->st.m, g->alt.m);
-    std::swap(ctx->st.t, g->alt.t);
-}
-
 // Ordered on the context's stream: the copy lands before the next rebuild's
 // reordering kernel reads the ids (a copy on the legacy stream would not be
 // ordered with a non-blocking stream).
@@ -1121,7 +1110,12 @@ RbSim rb_sim(hh_ctx *ctx, GTreeBuf *g, double t)
 // trade places.
 void swap_state(hh_ctx *ctx, GTreeBuf *g)
 {
-    hh_gtree_swap(ctx);
+    std::swap(ctx->st.x, g->alt.x);
+    std::swap(ctx->st.v, g->alt.v);
+    std::swap(ctx->st.a, g->alt.a);
+    std::swap(ctx->st.jk, g->alt.jk);
+    std::swap(ctx->st.m, g->alt.m);
+    std::swap(ctx->st.t, g->alt.t);
     std::swap(ctx->st.dt, g->alt.dt);
     std::swap(g->ids, g->ids2);
     ctx->ids_on_device = true;  // (whether the build succeeds or not)

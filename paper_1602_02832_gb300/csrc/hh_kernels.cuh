@@ -1743,41 +1743,49 @@ static __global__ void k_adopt_forces(State s, DevScalars *ds)
 }
 
 // A load through the second set of state buffers: checks x, v (finite: bit 0 of
-// *bad) and m (finite and > 0: bit 1) of n particles and writes the rest.
-static __global__ void k_load_check(State s, int64_t n, double t, int32_t *bad)
+// *bad) and m (finite and > 0: bit 1) of n particles there.
+static __global__ void k_load_check(State s, int64_t n, int32_t *bad)
 {
     int32_t wrong = 0;
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
         for (int d = 0; d < 3; d++) {
             const uint32_t x = f64_hi(s.x[d * s.cap_j + q]), v = f64_hi(s.v[d * s.cap_j + q]);
             if ((x & 0x7ff00000u) == 0x7ff00000u || (v & 0x7ff00000u) == 0x7ff00000u) wrong |= 1;
-            s.a[d * s.cap_j + q] = s.jk[d * s.cap_j + q] = 0.0;
         }
         const long long m = __double_as_longlong(s.m[q]);  // (positive and finite, as an integer)
         if (m <= 0 || m >= 0x7ff0000000000000ll) wrong |= 2;
-        s.t[q] = t;
     }
     if (wrong) atomicOr(bad, wrong);
 }
 
-// Then the base records of the mixed form, if all was right, and the verdict.
-static __global__ void k_load_base(State s, int64_t n, const int32_t *bad, volatile int32_t *verdict)
+// What a load of particle q at time t leaves besides x, v and m.
+__device__ __forceinline__ void load_rest(const State &s, int64_t q, double t)
+{
+    for (int d = 0; d < 3; d++) s.a[d * s.cap_j + q] = s.jk[d * s.cap_j + q] = 0.0;
+    s.t[q] = t;
+    if (s.base) refresh_base(s, q);
+}
+
+// Then, if all was right, the particles from there into the state, and the verdict.
+static __global__ void k_load_checked(State from, State s, int64_t n, double t, const int32_t *bad, volatile int32_t *verdict)
 {
     const int32_t wrong = *bad;
     if (blockIdx.x == 0 && threadIdx.x == 0) *verdict = wrong;
-    if (wrong || !s.base) return;
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x)
-        refresh_base(s, q);
+    if (wrong) return;
+    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
+        for (int d = 0; d < 3; d++) {
+            s.x[d * s.cap_j + q] = from.x[d * from.cap_j + q];
+            s.v[d * s.cap_j + q] = from.v[d * from.cap_j + q];
+        }
+        s.m[q] = from.m[q];
+        load_rest(s, q, t);
+    }
 }
 
-// What a load of n particles at time t leaves besides x, v and m.
 static __global__ void k_load_rest(State s, int64_t n, double t)
 {
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
-        for (int d = 0; d < 3; d++) s.a[d * s.cap_j + q] = s.jk[d * s.cap_j + q] = 0.0;
-        s.t[q] = t;
-        if (s.base) refresh_base(s, q);
-    }
+    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x)
+        load_rest(s, q, t);
 }
 
 static __global__ void k_refresh_base(State s, int64_t first, int64_t n)

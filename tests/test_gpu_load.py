@@ -90,3 +90,37 @@ def test_ids_after_lists_of_fewer_particles(hh):
     c.hh_set_lists(10, 10, np.array([0, 10]), np.arange(10, dtype=np.int32), np.zeros(10, np.int32))
     assert np.array_equal(c.hh_get_ids(), np.arange(10))
     c.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("n_new", [1500, 900])
+def test_load_leaves_the_entries_behind_its_particles(hh, prec, n_new):
+    # a program's own nodes (and particles beyond the loaded ones) stay as set,
+    # with and without a device builder: lists over them give the same forces
+    P = hh.HH_FP64 if prec == "fp64" else hh.HH_MIXED
+    x, v, m = synth.plummer(1500, 21)
+    y, u, k = synth.plummer(n_new, 22)
+    out = []
+    for dev in (True, False):
+        c = _ctx(hh, P, 1500)
+        c.hh_set_rebuild_device(dev)
+        c.hh_load_particles(x.T, v.T, m)
+        c.hh_rebuild(0.0)
+        rng = np.random.default_rng(23)
+        J = [rng.normal(size=(3, 2000)) for _ in range(4)]
+        mj = rng.uniform(0.5, 1.0, 2000) / 2000
+        c.hh_set_j(0, *J, mj, np.zeros(2000))
+        c.hh_load_particles(y.T, u.T, k)
+        off = np.arange(0, 51) * 400
+        idx = np.sort(rng.integers(0, 2000, (50, 400)), axis=1).astype(np.int32).ravel()
+        c.hh_set_lists(1500, 2000, off, idx, (np.arange(1500) // 30).astype(np.int32))
+        j = c.hh_get_j(0, 2000)
+        for q, f in enumerate(("x", "v", "a", "jk")):
+            assert np.array_equal(j[f][:, n_new:], J[q][:, n_new:]), (dev, f)
+        assert np.array_equal(j["m"][n_new:], mj[n_new:]) and np.array_equal(j["m"][:n_new], k)
+        assert np.array_equal(j["x"][:, :n_new], y.T) and not j["a"][:, :n_new].any()
+        c.hh_predict(2.0 ** -10)
+        out.append(c.hh_force(np.arange(1500, dtype=np.int32)))
+        c.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
