@@ -331,7 +331,8 @@ __device__ __forceinline__ int due_count(const SimDesc &sd, double tnow)
 // extra phase and grid barrier (a few microseconds): at least kListModeMinJ
 // entries.  (Many small simulations together gain nothing from it: their
 // every-entry passes are short and run side by side.)  It changes no result:
-// a predicted record is the same whoever computes it.
+// a predicted record is the same whoever computes it, and the plain form's list
+// parts follow this choice wherever the simulation is in the batch.
 constexpr int64_t kListModeMinJ = 1 << 18;
 
 __device__ __forceinline__ bool list_mode_of(const SimDesc &sd, double tnow, int due)
@@ -660,12 +661,15 @@ __global__ void __launch_bounds__(kBlock, 1) k_batch(BatchDev B)
                     // 1024, N = 65536: 86.3 -> 79.2 us; below 512 the step
                     // lacks items), and of work_item's, twice from 4096 (690 ->
                     // 659 us; half there: 745 us) and four times from 16384
-                    // (2066 -> 1898 us; twice 1948, eight times 1906).  (Not in
-                    // list mode: its prediction covers parts of the plain rule.)
+                    // (2066 -> 1898 us; twice 1948, eight times 1906).  (Not
+                    // where list mode applies: its prediction covers parts of
+                    // the plain rule.  Asked of the simulation's own numbers,
+                    // also where the step then predicts every entry: its
+                    // sums do not depend on its place in the batch.)
                     int work = sd.work, pj = sd.pj;
                     if (sd.work_split > 0 || sd.pj_small > 0) {
                         const int due = __reduce_add_sync(0xffffffffu, lane >= kmin_of(tnow) ? cnt : 0);
-                        const bool longer = kPlain && sd.work_split > 0 && work <= (1 << 28) && !cached_list_mode(sc, s);
+                        const bool longer = kPlain && sd.work_split > 0 && work <= (1 << 28) && !list_mode_of(sd, tnow, due);
                         if (sd.work_split > 0 && due < sd.work_split) {
                             work = kPlain ? kMedWork * sd.pj : 0;
                             if (kPlain) pj = 32;
