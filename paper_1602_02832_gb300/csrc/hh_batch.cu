@@ -1279,7 +1279,9 @@ int hh_loop_run(hh_ctx *ctx, double t_end)
     // hh_advance uses parts of tile_j or of work_item's rule only
     if (d.work_split > 0) d.work = d.work_split = 0;
     d.pj_small = 0;
-    d.lbar = int64_t(1) << 40;  // and predicts every entry at every step (no list mode, list_steps stays)
+    // and predicts every entry at every step (no list mode, list_steps stays): a due
+    // particle counts as all entries, so list_mode_of's product stays below 2^62
+    d.lbar = ctx->nj;
     int64_t *base = reinterpret_cast<int64_t *>(b->h_blk + L.base);  // jbase, pbase, tbase: two entries each
     base[0] = base[2] = base[4] = 0;
     base[1] = ctx->nj;

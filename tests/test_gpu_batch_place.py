@@ -58,3 +58,19 @@ def test_a_list_mode_step_at_any_place(hh, prec, own):
         assert np.array_equal(states[0][k], states[1][k]), k
     for c in small:
         c.close()
+
+
+def test_an_advance_of_many_particles_predicts_every_entry(hh):
+    # 2^22 particles due at once: hh_advance does not take list steps, however many are due
+    n = 1 << 22
+    cfg = hh.hh_config_default()
+    with hh.Context(cfg, n, n, n // 16, n // 32) as c:
+        x = np.stack([np.arange(n) % 2048.0, np.arange(n) // 2048.0, np.zeros(n)])
+        z = np.zeros((3, n))
+        c.hh_set_j(0, x, z, z, z, np.full(n, 1.0 / n), np.zeros(n))
+        idx = (np.arange(n // 32)[:, None] * 32 + np.arange(2)).astype(np.int32).ravel()
+        c.hh_set_lists(n, n, np.arange(n // 32 + 1) * 2, idx, (np.arange(n) // 32).astype(np.int32))
+        c.hh_set_dt(np.full(n, 2.0 ** -7))
+        assert c.hh_advance(2.0 ** -7) == 1
+        k = c.hh_get_counters()
+    assert k["particle_steps"] == n and k["list_steps"] == 0
