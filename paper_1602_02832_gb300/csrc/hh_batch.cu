@@ -747,10 +747,13 @@ __global__ void __launch_bounds__(kBlock, 1) k_batch(BatchDev B)
                         maxc = max(maxc, (min(plen, sd.lmax) + 31) / 32);
                     }
             }
-            const int64_t n_tasks = (int64_t)n_items * maxc;
+            // (and one task an item for the due particles of a tile, which its
+            // list need not hold)
+            const int per = maxc + 1;
+            const int64_t n_tasks = (int64_t)n_items * per;
             for (int64_t task = w0; task < n_tasks; task += nw) {
-                const int64_t i = task / maxc;
-                const int c = (int)(task - i * maxc);
+                const int64_t i = task / per;
+                const int c = (int)(task - i * per);
                 const WorkItem &it = items[i];
                 const int s = it.part_sim >> 16;
                 if (!cached_list_mode(sc, s)) continue;  // warp-uniform
@@ -758,7 +761,10 @@ __global__ void __launch_bounds__(kBlock, 1) k_batch(BatchDev B)
                 const int64_t lb = it.gb + (int64_t)(it.part_sim & 0xFFFF) * it.part_len;
                 const int64_t le = min(it.ge, lb + (int64_t)it.part_len);
                 const int64_t e = lb + 32 * (int64_t)c + lane;
-                if (e < le) predict_entry<Rec>(sd.st, (Rec *)sd.rec, sd.L.idx[e], cached_time(sc, B.sims, s, par));
+                const bool own = c == maxc && (it.part_sim & 0xFFFF) == 0 && ((it.mask >> lane) & 1u);
+                if (own || (c < maxc && e < le))
+                    predict_entry<Rec>(sd.st, (Rec *)sd.rec, own ? it.p_begin + lane : sd.L.idx[e],
+                                       cached_time(sc, B.sims, s, par));
             }
             if (!grid_sync(B.bs)) return;
         }

@@ -38,7 +38,7 @@ def _listed(hh, prec, n, nj, n_list, group, seed, own=True, **over):
 
 
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
-@pytest.mark.parametrize("own", [True])
+@pytest.mark.parametrize("own", [True, False])
 def test_a_list_mode_step_at_any_place(hh, prec, own):
     # 512 due particles with lists of 200 entries among 2^18: predicted from the lists alone (2^18 > 512 * 200 * 2)
     # where the step's data are kept in shared memory, entry by entry where they are not
