@@ -222,11 +222,13 @@ int hh_step(hh_ctx *ctx, double *t_next_out, int32_t *n_act_out);
  * 256 steps (the kernel of hh_batch_run, with the same results as the graph
  * loop: list parts of tile_j, or of work_item when work_split is 0, every
  * entry predicted at every step).  Contexts that advance at the same time
- * from several threads share the SMs.  With hh_force_timing on, with dt_min
- * below 2^-31 or dt_max above 1, and for a state that breaks the block rule
- * (see hh_batch_run), a CUDA graph of unrolled block steps is replayed instead
- * (each kernel becomes a no-op once done).  The first call allocates the launch's buffers (some 40 KB, counted
- * in hh_ctx_device_bytes).  *n_steps_out (may be NULL) receives the number of
+ * from several threads share the SMs (those that batch launches leave free,
+ * see hh_batch_set_ctas, if there are any).  With hh_force_timing on, with
+ * dt_min below 2^-31 or dt_max above 1, and for a state that breaks the block
+ * rule (see hh_batch_run), a CUDA graph of unrolled block steps is replayed
+ * instead (each kernel becomes a no-op once done).  The first call allocates
+ * the launch's buffers (some 40 KB, counted in hh_ctx_device_bytes).
+ * *n_steps_out (may be NULL) receives the number of
  * block steps taken.  Errors: HH_ESTATE without lists and steps; HH_EINVAL
  * for a NaN t_end or an error found on the device; HH_ETIMEOUT for a grid
  * barrier that gave up, or if the replays stop making progress; HH_ECUDA. */

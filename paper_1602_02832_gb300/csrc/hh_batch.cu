@@ -1118,6 +1118,22 @@ extern "C" int hh_batch_destroy(hh_batch *b)
     return HH_OK;
 }
 
+namespace {
+
+// What runs on each device's SMs in persistent launches: CTAs (one per SM) of
+// hh_batch_run, and contexts in hh_advance.
+std::atomic<int> g_batch_ctas[64], g_loops[64];
+
+// Counts `k` while in scope.
+struct Running {
+    std::atomic<int> &n;
+    int k;
+    Running(std::atomic<int> *a, int device, int k_) : n(a[unsigned(device) % 64u]), k(k_) { n.fetch_add(k); }
+    ~Running() { n.fetch_sub(k); }
+};
+
+}  // namespace
+
 extern "C" int hh_batch_run(hh_batch *b, int32_t n, hh_ctx *const *ctxs, const double *t_end, int32_t max_steps,
                             int32_t *steps_out, double *t_next_out, double *step_us_out, double *phase_us_out)
 {
@@ -1168,6 +1184,7 @@ extern "C" int hh_batch_run(hh_batch *b, int32_t n, hh_ctx *const *ctxs, const d
     hdr->max_steps = max_steps;
     hdr->items = b->d_items;
     std::memset(b->h_blk + Ly.bs, 0, sizeof(BatchScalars));
+    const Running running(g_batch_ctas, b->device, b->grid);
     if (cudaGraphLaunch(b->graph, b->stream) != cudaSuccess) {
         const cudaError_t e = cudaGetLastError();
         return bfail(b, HH_ECUDA, std::string("hh_batch_run: launch: ") + cudaGetErrorString(e));
@@ -1222,11 +1239,14 @@ constexpr int kLoopSteps = 256;
 // 1.37 ms on 152, N = 4096 2.8 / 4.2 ms on 128 / 152; the SMs left over run other
 // contexts' launches.  Contexts that advance at the same time (other threads)
 // share the SMs, so that their loops run side by side instead of one after the
-// other: a cooperative launch only starts when all its CTAs fit.
-std::atomic<int> g_loops[64];
-
-int loop_ctas(const hh_ctx *ctx, int sms, int running)
+// other: a cooperative launch only starts when all its CTAs fit.  For the same
+// reason they share the SMs that batch launches leave free (hh_batch_set_ctas),
+// if there are any: beside a batch on all SMs but 16, a quarter interval of N =
+// 1024 takes 0.37 ms, where a launch of 32 CTAs waited 15.7 ms for the batch to
+// end (three kernels a step, which need not fit together: 2.4 ms).
+int loop_ctas(const hh_ctx *ctx, int sms, int batch, int running)
 {
+    if (batch < sms) sms -= batch;
     const int64_t want = std::max<int64_t>(16, ctx->n / (ctx->cfg.precision == HH_MIXED ? 32 : 16));
     return int(std::min<int64_t>(want, std::max(1, sms / std::max(1, running))));
 }
@@ -1299,13 +1319,9 @@ int hh_loop_run(hh_ctx *ctx, double t_end)
     hdr->items = ctx->cap_parts >= int64_t(b->sms) * kGroups ? ctx->items : b->items;
     BatchDev B = batch_dev(L, b->d_blk, 1);
     void *args[] = {&B};
-    struct Running {  // contexts of this device in their loops
-        std::atomic<int> &n;
-        explicit Running(std::atomic<int> &c) : n(c) { n.fetch_add(1); }
-        ~Running() { n.fetch_sub(1); }
-    } running(g_loops[unsigned(ctx->device) % 64u]);
+    const Running running(g_loops, ctx->device, 1);
     for (bool first = true;; first = false) {  // (only before any step was taken is the loop left to the caller)
-        const int grid = loop_ctas(ctx, b->sms, running.n.load());
+        const int grid = loop_ctas(ctx, b->sms, g_batch_ctas[unsigned(ctx->device) % 64u].load(), running.n.load());
         std::memset(b->h_blk + L.bs, 0, sizeof(BatchScalars));
         cudaError_t e = cudaMemcpyAsync(b->d_blk, b->h_blk, L.up_bytes(), cudaMemcpyHostToDevice, ctx->stream);
         if (e == cudaSuccess) e = cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kBlock), args, smem, ctx->stream);
