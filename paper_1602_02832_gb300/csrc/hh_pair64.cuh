@@ -184,6 +184,12 @@ constexpr int kMaxExp = 1223;  // 2^200: largest separation and velocity taken h
 constexpr int kMinExp = 128;   // smallest block exponent: anything below counts as zero against it
 
 // kDown = 2: component 2^(e - 1084), largest in [2^61, 2^62); each more place halves that.
+// The last bit is always set: what the shift cut off is then wrong by at most one
+// unit either way, without a bias, and the ones' complement with that bit set is
+// exactly -x (with no carry to pay for), so that f(-d, -w) = -f(d, w).  (Ones'
+// complement alone, -x - 1, leant every negative component and broke that in half
+// of all pairs; a full negation costs 4% of an evaluation of N = 65536, the bit and
+// the test for a vector of zeros 1.5%: 3.23 -> 3.28 ms.)
 template <int kDown>
 HH_HD void unpack_vec(const double *d, Vec64 &v)
 {
@@ -196,8 +202,8 @@ HH_HD void unpack_vec(const double *d, Vec64 &v)
         // 1.mantissa left-aligned in 64 bits, then down to its place
         const uint64_t m = ((((uint64_t)hi << 32) | lo) << 11) | 0x8000000000000000ull;
         const uint64_t x = shr64(m, base - (int)(a[k] >> 20));
-        const uint32_t neg = (uint32_t)((int32_t)hi >> 31);  // (-x - 1 for -x: one unit in 2^57 or more)
-        const uint32_t xl = lo32(x) ^ neg;
+        const uint32_t neg = (uint32_t)((int32_t)hi >> 31);
+        const uint32_t xl = (lo32(x) ^ neg) | 1u;
         v.k[k].l = (int32_t)xl;
         v.k[k].h = (int32_t)((hi32(x) ^ neg) + (xl >> 31));
     }
@@ -453,17 +459,19 @@ HH_HD void pair_add(const double *d, const double *w, double m, uint64_t mb, boo
     sa -= da;
     sj -= dj;
     const uint32_t out = umax(umax((uint32_t)(sa - smin), (uint32_t)(sj - smin)), (uint32_t)(sp - smin));
-    if (out <= (uint32_t)(32 - smin) && !self && (uint32_t)(D.e - eps.dmin) <= (uint32_t)(kMaxExp - eps.dmin) &&
-        W.e <= kMaxExp && hi32(mb) != 0u) {
+    const bool far = (uint32_t)(D.e - eps.dmin) > (uint32_t)(kMaxExp - eps.dmin);
+    // (W.e above kMinExp: the last bits of a vector of zeros are no velocity)
+    if (out <= (uint32_t)(32 - smin) && !self && !far && (uint32_t)(W.e - kMinExp - 1) < (uint32_t)(kMaxExp - kMinExp) &&
+        hi32(mb) != 0u) {
         sum_put<3>(A.a, ta, sa);
         sum_put<3>(A.j, tj, sj);
         sum_put<1>(A.p, tp, sp);
     } else if (!self) {
-        if ((uint32_t)(D.e - eps.dmin) > (uint32_t)(kMaxExp - eps.dmin) || W.e > kMaxExp || hi32(mb) == 0u) {
+        if (far || W.e > kMaxExp || hi32(mb) == 0u) {
             A.bad = true;
         } else {
             sum_any<3>(A.a, ta, sa, smin);
-            sum_any<3>(A.j, tj, sj, smin);
+            if (W.e > kMinExp) sum_any<3>(A.j, tj, sj, smin);
             sum_any<1>(A.p, tp, sp, smin);
         }
     }
