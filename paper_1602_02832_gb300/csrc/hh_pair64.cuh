@@ -440,10 +440,8 @@ HH_HD void pair_add(const double *d, const double *w, double m, uint64_t mb, boo
     // rho in units of the components, times 2^64
     int64_t G = mul_dig(dig(RW), dig((int64_t)Z));
     G = sar64(G, sh);
-    G = (int64_t)((uint64_t)G * 12ull);
-    Dig N = dig(G);
-    N.h = -N.h;
-    N.l = -N.l;
+    G = -(int64_t)((uint64_t)G * 12ull);  // (negated here: a digit of -2^31 has no negative)
+    const Dig N = dig(G);
     for (int k = 0; k < 3; k++) {
         const Dig t = dig(ta[k]);
         int64_t mid = mad_s(U.h, W.k[k].l, 0x80000000ll);

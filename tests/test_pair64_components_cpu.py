@@ -1,6 +1,6 @@
 """Single components of the plain form's integer pair term (csrc/hh_pair64.cuh), compiled for the host.
 
-A pair seen from its other end gives the negative of every component, to the last bit."""
+A pair seen from its other end gives the negative of every component, to the last bit; every digit has its negative."""
 import ctypes as C
 import os
 import subprocess
@@ -70,3 +70,17 @@ def test_a_pair_from_its_other_end(pair_sums, eps2, kind):
         assert np.array_equal(a[:6], -b[:6]) and a[6] == b[6], (i, a, b)
         if kind == "at rest":
             assert not a[3:6].any()
+
+
+def test_a_digit_without_a_negative(pair_sums):
+    # found by search (one pair in 2^32): the jerk's factor of the separation has the low digit -2^31
+    h = [float.fromhex(s) for s in ("0x1.821fa0ffd6076p-1", "0x1.6f6334dacc0ap-4", "-0x1.f74ed4f41876p-5",
+                                    "0x1.e940d71cb38b8p-1", "-0x1.e8e0238142a64p-1", "-0x1.fc7cb8a0e6c4cp-2")]
+    d, w = np.array(h[:3], dtype=np.longdouble), np.array(h[3:], dtype=np.longdouble)
+    r2 = (d * d).sum()
+    u = 1 / (r2 * np.sqrt(r2))
+    jerk = u * (w - 3 * (d * w).sum() / r2 * d)
+    got, left = pair_sums(d[None], w[None], np.ones(1), 0.0)
+    assert not left
+    # as in every pair: 2^-51 of |u w|
+    assert (np.abs(got[3:6] - jerk) <= 2.0 ** -51 * u * np.sqrt((w * w).sum())).all()
