@@ -333,14 +333,17 @@ HH_HD double sum_get(uint64_t u, int64_t o, int e)
     const int z = clz32(hi32(c));
     uint64_t m = (c << z) | (z ? w0 >> (32 - z) : 0u);
     e += 96 - z;  // value = m 2^(e - 64) with the top bit of m set
-    if (e < -1000) return 0.0;                                       // below the normal range
+    const bool small = e < -1021;  // below the normal range: 2^128 times the value, scaled down by one product
+    if (small) e += 128;
+    if (e < -1021) return 0.0;
     if (e > 1024) return f64_of(neg ? 0xfff00000u : 0x7ff00000u, 0u);  // beyond it
     // round to 53 bits, ties to even (bits below the 64 kept ones are dropped)
     const uint64_t lsb = (m >> 11) & 1ull;
     m = (m >> 11) + ((((m & 0x7ffull) + lsb) > 0x400ull) ? 1ull : 0ull);
     // m in [2^52, 2^53]; the exponent field carries a round-up to 2^53
     const uint64_t b = ((uint64_t)(e - 1 + 1022) << 52) + m;
-    return f64_of(hi32(b) | (neg ? 0x80000000u : 0u), lo32(b));
+    const double x = f64_of(hi32(b) | (neg ? 0x80000000u : 0u), lo32(b));
+    return small ? x * 0x1p-128 : x;
 }
 
 struct AccI64 {

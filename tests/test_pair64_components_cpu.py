@@ -84,3 +84,20 @@ def test_a_digit_without_a_negative(pair_sums):
     assert not left
     # as in every pair: 2^-51 of |u w|
     assert (np.abs(got[3:6] - jerk) <= 2.0 ** -51 * u * np.sqrt((w * w).sum())).all()
+
+
+@pytest.mark.parametrize("scale", [-250, -306, -312, -320, -330, -334, -345, -380, -386, -420])
+def test_results_near_the_end_of_the_range(pair_sums, scale):
+    # the jerk of a light pair far away and nearly at rest, down to subnormal numbers and zero
+    d, w, m = np.array([[1.5, -0.75, 0.3]]) * 2.0 ** 170, np.array([[0.3, 0.2, -1.1]]) * 2.0 ** scale, np.array([1.25 * 2.0 ** -180])
+    e = 2.0 ** -1074
+    L = np.longdouble
+    D, W = d[0].astype(L), w[0].astype(L)
+    r2 = (D * D).sum()
+    u = L(m[0]) / (r2 * np.sqrt(r2))
+    ref = np.concatenate([u * D, u * (W - 3 * (D * W).sum() / r2 * D)])
+    size = np.array([u * np.sqrt(r2)] * 3 + [u * np.sqrt((W * W).sum())] * 3)
+    got, left = pair_sums(d, w, m, 0.0)
+    assert not left
+    # 2^-51 of the sizes, or the spacing of subnormal numbers (two roundings)
+    assert (np.abs(got[:6] - ref) <= 2.0 ** -51 * size + 2 * e).all()
