@@ -51,7 +51,13 @@ extern "C" {
 #define HH_ETIMEOUT (-4) /* a bounded device-side wait gave up */
 #define HH_ESTATE (-5)   /* calls made in the wrong order (e.g. force before lists) */
 
-#define HH_FP64 0  /* plain form: FP64 prediction, pairwise arithmetic and sums */
+#define HH_FP64 0  /* plain form: FP64 prediction and i-j differences; pair terms and their sums
+                      over a list part in 64-bit integers, at least as accurate as in FP64: a
+                      term to about 2^-57 of its vector's largest component, f(-d, -w) =
+                      -f(d, w) exactly.  A part is summed in FP64 where a particle's terms in
+                      one component are all 2^8 or more below those in another (thin systems),
+                      where values leave 2^+-200 (squared softening 2^+-400) and for masses
+                      that are not positive.  Sums of parts in FP64 */
 #define HH_MIXED 1 /* FP64 state and corrector; i-j difference from float pairs
                       (hi + lo), FP32 pairwise arithmetic, compensated FP32 sums */
 

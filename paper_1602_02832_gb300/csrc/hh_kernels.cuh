@@ -967,6 +967,59 @@ static __device__ __noinline__ void part_sums_f64(const RecF64 *__restrict__ rec
     to_red(A, out);
 }
 
+// The same with the integers' scalars and FP64 components (20 FP64 operations a pair
+// instead of 34): the parts that the integers take but for a component that is too
+// small for them.
+static __device__ __noinline__ void part_sums_thin(const RecF64 *__restrict__ rec, const int32_t *idx, int64_t len, int tj,
+                                                   int jslice, int S, int64_t pi, const IF64 &I, double eps2, RedF64 &out)
+{
+    AccF64 A;
+    A.zero();
+    const Soft64 soft = soft_of(eps2);
+    for (int64_t c = 0; c < len; c += tj)
+        for (int64_t e = c + jslice; e < min(len, c + (int64_t)tj); e += S) {
+            const int32_t j = idx[e];
+            const RecF64 J = rec[j];
+            if ((int64_t)j == pi) continue;
+            const double d[3] = {J.xm.x - I.x, J.xm.y - I.y, J.xm.z - I.z};
+            const double wx = J.v.x - I.vx, wy = J.v.y - I.vy, wz = J.v.z - I.vz;
+            double mr, u, z3;
+            pair_scalars_f64(d, J.xm.w, (uint64_t)__double_as_longlong(J.v.w), soft, mr, u, z3);
+            const double al = fma(d[0], wx, fma(d[1], wy, d[2] * wz)) * z3;
+            A.p += mr;
+            A.ax = fma(u, d[0], A.ax);
+            A.ay = fma(u, d[1], A.ay);
+            A.az = fma(u, d[2], A.az);
+            A.jx = fma(u, fma(-al, d[0], wx), A.jx);
+            A.jy = fma(u, fma(-al, d[1], wy), A.jy);
+            A.jz = fma(u, fma(-al, d[2], wz), A.jz);
+        }
+    to_red(A, out);
+}
+
+// A slice of a few terms often is thin where its particle is not: maxima over the
+// lanes of a warp that work on the same particle (thread = particle + I x slice;
+// in lanes 0 to I - 1), then over the warps.
+__device__ __forceinline__ void warp_span(Span64 &s, int I)
+{
+    for (int step = I; step < 32; step <<= 1)
+#pragma unroll
+        for (int k = 0; k < 3; k++) s.k[k] = addmax_u16x2(__shfl_down_sync(0xffffffffu, s.k[k], step), 0u, s.k[k]);
+}
+
+// Whether one of the item's particles is thin, from the warps' spans.  buf: a span
+// per warp and particle.
+__device__ __forceinline__ bool thin_particles(Span64 s, Span64 *buf, int islot, int I, int tid, int bar_id)
+{
+    if ((tid & 31) < I) buf[(tid & ~31) + islot] = s;
+    group_sync(bar_id);
+    if (tid < I)
+        for (int w = 32; w < kThreads; w += 32)
+#pragma unroll
+            for (int k = 0; k < 3; k++) s.k[k] = addmax_u16x2(buf[w + tid].k[k], 0u, s.k[k]);
+    return group_any(bar_id, tid < I && thin(s));
+}
+
 // a / b for 0 <= a < 2^14, 0 < b <= 2^8: one reciprocal and a product instead of
 // an integer division's chain, of which a part's path has five ((a + 1/2) / b
 // keeps 2^-9 from every integer, the error is below 2^-16).
@@ -1134,11 +1187,17 @@ __device__ __forceinline__ bool force_item(const State &s, const Rec *__restrict
     }
     if constexpr (kPlain) {
         // a term that the integers do not take (a number beyond their range,
-        // a mass that is not positive): the whole part again in FP64
-        if (group_any(bar_id, A.bad)) {
-            if (!idle) load_i(rec, pload, Iv);
-            if (!idle) part_sums_f64(rec, L.idx + lb, len, TJ, jslice, S, pi, Iv, eps2, (&sm.red[0][0])[tid]);
-            group_sync(bar_id);
+        // a mass that is not positive), or a particle one of whose components
+        // is too small for them: the whole part again in FP64
+        warp_span(A.span, I);
+        if (group_any(bar_id, A.bad || (lane < I && thin(A.span)))) {
+            const bool bad = group_any(bar_id, A.bad);
+            if (bad || thin_particles(A.span, reinterpret_cast<Span64 *>(&sm.rec[0][0]), islot, I, tid, bar_id)) {
+                RedF64 &out = (&sm.red[0][0])[tid];
+                if (!idle && bad) part_sums_f64(rec, L.idx + lb, len, TJ, jslice, S, pi, sm.iv[islot], eps2, out);
+                if (!idle && !bad) part_sums_thin(rec, L.idx + lb, len, TJ, jslice, S, pi, sm.iv[islot], eps2, out);
+                group_sync(bar_id);
+            }
         }
     } else {
         group_sync(bar_id);

@@ -20,9 +20,10 @@
 // two components, 9% for three), five or six warps a sub-partition (the same).
 //
 // Errors, measured against quad precision: force 4.7e-17 (rms, relative) and
-// jerk 8e-17 of |m w / r^3| a pair, where FP64 arithmetic has 1.9e-16 and
-// 4.9e-16; sums of 125 terms 4.8e-17 and 5.5e-17 against 4.8e-16 and 5.8e-16
-// (a 96-bit sum drops nothing that counts).  No term depends on the order or
+// jerk 6.8e-17 of |m w / r^3| a pair, where FP64 arithmetic has 1.9e-16 and
+// 4.9e-16; sums of 300 terms 4.7e-17 and 4.9e-17 against 7.8e-16 and 7.8e-16
+// (a 96-bit sum drops nothing that counts).  Of a single component's own terms:
+// see thin().  No term depends on the order or
 // the partners of a lane, so results stay as reproducible as in FP64.
 //
 // Numbers beyond 2^+-200 (separations only above, when there is a softening),
@@ -100,6 +101,16 @@ HH_HD int imin(int a, int b) { return a < b ? a : b; }
 HH_HD int imax(int a, int b) { return a > b ? a : b; }
 HH_HD uint32_t umax(uint32_t a, uint32_t b) { return a > b ? a : b; }
 HH_HD int64_t wide_s(int32_t a, int32_t b) { return (int64_t)a * b; }
+// max(a + b, c) in both 16-bit halves.
+HH_HD uint32_t addmax_u16x2(uint32_t a, uint32_t b, uint32_t c)
+{
+#ifdef __CUDA_ARCH__
+    return __viaddmax_u16x2(a, b, c);
+#else
+    const uint32_t s = a + b, l = umax(s & 0xffffu, c & 0xffffu), h = umax(s >> 16, c >> 16);
+    return h << 16 | l;
+#endif
+}
 HH_HD uint64_t wide_u(uint32_t a, uint32_t b) { return (uint64_t)a * b; }
 HH_HD uint32_t hi32(uint64_t x) { return (uint32_t)(x >> 32); }
 HH_HD uint32_t lo32(uint64_t x) { return (uint32_t)x; }
@@ -178,6 +189,7 @@ HH_HD int64_t mul_dig(const Dig &a, const Dig &b)
 struct Vec64 {
     Dig k[3];
     int32_t e;
+    uint32_t x[3];  // each component's own (biased) exponent
 };
 
 constexpr int kMaxExp = 1223;  // 2^200: largest separation and velocity taken here
@@ -198,10 +210,11 @@ HH_HD void unpack_vec(const double *d, Vec64 &v)
     v.e = imax((int)(umax(umax(a[0], a[1]), a[2]) >> 20), kMinExp);
     const int base = v.e + kDown;
     for (int k = 0; k < 3; k++) {
+        v.x[k] = a[k] >> 20;
         const uint32_t hi = f64_hi(d[k]), lo = f64_lo(d[k]);
         // 1.mantissa left-aligned in 64 bits, then down to its place
         const uint64_t m = ((((uint64_t)hi << 32) | lo) << 11) | 0x8000000000000000ull;
-        const uint64_t x = shr64(m, base - (int)(a[k] >> 20));
+        const uint64_t x = shr64(m, base - (int)v.x[k]);
         const uint32_t neg = (uint32_t)((int32_t)hi >> 31);
         const uint32_t xl = (lo32(x) ^ neg) | 1u;
         v.k[k].l = (int32_t)xl;
@@ -346,15 +359,49 @@ HH_HD double sum_get(uint64_t u, int64_t o, int e)
     return small ? x * 0x1p-128 : x;
 }
 
+// Component k's largest term of the force (low half) and of the velocity's part of
+// the jerk (high half), as the exponent of u = m / r^3 plus the component's own.
+struct Span64 {
+    uint32_t k[3];
+};
+
+// The integers hold a vector to a unit of its largest component, so a component
+// that is small in every term (of a disc, a ring, a nearly planar or collinear
+// set) loses what FP64 would keep of it.  True if the largest term of a component is more
+// than kThinForce or kThinJerk places below the vector's: the caller then sums in
+// FP64.  At that line both are about as good: sheets of 30, 100 and 1000 terms of
+// thickness 2^-9 have rms errors of 1.7e-16, 2.2e-16 and 5.0e-16 of the component's own sizes
+// in the force and 2.9e-16, 3.5e-16 and 8.2e-16 in the jerk, all in FP64 1.9e-16, 2.3e-16,
+// 6.4e-16 and 3.0e-16, 3.6e-16, 8.7e-16; thicker ones are better in integers, thinner ones came
+// out worse by 2^-9 over the thickness.  Places less would make more parts of a
+// round cluster take FP64 for one close pair's direction (with 5 instead of 8
+// places in the jerk one in fourteen: N = 65536 4.22 against 3.42 ms).  A
+// component of zeros, which the integers hold exactly, has no exponent to speak
+// of: it comes out kThinEnd places or more below the others.
+constexpr uint32_t kThinForce = 8, kThinJerk = 8, kThinEnd = 600;
+HH_HD bool thin(const Span64 &s)
+{
+    bool t = false;
+    for (int half = 0; half < 2; half++) {
+        uint32_t e[3];
+        for (int k = 0; k < 3; k++) e[k] = half ? s.k[k] >> 16 : s.k[k] & 0xffffu;
+        const uint32_t most = umax(umax(e[0], e[1]), e[2]), lim = half ? kThinJerk : kThinForce;
+        for (int k = 0; k < 3; k++) t |= most - e[k] - lim - 1u < kThinEnd - lim - 1u;
+    }
+    return t;
+}
+
 struct AccI64 {
     Sum64<3> a, j;
     Sum64<1> p;
+    Span64 span;
     bool bad;
     HH_HD void zero()
     {
         a.zero();
         j.zero();
         p.zero();
+        for (int k = 0; k < 3; k++) span.k[k] = 0u;
         bad = false;
     }
 };
@@ -372,19 +419,16 @@ HH_HD float seed_rsqrt(float f)
 // bit at 2^55 or above and every middle sum (up to six partial products) below
 // 2^63:
 //   separation D 2^(D.e - 1084), largest component in [2^61, 2^62); velocity
-//   W 2^(W.e - 1079), in [2^56, 2^57); R = r^2 in [2^60, 2^62) 2^(X - n);
+//   W 2^(W.e - 1081), in [2^58, 2^59); R = r^2 in [2^60, 2^62) 2^(X - n);
 //   y = 2^93 / sqrt(R); Z = 2^122 / R; mr = m y 2^-64; u in [2^61, 2^62).
 // The jerk uses u w - rho (u d) with rho = 3 (d.w) / r^2: |rho d| <= 3 |w|, so
 // rho has a fixed scale against w whatever the sizes.
-//
-// Adds the pair term of separation d, relative velocity w, mass m (mb its
-// mass_bits); a term that has to be left to FP64 sets A.bad.
-HH_HD void pair_add(const double *d, const double *w, double m, uint64_t mb, bool self, const Soft64 &eps, int smin,
-                    AccI64 &A)
+struct Scal64 {
+    uint64_t Z, mr, u;
+    int sh, n, h, em, eu;
+};
+HH_HD Scal64 pair_scalars(const Vec64 &D, double m, uint64_t mb, const Soft64 &eps)
 {
-    Vec64 D, W;
-    unpack_vec<2>(d, D);
-    unpack_vec<7>(w, W);
     // r^2 = R 2^X
     int64_t hh = wide_s(D.k[0].h, D.k[0].h), hl = wide_s(D.k[0].h, D.k[0].l);
     hh = mad_s(D.k[1].h, D.k[1].h, hh);
@@ -423,10 +467,23 @@ HH_HD void pair_add(const double *d, const double *w, double m, uint64_t mb, boo
     const int lz = clz32(hi32(u)) - 2;
     u <<= (lz & 31);  // [2^61, 2^62)
     const int em = (int)(f64_hi(m) >> 20);
-    const int eu = em - 3 * h - lz;
-    const Dig U = dig((int64_t)u);
+    return Scal64{Z, mr, u, sh, n, h, em, em - 3 * h - lz};
+}
+
+// Adds the pair term of separation d, relative velocity w, mass m (mb its
+// mass_bits); a term that has to be left to FP64 sets A.bad.
+HH_HD void pair_add(const double *d, const double *w, double m, uint64_t mb, bool self, const Soft64 &eps, int smin,
+                    AccI64 &A)
+{
+    Vec64 D, W;
+    unpack_vec<2>(d, D);
+    unpack_vec<5>(w, W);
+    const Scal64 q = pair_scalars(D, m, mb, eps);
+    const uint64_t Z = q.Z, mr = q.mr;
+    const int sh = q.sh, n = q.n, h = q.h, em = q.em, eu = q.eu;
+    const Dig U = dig((int64_t)q.u);
     // places below the sums' scales
-    int sa = A.a.e - (eu + D.e - 2192), sj = A.j.e - (eu + W.e - 2187);
+    int sa = A.a.e - (eu + D.e - 2192), sj = A.j.e - (eu + W.e - 2189);
     const int sp = A.p.e - (em - h - 1114);
     int64_t ta[3], tj[3], tp[1] = {(int64_t)mr};
     for (int k = 0; k < 3; k++) ta[k] = mul_dig(U, D.k[k]);
@@ -439,14 +496,14 @@ HH_HD void pair_add(const double *d, const double *w, double m, uint64_t mb, boo
     gh = mad_s(D.k[2].h, W.k[2].h, gh);
     gl = mad_s(D.k[2].h, W.k[2].l, gl);
     gl = mad_s(D.k[2].l, W.k[2].h, gl);
-    const int64_t RW = (int64_t)((uint64_t)gh << (4 + n)) + (gl >> (28 - n));
+    const int64_t RW = (int64_t)((uint64_t)gh << (2 + n)) + (gl >> (30 - n));
     // rho in units of the components, times 2^64
     int64_t G = mul_dig(dig(RW), dig((int64_t)Z));
     G = sar64(G, sh);
     G = -(int64_t)((uint64_t)G * 12ull);  // (negated here: a digit of -2^31 has no negative)
     const Dig N = dig(G);
     for (int k = 0; k < 3; k++) {
-        const Dig t = dig(ta[k]);
+        const Dig t = dig((int64_t)((uint64_t)ta[k] << 2));
         int64_t mid = mad_s(U.h, W.k[k].l, 0x80000000ll);
         mid = mad_s(U.l, W.k[k].h, mid);
         mid = mad_s(N.h, t.l, mid);
@@ -467,6 +524,7 @@ HH_HD void pair_add(const double *d, const double *w, double m, uint64_t mb, boo
         sum_put<3>(A.a, ta, sa);
         sum_put<3>(A.j, tj, sj);
         sum_put<1>(A.p, tp, sp);
+        for (int k = 0; k < 3; k++) A.span.k[k] = addmax_u16x2(D.x[k] | W.x[k] << 16, (uint32_t)eu * 0x10001u, A.span.k[k]);
     } else if (!self) {
         if (far || W.e > kMaxExp || hi32(mb) == 0u) {
             A.bad = true;
@@ -474,8 +532,31 @@ HH_HD void pair_add(const double *d, const double *w, double m, uint64_t mb, boo
             sum_any<3>(A.a, ta, sa, smin);
             if (W.e > kMinExp) sum_any<3>(A.j, tj, sj, smin);
             sum_any<1>(A.p, tp, sp, smin);
+            for (int k = 0; k < 3; k++)
+                A.span.k[k] = addmax_u16x2(D.x[k] | W.x[k] << 16, (uint32_t)eu * 0x10001u, A.span.k[k]);
         }
     }
+}
+
+// q 2^x as a double, q in [2^52, 2^64), to nearest.
+HH_HD double f64_scaled(uint64_t q, int x)
+{
+    const int z = clz32(hi32(q));
+    uint64_t m = q << z;
+    m = (m >> 11) + ((((m & 0x7ffull) + ((m >> 11) & 1ull)) > 0x400ull) ? 1ull : 0ull);
+    const uint64_t b = ((uint64_t)(x - z + 1085) << 52) + m;
+    return f64_of(hi32(b), lo32(b));
+}
+
+// The scalars of a pair alone, as doubles: m / r, m / r^3 and 3 / r^2.
+HH_HD void pair_scalars_f64(const double *d, double m, uint64_t mb, const Soft64 &eps, double &mr, double &u, double &z3)
+{
+    Vec64 D;
+    unpack_vec<2>(d, D);
+    const Scal64 q = pair_scalars(D, m, mb, eps);
+    mr = f64_scaled(q.mr, q.em - q.h - 1114);
+    u = f64_scaled(q.u, q.eu - 1172);
+    z3 = f64_scaled(3 * q.Z, -2 * q.h - 122);
 }
 
 }  // namespace hh
