@@ -186,7 +186,12 @@ int hh_predict(hh_ctx *ctx, double t);
  * hh_predict, each particle summing over its group's list and skipping its
  * own entry.  Outputs host SoA acc[3][n_act], jerk[3][n_act], pot[n_act]
  * (any of them may be NULL).  The results also stay on the device for
- * hh_correct.  hh_force_dev takes device arrays (i_idx included) used on the
+ * hh_correct.  A particle's sums are rounded in an order that depends on its
+ * list, on how many particles of its tile are in i_idx, on the configuration's
+ * list parts and, in the plain form, on n_act: large evaluations (from about
+ * 10^4 parts of tile_j on) take parts of two or four times tile_j, so that a
+ * particle's result may differ from hh_step's, or from a small evaluation's, in
+ * the last bits.  The same call gives the same bits.  hh_force_dev takes device arrays (i_idx included) used on the
  * context's stream.  Errors: HH_ESTATE without lists, or when the j
  * entries, lists or particle state changed (hh_set_j, hh_set_lists,
  * hh_correct, hh_advance, hh_rebuild, a batch run) after the last

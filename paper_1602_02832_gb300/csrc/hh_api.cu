@@ -317,17 +317,21 @@ int ensure_graph(hh_ctx *ctx)
 
 // List parts of an explicit evaluation in the plain form: tile_j entries, or
 // two or four times that where the evaluation has eight parts of that length
-// for every group that works on them all the same (a part's start and end cost
-// about six of its thread's pairs, tile_j = 256 entries of a tile of 14 are 28:
-// N = 65536 takes 3.23 ms against 3.37 ms; four or two parts per group, or up to
-// eight times tile_j: the same).  The mixed form's sums follow its parts, which stay.
+// for every group of a GB300 that works on them all the same (a part's start and
+// end cost about six of its thread's pairs, tile_j = 256 entries of a tile of 14
+// are 28: N = 65536 takes 3.23 ms against 3.37 ms; four or two parts per group, or
+// up to eight times tile_j: the same).  The mixed form's sums follow its parts,
+// which stay.  (A constant number of groups, so that results do not follow the
+// SMs of the device at hand.)
+constexpr double kPartGroups = 608.0;
+
 int part_shift(const hh_ctx *ctx, int32_t n_act)
 {
     if (ctx->cfg.precision != HH_FP64 || ctx->n_groups < 1) return 0;
     const double tiles = std::min(n_act, ctx->n_tiles);
     const double parts = tiles * (double(ctx->list_len) / ctx->n_groups) / ctx->part_len;
     int shift = 0;
-    while (shift < 2 && parts >= 8.0 * ctx->force_grid * (2 << shift)) shift++;
+    while (shift < 2 && parts >= 8.0 * kPartGroups * (2 << shift)) shift++;
     return shift;
 }
 

@@ -860,8 +860,9 @@ __device__ __forceinline__ void fold_chunk(AccMix &A) { A.fold(); }
 // into several parts leaves per-part sums in the partials buffer; the group
 // that finishes a tile's last part (acquire-release arrival counter: no
 // waiting) adds the parts in part order.  So each particle's result depends
-// only on its list, its tile's active count and the part length, never on
-// scheduling.
+// only on its list, its tile's active count and the part length (which follows
+// the configuration and, in the plain form's large evaluations and steps, the
+// number of active particles), never on scheduling.
 // Asynchronous global -> shared copies (16 B each) for chunk staging,
 // cached in L1: the 16-byte pieces of one record, and the records of
 // neighbouring list entries (consecutive particles of a leaf, sibling
