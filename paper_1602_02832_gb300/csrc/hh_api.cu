@@ -768,7 +768,6 @@ int set_lists_core(hh_ctx *ctx, int64_t n_particles, int64_t n_j, int32_t n_grou
     ctx->n_tiles = int32_t(tiles.size());
     ctx->total_parts = total_parts;
     ctx->small_parts = small_parts;
-    ctx->h_group_of.assign(group_of, group_of + n_particles);
     if (int64_t(ctx->ids.size()) != n_particles) {
         ctx->ids.resize(size_t(n_particles));
         for (int64_t q = 0; q < n_particles; q++) ctx->ids[size_t(q)] = q;

@@ -101,7 +101,6 @@ struct hh_ctx {
     bool ids_on_device = false;  // particle ids kept by the device builder (the host's are old)
     bool ids_on_both = false;    // the builder's ids and the host's are the same
     std::vector<int64_t> ids;  // slot -> particle id
-    std::vector<int32_t> h_group_of;
     // grid shapes
     int n_sm = 0, force_grid = 0, elem_grid = 0;
     LoopBuf *loop = nullptr;   // buffers of the persistent loop (first hh_advance)

@@ -54,8 +54,6 @@ __device__ __forceinline__ uint64_t spread_bits(uint32_t v)
     return x;
 }
 
-__device__ __forceinline__ int digit_at(uint64_t key, int depth) { return int((key >> (3 * (kBits - 1 - depth))) & 7u); }
-
 // Peano-Hilbert key of a cell of the 2^21 grid (Skilling 2004): the low bit
 // fields are mapped level by level into each sub-cube's frame, Gray-coded,
 // and the resulting transposed index is interleaved like a Morton key.

@@ -300,15 +300,6 @@ __device__ __forceinline__ void predict_xv(double D, double x, double v, double 
     vp = v + D * (a + h * j);
 }
 
-__device__ __forceinline__ void predict_one(const State &s, int64_t e, double tnow, double xp[3], double vp[3])
-{
-    const double D = tnow - s.t[e];
-#pragma unroll
-    for (int d = 0; d < 3; d++)
-        predict_xv(D, s.x[d * s.cap_j + e], s.v[d * s.cap_j + e], s.a[d * s.cap_j + e], s.jk[d * s.cap_j + e], xp[d],
-                   vp[d]);
-}
-
 template <typename Rec>
 __device__ __forceinline__ void store_rec(Rec *out, int64_t e, const double xp[3], const double vp[3], double m);
 
@@ -455,7 +446,7 @@ __device__ __forceinline__ RecMix mix_from_base(const BaseMix &b, float D, int64
 
 // Inputs of one entry's prediction, loaded ahead of its arithmetic so that a
 // thread can keep several entries' loads in flight (pred_load, then
-// pred_store: the same arithmetic as predict_one / mix_from_base).
+// pred_store).
 template <typename Rec>
 struct PredIn;
 template <>
@@ -718,17 +709,6 @@ __device__ __forceinline__ void interact(const IMix &I, const RecMix &J, bool se
 }
 
 // ---------------------------------------------- cross-slice reductions
-__device__ __forceinline__ void acc_shfl_add(AccF64 &A, int off)
-{
-    A.ax += __shfl_xor_sync(0xffffffffu, A.ax, off);
-    A.ay += __shfl_xor_sync(0xffffffffu, A.ay, off);
-    A.az += __shfl_xor_sync(0xffffffffu, A.az, off);
-    A.jx += __shfl_xor_sync(0xffffffffu, A.jx, off);
-    A.jy += __shfl_xor_sync(0xffffffffu, A.jy, off);
-    A.jz += __shfl_xor_sync(0xffffffffu, A.jz, off);
-    A.p += __shfl_xor_sync(0xffffffffu, A.p, off);
-}
-
 __device__ __forceinline__ F2 f2_shfl(F2 a, int off)
 {
     F2 b;
@@ -748,23 +728,6 @@ __device__ __forceinline__ void acc_shfl_add(AccMix &A, int off)
 // Adds the partner's sums (lane + delta) into this lane's where `take`; every
 // lane takes part in the shuffles.  The receiving lane's sums come first, so
 // the order of every addition is fixed.
-__device__ __forceinline__ double shfl_down_take(double x, int delta, bool take)
-{
-    const double o = __shfl_down_sync(0xffffffffu, x, delta);
-    return take ? x + o : x;
-}
-
-__device__ __forceinline__ void acc_shfl_down_add(AccF64 &A, int delta, bool take)
-{
-    A.ax = shfl_down_take(A.ax, delta, take);
-    A.ay = shfl_down_take(A.ay, delta, take);
-    A.az = shfl_down_take(A.az, delta, take);
-    A.jx = shfl_down_take(A.jx, delta, take);
-    A.jy = shfl_down_take(A.jy, delta, take);
-    A.jz = shfl_down_take(A.jz, delta, take);
-    A.p = shfl_down_take(A.p, delta, take);
-}
-
 __device__ __forceinline__ F2 f2_shfl_down_take(F2 a, int delta, bool take)
 {
     F2 o;
@@ -808,8 +771,6 @@ __device__ __forceinline__ void to_red(const AccMix &A, RedMix &r)
 {
     r.v[0] = A.Ax; r.v[1] = A.Ay; r.v[2] = A.Az; r.v[3] = A.Jx; r.v[4] = A.Jy; r.v[5] = A.Jz; r.v[6] = A.P;
 }
-__device__ __forceinline__ double red_get(const RedF64 &r, int q) { return r.v[q]; }
-__device__ __forceinline__ double red_get(const RedMix &r, int q) { return (double)r.v[q].h + (double)r.v[q].l; }
 // partial sums written by other CTAs are read through L2 (bypassing L1)
 // One component of a reduction record (double, or an FP32 pair).
 __device__ __forceinline__ double shfl_down_e(double v, int d) { return __shfl_down_sync(0xffffffffu, v, d); }
@@ -1023,7 +984,8 @@ __device__ __forceinline__ bool thin_particles(Span64 s, Span64 *buf, int islot,
 
 // a / b for 0 <= a < 2^14, 0 < b <= 2^8: one reciprocal and a product instead of
 // an integer division's chain, of which a part's path has five ((a + 1/2) / b
-// keeps 2^-9 from every integer, the error is below 2^-16).
+// is at least 1 / (2 b) from every integer, and the quotient's error, two units of
+// FP32, at most (a + 1/2) / b 2^-22: less as long as a < 2^20).
 __device__ __forceinline__ int small_div(int a, int b) { return (int)__fdividef((float)a + 0.5f, (float)b); }
 
 // item = (tile, part | sim << 16, active mask, parts of the tile); tid is

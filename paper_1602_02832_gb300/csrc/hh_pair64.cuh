@@ -97,7 +97,6 @@ HH_HD int clz32(uint32_t a)
     return a ? __builtin_clz(a) : 32;
 #endif
 }
-HH_HD int imin(int a, int b) { return a < b ? a : b; }
 HH_HD int imax(int a, int b) { return a > b ? a : b; }
 HH_HD uint32_t umax(uint32_t a, uint32_t b) { return a > b ? a : b; }
 HH_HD int64_t wide_s(int32_t a, int32_t b) { return (int64_t)a * b; }
@@ -276,12 +275,13 @@ struct Sum64 {
     }
 };
 
-// Where a sum puts its first term (and one too large for it): 24 places below
-// the top of the window leave 2^16 and more of room for larger ones, so that a
-// thread's terms rarely move the scale (a move costs as much as a pair, and one
-// lane's move holds up its warp; with 4 places of room instead of about 18 an
+// Where a sum puts its first term (and one too large for it): 24 places below the
+// top of the window leave room for terms 2^(24 - smin) larger, so that a thread's
+// terms rarely move the scale (a move costs as much as a pair, and one lane's
+// move holds up its warp; with 4 places of room instead of about 18 an
 // evaluation of N = 65536 took 3.53 ms against 3.41 ms), and 8 bits below the first
-// term's last one for smaller ones.
+// term's last one for smaller ones.  (smin is 5 for 256 entries of a tile of 14, 7
+// for 1024: 2^19 and 2^17; the least room is 2^14, 2048 entries of a full tile.)
 constexpr int kPlace = 24;
 
 // sum += t 2^(e - s), smin <= s <= 32 (smin: the bits of the number of terms, at least 2)
