@@ -164,6 +164,13 @@ __device__ __forceinline__ const RbSim &rb_sim_of(const RbSim &one, const RbSim 
 }
 #define RB_SIM                                                      \
     after_previous();                                               \
+    RB_RECORD
+// (in front of a CUB call: its kernels are placed when this one has ended, as
+// they expect of a kernel that knows nothing of dependent launches)
+#define RB_SIM_BEFORE_CUB                                           \
+    wait_previous();                                                \
+    RB_RECORD
+#define RB_RECORD                                                   \
     __shared__ __align__(16) unsigned char rb_rec_[sizeof(RbSim)]; \
     const RbSim &a = rb_sim_of<kMany>(one, many, rb_rec_)
 
@@ -230,7 +237,7 @@ __global__ void k_box(RB_ARGS)
 template <bool kMany>
 __global__ void k_keys(RB_ARGS)
 {
-    RB_SIM;
+    RB_SIM_BEFORE_CUB;
     const State &s = a.st;
     const Box *b = a.box;
     double lo[3], side = 0.0;
@@ -319,7 +326,7 @@ __device__ __forceinline__ bool more_than(const uint64_t *key, int64_t n, int64_
 template <bool kMany>
 __global__ void k_chains(RB_ARGS)
 {
-    RB_SIM;
+    RB_SIM_BEFORE_CUB;
     const uint64_t *key = a.key2;
     if (blockIdx.x == 0 && threadIdx.x == 0) a.cnt[a.n] = 0;  // terminal entry of the scan
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -740,7 +747,9 @@ __global__ void k_paths(RB_ARGS)
 template <bool kMany, bool kWrite>
 __global__ void __launch_bounds__(kWalkThreads) k_lists(RB_ARGS)
 {
-    RB_SIM;
+    if (kWrite) after_previous();
+    else wait_previous();  // (the scan follows)
+    RB_RECORD;
     __shared__ CellRec s_cell[kWalkStage];
     const int32_t R = a.R, n_row = (a.G + kWalkThreads - 1) / kWalkThreads;
     const int64_t n = a.n;
@@ -812,7 +821,7 @@ __global__ void __launch_bounds__(kWalkThreads) k_lists(RB_ARGS)
 template <bool kMany>
 __global__ void k_tile_counts(RB_ARGS)
 {
-    RB_SIM;
+    RB_SIM_BEFORE_CUB;
     const int32_t G = a.G, R = a.R;
     const int64_t *scan_p = a.pscan2, *scan_n = a.pscan2 + a.pairs + 1;
     const int64_t base = scan_p[0] + scan_n[0];
