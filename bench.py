@@ -803,6 +803,38 @@ def _cpu_baseline(a, state, cfg3=None):
     return out
 
 
+# sections of the record beside the contract's keys, and what the printed line keeps of each
+SHORT = {"roofline": ("kernel", "bound", "achieved", "peak", "unit", "frac", "traffic"),
+         "cpu_baseline": ("value", "unit", "cores", "kind"),
+         "mixed": ("value", "block_steps_per_s", "ms_per_step", "speedup_vs_plain"),
+         "config3": ("value", "equiv_tflops", "run_s", "device_gb"),
+         "batched": ("clusters", "wall_s", "block_steps_per_s", "interactions_per_s"),
+         "serving": ("requests_arrived", "completed", "block_steps_per_s"),
+         "serving_sustained": ("requests_arrived", "completed", "block_steps_per_s")}
+
+
+def short_line(line):
+    """The line for standard output: the contract's keys as they are, a few figures (6 digits) of every other section,
+    latencies as p50 and p99.  Below 3 KB, so that a log's tail holds it; the whole record goes to standard error."""
+    def figure(v):
+        return float(f"{v:.6g}") if isinstance(v, float) else v
+
+    def latency(d):
+        return {k: {w: figure(u[w]) for w in ("p50", "p99")} for k, u in d.items() if isinstance(u, dict) and "p50" in u}
+
+    out = {}
+    for k, v in line.items():
+        if k in ("config", "e2e", "clocks") or not isinstance(v, (dict, list)):
+            out[k] = v
+        elif k in SHORT:
+            out[k] = {**{q: figure(v[q]) for q in SHORT[k] if q in v}, **latency(v)}
+        elif k == "block_step_latency_us":
+            out.update(latency({k: v}))
+        elif k == "config1":
+            out[k] = {q: figure(u["interactions_per_s"]) for q, u in v.items() if isinstance(u, dict)}
+    return out
+
+
 def main_reference(a):
     """The FP64 oracle as the reference arm, on the host cores: the same
     workload run from t = 0 to the start of the GPU arm's timed window (W
@@ -979,7 +1011,8 @@ def main():
         line["clocks"] = clk.summary()
         if cpu:
             line["cpu_baseline"] = cpu
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(short_line(line)), flush=True)
     if world > 1:
         dist.barrier()
         dist.destroy_process_group()
