@@ -10,10 +10,10 @@
 // separation, the relative velocity and every scalar as 64-bit numbers in two
 // signed 32-bit digits, the sums in 96 bits with an exponent of their own.
 // A micro-benchmark of the pair loop (4 warps per sub-partition, records in
-// shared memory) went from 2280 to 650 cycles a warp and pair; one evaluation of
-// N = 65536 particles (theta 0.5 lists) from 11.5 to 3.95 ms, a tree interval of
-// its block steps from 90.8 to 55.6 ms.  What bounds it now is the integer
-// multiply-add pipe (71% busy; the ALU pipe 61%, FP64 59%, issue 58%) and the
+// shared memory) went from 2280 to 690 cycles a warp and pair; one evaluation of
+// N = 65536 particles (theta 0.5 lists) from 11.5 to 3.34 ms, a tree interval of
+// its block steps from 90.8 to 49.9 ms.  What bounds it now is the integer
+// multiply-add pipe (70% busy; the ALU pipe 61%, FP64 56%, issue 58%) and the
 // latency of its chains with 4 warps a sub-partition.  Taken back: the next
 // pair's differences one iteration ahead (its registers: 6% slower), unpacking
 // by FP64-to-integer conversions (64 cycles each on the FP64 pipe: 1% slower for
